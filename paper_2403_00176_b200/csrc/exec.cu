@@ -933,10 +933,10 @@ struct Builder {
       k::ChainBatch cb;
       std::vector<Ptr> base;      // per operand: pointer of the table's first request
       Ptr out;
-      bool vec = true;            // every request qualifies for the 8-wide kernel
-      bool vec16 = true;          // ... and has a last extent that is a multiple of 16
+      bool out_vec = true;        // every request's output starts on a 16-byte boundary relative to the first's
       int max_cols = 0;
     };
+    const int64_t tile = 256 * k::CHAIN_NV * (proto.out_bf16 ? 8 : 4);     // outputs per CTA of chain_elementwise
     auto fresh = [&]() { Pending q; q.cb = proto; q.base.assign(1 + k::CHAIN_MAX_OPS, Ptr()); return q; };
     Pending cur = fresh();
     auto flush = [&]() {
@@ -950,18 +950,17 @@ struct Builder {
         cb.out = x.resolve(q.out);
         if (red == 2) { cb.gamma = x.resolve(pg); cb.beta = x.resolve(pb); }
         if (!red) {
-          const unsigned grid = static_cast<unsigned>(std::max<long long>(1, std::min<long long>((cb.total + 255) / 256, 148 * 32)));
-          if (q.vec && q.vec16) {
-            // two vectors per item: the table was filled in units of 8 elements
-            for (int i = 0; i < cb.n_req; ++i) cb.r[i].first /= 2;
-            cb.total /= 2;
-            const unsigned g16 = static_cast<unsigned>(std::max<long long>(1, std::min<long long>((cb.total + 255) / 256, 148 * 32)));
-            k::chain_elementwise_vec<2><<<g16, 256, 0, x.stream>>>(cb);
-            for (int i = 0; i < cb.n_req; ++i) cb.r[i].first *= 2;
-            cb.total *= 2;
-          } else if (q.vec) k::chain_elementwise_vec<1><<<grid, 256, 0, x.stream>>>(cb);
-          else k::chain_elementwise<<<grid, 256, 0, x.stream>>>(cb);
-        } else if (q.max_cols <= k::ROWRED_WARP_COLS) {
+          // an item reads and writes 16-byte vectors: a caller's buffer that is not 16-byte aligned is read (written)
+          // one element at a time
+          cb.vec_ok = q.out_vec && (reinterpret_cast<uintptr_t>(cb.out) & 15) == 0;
+          for (int kx = 0; kx <= k::CHAIN_MAX_OPS; ++kx)
+            if (has_ptr[kx] && (reinterpret_cast<uintptr_t>(cb.base[kx]) & 15))
+              for (int i = 0; i < cb.n_req; ++i) if (cb.r[i].cls[kx] == k::CC_FLAT || cb.r[i].cls[kx] == k::CC_VEC) cb.vec_ok = 0;
+          const dim3 grid(static_cast<unsigned>(cb.total));
+          return cb.out_bf16 ? launch_pdl(k::chain_elementwise<true>, grid, dim3(256), 0, x.stream, cb)
+                             : launch_pdl(k::chain_elementwise<false>, grid, dim3(256), 0, x.stream, cb);
+        }
+        if (q.max_cols <= k::ROWRED_WARP_COLS) {
           const size_t smem = static_cast<size_t>(q.max_cols) * 4 * 8;
           if (smem > 48 * 1024) { static bool once = (cudaFuncSetAttribute(k::chain_rowreduce_warp, cudaFuncAttributeMaxDynamicSharedMemorySize, k::ROWRED_WARP_COLS * 32), true); (void)once; }
           const unsigned grid = static_cast<unsigned>(std::max<long long>(1, std::min<long long>((cb.total + 7) / 8, 148 * 8)));
@@ -984,7 +983,7 @@ struct Builder {
       if (red && od[3] * 4 > 200 * 1024) return fail(E_UNSUPPORTED_OP, "row too long for the row-reduction kernel");
       // this request's operands: pointer, strides (0 on broadcast dims: read in place)
       std::vector<Ptr> ptrs(1 + k::CHAIN_MAX_OPS);
-      int strides[1 + k::CHAIN_MAX_OPS][4] = {};
+      int64_t strides[1 + k::CHAIN_MAX_OPS][4] = {};
       for (int kx = 0; kx <= k::CHAIN_MAX_OPS; ++kx) {
         const int t = opnd[kx];
         if (t < 0 || g.tensors[t].kind == TKind::FCONST) continue;
@@ -995,13 +994,17 @@ struct Builder {
           const int src = i - (4 - rk);
           const int64_t st = (src >= 0 && v.dims[src] != 1) ? v.strides[src] : 0;
           if (st >= (int64_t(1) << 31) || st < 0) return fail(E_UNSUPPORTED_OP, "chain operand stride out of range");
-          strides[kx][i] = static_cast<int>(st);
+          strides[kx][i] = st;
         }
         ptrs[kx] = ptr_of(t, rr);
       }
       Ptr pout = ptr_of(G.out, r);
+      const int64_t total = numel(ov.dims);
+      const long long items = red ? od[0] * od[1] * od[2] : (total + tile - 1) / tile;
+      // flat indices are 32-bit, and a tile may reach past the last element
+      if ((red ? items : total + tile) >= (int64_t(1) << 31)) return fail(E_UNSUPPORTED_OP, "chain request above 2^31 elements");
       // does it fit the open table?
-      bool fits = cur.cb.n_req < k::CHAIN_MAX_REQ;
+      bool fits = cur.cb.n_req < k::CHAIN_MAX_REQ && (red || cur.cb.total + items < (1ll << 31));
       if (fits && cur.cb.n_req) {
         if (!same_base(pout, cur.out)) fits = false;
         for (int kx = 0; kx <= k::CHAIN_MAX_OPS && fits; ++kx)
@@ -1010,37 +1013,53 @@ struct Builder {
       if (!fits) flush();
       if (!cur.cb.n_req) { cur.out = pout; for (int kx = 0; kx <= k::CHAIN_MAX_OPS; ++kx) cur.base[kx] = ptrs[kx]; }
       k::ChainReq& R = cur.cb.r[cur.cb.n_req++];
+      // Collapse dims i and i + 1 where every operand steps through them as through one dim; the merged dim takes
+      // the place of i + 1, the dims in front move right (row reductions keep their last dim).
+      if (!red) {
+        int i = 2;      // candidate; what has been merged so far sits in dim i + 1
+        for (int step = 0; step < 3 && i >= 0; ++step) {
+          bool can = true;
+          if (od[i] != 1 && od[i + 1] != 1)
+            for (int kx = 0; kx <= k::CHAIN_MAX_OPS && can; ++kx)
+              if (has_ptr[kx] && strides[kx][i] != strides[kx][i + 1] * od[i + 1]) can = false;
+          if (!can) { --i; continue; }
+          for (int kx = 0; kx <= k::CHAIN_MAX_OPS; ++kx) {
+            if (od[i + 1] == 1) strides[kx][i + 1] = strides[kx][i];
+            for (int j = i; j > 0; --j) strides[kx][j] = strides[kx][j - 1];
+            strides[kx][0] = 0;
+          }
+          od[i + 1] *= od[i];
+          for (int j = i; j > 0; --j) od[j] = od[j - 1];
+          od[0] = 1;
+        }
+      }
       const int oesz = dtype_size(O.dtype);
       for (int i = 0; i < 4; ++i) R.dim[i] = static_cast<int>(od[i]);
+      R.numel = red ? 0 : static_cast<int>(total);
       R.out_off = (pout.off - cur.out.off) / oesz;
-      bool vec = !red && od[3] % 8 == 0 && R.out_off % 8 == 0 && cur.out.off % 16 == 0;
+      if ((pout.off - cur.out.off) % 16) cur.out_vec = false;
+      R.fast = od[3] * oesz >= 16;
+      R.first_vec = -1;
+      const int64_t flat[4] = {od[1] * od[2] * od[3], od[2] * od[3], od[3], 1};
       for (int kx = 0; kx <= k::CHAIN_MAX_OPS; ++kx) {
         const int t = opnd[kx];
+        R.cls[kx] = k::CC_SCALAR;
         if (t < 0 || g.tensors[t].kind == TKind::FCONST) continue;
         const int esz = dtype_size(g.tensors[t].dtype);
         R.off[kx] = (ptrs[kx].off - cur.base[kx].off) / esz;
-        for (int i = 0; i < 4; ++i) R.stride[kx][i] = strides[kx][i];
-        if (strides[kx][3] == 1 || od[3] == 1) {
-          // read as 8-element vectors: every address a multiple of 16 bytes (32 for fp32 pairs of float4)
-          if (od[3] != 1 && (R.off[kx] % 8 || strides[kx][0] % 8 || strides[kx][1] % 8 || strides[kx][2] % 8 || cur.base[kx].off % 16)) vec = false;
-        } else if (strides[kx][3] != 0) vec = false;
-      }
-      const long long items = red ? od[0] * od[1] * od[2] : (vec && cur.vec ? numel(ov.dims) / 8 : numel(ov.dims));
-      if ((red ? items : numel(ov.dims)) >= (int64_t(1) << 31)) return fail(E_UNSUPPORTED_OP, "chain request above 2^31 elements");
-      if (!red && cur.vec && !vec) {
-        // the table falls back to one element per item: recount the earlier requests
-        long long first = 0;
-        for (int q = 0; q + 1 < cur.cb.n_req; ++q) {
-          cur.cb.r[q].first = first;
-          first += static_cast<long long>(cur.cb.r[q].dim[0]) * cur.cb.r[q].dim[1] * cur.cb.r[q].dim[2] * cur.cb.r[q].dim[3];
-        }
-        cur.cb.total = first;
-        cur.vec = false;
+        for (int i = 0; i < 4; ++i) R.stride[kx][i] = static_cast<int>(strides[kx][i]);
+        const bool aligned = (ptrs[kx].off - cur.base[kx].off) % 16 == 0;
+        bool is_flat = aligned;
+        for (int i = 0; i < 4; ++i) if (od[i] != 1 && strides[kx][i] != flat[i]) is_flat = false;
+        bool is_vec = aligned && strides[kx][3] == 1 && od[3] % 8 == 0;
+        for (int i = 0; i < 3; ++i) if (strides[kx][i] % 8) is_vec = false;
+        R.cls[kx] = is_flat ? k::CC_FLAT : (strides[kx][3] == 0 || od[3] == 1) ? k::CC_BCAST : is_vec ? k::CC_VEC : k::CC_INNER;
+        if (R.cls[kx] == k::CC_INNER || (R.cls[kx] != k::CC_BCAST && esz != oesz)) R.fast = 0;
+        if (R.cls[kx] != k::CC_BCAST && R.first_vec < 0) R.first_vec = kx;
       }
       R.first = cur.cb.total;
-      cur.cb.total += (!red && !cur.vec) ? numel(ov.dims) : items;
+      cur.cb.total += items;
       cur.max_cols = std::max(cur.max_cols, static_cast<int>(od[3]));
-      if (od[3] % 16) cur.vec16 = false;
     }
     flush();
     return OK;

@@ -149,7 +149,6 @@ __global__ void __launch_bounds__(256) layernorm_bf16(const __nv_bfloat16* __res
   const uint4* xr = reinterpret_cast<const uint4*>(x + row * D);
   float v[CH][8];
   float s = 0.f;
-#pragma unroll
   // all loads of the row first, unconditionally (a lane past the row's end re-reads the last vector and
   // discards it): guarded loads would sit in basic blocks of their own and wait for one another
   uint4 u4[CH];
@@ -285,22 +284,31 @@ __global__ void __launch_bounds__(256) splitk_ln_finish(const float* __restrict_
 // right-alignment); every operand is read through its own strides, 0 on the dims RDP resolved to "broadcast".
 // All requests of a batch run in ONE launch through a request table (up to CHAIN_MAX_REQ entries): the operands of
 // the requests live in the same packed buffers, so an entry is extents, element offsets and strides.
-//   chain_elementwise_vec   work item = 8 or 16 consecutive outputs along the last dim: 128-bit loads / stores, operands
-//                           broadcast along the last dim fetched once per item; (row, column) decomposition in 32-bit
-//                           arithmetic, one division chain per item instead of per element
-//   chain_elementwise       work item = one output (any strides, any extents): the fallback
+//   chain_elementwise       no trailing reduction: vectors over the flat output index, see the kernel
 //   chain_rowreduce_warp    a warp per row (rows up to ROWRED_WARP_COLS), the row staged in the warp's slice of shared
 //                           memory, statistics by shuffles: no CTA barrier, eight rows in flight per CTA
 //   chain_rowreduce         a CTA per row for longer rows
+constexpr int CHAIN_NV = 4;                  // chain_elementwise: 16-byte vectors per thread
 constexpr int CHAIN_MAX_OPS = 8;
 constexpr int CHAIN_MAX_REQ = 8;
 constexpr int ROWRED_WARP_COLS = 2048;
 enum ChainOp : int { C_ADD = 0, C_SUB, C_RSUB, C_MUL, C_DIV, C_RDIV, C_RELU, C_GELU, C_SIGMOID };
 enum ChainRed : int { RED_NONE = 0, RED_SOFTMAX = 1, RED_LAYERNORM = 2 };
 
+// How an operand is read by chain_elementwise, per request.
+//   FLAT   laid out like the output: element e of the output reads element e of the operand, 16-byte vectors
+//   BCAST  one value along the last (collapsed) dim
+//   VEC    unit stride along the last dim and 16-byte vectors wherever a column is a multiple of 8 (a bias row)
+//   INNER  anything else: one load per element
+//   SCALAR a constant of the graph (base == nullptr)
+enum ChainCls : int { CC_FLAT = 0, CC_BCAST = 1, CC_INNER = 2, CC_SCALAR = 3, CC_VEC = 4 };
 struct ChainReq {
-  int dim[4];                               // output extents
-  long long first;                          // first work item of this request in the launch
+  int dim[4];                               // output extents (chain_elementwise: adjacent dims collapsed where every operand allows)
+  int numel;                                // chain_elementwise: elements of the output
+  int first_vec;                            // chain_elementwise: first operand that is not one value along a row, -1 if none
+  int fast;                                 // chain_elementwise: no operand is CC_INNER, all are of the output's type, rows are a vector or longer
+  int cls[1 + CHAIN_MAX_OPS];               // ChainCls
+  long long first;                          // first work item of this request in the launch (chain_elementwise: first tile)
   long long out_off;                        // elements from `out`
   long long off[1 + CHAIN_MAX_OPS];         // elements from base[k]; k = 0 is in0, k = 1 + i operand i
   int stride[1 + CHAIN_MAX_OPS][4];         // elements
@@ -316,7 +324,8 @@ struct ChainBatch {
   int red;
   const void* gamma; const void* beta; int gb_bf16; float eps;
   int n_req;
-  long long total;                          // work items of all requests
+  int vec_ok;                               // chain_elementwise: `out` is 16-byte aligned
+  long long total;                          // work items of all requests (chain_elementwise: tiles)
   ChainReq r[CHAIN_MAX_REQ];
 };
 
@@ -357,123 +366,200 @@ __device__ __forceinline__ void chain_store1(const ChainBatch& p, long long lin,
   else reinterpret_cast<float*>(p.out)[lin] = v;
 }
 
-// eight consecutive elements of operand k along the last dim (stride 1, 16-byte aligned), or one broadcast value
-__device__ __forceinline__ void chain_load8(const ChainBatch& p, const ChainReq& R, int k, int i0, int i1, int i2, int i3, float* w) {
-  if (!p.base[k]) {
-#pragma unroll
-    for (int t = 0; t < 8; ++t) w[t] = p.scalar[k];
-    return;
+__device__ __forceinline__ void chain_split_row(const ChainReq& R, int row, int* i0, int* i1, int* i2) {
+  *i0 = 0; *i1 = 0; *i2 = row;
+  if (R.dim[0] * R.dim[1] > 1) {        // after collapsing, most chains have one leading dim left
+    const unsigned t2 = static_cast<unsigned>(row) / static_cast<unsigned>(R.dim[2]);
+    *i2 = row - static_cast<int>(t2) * R.dim[2];
+    *i0 = static_cast<int>(t2 / static_cast<unsigned>(R.dim[1]));
+    *i1 = static_cast<int>(t2) - *i0 * R.dim[1];
   }
-  const long long off = R.off[k] + static_cast<long long>(i0) * R.stride[k][0] + static_cast<long long>(i1) * R.stride[k][1] +
-                        static_cast<long long>(i2) * R.stride[k][2] + static_cast<long long>(i3) * R.stride[k][3];
-  if (R.stride[k][3] == 0) {
-    const float x = p.is_bf16[k] ? __bfloat162float(reinterpret_cast<const __nv_bfloat16*>(p.base[k])[off]) : reinterpret_cast<const float*>(p.base[k])[off];
-#pragma unroll
-    for (int t = 0; t < 8; ++t) w[t] = x;
-  } else if (p.is_bf16[k]) {
-    const uint4 u = *reinterpret_cast<const uint4*>(reinterpret_cast<const __nv_bfloat16*>(p.base[k]) + off);
+}
+
+template <bool BF16> struct ChainVec;     // one 16-byte vector
+template <> struct ChainVec<true> {
+  static constexpr int E = 8;
+  using Raw = uint4;
+  __device__ static void unpack(const Raw& u, float* f) {
     const __nv_bfloat162* h = reinterpret_cast<const __nv_bfloat162*>(&u);
 #pragma unroll
-    for (int t = 0; t < 4; ++t) { const float2 f = __bfloat1622float2(h[t]); w[2 * t] = f.x; w[2 * t + 1] = f.y; }
-  } else {
-    const float4 a = *reinterpret_cast<const float4*>(reinterpret_cast<const float*>(p.base[k]) + off);
-    const float4 c = *reinterpret_cast<const float4*>(reinterpret_cast<const float*>(p.base[k]) + off + 4);
-    w[0] = a.x; w[1] = a.y; w[2] = a.z; w[3] = a.w; w[4] = c.x; w[5] = c.y; w[6] = c.z; w[7] = c.w;
+    for (int t = 0; t < 4; ++t) { const float2 q = __bfloat1622float2(h[t]); f[2 * t] = q.x; f[2 * t + 1] = q.y; }
   }
-}
+  __device__ static Raw pack(const float* f) {
+    Raw u;
+    __nv_bfloat162* h = reinterpret_cast<__nv_bfloat162*>(&u);
+#pragma unroll
+    for (int t = 0; t < 4; ++t) h[t] = __floats2bfloat162_rn(f[2 * t], f[2 * t + 1]);
+    return u;
+  }
+};
+template <> struct ChainVec<false> {
+  static constexpr int E = 4;
+  using Raw = float4;
+  __device__ static void unpack(const Raw& u, float* f) { f[0] = u.x; f[1] = u.y; f[2] = u.z; f[3] = u.w; }
+  __device__ static Raw pack(const float* f) { return make_float4(f[0], f[1], f[2], f[3]); }
+};
 
-// The host selects this kernel only if, for every request, dim[3] % (8 * NV) == 0, every operand's last-dim stride is
-// 0 or 1, and all offsets and leading strides of stride-1 operands (and the output offset) are multiples of 8
-// elements.  NV = 8-element vectors per work item (1 or 2): the index arithmetic is paid once per item.
-template <int NV>
-__global__ void __launch_bounds__(256) chain_elementwise_vec(const __grid_constant__ ChainBatch p) {
-  for (long long item = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x; item < p.total;
-       item += static_cast<long long>(gridDim.x) * blockDim.x) {
-    const ChainReq& R = p.r[chain_find_req(p, item)];
-    const unsigned li = static_cast<unsigned>(item - R.first);      // the host keeps a request below 2^31 items
-    const unsigned cv = static_cast<unsigned>(R.dim[3]) / (8 * NV);
-    unsigned row = li / cv;
-    const int i3 = static_cast<int>(li - row * cv) * (8 * NV);
-    const unsigned d2 = R.dim[2], d1 = R.dim[1];
-    const unsigned t2 = row / d2;
-    const int i2 = static_cast<int>(row - t2 * d2);
-    const unsigned t1 = t2 / d1;
-    const int i1 = static_cast<int>(t2 - t1 * d1), i0 = static_cast<int>(t1);
-    // While every operand so far is broadcast along the last dim the values of an item are one value: that prefix
-    // of the chain (Fig. 4: Sigmoid of the [I,1,1] operand) is evaluated once per item, not once per element.
-    float v[NV][8], w[NV][8];
-    int k0 = 0;
-    if (!p.base[0] || R.stride[0][3] == 0) {
-      float u = chain_load1(p, R, 0, i0, i1, i2, i3);
-      for (; k0 < p.n_ops; ++k0) {
-        const int op = p.op[k0];
-        if (op < C_RELU && p.base[1 + k0] && R.stride[1 + k0][3] != 0) break;
-        u = chain_apply(op, u, op >= C_RELU ? 0.f : chain_load1(p, R, 1 + k0, i0, i1, i2, i3));
-      }
+// The NV vectors of one thread: vector n is the outputs from flat index e + n * 256 vectors on.  No operand is CC_INNER
+// (the host's `fast`).  UNI: all lie in row `row`, vector 0 at column i3.  Otherwise every vector finds its own row; one
+// that reaches past the row's end takes broadcast operands from two rows (rows are at least a vector long then), one that
+// lies past the last element (n >= live) is read from where vector 0 is and not stored.
+template <bool BF16, bool UNI>
+__device__ __forceinline__ void chain_eval_vec(const ChainBatch& p, const ChainReq& R, int e, int row, int i3, int live) {
+  using V = ChainVec<BF16>;
+  constexpr int E = V::E, NV = CHAIN_NV, NR = UNI ? 1 : NV;
+  int i0[NR], i1[NR], i2[NR], col[NR], cut[NR];     // cut: elements of the vector before the row's end
 #pragma unroll
-      for (int n = 0; n < NV; ++n)
+  for (int n = 0; n < NR; ++n) {
+    int r = row;
+    col[n] = i3;
+    if constexpr (!UNI) {
+      const int en = n < live ? e + n * (256 * E) : e;
+      r = static_cast<int>(static_cast<unsigned>(en) / static_cast<unsigned>(R.dim[3]));
+      col[n] = en - r * R.dim[3];
+    }
+    cut[n] = UNI ? E : R.dim[3] - col[n];
+    chain_split_row(R, r, &i0[n], &i1[n], &i2[n]);
+  }
+  auto one_value = [&](int k) { return R.cls[k] == CC_BCAST || R.cls[k] == CC_SCALAR; };
+  auto load = [&](int k, typename V::Raw* u) {
+    const char* base = static_cast<const char*>(p.base[k]) + R.off[k] * (16 / E);
+    if (R.cls[k] == CC_FLAT) {
+      const typename V::Raw* src = reinterpret_cast<const typename V::Raw*>(base) + e / E;
 #pragma unroll
-        for (int t = 0; t < 8; ++t) v[n][t] = u;
+      for (int n = 0; n < NV; ++n) u[n] = src[(UNI || n < live) ? n * 256 : 0];
     } else {
 #pragma unroll
-      for (int n = 0; n < NV; ++n) chain_load8(p, R, 0, i0, i1, i2, i3 + 8 * n, v[n]);
+      for (int n = 0; n < NV; ++n) {
+        const int m = UNI ? 0 : n;
+        const long long off = static_cast<long long>(i0[m]) * R.stride[k][0] + static_cast<long long>(i1[m]) * R.stride[k][1] +
+                              static_cast<long long>(i2[m]) * R.stride[k][2] + col[m] + (UNI ? n * (256 * E) : 0);
+        u[n] = reinterpret_cast<const typename V::Raw*>(base)[off / E];
+      }
     }
-    for (int k = k0; k < p.n_ops; ++k) {
+  };
+  // one value of operand k for the row of vector n, or for the row after it
+  auto value = [&](int k, int n) { return chain_load1(p, R, k, i0[n], i1[n], i2[n], 0); };
+  auto value_after = [&](int k, int n) {
+    int a0 = i0[n], a1 = i1[n], a2 = i2[n] + 1;
+    if (a2 == R.dim[2]) { a2 = 0; if (++a1 == R.dim[1]) { a1 = 0; ++a0; } }
+    return chain_load1(p, R, k, a0, a1, a2, 0);
+  };
+  float v[NV][E];
+  typename V::Raw u[NV];
+  // the first vector operand is requested before anything else is worked out
+  if (R.first_vec >= 0) load(R.first_vec, u);
+  int k0 = 0;
+  // While every operand so far is one value along the row the values of a vector are one value (two where it straddles
+  // rows): that prefix of the chain (Fig. 4: Sigmoid of the [I,1,1] operand) is not evaluated for every element.
+  if (one_value(0)) {
+    k0 = R.first_vec < 0 ? p.n_ops : R.first_vec - 1;
+    float x[NR], y[NR];
+#pragma unroll
+    for (int n = 0; n < NR; ++n) { x[n] = value(0, n); y[n] = (UNI || cut[n] >= E) ? x[n] : value_after(0, n); }
+    for (int k = 0; k < k0; ++k) {
       const int op = p.op[k];
-      if (op < C_RELU) {
 #pragma unroll
-        for (int n = 0; n < NV; ++n) chain_load8(p, R, 1 + k, i0, i1, i2, i3 + 8 * n, w[n]);
-      }
-      // the operator is chosen once per item; the elements run through straight-line code
-      switch (op) {
-#define SOD2_CHAIN_CASE(OP_)                                                                                   \
-        case OP_:                                                                                              \
-          _Pragma("unroll") for (int n = 0; n < NV; ++n)                                                       \
-            _Pragma("unroll") for (int t = 0; t < 8; ++t) v[n][t] = chain_apply(OP_, v[n][t], w[n][t]);        \
-          break;
-        SOD2_CHAIN_CASE(C_ADD)
-        SOD2_CHAIN_CASE(C_SUB)
-        SOD2_CHAIN_CASE(C_RSUB)
-        SOD2_CHAIN_CASE(C_MUL)
-        SOD2_CHAIN_CASE(C_DIV)
-        SOD2_CHAIN_CASE(C_RDIV)
-        SOD2_CHAIN_CASE(C_RELU)
-        SOD2_CHAIN_CASE(C_GELU)
-        default:
-        SOD2_CHAIN_CASE(C_SIGMOID)
-#undef SOD2_CHAIN_CASE
+      for (int n = 0; n < NR; ++n) {
+        const float w = op >= C_RELU ? 0.f : value(1 + k, n);
+        x[n] = chain_apply(op, x[n], w);
+        if (!UNI) y[n] = cut[n] >= E ? x[n] : chain_apply(op, y[n], op >= C_RELU ? 0.f : value_after(1 + k, n));
       }
     }
-    const long long lin = R.out_off + static_cast<long long>(li) * (8 * NV);
 #pragma unroll
-    for (int n = 0; n < NV; ++n) {
-      if (p.out_bf16) {
-        uint4 o;
-        __nv_bfloat162* oh = reinterpret_cast<__nv_bfloat162*>(&o);
+    for (int n = 0; n < NV; ++n)
 #pragma unroll
-        for (int t = 0; t < 4; ++t) oh[t] = __floats2bfloat162_rn(v[n][2 * t], v[n][2 * t + 1]);
-        *reinterpret_cast<uint4*>(reinterpret_cast<__nv_bfloat16*>(p.out) + lin + 8 * n) = o;
-      } else {
-        float* o = reinterpret_cast<float*>(p.out) + lin + 8 * n;
-        *reinterpret_cast<float4*>(o) = make_float4(v[n][0], v[n][1], v[n][2], v[n][3]);
-        *reinterpret_cast<float4*>(o + 4) = make_float4(v[n][4], v[n][5], v[n][6], v[n][7]);
-      }
+      for (int t = 0; t < E; ++t) v[n][t] = UNI ? x[0] : t < cut[n % NR] ? x[n % NR] : y[n % NR];
+  } else {
+#pragma unroll
+    for (int n = 0; n < NV; ++n) V::unpack(u[n], v[n]);
+  }
+#pragma unroll 1
+  for (int k = k0; k < p.n_ops; ++k) {
+    const int op = p.op[k];
+    if (op >= C_RELU) {
+      // the operator is chosen once per thread; the elements run through straight-line code
+#define SOD2_CHAIN_UNARY(OP_) { _Pragma("unroll") for (int n = 0; n < NV; ++n) _Pragma("unroll") for (int t = 0; t < E; ++t) v[n][t] = chain_apply(OP_, v[n][t], 0.f); }
+      if (op == C_RELU) SOD2_CHAIN_UNARY(C_RELU)
+      else if (op == C_GELU) SOD2_CHAIN_UNARY(C_GELU)
+      else SOD2_CHAIN_UNARY(C_SIGMOID)
+#undef SOD2_CHAIN_UNARY
+      continue;
+    }
+    float x[NR], y[NR];
+    const bool one = one_value(1 + k);
+    if (one) {
+#pragma unroll
+      for (int n = 0; n < NR; ++n) { x[n] = value(1 + k, n); y[n] = (UNI || cut[n] >= E) ? x[n] : value_after(1 + k, n); }
+    } else if (1 + k != R.first_vec) {
+      load(1 + k, u);
+    }
+    switch (op) {
+#define SOD2_CHAIN_CASE(OP_)                                                                                   \
+      case OP_:                                                                                                \
+        _Pragma("unroll") for (int n = 0; n < NV; ++n) {                                                       \
+          float w[E];                                                                                          \
+          V::unpack(u[n], w);                                                                                  \
+          _Pragma("unroll") for (int t = 0; t < E; ++t)                                                        \
+            v[n][t] = chain_apply(OP_, v[n][t], !one ? w[t] : (UNI || t < cut[n % NR]) ? x[n % NR] : y[n % NR]); \
+        }                                                                                                      \
+        break;
+      SOD2_CHAIN_CASE(C_ADD)
+      SOD2_CHAIN_CASE(C_SUB)
+      SOD2_CHAIN_CASE(C_RSUB)
+      SOD2_CHAIN_CASE(C_MUL)
+      SOD2_CHAIN_CASE(C_DIV)
+      default:
+      SOD2_CHAIN_CASE(C_RDIV)
+#undef SOD2_CHAIN_CASE
     }
   }
+  typename V::Raw* dst = reinterpret_cast<typename V::Raw*>(static_cast<char*>(p.out) + R.out_off * (16 / E)) + e / E;
+#pragma unroll
+  for (int n = 0; n < NV; ++n)
+    if (UNI || n < live) dst[n * 256] = V::pack(v[n]);
 }
 
-// fallback: one thread per output element, grid-stride
-__global__ void __launch_bounds__(256) chain_elementwise(const __grid_constant__ ChainBatch p) {
-  for (long long item = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x; item < p.total;
-       item += static_cast<long long>(gridDim.x) * blockDim.x) {
-    const ChainReq& R = p.r[chain_find_req(p, item)];
-    long long r = item - R.first;
-    const int i3 = static_cast<int>(r % R.dim[3]); r /= R.dim[3];
-    const int i2 = static_cast<int>(r % R.dim[2]); r /= R.dim[2];
-    const int i1 = static_cast<int>(r % R.dim[1]);
-    const int i0 = static_cast<int>(r / R.dim[1]);
-    chain_store1(p, R.out_off + (item - R.first), chain_eval(p, R, i0, i1, i2, i3));
+// Elementwise chains, bound by HBM.  Work is cut over the FLAT output index, not over rows: a tile is 1024 16-byte
+// vectors of consecutive outputs of one request, a thread takes four of them, so neither a row length that is no
+// multiple of 8 nor a request of such rows among others costs the batch its 16-byte accesses.  The host collapses
+// adjacent dims wherever every operand allows it (Fig. 4: [I,J,K] -> [I, J*K]), so that most tiles lie inside one row:
+// then the row index and every broadcast operand are the same for the whole CTA and cost one evaluation per thread and
+// tile.  In the other tiles every vector finds its own row (its loads in flight with the others': one after the other
+// they made these tiles four round trips long, and the last of them the kernel's tail).  A request's last, incomplete
+// vector, rows shorter than a vector, operands of other strides and operands of mixed types go element by element.
+// Measured on B200, Fig. 4 chain in bf16, requests 64x128x784 + 37x101x333 + 64x77x1024 + 3x250x49 (51 MB):
+// 120 -> 16 us a pass (0.42 -> 3.2 TB/s): one request with rows of 333 or 49 used to put the whole batch on one element
+// per thread and three 64-bit divisions.  Now bound by HBM latency and instruction fetch in short CTAs, not by bytes.
+template <bool BF16>
+__global__ void __launch_bounds__(256, 4) chain_elementwise(const __grid_constant__ ChainBatch p) {
+  constexpr int E = ChainVec<BF16>::E, TILE = 256 * CHAIN_NV * E;
+  ptx::pdl_wait();
+  ptx::pdl_launch();
+  const ChainReq& R = p.r[chain_find_req(p, blockIdx.x)];
+  const int e0 = (static_cast<int>(blockIdx.x) - static_cast<int>(R.first)) * TILE;
+  const int inner = R.dim[3];
+  auto by_element = [&](int e) {
+    const int row = static_cast<int>(static_cast<unsigned>(e) / static_cast<unsigned>(inner));
+    int i0, i1, i2;
+    chain_split_row(R, row, &i0, &i1, &i2);
+    chain_store1(p, R.out_off + e, chain_eval(p, R, i0, i1, i2, e - row * inner));
+  };
+  if (!(p.vec_ok && R.fast)) {
+    for (int e = e0 + threadIdx.x; e < min(e0 + TILE, R.numel); e += 256) by_element(e);
+    return;
   }
+  const int row0 = static_cast<int>(static_cast<unsigned>(e0) / static_cast<unsigned>(inner));
+  const int col0 = e0 - row0 * inner;
+  const int d = threadIdx.x * E;
+  if (col0 + TILE <= inner) {
+    chain_eval_vec<BF16, true>(p, R, e0 + d, row0, col0 + d, CHAIN_NV);
+    return;
+  }
+  const int whole = R.numel / E * E;                     // the tail behind the last whole vector: one element per thread
+  const int left = whole - (e0 + d);
+  if (left > 0) chain_eval_vec<BF16, false>(p, R, e0 + d, 0, 0, min(CHAIN_NV, (left + 256 * E - 1) / (256 * E)));
+  if (whole >= e0 && whole < e0 + TILE && whole + static_cast<int>(threadIdx.x) < R.numel) by_element(whole + threadIdx.x);
 }
 
 __device__ __forceinline__ void chain_row_index(const ChainReq& R, long long row, int* i0, int* i1, int* i2) {
