@@ -210,11 +210,8 @@ sod2_status sod2_run(sod2_plan_t* p, const void* const* inputs, void* const* out
   for (size_t i = 0; i < G.outputs.size(); ++i) if (!outputs[i]) { p->h.err = "null output"; return SOD2_E_INVALID_ARG; }
   if (arena_bytes < p->p.arena_bytes) { p->h.err = "arena too small"; return SOD2_E_ARENA_TOO_SMALL; }
   if (reinterpret_cast<uintptr_t>(arena) & 255) { p->h.err = "arena must be 256-byte aligned"; return SOD2_E_MISALIGNED; }
-  for (int c : G.consts) {
-    bool used = false;
-    for (auto& grp : p->g->c.groups) for (int t : grp.ext_in) if (t == c) used = true;
-    if (used && !G.tensors[c].dev_ptr) { p->h.err = "constant " + G.tensors[c].name + " has no device data"; return SOD2_E_INVALID_ARG; }
-  }
+  for (int c : p->g->c.used_consts)
+    if (!G.tensors[c].dev_ptr) { p->h.err = "constant " + G.tensors[c].name + " has no device data"; return SOD2_E_INVALID_ARG; }
   int64_t inf[8] = {0};
   Status s = run_plan(&p->p, inputs, outputs, arena, arena_bytes, stream, inf);
   if (s != OK) p->h.err = p->p.err;
@@ -228,11 +225,8 @@ sod2_status sod2_run_graph(sod2_plan_t* p, const void* const* inputs, void* cons
   const Graph& G = p->g->c.g;
   for (size_t i = 0; i < G.inputs.size(); ++i) if (!inputs[i]) { p->h.err = "null input"; return SOD2_E_INVALID_ARG; }
   for (size_t i = 0; i < G.outputs.size(); ++i) if (!outputs[i]) { p->h.err = "null output"; return SOD2_E_INVALID_ARG; }
-  for (int c : G.consts) {
-    bool used = false;
-    for (auto& grp : p->g->c.groups) for (int t : grp.ext_in) if (t == c) used = true;
-    if (used && !G.tensors[c].dev_ptr) { p->h.err = "constant " + G.tensors[c].name + " has no device data"; return SOD2_E_INVALID_ARG; }
-  }
+  for (int c : p->g->c.used_consts)
+    if (!G.tensors[c].dev_ptr) { p->h.err = "constant " + G.tensors[c].name + " has no device data"; return SOD2_E_INVALID_ARG; }
   int64_t inf[8] = {0};
   Status s = run_plan_graph(&p->p, inputs, outputs, arena, arena_bytes, stream, inf);
   if (s != OK) p->h.err = p->p.err;
@@ -253,6 +247,7 @@ sod2_status sod2_run_exact(sod2_plan_t* p, const void* const* inputs, void* cons
   }
   int64_t inf[8] = {0};
   std::string err;
+  ++p->p.run_epoch;
   Status s = run_exact(&p->g->c, p->p.b, &p->p, inputs, outputs, arena, arena_bytes, stream, inf, &err);
   if (s != OK) p->h.err = err;
   if (info) {
@@ -464,14 +459,9 @@ sod2_status sod2_run_output_shape(sod2_plan_t* p, const void* arena, void* strea
   for (auto& d : T.S.dims) if (d.known() && e_has_runtime(G.cx, d.e)) need = true;
   if (need) {
     if (!arena) return SOD2_E_INVALID_ARG;
-    if (cudaStreamSynchronize(static_cast<cudaStream_t>(stream)) != cudaSuccess) return SOD2_E_CUDA;
-    for (size_t a = 0; a < G.cx.atoms.size(); ++a) {
-      if (G.cx.atoms[a].kind != AtomKind::SYM || !G.cx.atoms[a].runtime) continue;
-      long long v = 0;
-      const char* src = static_cast<const char*>(arena) + 256 + (a * p->p.n_req + r) * 8;
-      if (cudaMemcpy(&v, src, 8, cudaMemcpyDeviceToHost) != cudaSuccess) return SOD2_E_CUDA;
-      vals[a] = v;
-    }
+    if (read_counts(&p->p, arena, stream) != OK) return SOD2_E_CUDA;
+    for (size_t a = 0; a < G.cx.atoms.size(); ++a)
+      if (G.cx.atoms[a].kind == AtomKind::SYM && G.cx.atoms[a].runtime) vals[a] = p->p.counts[a * p->p.n_req + r];
   }
   if (rank) *rank = T.S.rank;
   for (int i = 0; i < T.S.rank; ++i) {

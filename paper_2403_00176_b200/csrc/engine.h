@@ -121,6 +121,7 @@ struct Compiled {
   // a = perm; Slice: a = start, b = step per axis of the input), so that planning touches no strings
   struct ViewParam { int op = -1; std::vector<int64_t> a, b; };   // op: 0 Transpose, 1 Reshape, 2 Slice
   std::vector<ViewParam> view_param;
+  std::vector<int> used_consts;       // constants some group reads: a run needs their device data
   std::vector<int> packed_consts;     // tensor ids
   std::vector<size_t> packed_off;     // byte offsets in the prepack workspace
   // entry i with packed_ln[i].gamma >= 0 is the weight of a GEMM whose A operand is a folded LayerNorm:
@@ -337,6 +338,13 @@ struct Plan {
   void* ev_fork = nullptr;                // cudaEvent_t
   void* ev_join = nullptr;                // cudaEvent_t
   std::vector<const void*> graph_key;     // inputs, outputs, arena the graph was captured with
+  // Run-time counts of the last run, read back by the first sod2_run_output_shape after it (read_counts).  They are kept
+  // only while the library can tell that no other run has happened: a run that a caller captured into a graph of its own
+  // may be replayed without a call, so such a plan reads the counts every time.
+  uint64_t run_epoch = 1, counts_epoch = 0;
+  const void* counts_arena = nullptr;
+  bool captured_by_caller = false;
+  std::vector<long long> counts;          // [atom][request], as in the arena header
   Plan() = default;
   Plan(const Plan&) = delete;
   Plan& operator=(const Plan&) = delete;
@@ -348,6 +356,8 @@ Status make_plan(const Compiled* c, const Binding* b, Plan* p);
 // pointer differs from the captured ones, then replayed on `stream`.  info[3] = 1 if this call captured.
 Status run_plan_graph(Plan* p, const void* const* inputs, void* const* outputs, void* arena, size_t arena_bytes, void* stream,
                       int64_t* info);
+// The counts in the arena header -> Plan::counts (synchronises `stream`).
+Status read_counts(Plan* p, const void* arena, void* stream);
 Status build_launches(Plan* p);   // exec.cu
 Status detect_chains(Plan* p);    // exec.cu: fills Plan::chains / chain_of from the resolved views
 // step_lo..step_hi: only these groups (positions in execution order) are enqueued (all by default); the arena header

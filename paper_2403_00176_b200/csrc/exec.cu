@@ -6,6 +6,7 @@
 #include <cstring>
 #include <functional>
 #include <map>
+#include <mutex>
 #include <set>
 
 #include "attention.cuh"
@@ -1312,28 +1313,47 @@ struct Builder {
     const Expr& ce = g.tensors[G.out].S.dims[1].e;
     const int sym = ce.terms.begin()->first[0].first;
     count_known_after(gi, G.out);
-    for (int r = 0; r < p.n_req; ++r) {
-      const View& v = p.views[G.a][r];
-      if (!v.contiguous()) return fail(E_UNSUPPORTED_OP, "NonZero needs a contiguous input");
-      k::NonZeroParams np{};
-      np.is_bf16 = X.dtype == DType::BF16;
-      np.numel = numel(v.dims);
-      np.rank = static_cast<int>(v.dims.size());
-      for (int i = 0; i < np.rank; ++i) np.dims[i] = v.dims[i];
-      np.nblocks = static_cast<int>((np.numel + k::NZ_BLOCK - 1) / k::NZ_BLOCK);
-      scratch_need = std::max(scratch_need, static_cast<size_t>(np.nblocks + 1) * 4);
-      Ptr px = ptr_of(G.a, r), po = ptr_of(G.out, r);
-      const size_t count_off = 256 + (static_cast<size_t>(sym) * p.n_req + r) * 8;
-      add(gi, 3, [=](const RunCtx& x) mutable {
-        np.x = x.resolve(px);
-        np.out = reinterpret_cast<long long*>(x.resolve(po));
-        np.block_count = reinterpret_cast<int*>(x.arena + x.plan->scratch_off[0]);
-        np.count_out = reinterpret_cast<long long*>(x.arena + count_off);
-        if (np.nblocks == 0) return cudaMemsetAsync(np.count_out, 0, 8, x.stream);
-        k::nonzero_count<<<np.nblocks, k::NZ_BLOCK, 0, x.stream>>>(np);
-        k::nonzero_scan<<<1, 1024, 0, x.stream>>>(np);
-        k::nonzero_write<<<np.nblocks, k::NZ_BLOCK, 0, x.stream>>>(np);
-        return cudaGetLastError();
+    for (int r0 = 0; r0 < p.n_req; r0 += k::NZ_MAX_REQ) {
+      k::NonZeroBatch nb{};
+      nb.n_req = std::min(k::NZ_MAX_REQ, p.n_req - r0);
+      nb.is_bf16 = X.dtype == DType::BF16;
+      nb.rank = X.S.rank;
+      struct Io { Ptr px, po; size_t count_off, mask_off, cnt_off; };
+      std::vector<Io> io(nb.n_req);
+      size_t need = 0;
+      int ctas = 0;
+      for (int i = 0; i < nb.n_req; ++i) {
+        const int r = r0 + i;
+        const View& v = p.views[G.a][r];
+        if (!v.contiguous()) return fail(E_UNSUPPORTED_OP, "NonZero needs a contiguous input");
+        k::NonZeroReq& R = nb.r[i];
+        R.numel = numel(v.dims);
+        for (int d = 0; d < 4; ++d) R.dims[d] = d < 4 - nb.rank ? 1 : std::max<int64_t>(v.dims[d - (4 - nb.rank)], 1);
+        const long long subs = (R.numel + k::NZ_SUB - 1) / k::NZ_SUB;
+        const long long per = std::max<long long>(1, (subs + k::NZ_MAX_CHUNKS - 1) / k::NZ_MAX_CHUNKS);
+        R.chunk = per * k::NZ_SUB;
+        R.chunks = static_cast<int>(std::max<long long>(1, (subs + per - 1) / per));   // an empty request still reports its count
+        R.first = ctas;
+        ctas += R.chunks;
+        io[i] = Io{ptr_of(G.a, r), ptr_of(G.out, r), 256 + (static_cast<size_t>(sym) * p.n_req + r) * 8, need, 0};
+        need += static_cast<size_t>(subs) * (k::NZ_SUB / 8);
+        io[i].cnt_off = need;
+        need += (static_cast<size_t>(R.chunks) * 4 + 15) & ~size_t(15);
+      }
+      scratch_need = std::max(scratch_need, need);
+      add(gi, 2, [=](const RunCtx& x) mutable {
+        char* scratch = x.arena + x.plan->scratch_off[0];
+        for (int i = 0; i < nb.n_req; ++i) {
+          k::NonZeroReq& R = nb.r[i];
+          R.x = x.resolve(io[i].px);
+          R.vec_ok = (reinterpret_cast<uintptr_t>(R.x) & 15) == 0;
+          R.out = reinterpret_cast<long long*>(x.resolve(io[i].po));
+          R.mask = reinterpret_cast<unsigned*>(scratch + io[i].mask_off);
+          R.count = reinterpret_cast<int*>(scratch + io[i].cnt_off);
+          R.count_out = reinterpret_cast<long long*>(x.arena + io[i].count_off);
+        }
+        cudaError_t e = launch_pdl(k::nonzero_mask, dim3(ctas), dim3(k::NZ_THREADS), 0, x.stream, nb);
+        return e != cudaSuccess ? e : launch_pdl(k::nonzero_write, dim3(ctas), dim3(k::NZ_THREADS), 0, x.stream, nb);
       });
     }
     return OK;
@@ -2129,7 +2149,6 @@ struct Builder {
     p.group_bytes.clear();
     p.gpu_launches = 0;
     p.rt_syms_after.assign(c.groups.size(), {});
-    // the fp32 row kernel and the elementwise chains have no bounded waits, tickets or device-side counts
     // a pooling group right after a layout change of the SAME tensor: neither reads what the other writes, and the
     // shared input stays live over both steps, so the arena plan (liveness by step) cannot hand the pooled output a
     // slot that the layout kernel still reads
@@ -2139,9 +2158,11 @@ struct Builder {
       if (Bg.kind == GKind::GAP && A.kind == GKind::LAYOUT && Bg.a == A.a && Bg.a != A.out && A.a != Bg.out && !p.side_group[gi - 1])
         p.side_group[gi] = 1;
     }
+    // the fp32 row kernel, the elementwise chains and NonZero (which writes its counts, never adds to them) have no
+    // bounded waits and no tickets
     p.uses_header = false;
     for (const Group& G : c.groups)
-      if (!((G.kind == GKind::GEMM && g.tensors[G.a].dtype == DType::F32) || G.kind == GKind::CHAIN || G.kind == GKind::BMM ||
+      if (!((G.kind == GKind::GEMM && g.tensors[G.a].dtype == DType::F32) || G.kind == GKind::CHAIN || G.kind == GKind::NONZERO || G.kind == GKind::BMM ||
             G.kind == GKind::SUMSQ || G.kind == GKind::TOPK || G.kind == GKind::GATHER || G.kind == GKind::FILL || G.kind == GKind::RESIZE)) p.uses_header = true;
     // SOD2_HOST_PROFILE: host time of building the launches, per group kind
     static const bool prof = getenv("SOD2_HOST_PROFILE") != nullptr;
@@ -2339,6 +2360,7 @@ Status run_plan_timed(Plan* p, const void* const* inputs, void* const* outputs, 
   if (reinterpret_cast<uintptr_t>(arena) & 255) { p->err = "arena must be 256-byte aligned"; return E_MISALIGNED; }
   RunCtx x{inputs, outputs, static_cast<char*>(arena), static_cast<char*>(p->c->packed_ws), static_cast<cudaStream_t>(stream), p};
   const size_t n = p->launches.size();
+  ++p->run_epoch;
   std::vector<cudaEvent_t> ev(2 * n);
   for (auto& e : ev) if (cudaEventCreate(&e) != cudaSuccess) { p->err = "cudaEventCreate failed"; return E_CUDA; }
   if (p->uses_header) cudaMemsetAsync(arena, 0, p->header_clear_bytes, x.stream);
@@ -2361,6 +2383,52 @@ Status run_plan_timed(Plan* p, const void* const* inputs, void* const* outputs, 
     }
   for (auto& e : ev) cudaEventDestroy(e);
   return st;
+}
+
+// Pinned host memory for reading counts back: a copy into pageable memory is staged by the driver and costs a second
+// round trip.  Blocks of one size, at most PINNED_MAX of them parked; a larger header takes a pageable copy.
+namespace {
+constexpr size_t PINNED_BYTES = 16 << 10, PINNED_MAX = 8;
+struct PinnedPool { std::mutex mu; std::vector<void*> parked; };
+PinnedPool& pinned_pool() { static PinnedPool* p = new PinnedPool; return *p; }   // never destroyed: plans may outlive the statics
+struct PinnedBlock {
+  void* p = nullptr;
+  PinnedBlock() {
+    PinnedPool& P = pinned_pool();
+    std::lock_guard<std::mutex> lk(P.mu);
+    if (!P.parked.empty()) { p = P.parked.back(); P.parked.pop_back(); return; }
+    if (cudaHostAlloc(&p, PINNED_BYTES, cudaHostAllocPortable) != cudaSuccess) { p = nullptr; cudaGetLastError(); }
+  }
+  ~PinnedBlock() {
+    if (!p) return;
+    PinnedPool& P = pinned_pool();
+    std::lock_guard<std::mutex> lk(P.mu);
+    if (P.parked.size() < PINNED_MAX) P.parked.push_back(p); else cudaFreeHost(p);
+  }
+};
+// copies `bytes` of device memory and waits for the stream
+bool read_back(void* dst, const void* src, size_t bytes, cudaStream_t st) {
+  if (bytes <= PINNED_BYTES) {
+    PinnedBlock b;
+    if (b.p) {
+      if (cudaMemcpyAsync(b.p, src, bytes, cudaMemcpyDeviceToHost, st) != cudaSuccess || cudaStreamSynchronize(st) != cudaSuccess) return false;
+      std::memcpy(dst, b.p, bytes);
+      return true;
+    }
+  }
+  return cudaMemcpyAsync(dst, src, bytes, cudaMemcpyDeviceToHost, st) == cudaSuccess && cudaStreamSynchronize(st) == cudaSuccess;
+}
+}  // namespace
+
+Status read_counts(Plan* p, const void* arena, void* stream) {
+  cudaStream_t st = static_cast<cudaStream_t>(stream);
+  if (!p->captured_by_caller && p->counts_epoch == p->run_epoch && p->counts_arena == arena)
+    return cudaStreamSynchronize(st) == cudaSuccess ? OK : E_CUDA;
+  p->counts.resize(p->c->g.cx.atoms.size() * static_cast<size_t>(p->n_req));
+  if (!read_back(p->counts.data(), static_cast<const char*>(arena) + 256, p->counts.size() * 8, st)) return E_CUDA;
+  p->counts_epoch = p->run_epoch;
+  p->counts_arena = arena;
+  return OK;
 }
 
 Plan::~Plan() {
@@ -2422,6 +2490,7 @@ Status run_plan_graph(Plan* p, const void* const* inputs, void* const* outputs, 
   } else {
     if (arena_bytes < p->arena_bytes) { p->err = "arena too small"; return E_ARENA_TOO_SMALL; }
   }
+  ++p->run_epoch;
   const cudaError_t el = cudaGraphLaunch(static_cast<cudaGraphExec_t>(p->graph_exec), static_cast<cudaStream_t>(stream));
   if (el != cudaSuccess) { p->err = std::string("graph launch failed: ") + cudaGetErrorString(el); return E_CUDA; }
   if (info) {
@@ -2439,6 +2508,16 @@ Status run_plan(Plan* p, const void* const* inputs, void* const* outputs, void* 
   if (reinterpret_cast<uintptr_t>(arena) & 255) { p->err = "arena must be 256-byte aligned"; return E_MISALIGNED; }
   if (p->c->packed_bytes && !p->c->packed_ws) { p->err = "weights are not prepacked"; return E_INVALID_ARG; }
   auto t0 = std::chrono::steady_clock::now();
+  ++p->run_epoch;
+  if (!p->captured_by_caller && stream != p->capture_stream) {
+    for (auto& syms : p->rt_syms_after)
+      if (!syms.empty()) {
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        if (cudaStreamIsCapturing(static_cast<cudaStream_t>(stream), &cap) != cudaSuccess) cudaGetLastError();
+        if (cap != cudaStreamCaptureStatusNone) p->captured_by_caller = true;
+        break;
+      }
+  }
   if (!p->sm_count_known) {
     int dev = 0, n = 0;
     if (cudaGetDevice(&dev) == cudaSuccess && cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && n > 0) p->sm_count = n;
@@ -2627,8 +2706,7 @@ Status run_exact(const Compiled* c, const Binding* b0, const Plan* bounded, cons
     launches += inf[1];
     if (k + 1 >= plan_stages.size() || st.newly.empty()) continue;
     // read the counts and bind the symbols: the next stage is planned at the true sizes
-    if (cudaMemcpyAsync(counts.data(), static_cast<const char*>(arena) + 256, counts.size() * 8, cudaMemcpyDeviceToHost, static_cast<cudaStream_t>(stream)) != cudaSuccess ||
-        cudaStreamSynchronize(static_cast<cudaStream_t>(stream)) != cudaSuccess) { *err = "cannot read the run-time counts"; return E_CUDA; }
+    if (!read_back(counts.data(), static_cast<const char*>(arena) + 256, counts.size() * 8, static_cast<cudaStream_t>(stream))) { *err = "cannot read the run-time counts"; return E_CUDA; }
     for (int r = 0; r < n_req; ++r)
       for (int a : st.newly) rt[r].push_back({a, counts[static_cast<size_t>(a) * n_req + r]});
   }

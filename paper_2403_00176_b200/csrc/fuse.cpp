@@ -815,7 +815,15 @@ static void index_shape_classes(Compiled* c) {
 Status form_groups(Compiled* c) {
   Fuser f(*c);
   Status s = f.run();
-  if (s == OK) { index_dim_exprs(c); index_view_params(c); index_shape_classes(c); }
+  if (s == OK) {
+    index_dim_exprs(c);
+    index_view_params(c);
+    index_shape_classes(c);
+    std::vector<char> read(c->g.tensors.size(), 0);
+    for (auto& G : c->groups) for (int t : G.ext_in) read[t] = 1;
+    c->used_consts.clear();
+    for (int t : c->g.consts) if (read[t]) c->used_consts.push_back(t);
+  }
   return s;
 }
 

@@ -184,79 +184,166 @@ __global__ void __launch_bounds__(256) topk_gather(const __grid_constant__ TopkP
 }
 
 // ---------------------------------------------------------------------------------------------
-// NonZero: int64 coordinates [rank, nnz] of the non-zero elements in row-major order.
-// Pass 1: per-block counts into scratch; pass 2 (one CTA): exclusive scan of the counts + total;
-// pass 3: each block rescans its flags and writes coordinates at its offset. nnz is known only
-// after pass 2, so the row pitch of the output (= nnz) is read from device memory in pass 3.
-constexpr int NZ_BLOCK = 1024;
-struct NonZeroParams {
-  const void* x; int is_bf16;
+// NonZero: int64 coordinates [rank, nnz] of the non-zero elements in row-major order, all requests of a batch in two
+// launches.  The row pitch of the output is nnz, so no coordinate can be written before everything is counted:
+//   nonzero_mask   reads the input once (16-byte loads), leaves one bit per element and a count per chunk in scratch
+//   nonzero_write  a CTA per chunk adds up the counts in front of its own (at most NZ_MAX_CHUNKS, from L2), expands its
+//                  bits into a list of element indices in shared memory and writes the coordinates from there, so that
+//                  neighbouring threads write neighbouring words
+// A chunk is NZ_SUB elements, more where a request would have over NZ_MAX_CHUNKS of them.
+// Bound by the 16 bytes written per element found and, below a few MB, by the two launches.
+// Measured on B200, 1024x1024 + 777x1333 + 3x4095 + 2048x768 in fp32 (38 MB): with three launches per request and one
+// element per thread 114 us on the device and 200 us with the counts read back; now 65 us with the counts read back.
+constexpr int NZ_THREADS = 256, NZ_SUB = NZ_THREADS * 32, NZ_MAX_CHUNKS = 2048, NZ_MAX_REQ = 8;
+struct NonZeroReq {
+  const void* x;
   long long numel;
-  int rank;
-  long long dims[4];
-  int* block_count;       // scratch [nblocks + 1]; after pass 2: exclusive offsets, [nblocks] = total
+  long long dims[4];      // leading extents are 1 below rank 4
+  long long chunk;        // elements per chunk, a multiple of NZ_SUB
+  unsigned* mask;         // scratch: one bit per element, whole NZ_SUBs
+  int* count;             // scratch: non-zero elements per chunk
   long long* out;         // [rank, nnz]
   long long* count_out;   // device word: nnz
-  int nblocks;
+  int first, chunks;      // first CTA of the request in the launch, number of its chunks (at least one)
+  int vec_ok;             // x is 16-byte aligned
 };
-__device__ __forceinline__ bool nz_flag(const NonZeroParams& p, long long i) {
-  if (i >= p.numel) return false;
-  return p.is_bf16 ? (__bfloat162float(reinterpret_cast<const __nv_bfloat16*>(p.x)[i]) != 0.0f)
-                   : (reinterpret_cast<const float*>(p.x)[i] != 0.0f);
+struct NonZeroBatch {
+  int n_req, is_bf16, rank;
+  NonZeroReq r[NZ_MAX_REQ];
+};
+__device__ __forceinline__ const NonZeroReq& nz_find(const NonZeroBatch& p) {
+  int ri = 0;
+  while (ri + 1 < p.n_req && static_cast<int>(blockIdx.x) >= p.r[ri + 1].first) ++ri;
+  return p.r[ri];
 }
-__global__ void __launch_bounds__(NZ_BLOCK) nonzero_count(NonZeroParams p) {
-  __shared__ int wc[32];
-  const long long i = static_cast<long long>(blockIdx.x) * NZ_BLOCK + threadIdx.x;
-  const unsigned bal = __ballot_sync(0xffffffffu, nz_flag(p, i));
-  if ((threadIdx.x & 31) == 0) wc[threadIdx.x >> 5] = __popc(bal);
+__device__ __forceinline__ int nz_block_sum(int v, int* warp_sums) {
+#pragma unroll
+  for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  if ((threadIdx.x & 31) == 0) warp_sums[threadIdx.x >> 5] = v;
   __syncthreads();
-  if (threadIdx.x == 0) {
-    int t = 0;
-    for (int w = 0; w < 32; ++w) t += wc[w];
-    p.block_count[blockIdx.x] = t;
+  int t = 0;
+#pragma unroll
+  for (int w = 0; w < NZ_THREADS / 32; ++w) t += warp_sums[w];
+  return t;
+}
+__global__ void __launch_bounds__(NZ_THREADS) nonzero_mask(const __grid_constant__ NonZeroBatch p) {
+  __shared__ int warp_sums[NZ_THREADS / 32];
+  const NonZeroReq& R = nz_find(p);
+  ptx::pdl_wait();
+  ptx::pdl_launch();
+  const int chunk = blockIdx.x - R.first, tid = threadIdx.x, lane = tid & 31;
+  const long long lo = chunk * R.chunk, hi = min(R.numel, lo + R.chunk);
+  int cnt = 0;
+  for (long long base = lo; base < hi; base += NZ_SUB) {
+    unsigned* words = R.mask + (base >> 5);
+    if (R.vec_ok && base + NZ_SUB <= R.numel) {
+      if (p.is_bf16) {
+        const uint4* src = reinterpret_cast<const uint4*>(reinterpret_cast<const __nv_bfloat16*>(R.x) + base);
+        uint4 u[4];
+#pragma unroll
+        for (int v = 0; v < 4; ++v) u[v] = src[v * NZ_THREADS + tid];
+#pragma unroll
+        for (int v = 0; v < 4; ++v) {     // eight elements per thread: four threads make a word
+          const unsigned q[4] = {u[v].x, u[v].y, u[v].z, u[v].w};
+          unsigned b = 0;
+#pragma unroll
+          for (int t = 0; t < 4; ++t) b |= ((q[t] & 0x7fffu) ? 1u : 0u) << (2 * t) | ((q[t] & 0x7fff0000u) ? 2u : 0u) << (2 * t);
+          b <<= 8 * (lane & 3);
+          b |= __shfl_xor_sync(0xffffffffu, b, 1);
+          b |= __shfl_xor_sync(0xffffffffu, b, 2);
+          if ((lane & 3) == 0) { words[(v * NZ_THREADS + tid) >> 2] = b; cnt += __popc(b); }
+        }
+      } else {
+        const float4* src = reinterpret_cast<const float4*>(reinterpret_cast<const float*>(R.x) + base);
+        float4 u[8];
+#pragma unroll
+        for (int v = 0; v < 8; ++v) u[v] = src[v * NZ_THREADS + tid];
+#pragma unroll
+        for (int v = 0; v < 8; ++v) {     // four elements per thread: eight threads make a word
+          unsigned b = (u[v].x != 0.f ? 1u : 0u) | (u[v].y != 0.f ? 2u : 0u) | (u[v].z != 0.f ? 4u : 0u) | (u[v].w != 0.f ? 8u : 0u);
+          b <<= 4 * (lane & 7);
+          b |= __shfl_xor_sync(0xffffffffu, b, 1);
+          b |= __shfl_xor_sync(0xffffffffu, b, 2);
+          b |= __shfl_xor_sync(0xffffffffu, b, 4);
+          if ((lane & 7) == 0) { words[(v * NZ_THREADS + tid) >> 3] = b; cnt += __popc(b); }
+        }
+      }
+      continue;
+    }
+    // the request's last piece, or a caller's buffer that is not 16-byte aligned: a warp makes a word at a time
+    for (int w = tid >> 5; w < NZ_SUB / 32; w += NZ_THREADS / 32) {
+      const long long i = base + w * 32 + lane;
+      bool f = false;
+      if (i < R.numel)
+        f = p.is_bf16 ? (__bfloat162float(reinterpret_cast<const __nv_bfloat16*>(R.x)[i]) != 0.0f) : (reinterpret_cast<const float*>(R.x)[i] != 0.0f);
+      const unsigned b = __ballot_sync(0xffffffffu, f);
+      if (lane == 0) { words[w] = b; cnt += __popc(b); }
+    }
   }
+  const int total = nz_block_sum(cnt, warp_sums);
+  if (tid == 0) R.count[chunk] = total;
 }
-__global__ void __launch_bounds__(1024) nonzero_scan(NonZeroParams p) {
-  // single CTA, sequential over chunks of 1024 block counts
-  __shared__ int wt[32];
-  __shared__ int carry_s;
-  if (threadIdx.x == 0) carry_s = 0;
-  __syncthreads();
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  for (int base = 0; base < p.nblocks; base += 1024) {
-    const int i = base + threadIdx.x;
-    const int v = i < p.nblocks ? p.block_count[i] : 0;
-    int inc = v;
+__global__ void __launch_bounds__(NZ_THREADS) nonzero_write(const __grid_constant__ NonZeroBatch p) {
+  __shared__ int sums[3][NZ_THREADS / 32];
+  __shared__ unsigned short list[NZ_SUB];
+  const NonZeroReq& R = nz_find(p);
+  const int chunk = blockIdx.x - R.first, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const long long lo = chunk * R.chunk, hi = min(R.numel, lo + R.chunk);
+  ptx::pdl_wait();
+  ptx::pdl_launch();
+  int before = 0, all = 0;
+  for (int j = tid; j < R.chunks; j += NZ_THREADS) { const int c = R.count[j]; all += c; before += j < chunk ? c : 0; }
+  before = nz_block_sum(before, sums[0]);
+  const long long nnz = nz_block_sum(all, sums[1]);
+  if (chunk == 0 && tid == 0) *R.count_out = nnz;
+  long long off = before;
+  for (long long base = lo; base < hi; base += NZ_SUB) {
+    unsigned m = R.mask[(base >> 5) + tid];
+    const int mine = __popc(m);
+    int inc = mine;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) { const int t = __shfl_up_sync(0xffffffffu, inc, o); if (lane >= o) inc += t; }
-    if (lane == 31) wt[warp] = inc;
+    __syncthreads();                     // the previous piece's list and sums have been read
+    if (lane == 31) sums[2][warp] = inc;
     __syncthreads();
-    int woff = 0;
-    for (int w = 0; w < warp; ++w) woff += wt[w];
-    const int carry = carry_s;
-    if (i < p.nblocks) p.block_count[i] = carry + woff + inc - v;
+    int at = inc - mine, cnt = 0;
+#pragma unroll
+    for (int w = 0; w < NZ_THREADS / 32; ++w) { const int t = sums[2][w]; at += w < warp ? t : 0; cnt += t; }
+    while (m) {
+      const int b = __ffs(m) - 1;
+      m &= m - 1;
+      list[at++] = static_cast<unsigned short>(tid * 32 + b);
+    }
     __syncthreads();
-    if (threadIdx.x == 1023) carry_s = carry + woff + inc;
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) { p.block_count[p.nblocks] = carry_s; *p.count_out = carry_s; }
-}
-__global__ void __launch_bounds__(NZ_BLOCK) nonzero_write(NonZeroParams p) {
-  __shared__ int wc[32];
-  const long long i = static_cast<long long>(blockIdx.x) * NZ_BLOCK + threadIdx.x;
-  const bool f = nz_flag(p, i);
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const unsigned bal = __ballot_sync(0xffffffffu, f);
-  if (lane == 0) wc[warp] = __popc(bal);
-  __syncthreads();
-  if (!f) return;
-  int off = p.block_count[blockIdx.x] + __popc(bal & ((1u << lane) - 1));
-  for (int w = 0; w < warp; ++w) off += wc[w];
-  const long long nnz = p.block_count[p.nblocks];
-  long long r = i;
-  for (int d = p.rank - 1; d >= 0; --d) {
-    p.out[static_cast<long long>(d) * nnz + off] = r % p.dims[d];
-    r /= p.dims[d];
+    long long* out = R.out + off;
+    if (R.numel < (1ll << 32)) {
+      const unsigned d1 = static_cast<unsigned>(R.dims[1]), d2 = static_cast<unsigned>(R.dims[2]), d3 = static_cast<unsigned>(R.dims[3]);
+      for (int j = tid; j < cnt; j += NZ_THREADS) {
+        const unsigned e = static_cast<unsigned>(base) + list[j];
+        long long* o = out + j + (p.rank - 1) * nnz;
+        unsigned q = e / d3;
+        *o = e - q * d3;
+        if (p.rank > 1) {
+          if (p.rank == 2) { o[-nnz] = q; continue; }
+          const unsigned q2 = q / d2;
+          o[-nnz] = q - q2 * d2;
+          if (p.rank == 3) { o[-2 * nnz] = q2; continue; }
+          const unsigned q1 = q2 / d1;
+          o[-2 * nnz] = q2 - q1 * d1;
+          o[-3 * nnz] = q1;
+        }
+      }
+    } else {
+      for (int j = tid; j < cnt; j += NZ_THREADS) {
+        long long e = base + list[j];
+        for (int d = p.rank - 1; d >= 0; --d) {
+          const long long ext = R.dims[4 - p.rank + d];
+          out[d * nnz + j] = e % ext;
+          e /= ext;
+        }
+      }
+    }
+    off += cnt;
   }
 }
 

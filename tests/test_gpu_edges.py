@@ -1,6 +1,7 @@
 """Kernel edges on the GPU: sizes at the ends of tiles, items and dispatch rules, against the oracle."""
 import numpy as np
 import pytest
+import torch
 
 from oracle import interp as O
 from paper_2403_00176_b200 import workloads as WL
@@ -29,3 +30,32 @@ def test_chain_vectors_that_straddle_rows_and_tails(dtype, tol):
         ref = O.run(ir, {}, req.inputs)["y"]
         assert outs[r]["y"].shape == ref.shape
         assert O.rel_err(outs[r]["y"], ref) <= tol, req.syms
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("rank", [1, 2, 3, 4])
+def test_nonzero_chunks_words_and_ranks(dtype, rank):
+    # pieces of 8192 elements +- 1 (32-element words, 16-byte vectors), a request of several chunks, ten requests (two
+    # tables), an all-zero one, negative zeros, ranks 1 to 4; the coordinates are whole numbers: exact
+    names = ["A", "B", "C", "D"][:rank]
+    ir = "".join(f"sym {n} 0 100000\n" for n in names) + f"input x {dtype} [{','.join(names)}]\nnode NonZero x -> nz\noutput nz\n"
+    rng = np.random.default_rng(31)
+    sizes = [1, 31, 33, 8191, 8192, 8193, 16400, 40001, 7, 640]
+    reqs = []
+    for i, n in enumerate(sizes):
+        shape = {1: (n,), 2: (max(n // 7, 1), 7), 3: (max(n // 15, 1), 5, 3), 4: (max(n // 40, 1), 2, 5, 4)}[rank]
+        x = bf16_round(rng.standard_normal(shape).astype(np.float32))
+        x[rng.uniform(size=shape) < (1.0 if i == 8 else 0.5)] = -0.0
+        reqs.append(Request(dict(zip(names, shape)), {"x": x}))
+    wl = WL.Workload("nonzero_edges", dtype, ir, {}, names, ["nz"], {"batch_fn": lambda j: reqs})
+    _, p, outs = run_batch(wl, reqs)
+    for r, req in enumerate(reqs):
+        assert np.array_equal(outs[r]["nz"], np.array(np.nonzero(req.inputs["x"]))), req.syms
+    # the counts are read once per run: another run on other data must be read again
+    p.in_dev[0].zero_()
+    p.run()
+    assert all(o["nz"].shape == (rank, 0) for o in p.outputs())
+    p.in_dev[0].copy_(torch.from_numpy(p.in_host[0]))
+    p.run_graph()
+    again = p.outputs()
+    assert all(np.array_equal(a["nz"], b["nz"]) for a, b in zip(again, outs))
