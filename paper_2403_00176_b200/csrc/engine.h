@@ -334,7 +334,8 @@ struct Plan {
   // groups that run beside their predecessor on a second stream (forked before the predecessor's first launch,
   // joined after their own last one): both only read what came before and write their own outputs
   std::vector<char> side_group;           // [group]
-  void* side_stream = nullptr;            // cudaStream_t
+  int side_device = 0;
+  void* side_stream = nullptr;            // cudaStream_t, from a pool (exec.cu)
   void* ev_fork = nullptr;                // cudaEvent_t
   void* ev_join = nullptr;                // cudaEvent_t
   std::vector<const void*> graph_key;     // inputs, outputs, arena the graph was captured with

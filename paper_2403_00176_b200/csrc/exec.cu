@@ -2431,27 +2431,56 @@ Status read_counts(Plan* p, const void* arena, void* stream) {
   return OK;
 }
 
+// Second streams (with their fork and join events) are parked between plans: a plan is made per batch, and creating
+// and destroying the three cost 55 + 60 us of host time, more than planning and launching a convolution stage.
+namespace {
+struct SideSet { int device; void *stream, *fork, *join; };
+constexpr size_t SIDE_MAX = 8;
+struct SidePool { std::mutex mu; std::vector<SideSet> parked; };
+SidePool& side_pool() { static SidePool* p = new SidePool; return *p; }           // never destroyed, as above
+}  // namespace
+
 Plan::~Plan() {
   if (graph_exec) cudaGraphExecDestroy(static_cast<cudaGraphExec_t>(graph_exec));
   if (capture_stream) cudaStreamDestroy(static_cast<cudaStream_t>(capture_stream));
-  if (side_stream) cudaStreamDestroy(static_cast<cudaStream_t>(side_stream));
-  if (ev_fork) cudaEventDestroy(static_cast<cudaEvent_t>(ev_fork));
-  if (ev_join) cudaEventDestroy(static_cast<cudaEvent_t>(ev_join));
+  if (side_stream) {
+    // work may still be in flight on it: whoever takes it next is ordered behind that
+    SidePool& P = side_pool();
+    std::lock_guard<std::mutex> lk(P.mu);
+    if (P.parked.size() < SIDE_MAX) {
+      P.parked.push_back(SideSet{side_device, side_stream, ev_fork, ev_join});
+    } else {
+      cudaStreamDestroy(static_cast<cudaStream_t>(side_stream));
+      cudaEventDestroy(static_cast<cudaEvent_t>(ev_fork));
+      cudaEventDestroy(static_cast<cudaEvent_t>(ev_join));
+    }
+  }
 }
 
-// The second stream and the two events of a plan with side groups (made outside any stream capture).
+// The second stream and the two events of a plan with side groups (taken outside any stream capture).
 static bool ensure_side_stream(Plan* p) {
   bool any = false;
   for (char c : p->side_group) any = any || c;
   if (!any || p->side_stream) return true;
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return false;
+  {
+    SidePool& P = side_pool();
+    std::lock_guard<std::mutex> lk(P.mu);
+    for (size_t i = 0; i < P.parked.size(); ++i)
+      if (P.parked[i].device == dev) {
+        const SideSet q = P.parked[i];
+        P.parked.erase(P.parked.begin() + i);
+        p->side_device = dev; p->side_stream = q.stream; p->ev_fork = q.fork; p->ev_join = q.join;
+        return true;
+      }
+  }
   cudaStream_t s;
   cudaEvent_t a, b;
   if (cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking) != cudaSuccess) return false;
-  if (cudaEventCreateWithFlags(&a, cudaEventDisableTiming) != cudaSuccess || cudaEventCreateWithFlags(&b, cudaEventDisableTiming) != cudaSuccess) {
-    cudaStreamDestroy(s);
-    return false;
-  }
-  p->side_stream = s; p->ev_fork = a; p->ev_join = b;
+  if (cudaEventCreateWithFlags(&a, cudaEventDisableTiming) != cudaSuccess) { cudaStreamDestroy(s); return false; }
+  if (cudaEventCreateWithFlags(&b, cudaEventDisableTiming) != cudaSuccess) { cudaEventDestroy(a); cudaStreamDestroy(s); return false; }
+  p->side_device = dev; p->side_stream = s; p->ev_fork = a; p->ev_join = b;
   return true;
 }
 
