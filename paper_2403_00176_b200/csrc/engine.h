@@ -1,8 +1,10 @@
 // Fused groups, per-request binding, arena memory plan and launch plan.
 #pragma once
 #include <initializer_list>
+#include <map>
 #include <memory>
 #include <new>
+#include <set>
 #include <string>
 #include <type_traits>
 #include <vector>
@@ -284,6 +286,22 @@ struct Ptr {                  // address resolved at run time
 
 struct Launch;                // defined in exec.cu
 
+// What building the launches of one group leaves for later groups (exec.cu); carried from stage to stage when the
+// groups of a graph are planned a few at a time.
+struct BuildState {
+  std::map<int, size_t> switch_aux;   // persistent side storage of a Switch (index lists), found again by the Combine
+                                      // through the gate tensor -> offset inside the aux region
+  size_t aux_need = 0;
+  std::set<int> partition_fused;      // gate tensors whose id partition is computed by the gate kernel
+  int n_tickets = 0;
+  // Per-sample channel sums carried from gate to gate (aux region): `gapsum_root` is the storage root whose
+  // current contents the table at `gapsum_aux` describes.  A gate on that storage skips the pooling pass; the
+  // last convolution of an in-place block (group index in gap_accum) adds the executed samples' new sums.
+  int gapsum_root = -1;
+  size_t gapsum_aux = 0;
+  std::map<int, size_t> gap_accum;    // convolution group -> offset of the table it accumulates into
+};
+
 struct Plan {
   const Compiled* c = nullptr;
   const Binding* b = nullptr;
@@ -316,11 +334,16 @@ struct Plan {
   // Staged planning (exact handling of execution-determined extents): `pinned` roots keep the arena offsets an
   // earlier stage gave them; `front_reserve` > 0 puts the group scratch (front_scratch bytes) and the Switch index
   // lists behind the header instead of behind the tensors, so that neither moves between stages.
-  std::vector<std::pair<int, size_t>> pinned;
+  struct Pinned { int t; size_t off; int64_t bytes; };
+  std::vector<Pinned> pinned;
   size_t front_reserve = 0, front_scratch = 0, header_end = 0;
   // a staged plan lays out only the tensors of its own steps: those defined at or before place_until_step and still
   // live at place_from_step (earlier ones are dead, later ones are planned by a later stage, at their true sizes)
   int place_from_step = 0, place_until_step = 1 << 30;
+  // ... and resolves and builds only its own groups: which tensor owns which bytes and how long it lives do not depend
+  // on the counts and are taken from the bounded plan
+  const Plan* stage_of = nullptr;
+  BuildState* build_state = nullptr;
   // [group] run-time symbols (atom ids) whose counts are in the arena header once the group has run: a gate whose
   // kernel also partitions the sample ids, a Switch that partitions them itself, a NonZero
   std::vector<std::vector<int>> rt_syms_after;

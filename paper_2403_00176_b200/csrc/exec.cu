@@ -175,7 +175,7 @@ cudaError_t gemm_pair_dispatch(int act, bool res, dim3 grid, cudaStream_t st, co
   }
 }
 
-struct Builder {
+struct Builder : BuildState {
   Plan& p;
   const Compiled& c;
   const Graph& g;
@@ -1811,17 +1811,6 @@ struct Builder {
     rc.b = static_cast<int>(v1 - v0);
     return rc;
   }
-  // persistent side storage of a Switch (index lists), found again by the Combine through the gate tensor
-  std::map<int, size_t> switch_aux;   // gate tensor -> offset inside the aux region
-  size_t aux_need = 0;
-  std::set<int> partition_fused;      // gate tensors whose id partition is computed by the gate kernel
-  int n_tickets = 0;
-  // Per-sample channel sums carried from gate to gate (aux region): `gapsum_root` is the storage root whose
-  // current contents the table at `gapsum_aux` describes.  A gate on that storage skips the pooling pass; the
-  // last convolution of an in-place block (group index in gap_accum) adds the executed samples' new sums.
-  int gapsum_root = -1;
-  size_t gapsum_aux = 0;
-  std::map<int, size_t> gap_accum;    // convolution group -> offset of the table it accumulates into
 
   // ------------------------------------------------------------------------------ gate (decision scalar)
   Status build_gate(int gi, const Group& G) {
@@ -1879,7 +1868,7 @@ struct Builder {
         for (size_t ci = 0; ci < c.groups.size() && writer < 0; ++ci) {
           const Group& Cb = c.groups[ci];
           if (Cb.kind != GKind::COMBINE || Cb.gate != G.out || c.storage[Cb.out].kind != Storage::ALIAS) continue;
-          if (p.views[Cb.out].empty() || p.root_of[Cb.out] != xroot) continue;
+          if (p.root_of[Cb.out] != xroot) continue;
           in_place = true;
           for (size_t wi = 0; wi < c.groups.size(); ++wi) {
             const Group& Wg = c.groups[wi];
@@ -2176,7 +2165,10 @@ struct Builder {
         for (int k = 0; k < 32; ++k) if (n[k]) fprintf(stderr, "[sod2] launches: %-10s %3d groups %.1f us\n", gkind_name(static_cast<GKind>(k)), n[k], us[k]);
       }
     } kt(prof);
-    for (size_t gi = 0; gi < c.groups.size(); ++gi) {
+    if (p.build_state) static_cast<BuildState&>(*this) = *p.build_state;
+    const size_t first_group = p.stage_of ? static_cast<size_t>(p.place_from_step) : 0;
+    const size_t end_group = p.stage_of ? std::min(c.groups.size(), static_cast<size_t>(p.place_until_step) + 1) : c.groups.size();
+    for (size_t gi = first_group; gi < end_group; ++gi) {
       const Group& G = c.groups[gi];
       Status s = OK;
       struct Tick {
@@ -2188,7 +2180,7 @@ struct Builder {
         // the first member builds the launch for the whole chain
         if (p.chains[p.chain_of[gi]].groups.front() == static_cast<int>(gi)) s = build_gemm_chain(p.chain_of[gi]);
         if (s != OK) return s;
-        cost(G);
+        if (!p.stage_of) cost(G);
         continue;
       }
       switch (G.kind) {
@@ -2213,8 +2205,9 @@ struct Builder {
         default: return fail(E_UNSUPPORTED_OP, std::string("no executor yet for group kind ") + gkind_name(G.kind));
       }
       if (s != OK) return s;
-      cost(G);
+      if (!p.stage_of) cost(G);
     }
+    if (p.build_state) *p.build_state = *this;
     if (p.front_reserve) {
       // staged plan: scratch and index lists at the fixed places behind the header that the first stage chose
       const size_t sc = (scratch_need + 255) & ~size_t(255), ax = (aux_need + 255) & ~size_t(255);
@@ -2683,6 +2676,7 @@ Status run_exact(const Compiled* c, const Binding* b0, const Plan* bounded, cons
   std::vector<std::vector<std::pair<int, int64_t>>> rt(n_req);
   int64_t plan_ns = 0, launches = 0, stages = 0;
   size_t peak_extent = 0;
+  BuildState built;
   auto make_stage = [&](const Plan* prev, int first_step, int last_step) -> Status {
     auto tp = std::chrono::steady_clock::now();
     std::unique_ptr<Binding> nb(new Binding());
@@ -2693,10 +2687,12 @@ Status run_exact(const Compiled* c, const Binding* b0, const Plan* bounded, cons
     np->front_scratch = front_scratch;
     np->place_from_step = first_step;
     np->place_until_step = last_step;
+    np->stage_of = bounded;
+    np->build_state = &built;
     if (prev)
       for (size_t t = 0; t < prev->roots.size(); ++t) {
         const RootBuf& R = prev->roots[t];
-        if (R.where == RootBuf::ARENA && R.def_step >= 0 && R.def_step < first_step && R.last_step >= first_step) np->pinned.push_back({static_cast<int>(t), R.arena_off});
+        if (R.where == RootBuf::ARENA && R.def_step >= 0 && R.def_step < first_step && R.last_step >= first_step) np->pinned.push_back({static_cast<int>(t), R.arena_off, R.bytes});
       }
     s = make_plan(c, nb.get(), np.get());
     if (s != OK) { *err = np->err; return s; }

@@ -409,6 +409,7 @@ struct Planner {
     p.views.reset(T, p.n_req);   // rows are made per tensor when it is resolved
     p.root_of.assign(T, -1);
     p.roots.assign(T, RootBuf());
+    if (p.stage_of) return run_stage();
     // resolve every tensor a group touches
     for (auto& G : c.groups) {
       if (G.kind == GKind::UNSUPPORTED) return fail(E_UNSUPPORTED_OP, "group around " + g.nodes[G.nodes[0]].op + ": " + G.why);
@@ -459,6 +460,24 @@ struct Planner {
       fprintf(stderr, "[sod2] plan: views %.1f us (%d tensors, %d table rows filled), liveness %.1f us, arena %.1f us\n", us(t0, t1), n_res, n_rep, us(t1, t2), us(t2, t3));
     }
     return s;
+  }
+
+  // A stage of a staged plan: its own groups only.
+  Status run_stage() {
+    const Plan& B = *p.stage_of;
+    p.root_of = B.root_of;
+    for (size_t t = 0; t < p.roots.size(); ++t) { p.roots[t].def_step = B.roots[t].def_step; p.roots[t].last_step = B.roots[t].last_step; }
+    for (auto& pin : p.pinned) { p.roots[pin.t].where = RootBuf::ARENA; p.roots[pin.t].bytes = pin.bytes; }
+    const int last = std::min(p.place_until_step, static_cast<int>(c.groups.size()) - 1);
+    for (int s = p.place_from_step; s <= last; ++s) {
+      const Group& G = c.groups[s];
+      for (int t : G.ext_in) { Status st = resolve(t); if (st != OK) return st; }
+      for (int t : G.ext_out) { Status st = resolve(t); if (st != OK) return st; }
+    }
+    p.chain_of = B.chain_of;
+    p.chains = B.chains;
+    p.chain_counter_words = B.chain_counter_words;
+    return plan_arena(static_cast<int>(c.groups.size()));
   }
 
   // Peak-first greedy: place the tensors live at the peak step contiguously, then walk forward
@@ -523,13 +542,13 @@ struct Planner {
     std::vector<char> done(p.roots.size(), 0);
     // 0. tensors an earlier stage has already placed (and filled) stay where they are
     for (auto& pin : p.pinned) {
-      const int t = pin.first;
+      const int t = pin.t;
       if (t < 0 || t >= static_cast<int>(p.roots.size()) || p.roots[t].where != RootBuf::ARENA || p.roots[t].def_step < 0) continue;
       if (std::find(ids.begin(), ids.end(), t) == ids.end()) continue;
-      if (pin.second < HEADER) return fail(E_INTERNAL, "pinned tensor inside the arena header");
-      p.roots[t].arena_off = pin.second;
-      placed.push_back({pin.second, sz(t), p.roots[t].def_step, p.roots[t].last_step});
-      top = std::max(top, pin.second + sz(t));
+      if (pin.off < HEADER) return fail(E_INTERNAL, "pinned tensor inside the arena header");
+      p.roots[t].arena_off = pin.off;
+      placed.push_back({pin.off, sz(t), p.roots[t].def_step, p.roots[t].last_step});
+      top = std::max(top, pin.off + sz(t));
       done[t] = 1;
     }
     // 1. live set at the peak, in (def step, id) order
