@@ -102,6 +102,7 @@ def _load() -> C.CDLL:
 
 
 lib = _load()
+from . import _sod2calls as _calls  # noqa: E402  (the per-batch calls; links to the library loaded above)
 EXPORTS = ["sod2_graph_create", "sod2_graph_destroy", "sod2_graph_set_const", "sod2_graph_prepack_bytes",
            "sod2_graph_prepack", "sod2_bind_dims", "sod2_binding_destroy", "sod2_plan", "sod2_plan_destroy", "sod2_graph_set_plan_cache", "sod2_plan_cached",
            "sod2_run", "sod2_run_graph", "sod2_run_exact", "sod2_run_timed", "sod2_run_timed_repeat", "sod2_plan_device_status", "sod2_plan_poison_arena", "sod2_plan_check_guards", "sod2_graph_tensor_info", "sod2_graph_tensor_value", "sod2_graph_tensor_dtype",
@@ -161,6 +162,7 @@ class Graph:
         h = C.c_void_p()
         _check(lib.sod2_graph_create(raw, len(raw), opt_flags, C.byref(h)))
         self.h = h
+        self._addr = h.value
         self._keep = []
 
     def __del__(self):
@@ -196,9 +198,9 @@ class Graph:
         hb, hp, ab, hit = C.c_void_p(), C.c_void_p(), C.c_size_t(), C.c_int()
         _check(lib.sod2_plan_cached(self.h, n_req, n_sym, names, vals, C.byref(hb), C.byref(hp), C.byref(ab), C.byref(hit)), self.h)
         b = Binding.__new__(Binding)
-        b.graph, b.h, b.n_req, b.borrowed = self, hb, n_req, True
+        b.graph, b._addr, b.n_req, b.borrowed = self, hb.value, n_req, True
         p = Plan.__new__(Plan)
-        p.binding, p.graph, p.h, p.arena_bytes, p.borrowed = b, self, hp, ab.value, True
+        p.binding, p.graph, p._addr, p.arena_bytes, p.borrowed = b, self, hp.value, ab.value, True
         return b, p, bool(hit.value)
 
     def bind_dims(self, sym_names: Sequence[str], values: Sequence[Sequence[int]]) -> "Binding":
@@ -259,24 +261,32 @@ class Graph:
         _check(lib.sod2_graph_reanalyse(self.h, arr, len(order)), self.h)
 
 
-class Binding:
+class _Handle:
+    """A library handle: `_addr` for the per-batch calls, `h` for ctypes."""
+
+    _addr = None
+    borrowed = False
+
+    @property
+    def h(self) -> C.c_void_p:
+        return C.c_void_p(self._addr)
+
+
+class Binding(_Handle):
     """sod2_binding handle (per-request symbol values)."""
 
     def __init__(self, graph: Graph, sym_names: Sequence[str], values: Sequence[Sequence[int]]):
         self.graph = graph
-        n_req, n_sym = len(values), len(sym_names)
-        names = (C.c_char_p * max(n_sym, 1))(*[s.encode() for s in sym_names])
-        flat = [int(v) for row in values for v in row]
-        vals = (C.c_int64 * max(len(flat), 1))(*flat)
-        h = C.c_void_p()
-        _check(lib.sod2_bind_dims(graph.h, n_req, n_sym, names, vals, C.byref(h)), graph.h)
-        self.h = h
-        self.n_req = n_req
+        status, addr = _calls.bind(graph._addr, sym_names, values)
+        if status:
+            _check(status, graph.h)
+        self._addr = addr
+        self.n_req = len(values)
 
     def __del__(self):
-        if getattr(self, "h", None) and lib is not None and not getattr(self, "borrowed", False):   # lib is None at shutdown
-            lib.sod2_binding_destroy(self.h)
-            self.h = None
+        if self._addr and _calls is not None and not self.borrowed:   # _calls is None at shutdown
+            _calls.binding_destroy(self._addr)
+            self._addr = None
 
     def shape(self, request: int, tensor: str) -> List[int]:
         dims = (C.c_int64 * 16)()
@@ -288,46 +298,40 @@ class Binding:
         return Plan(self)
 
 
-class Plan:
+class Plan(_Handle):
     """sod2_plan_t handle (arena plan + launch plan)."""
 
     def __init__(self, binding: Binding):
         self.binding = binding
         self.graph = binding.graph
-        h = C.c_void_p()
-        ab = C.c_size_t()
-        _check(lib.sod2_plan(self.graph.h, binding.h, C.byref(h), C.byref(ab)), self.graph.h)
-        self.h = h
-        self.arena_bytes = ab.value
+        status, addr, self.arena_bytes = _calls.plan(self.graph._addr, binding._addr)
+        if status:
+            _check(status, self.graph.h)
+        self._addr = addr
 
     def __del__(self):
-        if getattr(self, "h", None) and lib is not None and not getattr(self, "borrowed", False):   # lib is None at shutdown
-            lib.sod2_plan_destroy(self.h)
-            self.h = None
+        if self._addr and _calls is not None and not self.borrowed:   # _calls is None at shutdown
+            _calls.plan_destroy(self._addr)
+            self._addr = None
+
+    def _run(self, how, inputs, outputs, arena, arena_bytes, stream) -> RunInfo:
+        info = RunInfo()
+        status = _calls.run(how, self._addr, inputs, outputs, arena, arena_bytes, stream, info)
+        if status:
+            _check(status, self.h)
+        return info
 
     def run(self, inputs: Sequence[int], outputs: Sequence[int], arena: int, arena_bytes: int, stream: int) -> RunInfo:
-        ins = (C.c_void_p * max(len(inputs), 1))(*inputs)
-        outs = (C.c_void_p * max(len(outputs), 1))(*outputs)
-        info = RunInfo()
-        _check(lib.sod2_run(self.h, ins, outs, C.c_void_p(arena), arena_bytes, C.c_void_p(stream), C.byref(info)), self.h)
-        return info
+        return self._run(0, inputs, outputs, arena, arena_bytes, stream)
 
     def run_graph(self, inputs: Sequence[int], outputs: Sequence[int], arena: int, arena_bytes: int, stream: int) -> RunInfo:
         """The same inference as one CUDA graph (captured on first use and when a buffer pointer changes)."""
-        ins = (C.c_void_p * max(len(inputs), 1))(*inputs)
-        outs = (C.c_void_p * max(len(outputs), 1))(*outputs)
-        info = RunInfo()
-        _check(lib.sod2_run_graph(self.h, ins, outs, C.c_void_p(arena), arena_bytes, C.c_void_p(stream), C.byref(info)), self.h)
-        return info
+        return self._run(1, inputs, outputs, arena, arena_bytes, stream)
 
     def run_exact(self, inputs: Sequence[int], outputs: Sequence[int], arena: int, arena_bytes: int, stream: int) -> RunInfo:
         """The inference with exact handling of execution-determined extents: counts read back after every Switch /
         NonZero, the remaining sub-graphs planned again at their true sizes (synchronises the stream at each)."""
-        ins = (C.c_void_p * max(len(inputs), 1))(*inputs)
-        outs = (C.c_void_p * max(len(outputs), 1))(*outputs)
-        info = RunInfo()
-        _check(lib.sod2_run_exact(self.h, ins, outs, C.c_void_p(arena), arena_bytes, C.c_void_p(stream), C.byref(info)), self.h)
-        return info
+        return self._run(2, inputs, outputs, arena, arena_bytes, stream)
 
     def run_timed(self, inputs: Sequence[int], outputs: Sequence[int], arena: int, arena_bytes: int, stream: int, reps: int = 1) -> List[float]:
         """Device time per fused group (ms).  reps > 1: every launch repeated back to back, time divided by reps."""
@@ -388,8 +392,7 @@ class Plan:
         return bool(v.value)
 
     def output_shape(self, arena: int, stream: int, request: int, output: int) -> List[int]:
-        dims = (C.c_int64 * 16)()
-        rank = C.c_int()
-        _check(lib.sod2_run_output_shape(self.h, C.c_void_p(arena), C.c_void_p(stream), request, output, dims,
-                                         C.byref(rank)), self.h)
-        return list(dims[: rank.value])
+        dims = _calls.output_shape(self._addr, arena, stream, request, output)
+        if not isinstance(dims, list):
+            _check(dims, self.h)
+        return dims

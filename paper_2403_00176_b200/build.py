@@ -1,22 +1,24 @@
-"""Builds libsod2.so (host core + sm_100a kernels + C ABI) in-tree with nvcc."""
+"""Builds libsod2.so (host core + sm_100a kernels + C ABI) and the Python module over its per-batch calls, in-tree."""
 from __future__ import annotations
 
 import os
 import subprocess
 import sys
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libsod2.so")
+CALLS = os.path.join(HERE, "_sod2calls" + (sysconfig.get_config_var("EXT_SUFFIX") or ".so"))
 SOURCES = ["expr.cpp", "rdp.cpp", "fuse.cpp", "sep.cpp", "plan.cpp", "capi.cpp", "exec.cu", "noalloc.cu", "selftest_mma.cu"]
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
               "-Xcompiler", "-fPIC,-Wall,-Wno-unused-function", "--expt-relaxed-constexpr"]
 
 
 def _stale() -> bool:
-    if not os.path.exists(LIB):
+    if not os.path.exists(LIB) or not os.path.exists(CALLS):
         return True
-    t = os.path.getmtime(LIB)
+    t = min(os.path.getmtime(LIB), os.path.getmtime(CALLS))
     for root in (CSRC, os.path.join(HERE, "..", "include")):
         for f in os.listdir(root):
             if os.path.getmtime(os.path.join(root, f)) > t:
@@ -45,10 +47,15 @@ def build(force: bool = False, verbose: bool = False) -> str:
             raise RuntimeError(f"nvcc failed on {s}:\n{out}")
         if verbose and out.strip():
             print(out)
-    link = [nvcc, "-shared", "-o", LIB, *objs, "-gencode", "arch=compute_100a,code=sm_100a"]
+    link = [nvcc, "-shared", "-Xlinker", "-soname=libsod2.so", "-o", LIB, *objs, "-gencode", "arch=compute_100a,code=sm_100a"]
     r = subprocess.run(link, stdout=subprocess.PIPE, stderr=subprocess.STDOUT, text=True)
     if r.returncode != 0:
         raise RuntimeError(f"link failed:\n{r.stdout}")
+    cmd = [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared", "-Wall", "-I", sysconfig.get_paths()["include"],
+           os.path.join(CSRC, "pymodule.cpp"), "-o", CALLS, LIB, "-Wl,-rpath,$ORIGIN"]
+    r = subprocess.run(cmd, stdout=subprocess.PIPE, stderr=subprocess.STDOUT, text=True)
+    if r.returncode != 0:
+        raise RuntimeError(f"building the Python module failed:\n{r.stdout}")
     return LIB
 
 
