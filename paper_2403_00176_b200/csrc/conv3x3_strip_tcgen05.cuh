@@ -1,0 +1,291 @@
+// 3x3 / stride 1 / pad 1 convolution, 64 -> 64 channels (channels-last, bf16, tcgen05), in vertical strips.
+//
+// An MMA of N = 64 columns occupies the tensor pipe for about 72 cycles, one of N = 192 for 96: with one tap per
+// instruction a 64-channel layer cannot pass half of the pipe's rate.  Here an instruction carries the three dy taps of
+// one dx: the operand B is [dy = 2 | dy = 1 | dy = 0] x 64 output channels, and the result is what input row i gives to
+// the output rows i - 1, i and i + 1, whose accumulators lie side by side in tensor memory (a ring of eight 64-column
+// blocks; where the three blocks wrap around its end the instruction is cut in two).  The dx taps are the same rows of
+// shared memory through descriptors whose start address is shifted by a pixel.  So a CTA walks down a column of tiles
+// of 128 pixels, every input row is loaded ONCE per strip (one box of 130 pixels, zero-filled outside the image = the
+// padding), and takes 12 instructions instead of 36.
+//
+// Work is the list of all (request, image, column tile, row) tiles in that order; CTA b takes an equal, contiguous
+// share, which it walks in segments that do not leave their column.  A segment of L rows costs L + 2 input rows.
+//
+// Warps: 0 activation and weight TMA, 1 MMA issuer, 2 staging agent (residual prefetch + output stores), 4..19
+// epilogue: two groups of eight that take alternate rows (a row's accumulator -> activation -> residual -> staging is a
+// chain of about 2000 cycles against 1300 of the main loop).
+// SOD2_STRIP_FIGURES
+#pragma once
+#include <cuda.h>
+#include <cuda_bf16.h>
+#include "conv3x3_tcgen05.cuh"
+
+namespace sod2 {
+namespace k {
+
+constexpr int STRIP_THREADS = 640;
+constexpr int STRIP_STAGES = 5;              // input rows in flight
+constexpr int STRIP_NSB = 4;                 // staging buffers
+constexpr int STRIP_BLOCKS = 8;              // accumulator ring: 8 x 64 columns
+constexpr int STRIP_TAP = 64 * 128;          // one tap of the weights: 64 output channels x 64 input channels
+constexpr int STRIP_W = 9 * STRIP_TAP;
+constexpr int STRIP_SMEM = STRIP_W + STRIP_STAGES * C3_A_SLOT + STRIP_NSB * CONV_STAGE_OUT + 256 /*bias*/ +
+                           8 * (2 * STRIP_STAGES + 2 * STRIP_BLOCKS + 2 * STRIP_NSB + 1) + 16 + 1024 /*alignment*/;
+
+// B.tx: {64, W, H, N}, box {64, 130, 1, 1};  tmW: k-chunk view {64, 64, 9} of the weights in (dy, dx, ci) order, box
+// {64, 64, 1};  B.to / B.tr: {64, W, H, N}, box {64, 128, 1, 1}.  B.tile_start as for the row-halo kernel.
+template <int ACT, bool HASRES>
+__global__ void __launch_bounds__(STRIP_THREADS, 1)
+conv3x3_strip_bf16_tcgen05(const __grid_constant__ Conv3Batch B, const __grid_constant__ CUtensorMap tmW, ConvParams p) {
+  constexpr int NSB = STRIP_NSB, NB = STRIP_BLOCKS, ST = STRIP_STAGES;
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* wres = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  uint8_t* rows = wres + STRIP_W;
+  uint8_t* out_stage = rows + ST * C3_A_SLOT;
+  float* bias_s = reinterpret_cast<float*>(out_stage + NSB * CONV_STAGE_OUT);   // [64]
+  uint64_t* full = reinterpret_cast<uint64_t*>(bias_s + 64);
+  uint64_t* empty = full + ST;
+  uint64_t* tmem_full = empty + ST;
+  uint64_t* tmem_empty = tmem_full + NB;
+  uint64_t* res_full = tmem_empty + NB;
+  uint64_t* stage_ready = res_full + NSB;
+  uint64_t* w_full = stage_ready + NSB;
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(w_full + 1);
+  volatile int* dead = reinterpret_cast<volatile int*>(tmem_slot + 1);
+
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < ST; ++s) { ptx::mbar_init(&full[s], 1); ptx::mbar_init(&empty[s], 1); }
+    for (int b = 0; b < NB; ++b) { ptx::mbar_init(&tmem_full[b], 1); ptx::mbar_init(&tmem_empty[b], 8); }
+    for (int b = 0; b < NSB; ++b) { ptx::mbar_init(&res_full[b], 1); ptx::mbar_init(&stage_ready[b], 8); }
+    ptx::mbar_init(w_full, 1);
+    *dead = 0;
+    ptx::fence_barrier_init();
+    ptx::fence_proxy_async();
+    ptx::prefetch_tmap(&tmW);
+    for (int r = 0; r < B.n_req; ++r) {
+      ptx::prefetch_tmap(&B.tx[r]);
+      ptx::prefetch_tmap(&B.to[r]);
+      if (HASRES) ptx::prefetch_tmap(&B.tr[r]);
+    }
+  }
+  if (threadIdx.x >= 64 && threadIdx.x < 128) bias_s[threadIdx.x - 64] = p.bias ? __bfloat162float(p.bias[threadIdx.x - 64]) : 0.0f;
+  if (warp == 3) { ptx::tmem_alloc(tmem_slot, 512); ptx::tmem_relinquish(); }
+  ptx::tc_fence_before();
+  __syncthreads();
+  ptx::tc_fence_after();
+  const uint32_t tmem = *tmem_slot;
+  // the weights do not depend on the previous kernel; tap (dy, dx) goes to slot dx * 3 + 2 - dy
+  if (warp == 0 && lane == 0) {
+    ptx::mbar_expect_tx(w_full, STRIP_W);
+    for (int dx = 0; dx < 3; ++dx)
+      for (int dy = 2; dy >= 0; --dy) ptx::tma_load_3d(wres + (dx * 3 + 2 - dy) * STRIP_TAP, &tmW, 0, 0, dy * 3 + dx, w_full);
+  }
+  ptx::pdl_wait();
+  ptx::pdl_launch();
+  int total = B.tile_start[B.n_req];
+  if (p.n_img_ptr) {   // gated sub-batch (single request): the image count is on the device
+    const int n_img = min(p.n_img, max(0, p.cnt_a + p.cnt_b * static_cast<int>(*p.n_img_ptr)));
+    total = ((B.Wo[0] + 127) / 128) * B.Ho[0] * n_img;
+  }
+  const int begin = static_cast<int>(static_cast<long long>(total) * blockIdx.x / gridDim.x);
+  const int end = static_cast<int>(static_cast<long long>(total) * (blockIdx.x + 1) / gridDim.x);
+
+  // tile index -> request, image, row, first pixel; rows of a column vary fastest
+  auto decode = [&](int t, int* img, int* row, int* w0) -> int {
+    int r = 0;
+    while (r + 1 < B.n_req && t >= B.tile_start[r + 1]) ++r;
+    t -= B.tile_start[r];
+    const int per_img = ((B.Wo[r] + 127) / 128) * B.Ho[r];
+    *img = t / per_img;
+    const int rem = t - *img * per_img;
+    const int wt = rem / B.Ho[r];
+    *row = rem - wt * B.Ho[r];
+    *w0 = wt * 128;
+    return r;
+  };
+
+  if (warp == 0) {
+    if (lane == 0) {
+      // ---- input rows: a segment's L output rows need the L + 2 rows around them
+      int n = 0;
+      for (int t = begin; t < end;) {
+        int img, row, w0;
+        const int rq = decode(t, &img, &row, &w0);
+        const int len = min(end - t, B.Ho[rq] - row);
+        if (p.in_ids) img = p.in_ids[img];
+        for (int i = row - 1; i <= row + len; ++i, ++n) {
+          const int s = n % ST;
+          if (n >= ST) ptx::mbar_wait(&empty[s], ((n / ST) - 1) & 1, dead);
+          ptx::mbar_expect_tx(&full[s], C3_A_BYTES);
+          ptx::tma_load_4d(rows + s * C3_A_SLOT, &B.tx[rq], 0, w0 - 1, i, img, &full[s]);
+        }
+        t += len;
+      }
+    }
+  } else if (warp == 1) {
+    if (lane == 0) {
+      // ---- MMA issuer.  Output row o of the segment accumulates in block (j + o) % 8; input row ii (counted from the
+      // row above the segment) gives to the output rows ii - 2 (dy = 2), ii - 1 and ii, as far as they belong to the
+      // segment.  Row ii is touched for the first time: its very first instruction does not accumulate.
+      auto idesc = [](int blocks) { return ptx::idesc_bf16(128, 0) | static_cast<uint32_t>(blocks) << 20; };   // N = 64 * blocks
+      ptx::mbar_wait(w_full, 0, dead);
+      const uint64_t wdesc = ptx::smem_desc_sw128(ptx::smem_u32(wres));
+      constexpr uint64_t TAP = STRIP_TAP >> 4;
+      int n = 0, j = 0;
+      for (int t = begin; t < end;) {
+        int img, row, w0;
+        const int rq = decode(t, &img, &row, &w0);
+        const int len = min(end - t, B.Ho[rq] - row);
+        for (int ii = 0; ii < len + 2; ++ii, ++n) {
+          const bool fresh = ii < len;
+          const int lo = max(ii - 2, 0), cnt = min(ii, len - 1) - lo + 1;
+          const int b0 = (j + lo) % NB;
+          const int c1 = min(cnt, NB - b0), c2 = cnt - c1;            // blocks before and behind the ring's end
+          const uint64_t wb = wdesc + (lo - (ii - 2)) * TAP;
+          const uint32_t d1 = tmem + b0 * 64;
+          const uint32_t i1 = idesc(c1), i2 = idesc(c2);
+          if (fresh && j + ii >= NB) ptx::mbar_wait(&tmem_empty[(j + ii) % NB], (((j + ii) / NB) - 1) & 1, dead);
+          const int s = n % ST;
+          ptx::mbar_wait(&full[s], (n / ST) & 1, dead);
+          ptx::tc_fence_after();
+          const uint64_t ad = ptx::smem_desc_sw128(ptx::smem_u32(rows + s * C3_A_SLOT));
+          if (fresh) {
+            const int old = cnt - 1, o1 = min(old, c1), o2 = old - o1;
+            if (o1) ptx::mma_bf16(d1, ad, wb, idesc(o1), 1);
+            if (o2) ptx::mma_bf16(tmem, ad, wb + o1 * TAP, idesc(o2), 1);
+            ptx::mma_bf16(tmem + ((j + ii) % NB) * 64, ad, wb + old * TAP, idesc(1), 0);
+          } else {
+            ptx::mma_bf16(d1, ad, wb, i1, 1);
+            if (c2) ptx::mma_bf16(tmem, ad, wb + c1 * TAP, i2, 1);
+          }
+          if (c2 == 0) {
+#pragma unroll
+            for (int q = 1; q < 12; ++q) ptx::mma_bf16(d1, ad + (q >> 2) * 8 + 2 * (q & 3), wb + (q >> 2) * (3 * TAP) + 2 * (q & 3), i1, 1);
+          } else {
+            const uint64_t wc = wb + c1 * TAP;
+#pragma unroll
+            for (int q = 1; q < 12; ++q) {
+              ptx::mma_bf16(d1, ad + (q >> 2) * 8 + 2 * (q & 3), wb + (q >> 2) * (3 * TAP) + 2 * (q & 3), i1, 1);
+              ptx::mma_bf16(tmem, ad + (q >> 2) * 8 + 2 * (q & 3), wc + (q >> 2) * (3 * TAP) + 2 * (q & 3), i2, 1);
+            }
+          }
+          ptx::mma_commit(&empty[s]);
+          if (ii >= 2) ptx::mma_commit(&tmem_full[(j + ii - 2) % NB]);
+        }
+        j += len;
+        t += len;
+      }
+    }
+  } else if (warp == 2) {
+    if (lane == 0) {
+      // ---- staging agent: unit u = this CTA's u-th tile, in buffer u % NSB.  prepare(u) hands the buffer to the
+      // epilogue warps: with a residual it is TMA-loaded into the buffer (updated in place), otherwise a plain arrive.
+      // The buffer of unit u - 1 is free for unit u + NSB - 1 once its store, issued one unit ago, has read it.
+      const int U = end - begin;
+      auto prepare = [&](int u) {
+        const int bsel = u % NSB;
+        if (HASRES) {
+          int img, row, w0;
+          const int rq = decode(begin + u, &img, &row, &w0);
+          ptx::mbar_expect_tx(&res_full[bsel], CONV_STAGE_OUT);
+          ptx::tma_load_4d(out_stage + bsel * CONV_STAGE_OUT, &B.tr[rq], 0, w0, row, p.res_ids ? p.res_ids[img] : img, &res_full[bsel]);
+        } else {
+          ptx::mbar_arrive(&res_full[bsel]);
+        }
+      };
+      for (int u = 0; u < NSB && u < U; ++u) prepare(u);
+      for (int u = 0; u < U; ++u) {
+        const int bsel = u % NSB;
+        int img, row, w0;
+        const int rq = decode(begin + u, &img, &row, &w0);
+        const int img_o = p.out_ids ? p.out_ids[img] : img;
+        ptx::mbar_wait(&stage_ready[bsel], (u / NSB) & 1, dead);
+        tma_store_4d(&B.to[rq], out_stage + bsel * CONV_STAGE_OUT, 0, w0, row, img_o);
+        bulk_commit();
+        if (u >= 1 && u + NSB - 1 < U) {
+          asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
+          prepare(u + NSB - 1);
+        }
+      }
+      bulk_wait0();
+    }
+  } else if (warp >= 4) {
+    // ---- epilogue: group g (eight warps) takes the tiles j = g, g + 2, ...; warp (q, half) of a group owns TMEM lanes
+    // 32q..32q+31 and a 32-column half, a thread one pixel
+    const int g = (warp - 4) >> 3, e = (warp - 4) & 7;
+    const int q = warp & 3, half = e >> 2;
+    const int et = threadIdx.x - 128 - g * 256;
+    const int row = q * 32 + lane;
+    const float relu2_floor = p.act2 == ACT_RELU ? 0.0f : -INFINITY;
+    auto group_bar = [&]() { asm volatile("bar.sync %0, 256;" ::"r"(1 + g) : "memory"); };
+    const float4* bp4 = reinterpret_cast<const float4*>(bias_s + half * 32);
+    for (int j = g; j < end - begin; j += 2) {
+      const int blk = j % NB, bsel = j % NSB;
+      if (e == 0) ptx::mbar_wait_warp(&tmem_full[blk], (j / NB) & 1, dead);   // one polling warp, the others park at the barrier
+      group_bar();
+      ptx::tc_fence_after();
+      uint32_t r[32];
+      ptx::tmem_ld32(tmem + (static_cast<uint32_t>(q * 32) << 16) + blk * 64 + half * 32, r);
+      ptx::tmem_ld_wait();
+      ptx::tc_fence_before();
+      __syncwarp();
+      if (lane == 0) ptx::mbar_arrive(&tmem_empty[blk]);
+      float v[32];
+#pragma unroll
+      for (int i4 = 0; i4 < 8; ++i4) {
+        const float4 b4 = bp4[i4];
+        v[4 * i4] = apply_act<ACT>(__uint_as_float(r[4 * i4]) + b4.x);
+        v[4 * i4 + 1] = apply_act<ACT>(__uint_as_float(r[4 * i4 + 1]) + b4.y);
+        v[4 * i4 + 2] = apply_act<ACT>(__uint_as_float(r[4 * i4 + 2]) + b4.z);
+        v[4 * i4 + 3] = apply_act<ACT>(__uint_as_float(r[4 * i4 + 3]) + b4.w);
+      }
+      uint8_t* obase = out_stage + bsel * CONV_STAGE_OUT + row * 128;
+      ptx::mbar_wait_warp(&res_full[bsel], (j / NSB) & 1, dead);
+      uint4 pk[4];
+      if constexpr (HASRES) {
+        uint4 rv[4];      // loads together, then the arithmetic, then the stores (one buffer: never reordered by the compiler)
+#pragma unroll
+        for (int u = 0; u < 4; ++u) rv[u] = *reinterpret_cast<const uint4*>(obase + (((half * 4 + u) ^ (row & 7)) << 4));
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const __nv_bfloat162* h = reinterpret_cast<const __nv_bfloat162*>(&rv[u]);
+          __nv_bfloat162* oh = reinterpret_cast<__nv_bfloat162*>(&pk[u]);
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            const float2 f = __bfloat1622float2(h[i]);
+            oh[i] = __floats2bfloat162_rn(fmaxf(v[u * 8 + 2 * i] + f.x, relu2_floor), fmaxf(v[u * 8 + 2 * i + 1] + f.y, relu2_floor));
+          }
+        }
+      } else {
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          __nv_bfloat162* oh = reinterpret_cast<__nv_bfloat162*>(&pk[u]);
+#pragma unroll
+          for (int i = 0; i < 4; ++i) oh[i] = __floats2bfloat162_rn(v[u * 8 + 2 * i], v[u * 8 + 2 * i + 1]);
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < 4; ++u) *reinterpret_cast<uint4*>(obase + (((half * 4 + u) ^ (row & 7)) << 4)) = pk[u];
+      if (p.gap_sum) {
+        group_bar();                               // every row of the tile is in the staging buffer
+        int img, trow, w0;
+        const int rq = decode(begin + j, &img, &trow, &w0);
+        const int img_o = p.out_ids ? p.out_ids[img] : img;
+        const int wo = B.Wo[rq];
+        gap_accumulate_tile(out_stage + bsel * CONV_STAGE_OUT, et, p.gap_sum + static_cast<long long>(img_o) * 64, [&](int px) { return w0 + px < wo; });
+      }
+      ptx::fence_proxy_async();
+      __syncwarp();
+      if (lane == 0) ptx::mbar_arrive(&stage_ready[bsel]);
+    }
+  }
+  ptx::tc_fence_before();
+  __syncthreads();
+  if (warp == 3) ptx::tmem_dealloc(tmem, 512);
+  if (threadIdx.x == 0 && *dead && p.status) atomicExch(p.status, 1);
+}
+
+}  // namespace k
+}  // namespace sod2

@@ -5,8 +5,7 @@
 // are the same rows read through operand descriptors whose start address is shifted by dx rows (the
 // tensor core applies the 128-byte swizzle to absolute shared-memory addresses, so a start that is not
 // a multiple of 8 rows is fine).  Each input pixel therefore crosses L2 -> SM three times instead of
-// nine, and a stage carries 12 MMAs.  With RES (Cin = 64 and the 9 weight taps fit in shared memory) the
-// weights are loaded once per CTA and stay resident; otherwise they stream with the activations.
+// nine, and a stage carries 12 MMAs.  The weights stream with the activations.  (64 -> 64 channels: the strip kernel.)
 // Warps: 0 activation TMA, 1 weight TMA, 2 staging agent (residual prefetch + output stores), 3 and 12
 // MMA issuers (one TMEM accumulator each, alternate tiles), 4..11 epilogue.
 #pragma once
@@ -32,29 +31,25 @@ struct Conv3Batch {
   int Ho[C3_MAX_REQ], Wo[C3_MAX_REQ];
 };
 
-template <int BN, bool RES, int STAGES>
+template <int BN, int STAGES>
 struct Conv3Smem {
-  static constexpr int B_STAGE = RES ? 0 : 3 * BN * 128;
-  static constexpr int STAGE_BYTES = C3_A_SLOT + B_STAGE;
-  static constexpr int W_RES = RES ? 9 * BN * 128 : 0;
-  static constexpr int NSB = (BN == 128 && !RES) ? 1 : 2;   // staging buffers (what fits next to the ring)
-  static constexpr int TOTAL = W_RES + STAGES * STAGE_BYTES + NSB * CONV_STAGE_OUT + 896 + 2048 + 128;
+  static constexpr int STAGE_BYTES = C3_A_SLOT + 3 * BN * 128;
+  static constexpr int NSB = BN == 128 ? 1 : 2;   // staging buffers (what fits next to the ring)
+  static constexpr int TOTAL = STAGES * STAGE_BYTES + NSB * CONV_STAGE_OUT + 896 + 2048 + 128;
 };
 
 // B.tx: {Cin, W, H, N}, box {64, 130, 1, 1};  tmW: k-chunk view {64, Cout, K/64} of the weights in
 // (dy, channel chunk, dx, ci) order, box {64, BN, 3};  B.to / B.tr: {Cout, W, H, N}, box {64, 128, 1, 1}.
 // p.Ho / p.Wo / p.n_img are unused (per request in B); a run-time image count (p.n_img_ptr) is only
 // honoured for single-request launches and then replaces B.tile_start[1].
-template <int BN, bool RES, int STAGES, int ACT, bool HASRES>
+template <int BN, int STAGES, int ACT, bool HASRES>
 __global__ void __launch_bounds__(CONV3_THREADS, 1)
 conv3x3_rows_bf16_tcgen05(const __grid_constant__ Conv3Batch B, const __grid_constant__ CUtensorMap tmW, ConvParams p) {
-  using S = Conv3Smem<BN, RES, STAGES>;
+  using S = Conv3Smem<BN, STAGES>;
   constexpr int PASSES = BN / 64;
   constexpr int NSB = S::NSB;
   extern __shared__ uint8_t smem_raw[];
-  uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  uint8_t* wres = base;
-  uint8_t* tiles = base + S::W_RES;
+  uint8_t* tiles = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint8_t* out_stage = tiles + STAGES * S::STAGE_BYTES;
   float* bias_s = reinterpret_cast<float*>(out_stage + NSB * CONV_STAGE_OUT);  // [2][256]
   uint64_t* full = reinterpret_cast<uint64_t*>(bias_s + 512);
@@ -63,18 +58,16 @@ conv3x3_rows_bf16_tcgen05(const __grid_constant__ Conv3Batch B, const __grid_con
   uint64_t* tmem_empty = tmem_full + 2;
   uint64_t* res_full = tmem_empty + 2;
   uint64_t* stage_ready = res_full + 2;
-  uint64_t* w_full = stage_ready + 2;
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(w_full + 1);
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(stage_ready + 2);
   volatile int* dead = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   constexpr uint32_t TMEM_COLS = 2 * BN < 32 ? 32 : 2 * BN;
 
   if (threadIdx.x == 0) {
-    for (int s = 0; s < STAGES; ++s) { ptx::mbar_init(&full[s], RES ? 1 : 2); ptx::mbar_init(&empty[s], 1); }
+    for (int s = 0; s < STAGES; ++s) { ptx::mbar_init(&full[s], 2); ptx::mbar_init(&empty[s], 1); }
     for (int b = 0; b < 2; ++b) { ptx::mbar_init(&tmem_full[b], 1); ptx::mbar_init(&tmem_empty[b], 8); }
     for (int b = 0; b < 2; ++b) { ptx::mbar_init(&res_full[b], 1); ptx::mbar_init(&stage_ready[b], 8); }
-    ptx::mbar_init(w_full, 1);
     *dead = 0;
     ptx::fence_barrier_init();
     ptx::fence_proxy_async();
@@ -90,11 +83,6 @@ conv3x3_rows_bf16_tcgen05(const __grid_constant__ Conv3Batch B, const __grid_con
   __syncthreads();
   ptx::tc_fence_after();
   const uint32_t tmem = *tmem_slot;
-  // the weights do not depend on the previous kernel: resident weights are fetched before the wait
-  if (RES && warp == 1 && lane == 0) {
-    ptx::mbar_expect_tx(w_full, 9 * BN * 128);
-    for (int dy = 0; dy < 3; ++dy) ptx::tma_load_3d(wres + dy * 3 * BN * 128, &tmW, 0, 0, dy * 3, w_full);
-  }
   ptx::pdl_wait();
   ptx::pdl_launch();
   int tiles_px = B.tile_start[B.n_req];
@@ -141,8 +129,8 @@ conv3x3_rows_bf16_tcgen05(const __grid_constant__ Conv3Batch B, const __grid_con
       }
     }
   } else if (warp == 1) {
-    if (!RES && lane == 0) {
-      // ---- B producer (streaming weights): the three dx taps of (dy, chunk) are consecutive k-chunks
+    if (lane == 0) {
+      // ---- B producer: the three dx taps of (dy, chunk) are consecutive k-chunks
       int n = 0;
       for (int t = blockIdx.x; t < num_tiles; t += gridDim.x) {
         const int n0 = (t / tiles_px) * BN;
@@ -165,7 +153,6 @@ conv3x3_rows_bf16_tcgen05(const __grid_constant__ Conv3Batch B, const __grid_con
       // in-order producer cannot refill a slot twice while an issuer still owns an earlier stage).
       constexpr uint32_t idesc = ptx::idesc_bf16(128, BN);
       const int me = warp == 3 ? 0 : 1;
-      if (RES) ptx::mbar_wait(w_full, 0, dead);
       int n = 0, j = 0;
       for (int t = blockIdx.x; t < num_tiles; t += gridDim.x, ++j) {
         const int acc = j & 1;
@@ -182,7 +169,7 @@ conv3x3_rows_bf16_tcgen05(const __grid_constant__ Conv3Batch B, const __grid_con
           ptx::tc_fence_after();
           if (me == 0) { SOD2_TRACE(1, 200 + ks) }
           const uint32_t a = ptx::smem_u32(tiles + s * S::STAGE_BYTES);
-          const uint32_t b = RES ? ptx::smem_u32(wres) + ks * 3 * BN * 128 : a + C3_A_SLOT;
+          const uint32_t b = a + C3_A_SLOT;
 #pragma unroll
           for (int dx = 0; dx < 3; ++dx) {
             const uint64_t ad = ptx::smem_desc_sw128(a + dx * 128);     // rows shifted by dx pixels

@@ -12,6 +12,7 @@
 #include "attention.cuh"
 #include "attention_tcgen05.cuh"
 #include "conv_tcgen05.cuh"
+#include "conv3x3_strip_tcgen05.cuh"
 #include "conv3x3_tcgen05.cuh"
 #include "conv_stem_tcgen05.cuh"
 #include "engine.h"
@@ -1574,7 +1575,9 @@ struct Builder : BuildState {
     // the table of per-sample channel sums this convolution adds its outputs to (the last convolution of an
     // in-place gated block), or SIZE_MAX
     const size_t gap_table = gap_accum.count(gi) ? gap_accum[gi] : SIZE_MAX;
-    // requests that take the row-halo kernel are collected and launched together (up to C3_MAX_REQ per launch)
+    // 64 -> 64 channels, 3x3, stride 1, pad 1: the strip kernel instead of the row-halo kernel
+    const bool strip = Cin == 64 && Cout == 64;
+    // requests that take the row-halo or strip kernel are collected and launched together (up to C3_MAX_REQ per launch)
     struct RowsReq { Ptr px, po, pr; int H, W, Ho, Wo, n_img, n_in_map, n_out_map, n_res_map; k::ConvParams cp; bool rt; size_t rt_slot; long long ids_in, ids_res, ids_out; };
     std::vector<RowsReq> rows_reqs;
     Ptr pw_all; pw_all.where = 5; pw_all.off = static_cast<int64_t>(pk);
@@ -1582,7 +1585,6 @@ struct Builder : BuildState {
     auto emit_rows = [&](std::vector<RowsReq> batch) {
       const bool hb = G.bias >= 0, hr = G.res >= 0;
       const int act = G.act;
-      const bool wres = Cin == 64 && Cout == 64;
       const int K = 9 * Cin;
       const Ptr pw = pw_all, pb = pb_all;
       struct Cache { std::vector<const void*> key; CUtensorMap tw; k::Conv3Batch B; };
@@ -1613,7 +1615,7 @@ struct Builder : BuildState {
             B.Ho[i] = q.Ho; B.Wo[i] = q.Wo;
           }
           B.tile_start[batch.size()] = ts;
-          if (!encode_bf16_kchunks(&cache->tw, Wp, Cout, K, K, bn, 3)) return cudaErrorInvalidValue;
+          if (!encode_bf16_kchunks(&cache->tw, Wp, Cout, K, K, bn, strip ? 1 : 3)) return cudaErrorInvalidValue;
           cache->key = key;
         }
         k::ConvParams cp = batch[0].cp;
@@ -1626,29 +1628,37 @@ struct Builder : BuildState {
         cp.out_ids = batch[0].ids_out >= 0 ? reinterpret_cast<const int*>(auxb + batch[0].ids_out) : nullptr;
         cp.gap_sum = (gap_table != SIZE_MAX && batch.size() == 1) ? reinterpret_cast<double*>(const_cast<char*>(auxb) + gap_table) : nullptr;
         const dim3 gd(static_cast<unsigned>(std::min<long long>(tiles, x.plan->sm_count)));
-        const int variant = ((wres ? 4 : 0) + (bn == 128 ? 2 : 0) + (act == 2 ? 1 : 0)) * 2 + (hr ? 1 : 0);
-#define SOD2_CONV3_CASE(V, BN_, RES_, ST_, ACT_, HR_)                                                                    \
+        if (strip) {
+#define SOD2_STRIP(ACT_, HR_)                                                                                                            \
+          {                                                                                                                              \
+            static bool once = (cudaFuncSetAttribute(k::conv3x3_strip_bf16_tcgen05<ACT_, HR_>, cudaFuncAttributeMaxDynamicSharedMemorySize, \
+                                                     k::STRIP_SMEM), true);                                                              \
+            (void)once;                                                                                                                  \
+            return launch_pdl(k::conv3x3_strip_bf16_tcgen05<ACT_, HR_>, gd, dim3(k::STRIP_THREADS), k::STRIP_SMEM, x.stream, cache->B, cache->tw, cp); \
+          }
+          if (act == 2) { if (hr) SOD2_STRIP(2, true) else SOD2_STRIP(2, false) }
+          else { if (hr) SOD2_STRIP(0, true) else SOD2_STRIP(0, false) }
+#undef SOD2_STRIP
+        }
+        const int variant = ((bn == 128 ? 2 : 0) + (act == 2 ? 1 : 0)) * 2 + (hr ? 1 : 0);
+#define SOD2_CONV3_CASE(V, BN_, ST_, ACT_, HR_)                                                                          \
         case V: {                                                                                                        \
-          constexpr int smem = k::Conv3Smem<BN_, RES_, ST_>::TOTAL;                                                       \
-          static bool once = (cudaFuncSetAttribute(k::conv3x3_rows_bf16_tcgen05<BN_, RES_, ST_, ACT_, HR_>,               \
+          constexpr int smem = k::Conv3Smem<BN_, ST_>::TOTAL;                                                             \
+          static bool once = (cudaFuncSetAttribute(k::conv3x3_rows_bf16_tcgen05<BN_, ST_, ACT_, HR_>,                     \
                                                    cudaFuncAttributeMaxDynamicSharedMemorySize, smem), true);             \
           (void)once;                                                                                                    \
-          launch_pdl(k::conv3x3_rows_bf16_tcgen05<BN_, RES_, ST_, ACT_, HR_>, gd, dim3(k::CONV3_THREADS), smem, x.stream, cache->B, cache->tw, cp); \
+          launch_pdl(k::conv3x3_rows_bf16_tcgen05<BN_, ST_, ACT_, HR_>, gd, dim3(k::CONV3_THREADS), smem, x.stream, cache->B, cache->tw, cp); \
         } break;
         switch (variant) {
-          SOD2_CONV3_CASE(0, 64, false, 4, 0, false)
-          SOD2_CONV3_CASE(1, 64, false, 4, 0, true)
-          SOD2_CONV3_CASE(2, 64, false, 4, 2, false)
-          SOD2_CONV3_CASE(3, 64, false, 4, 2, true)
-          SOD2_CONV3_CASE(4, 128, false, 3, 0, false)
-          SOD2_CONV3_CASE(5, 128, false, 3, 0, true)
-          SOD2_CONV3_CASE(6, 128, false, 3, 2, false)
-          SOD2_CONV3_CASE(7, 128, false, 3, 2, true)
-          SOD2_CONV3_CASE(8, 64, true, 7, 0, false)
-          SOD2_CONV3_CASE(9, 64, true, 7, 0, true)
-          SOD2_CONV3_CASE(10, 64, true, 7, 2, false)
+          SOD2_CONV3_CASE(0, 64, 4, 0, false)
+          SOD2_CONV3_CASE(1, 64, 4, 0, true)
+          SOD2_CONV3_CASE(2, 64, 4, 2, false)
+          SOD2_CONV3_CASE(3, 64, 4, 2, true)
+          SOD2_CONV3_CASE(4, 128, 3, 0, false)
+          SOD2_CONV3_CASE(5, 128, 3, 0, true)
+          SOD2_CONV3_CASE(6, 128, 3, 2, false)
           default:
-          SOD2_CONV3_CASE(11, 64, true, 7, 2, true)
+          SOD2_CONV3_CASE(7, 128, 3, 2, true)
         }
 #undef SOD2_CONV3_CASE
         return cudaGetLastError();
@@ -1694,7 +1704,9 @@ struct Builder : BuildState {
         if (best < 0 || padded < best) { best = padded; cp.TW = tw; cp.TH = th; }
       }
       // wide images with a 3x3 / stride 1 / pad 1 kernel: row-halo kernel (a tile is 128 pixels of one row)
-      const bool rows = ks == 3 && G.stride == 1 && G.pad == 1 && cp.Wo >= 96 && ((cp.Wo + 127) / 128) * 128 * 4 <= cp.Wo * 5;
+      // (the strip kernel's tiles are the same, at less than half of the cost of any other: from half-full tiles on)
+      const int padded_w = ((cp.Wo + 127) / 128) * 128;
+      const bool rows = ks == 3 && G.stride == 1 && G.pad == 1 && (strip ? padded_w <= cp.Wo * 2 : cp.Wo >= 96 && padded_w * 4 <= cp.Wo * 5);
       if (rows) { cp.TW = 128; cp.TH = 1; }
       if (cp.TW * G.stride > 256 || cp.TH * G.stride > 256) return fail(E_UNSUPPORTED_OP, "convolution stride too large for the TMA box");
       const int H = static_cast<int>(vx.dims[2]), Wd = static_cast<int>(vx.dims[3]);

@@ -4,9 +4,10 @@ import pytest
 import torch
 
 from oracle import interp as O
+from paper_2403_00176_b200 import binding as B
 from paper_2403_00176_b200 import workloads as WL
 from paper_2403_00176_b200.workloads import Request, bf16_round
-from tests.gpu_harness import run_batch
+from tests.gpu_harness import lockstep, run_batch
 
 pytestmark = pytest.mark.gpu
 
@@ -59,3 +60,19 @@ def test_nonzero_chunks_words_and_ranks(dtype, rank):
     p.run_graph()
     again = p.outputs()
     assert all(np.array_equal(a["nz"], b["nz"]) for a, b in zip(again, outs))
+
+
+@pytest.mark.parametrize("shapes", [[(1, 64)], [(2, 127), (3, 128)], [(9, 129)], [(70, 65), (1, 300), (5, 257), (3, 3), (40, 192)], [(300, 66)]])
+def test_conv_strips_segments_and_ring(shapes):
+    # strips of the 64 -> 64 channel kernel: one row, segments shorter and longer than the accumulator ring (8 rows) and
+    # the row ring, column tiles with one pixel, several requests in one launch beside one below its width rule
+    wl = WL.cfg4(blocks=2)
+    rng = np.random.default_rng(41)
+    reqs = [Request({"H": h, "W": w}, {"x": bf16_round(rng.uniform(-1, 1, (1, 64, h, w)).astype(np.float32))}) for h, w in shapes]
+    s, p, outs = run_batch(wl, reqs, opt_flags=B.OPT_NO_REUSE)
+    for r, req in enumerate(reqs):
+        errs = lockstep(wl, s, p, outs, r, BF16_TOL)
+        assert max(errs.values()) <= BF16_TOL, (req.syms, errs)
+    p.run()
+    for a, b in zip(outs, p.outputs()):
+        assert all(np.array_equal(a[n], b[n]) for n in a)
