@@ -12,10 +12,12 @@
 // Work is the list of all (request, image, column tile, row) tiles in that order; CTA b takes an equal, contiguous
 // share, which it walks in segments that do not leave their column.  A segment of L rows costs L + 2 input rows.
 //
-// Warps: 0 activation and weight TMA, 1 MMA issuer, 2 staging agent (residual prefetch + output stores), 4..19
-// epilogue: two groups of eight that take alternate rows (a row's accumulator -> activation -> residual -> staging is a
+// Warps: 0 activation and weight TMA, 1 and 3 MMA issuers (alternate rows), 2 staging agent (residual prefetch + output
+// stores), 4..19 epilogue: two groups of eight that take alternate rows (a row's accumulator -> activation -> residual -> staging is a
 // chain of about 2000 cycles against 1300 of the main loop).
-// SOD2_STRIP_FIGURES
+// Measured on B200, 640x480 + 416x416 + 224x608 + 544x320 (6976 tiles): 92 us a layer with one tap per instruction, 60 here;
+// a row takes about 1500 cycles of which the MMAs are 1170 (1730 where the window wraps), the rest is the hand-over
+// between the issuers.
 #pragma once
 #include <cuda.h>
 #include <cuda_bf16.h>
@@ -25,13 +27,47 @@ namespace sod2 {
 namespace k {
 
 constexpr int STRIP_THREADS = 640;
-constexpr int STRIP_STAGES = 5;              // input rows in flight
-constexpr int STRIP_NSB = 4;                 // staging buffers
 constexpr int STRIP_BLOCKS = 8;              // accumulator ring: 8 x 64 columns
 constexpr int STRIP_TAP = 64 * 128;          // one tap of the weights: 64 output channels x 64 input channels
 constexpr int STRIP_W = 9 * STRIP_TAP;
+constexpr int STRIP_STAGES = 5;              // input rows in shared memory
+constexpr int STRIP_NSB = 4;                 // staging buffers (even: a buffer belongs to one epilogue group)
 constexpr int STRIP_SMEM = STRIP_W + STRIP_STAGES * C3_A_SLOT + STRIP_NSB * CONV_STAGE_OUT + 256 /*bias*/ +
-                           8 * (2 * STRIP_STAGES + 2 * STRIP_BLOCKS + 2 * STRIP_NSB + 1) + 16 + 1024 /*alignment*/;
+                           8 * (2 * STRIP_STAGES + 2 * STRIP_BLOCKS + 2 * STRIP_NSB + 3) + 16 + 1024 /*alignment*/;
+
+// One MMA whose descriptors differ from the others' only in their start addresses (low words, in units of 16 bytes).
+template <int BLOCKS>
+__device__ __forceinline__ void strip_mma(uint32_t d, uint32_t a_lo, uint32_t b_lo, uint32_t accumulate) {
+  constexpr uint32_t desc_hi = (1024u >> 4) | 1u << 14 | 2u << 29;      // ptx::smem_desc_sw128: row-group stride, version, 128-byte swizzle
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t.reg .b64 ad, bd;\n\t"
+      "setp.ne.b32 p, %4, 0;\n\t"
+      "mov.b64 ad, {%1, %5};\n\t"
+      "mov.b64 bd, {%2, %5};\n\t"
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], ad, bd, %3, p;\n\t}"
+      ::"r"(d), "r"(a_lo), "r"(b_lo), "n"(ptx::idesc_bf16(128, 64 * BLOCKS)), "r"(accumulate), "n"(desc_hi)
+      : "memory");
+}
+// One input row: three dx taps of 64 input channels onto C1 accumulator blocks from d1 and C2 behind the ring's end; the
+// last of them starts from zero (in its own block dn) if FRESH.  Everything but the start addresses is a constant: the
+// issuing thread has one MMA's time (96 cycles) for all its arithmetic, beside epilogue warps on its scheduler.
+template <int C1, int C2, bool FRESH>
+__device__ __forceinline__ void strip_row(uint32_t d1, uint32_t d2, uint32_t dn, uint32_t a_lo, uint32_t b_lo) {
+  constexpr uint32_t TAP = STRIP_TAP >> 4;
+  constexpr int OLD = C1 + C2 - 1, O1 = OLD < C1 ? OLD : C1, O2 = OLD - O1;
+#pragma unroll
+  for (int q = 0; q < 12; ++q) {
+    const uint32_t a = a_lo + (q >> 2) * 8 + 2 * (q & 3), b = b_lo + (q >> 2) * (3 * TAP) + 2 * (q & 3);
+    if (FRESH && q == 0) {
+      if constexpr (O1 > 0) strip_mma<O1>(d1, a, b, 1);
+      if constexpr (O2 > 0) strip_mma<O2>(d2, a, b + O1 * TAP, 1);
+      strip_mma<1>(dn, a, b + OLD * TAP, 0);
+    } else {
+      strip_mma<C1>(d1, a, b, 1);
+      if constexpr (C2 > 0) strip_mma<C2>(d2, a, b + C1 * TAP, 1);
+    }
+  }
+}
 
 // B.tx: {64, W, H, N}, box {64, 130, 1, 1};  tmW: k-chunk view {64, 64, 9} of the weights in (dy, dx, ci) order, box
 // {64, 64, 1};  B.to / B.tr: {64, W, H, N}, box {64, 128, 1, 1}.  B.tile_start as for the row-halo kernel.
@@ -51,7 +87,8 @@ conv3x3_strip_bf16_tcgen05(const __grid_constant__ Conv3Batch B, const __grid_co
   uint64_t* res_full = tmem_empty + NB;
   uint64_t* stage_ready = res_full + NSB;
   uint64_t* w_full = stage_ready + NSB;
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(w_full + 1);
+  uint64_t* turn = w_full + 1;             // [2] the other issuer has issued its row
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(turn + 2);
   volatile int* dead = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -60,6 +97,7 @@ conv3x3_strip_bf16_tcgen05(const __grid_constant__ Conv3Batch B, const __grid_co
     for (int b = 0; b < NB; ++b) { ptx::mbar_init(&tmem_full[b], 1); ptx::mbar_init(&tmem_empty[b], 8); }
     for (int b = 0; b < NSB; ++b) { ptx::mbar_init(&res_full[b], 1); ptx::mbar_init(&stage_ready[b], 8); }
     ptx::mbar_init(w_full, 1);
+    for (int b = 0; b < 2; ++b) ptx::mbar_init(&turn[b], 1);
     *dead = 0;
     ptx::fence_barrier_init();
     ptx::fence_proxy_async();
@@ -117,62 +155,66 @@ conv3x3_strip_bf16_tcgen05(const __grid_constant__ Conv3Batch B, const __grid_co
         if (p.in_ids) img = p.in_ids[img];
         for (int i = row - 1; i <= row + len; ++i, ++n) {
           const int s = n % ST;
-          if (n >= ST) ptx::mbar_wait(&empty[s], ((n / ST) - 1) & 1, dead);
+          if (n >= ST) ptx::mbar_wait_parked(&empty[s], ((n / ST) - 1) & 1, dead);
           ptx::mbar_expect_tx(&full[s], C3_A_BYTES);
           ptx::tma_load_4d(rows + s * C3_A_SLOT, &B.tx[rq], 0, w0 - 1, i, img, &full[s]);
         }
         t += len;
       }
     }
-  } else if (warp == 1) {
-    if (lane == 0) {
-      // ---- MMA issuer.  Output row o of the segment accumulates in block (j + o) % 8; input row ii (counted from the
+  } else if (warp == 1 || warp == 3) {
+    {
+      // ---- MMA issuers: rows alternate between two threads.  One thread's commits, address arithmetic and barrier
+      // waits between two rows leave the tensor pipe idle for about 300 cycles; here the next row's thread has done its
+      // waiting while this row's is issuing, and starts on its word (`turn`, passed on before the commits).  The rows
+      // stay in order, so sums do not depend on timing.  (A thread may wait on `full` and `tmem_empty` for its own rows
+      // only: its row n - 2 was issued after every earlier row had seen its barriers, so at row n each barrier is at most
+      // one phase away from the one waited for.)
+      // Output row o of the segment accumulates in block (j + o) % 8; input row ii (counted from the
       // row above the segment) gives to the output rows ii - 2 (dy = 2), ii - 1 and ii, as far as they belong to the
       // segment.  Row ii is touched for the first time: its very first instruction does not accumulate.
-      auto idesc = [](int blocks) { return ptx::idesc_bf16(128, 0) | static_cast<uint32_t>(blocks) << 20; };   // N = 64 * blocks
-      ptx::mbar_wait(w_full, 0, dead);
+      ptx::mbar_wait_warp(w_full, 0, dead);
       const uint64_t wdesc = ptx::smem_desc_sw128(ptx::smem_u32(wres));
-      constexpr uint64_t TAP = STRIP_TAP >> 4;
+      const int me = warp == 1 ? 0 : 1;
       int n = 0, j = 0;
       for (int t = begin; t < end;) {
         int img, row, w0;
         const int rq = decode(t, &img, &row, &w0);
         const int len = min(end - t, B.Ho[rq] - row);
         for (int ii = 0; ii < len + 2; ++ii, ++n) {
+          const int s = n % ST;
+          if ((n & 1) != me) continue;
           const bool fresh = ii < len;
           const int lo = max(ii - 2, 0), cnt = min(ii, len - 1) - lo + 1;
           const int b0 = (j + lo) % NB;
           const int c1 = min(cnt, NB - b0), c2 = cnt - c1;            // blocks before and behind the ring's end
-          const uint64_t wb = wdesc + (lo - (ii - 2)) * TAP;
+          const uint64_t wb = wdesc + (lo - (ii - 2)) * (STRIP_TAP >> 4);
           const uint32_t d1 = tmem + b0 * 64;
-          const uint32_t i1 = idesc(c1), i2 = idesc(c2);
-          if (fresh && j + ii >= NB) ptx::mbar_wait(&tmem_empty[(j + ii) % NB], (((j + ii) / NB) - 1) & 1, dead);
-          const int s = n % ST;
-          ptx::mbar_wait(&full[s], (n / ST) & 1, dead);
+          if (fresh && j + ii >= NB) ptx::mbar_wait_warp(&tmem_empty[(j + ii) % NB], (((j + ii) / NB) - 1) & 1, dead);
+          ptx::mbar_wait_warp(&full[s], (n / ST) & 1, dead);
+          if (n > 0) ptx::mbar_wait_warp(&turn[me], me ? (n >> 1) & 1 : ((n >> 1) - 1) & 1, dead);
           ptx::tc_fence_after();
           const uint64_t ad = ptx::smem_desc_sw128(ptx::smem_u32(rows + s * C3_A_SLOT));
-          if (fresh) {
-            const int old = cnt - 1, o1 = min(old, c1), o2 = old - o1;
-            if (o1) ptx::mma_bf16(d1, ad, wb, idesc(o1), 1);
-            if (o2) ptx::mma_bf16(tmem, ad, wb + o1 * TAP, idesc(o2), 1);
-            ptx::mma_bf16(tmem + ((j + ii) % NB) * 64, ad, wb + old * TAP, idesc(1), 0);
-          } else {
-            ptx::mma_bf16(d1, ad, wb, i1, 1);
-            if (c2) ptx::mma_bf16(tmem, ad, wb + c1 * TAP, i2, 1);
+          const uint32_t a_lo = static_cast<uint32_t>(ad), b_lo = static_cast<uint32_t>(wb);
+          const uint32_t dn = tmem + ((j + ii) % NB) * 64;
+          if (ptx::elect_one()) {
+          switch (c1 * 8 + c2 * 2 + (fresh ? 1 : 0)) {
+#define SOD2_STRIP_ROW(C1_, C2_) case C1_ * 8 + C2_ * 2: strip_row<C1_, C2_, false>(d1, tmem, dn, a_lo, b_lo); break; \
+                                 case C1_ * 8 + C2_ * 2 + 1: strip_row<C1_, C2_, true>(d1, tmem, dn, a_lo, b_lo); break;
+            SOD2_STRIP_ROW(3, 0)
+            SOD2_STRIP_ROW(2, 1)
+            SOD2_STRIP_ROW(1, 2)
+            SOD2_STRIP_ROW(2, 0)
+            SOD2_STRIP_ROW(1, 1)
+            SOD2_STRIP_ROW(1, 0)
+#undef SOD2_STRIP_ROW
           }
-          if (c2 == 0) {
-#pragma unroll
-            for (int q = 1; q < 12; ++q) ptx::mma_bf16(d1, ad + (q >> 2) * 8 + 2 * (q & 3), wb + (q >> 2) * (3 * TAP) + 2 * (q & 3), i1, 1);
-          } else {
-            const uint64_t wc = wb + c1 * TAP;
-#pragma unroll
-            for (int q = 1; q < 12; ++q) {
-              ptx::mma_bf16(d1, ad + (q >> 2) * 8 + 2 * (q & 3), wb + (q >> 2) * (3 * TAP) + 2 * (q & 3), i1, 1);
-              ptx::mma_bf16(tmem, ad + (q >> 2) * 8 + 2 * (q & 3), wc + (q >> 2) * (3 * TAP) + 2 * (q & 3), i2, 1);
-            }
-          }
+          ptx::tc_fence_before();
+          ptx::mbar_arrive(&turn[me ^ 1]);
           ptx::mma_commit(&empty[s]);
           if (ii >= 2) ptx::mma_commit(&tmem_full[(j + ii - 2) % NB]);
+          }
+          __syncwarp();
         }
         j += len;
         t += len;
@@ -183,14 +225,30 @@ conv3x3_strip_bf16_tcgen05(const __grid_constant__ Conv3Batch B, const __grid_co
       // ---- staging agent: unit u = this CTA's u-th tile, in buffer u % NSB.  prepare(u) hands the buffer to the
       // epilogue warps: with a residual it is TMA-loaded into the buffer (updated in place), otherwise a plain arrive.
       // The buffer of unit u - 1 is free for unit u + NSB - 1 once its store, issued one unit ago, has read it.
+      // Both walk the tiles with a cursor: decoding every tile (divisions, indexed parameters) made this thread the
+      // slowest of the kernel.
       const int U = end - begin;
-      auto prepare = [&](int u) {
-        const int bsel = u % NSB;
+      struct Cursor { int t, rq, img, row, w0, left; };
+      auto open = [&](Cursor& c, const int* ids) {
+        c.left = 0;
+        if (c.t >= end) return;
+        c.rq = decode(c.t, &c.img, &c.row, &c.w0);
+        c.left = min(end - c.t, B.Ho[c.rq] - c.row);
+        if (ids) c.img = ids[c.img];
+      };
+      auto next = [&](Cursor& c, const int* ids) {
+        ++c.t;
+        ++c.row;
+        if (--c.left == 0) open(c, ids);
+      };
+      Cursor in{begin, 0, 0, 0, 0, 0}, out{begin, 0, 0, 0, 0, 0};
+      if (HASRES) open(in, p.res_ids);
+      open(out, p.out_ids);
+      auto prepare = [&](int bsel) {
         if (HASRES) {
-          int img, row, w0;
-          const int rq = decode(begin + u, &img, &row, &w0);
           ptx::mbar_expect_tx(&res_full[bsel], CONV_STAGE_OUT);
-          ptx::tma_load_4d(out_stage + bsel * CONV_STAGE_OUT, &B.tr[rq], 0, w0, row, p.res_ids ? p.res_ids[img] : img, &res_full[bsel]);
+          ptx::tma_load_4d(out_stage + bsel * CONV_STAGE_OUT, &B.tr[in.rq], 0, in.w0, in.row, in.img, &res_full[bsel]);
+          next(in, p.res_ids);
         } else {
           ptx::mbar_arrive(&res_full[bsel]);
         }
@@ -198,16 +256,14 @@ conv3x3_strip_bf16_tcgen05(const __grid_constant__ Conv3Batch B, const __grid_co
       for (int u = 0; u < NSB && u < U; ++u) prepare(u);
       for (int u = 0; u < U; ++u) {
         const int bsel = u % NSB;
-        int img, row, w0;
-        const int rq = decode(begin + u, &img, &row, &w0);
-        const int img_o = p.out_ids ? p.out_ids[img] : img;
-        ptx::mbar_wait(&stage_ready[bsel], (u / NSB) & 1, dead);
-        tma_store_4d(&B.to[rq], out_stage + bsel * CONV_STAGE_OUT, 0, w0, row, img_o);
+        ptx::mbar_wait_parked(&stage_ready[bsel], (u / NSB) & 1, dead);
+        tma_store_4d(&B.to[out.rq], out_stage + bsel * CONV_STAGE_OUT, 0, out.w0, out.row, out.img);
         bulk_commit();
         if (u >= 1 && u + NSB - 1 < U) {
           asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
-          prepare(u + NSB - 1);
+          prepare((u + NSB - 1) % NSB);
         }
+        next(out, p.out_ids);
       }
       bulk_wait0();
     }
@@ -223,7 +279,7 @@ conv3x3_strip_bf16_tcgen05(const __grid_constant__ Conv3Batch B, const __grid_co
     const float4* bp4 = reinterpret_cast<const float4*>(bias_s + half * 32);
     for (int j = g; j < end - begin; j += 2) {
       const int blk = j % NB, bsel = j % NSB;
-      if (e == 0) ptx::mbar_wait_warp(&tmem_full[blk], (j / NB) & 1, dead);   // one polling warp, the others park at the barrier
+      if (e == 0) { if (lane == 0) ptx::mbar_wait_parked(&tmem_full[blk], (j / NB) & 1, dead); __syncwarp(); }   // one polling warp, the others park at the barrier
       group_bar();
       ptx::tc_fence_after();
       uint32_t r[32];
@@ -242,10 +298,10 @@ conv3x3_strip_bf16_tcgen05(const __grid_constant__ Conv3Batch B, const __grid_co
         v[4 * i4 + 3] = apply_act<ACT>(__uint_as_float(r[4 * i4 + 3]) + b4.w);
       }
       uint8_t* obase = out_stage + bsel * CONV_STAGE_OUT + row * 128;
+      uint4 rv[4];        // residual loads together, then the arithmetic, then the stores (never reordered by the compiler)
       ptx::mbar_wait_warp(&res_full[bsel], (j / NSB) & 1, dead);
       uint4 pk[4];
       if constexpr (HASRES) {
-        uint4 rv[4];      // loads together, then the arithmetic, then the stores (one buffer: never reordered by the compiler)
 #pragma unroll
         for (int u = 0; u < 4; ++u) rv[u] = *reinterpret_cast<const uint4*>(obase + (((half * 4 + u) ^ (row & 7)) << 4));
 #pragma unroll

@@ -88,6 +88,20 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volati
   return mbar_wait_limited(bar, parity, dead, SOD2_SPIN_LIMIT);
 }
 
+// The same for waits that are long and off the critical path: after the first test the thread is suspended by the
+// hardware (try_wait) instead of polling.  A polling thread takes a shared-memory cycle every 20 to 30; beside an MMA
+// stream that is bound by shared memory, five of them cost it a tenth of its rate.
+__device__ __forceinline__ bool mbar_wait_parked(uint64_t* bar, uint32_t parity, volatile int* dead) {
+  if (mbar_test_wait(bar, parity)) return true;
+#pragma unroll 1
+  for (uint32_t i = 0; i < SOD2_SPIN_LIMIT / 16; ++i) {
+    if (mbar_try_wait(bar, parity)) return true;
+    if ((i & 63u) == 63u && *dead) return false;
+  }
+  *dead = 1;
+  return false;
+}
+
 // The same wait for a whole warp: lane 0 polls, the others join (32 lanes polling one barrier serialise in the
 // shared-memory unit and triple the latency of a satisfied wait).  Must be called by all 32 lanes.
 __device__ __forceinline__ void mbar_wait_warp(uint64_t* bar, uint32_t parity, volatile int* dead) {
@@ -136,6 +150,21 @@ __device__ __forceinline__ void tmem_dealloc(uint32_t taddr, uint32_t ncols) {
 }
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
+
+// True in one lane of a warp whose 32 lanes are in step.  MMAs are issued under this and not under `lane == 0`, inside
+// loops that the whole warp runs: the operands of tcgen05.mma are uniform registers, and only behind elect.sync does the
+// compiler keep the address arithmetic there instead of moving every operand over for every instruction.  Measured on
+// B200 (cycles per 128x64x16 MMA with changing addresses; the pipe takes 48): `lane == 0` 56 alone and 97 beside sixteen
+// busy warps, elect.sync 48 and 53.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile(
+      "{\n\t.reg .pred q;\n\t.reg .b32 r;\n\t"
+      "elect.sync r|q, 0xffffffff;\n\t"
+      "selp.u32 %0, 1, 0, q;\n\t}"
+      : "=r"(p));
+  return p != 0;
+}
 
 // D[tmem] (+)= A[smem] * B[smem], bf16 inputs, fp32 accumulate; issued by one thread.
 __device__ __forceinline__ void mma_bf16(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t accumulate) {
