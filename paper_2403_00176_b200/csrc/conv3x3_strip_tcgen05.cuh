@@ -198,21 +198,21 @@ conv3x3_strip_bf16_tcgen05(const __grid_constant__ Conv3Batch B, const __grid_co
           const uint32_t a_lo = static_cast<uint32_t>(ad), b_lo = static_cast<uint32_t>(wb);
           const uint32_t dn = tmem + ((j + ii) % NB) * 64;
           if (ptx::elect_one()) {
-          switch (c1 * 8 + c2 * 2 + (fresh ? 1 : 0)) {
+            switch (c1 * 8 + c2 * 2 + (fresh ? 1 : 0)) {
 #define SOD2_STRIP_ROW(C1_, C2_) case C1_ * 8 + C2_ * 2: strip_row<C1_, C2_, false>(d1, tmem, dn, a_lo, b_lo); break; \
-                                 case C1_ * 8 + C2_ * 2 + 1: strip_row<C1_, C2_, true>(d1, tmem, dn, a_lo, b_lo); break;
-            SOD2_STRIP_ROW(3, 0)
-            SOD2_STRIP_ROW(2, 1)
-            SOD2_STRIP_ROW(1, 2)
-            SOD2_STRIP_ROW(2, 0)
-            SOD2_STRIP_ROW(1, 1)
-            SOD2_STRIP_ROW(1, 0)
+                                   case C1_ * 8 + C2_ * 2 + 1: strip_row<C1_, C2_, true>(d1, tmem, dn, a_lo, b_lo); break;
+              SOD2_STRIP_ROW(3, 0)
+              SOD2_STRIP_ROW(2, 1)
+              SOD2_STRIP_ROW(1, 2)
+              SOD2_STRIP_ROW(2, 0)
+              SOD2_STRIP_ROW(1, 1)
+              SOD2_STRIP_ROW(1, 0)
 #undef SOD2_STRIP_ROW
-          }
-          ptx::tc_fence_before();
-          ptx::mbar_arrive(&turn[me ^ 1]);
-          ptx::mma_commit(&empty[s]);
-          if (ii >= 2) ptx::mma_commit(&tmem_full[(j + ii - 2) % NB]);
+            }
+            ptx::tc_fence_before();
+            ptx::mbar_arrive(&turn[me ^ 1]);
+            ptx::mma_commit(&empty[s]);
+            if (ii >= 2) ptx::mma_commit(&tmem_full[(j + ii - 2) % NB]);
           }
           __syncwarp();
         }

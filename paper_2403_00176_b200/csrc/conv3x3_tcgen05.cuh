@@ -143,7 +143,7 @@ conv3x3_rows_bf16_tcgen05(const __grid_constant__ Conv3Batch B, const __grid_con
       }
     }
   } else if (warp == 3 || warp == 12) {
-    if (lane == 0) {
+    {
       // ---- two MMA issuers: warp 3 takes this CTA's even tiles (accumulator 0), warp 12 the odd ones
       // (accumulator 1).  A thread that waits on a barrier between MMAs leaves the tensor pipe idle for a
       // few hundred cycles; with two issuers one thread's wait is covered by the other's MMAs.  Both
@@ -158,28 +158,31 @@ conv3x3_rows_bf16_tcgen05(const __grid_constant__ Conv3Batch B, const __grid_con
         const int acc = j & 1;
         const bool mine = acc == me;
         if (mine) {
-          if (j >= 2) ptx::mbar_wait(&tmem_empty[acc], ((j >> 1) - 1) & 1, dead);
+          if (j >= 2) ptx::mbar_wait_warp(&tmem_empty[acc], ((j >> 1) - 1) & 1, dead);
           ptx::tc_fence_after();
         }
         const uint32_t d = tmem + acc * BN;
         for (int ks = 0; ks < kstages; ++ks, ++n) {
           const int s = n % STAGES;
-          ptx::mbar_wait(&full[s], (n / STAGES) & 1, dead);
+          ptx::mbar_wait_warp(&full[s], (n / STAGES) & 1, dead);
           if (!mine) continue;
           ptx::tc_fence_after();
           if (me == 0) { SOD2_TRACE(1, 200 + ks) }
           const uint32_t a = ptx::smem_u32(tiles + s * S::STAGE_BYTES);
           const uint32_t b = a + C3_A_SLOT;
+          if (ptx::elect_one()) {
 #pragma unroll
-          for (int dx = 0; dx < 3; ++dx) {
-            const uint64_t ad = ptx::smem_desc_sw128(a + dx * 128);     // rows shifted by dx pixels
-            const uint64_t bd = ptx::smem_desc_sw128(b + dx * (BN * 128));
+            for (int dx = 0; dx < 3; ++dx) {
+              const uint64_t ad = ptx::smem_desc_sw128(a + dx * 128);     // rows shifted by dx pixels
+              const uint64_t bd = ptx::smem_desc_sw128(b + dx * (BN * 128));
 #pragma unroll
-            for (int kk = 0; kk < 4; ++kk) ptx::mma_bf16(d, ad + 2 * kk, bd + 2 * kk, idesc, (ks | dx | kk) != 0);
+              for (int kk = 0; kk < 4; ++kk) ptx::mma_bf16(d, ad + 2 * kk, bd + 2 * kk, idesc, (ks | dx | kk) != 0);
+            }
+            ptx::mma_commit(&empty[s]);
+            if (ks + 1 == kstages) ptx::mma_commit(&tmem_full[acc]);
           }
-          ptx::mma_commit(&empty[s]);
+          __syncwarp();
         }
-        if (mine) ptx::mma_commit(&tmem_full[acc]);
         if (mine && me == 0) { SOD2_TRACE(1, 210) }
       }
     }

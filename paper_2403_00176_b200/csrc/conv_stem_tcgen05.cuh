@@ -248,28 +248,31 @@ conv_stem_bf16_tcgen05(const __grid_constant__ CUtensorMap tmW, const __grid_con
     }
     if constexpr (!TMA_PATCH) asm volatile("cp.async.wait_group 0;" ::: "memory");
   } else if (warp == 13) {
-    if (lane == 0) {
+    {
       // ---- MMA issuer
       constexpr uint32_t idesc = ptx::idesc_bf16(128, 64);
-      ptx::mbar_wait(w_full, 0, dead);
+      ptx::mbar_wait_warp(w_full, 0, dead);
       const uint32_t aW = ptx::smem_u32(sW);
       int it = 0;
       for (int t = blockIdx.x; t < n_tiles; t += gridDim.x, ++it) {
         const int b = it & 1;
-        ptx::mbar_wait(&a_full[b], (it >> 1) & 1, dead);
+        ptx::mbar_wait_warp(&a_full[b], (it >> 1) & 1, dead);
         SOD2_TRACE(1, 40)
-        if (it >= 2) ptx::mbar_wait(&acc_free[b], ((it >> 1) - 1) & 1, dead);
+        if (it >= 2) ptx::mbar_wait_warp(&acc_free[b], ((it >> 1) - 1) & 1, dead);
         SOD2_TRACE(1, 41)
         ptx::tc_fence_after();
         const uint32_t aA = ptx::smem_u32(sA + b * STEM_A_BYTES);
+        if (ptx::elect_one()) {
 #pragma unroll
-        for (int c = 0; c < 3; ++c) {
-          const uint64_t ad = ptx::smem_desc_sw128(aA + c * (128 * 128)), bd = ptx::smem_desc_sw128(aW + c * (64 * 128));
+          for (int c = 0; c < 3; ++c) {
+            const uint64_t ad = ptx::smem_desc_sw128(aA + c * (128 * 128)), bd = ptx::smem_desc_sw128(aW + c * (64 * 128));
 #pragma unroll
-          for (int kk = 0; kk < 4; ++kk) ptx::mma_bf16(tmem + b * 64, ad + 2 * kk, bd + 2 * kk, idesc, (c | kk) != 0);
+            for (int kk = 0; kk < 4; ++kk) ptx::mma_bf16(tmem + b * 64, ad + 2 * kk, bd + 2 * kk, idesc, (c | kk) != 0);
+          }
+          ptx::mma_commit(&a_free[b]);
+          ptx::mma_commit(&acc_full[b]);
         }
-        ptx::mma_commit(&a_free[b]);
-        ptx::mma_commit(&acc_full[b]);
+        __syncwarp();
         SOD2_TRACE(1, 42)
       }
     }

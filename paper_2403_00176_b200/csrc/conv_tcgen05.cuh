@@ -192,32 +192,35 @@ conv_igemm_bf16_tcgen05(const __grid_constant__ CUtensorMap tmX, const __grid_co
       }
     }
   } else if (warp == 3) {
-    if (lane == 0) {
-      // ---- MMA issuer
+    {
+      // ---- MMA issuer: the whole warp in step, one lane issues (ptx::elect_one)
       constexpr uint32_t idesc = ptx::idesc_bf16(128, BN);
       int n = 0, j = 0;
       for (int t = blockIdx.x; t < num_tiles; t += gridDim.x, ++j) {
         const int acc = j & 1;
-        if (j >= 2) ptx::mbar_wait(&tmem_empty[acc], ((j >> 1) - 1) & 1, dead);
+        if (j >= 2) ptx::mbar_wait_warp(&tmem_empty[acc], ((j >> 1) - 1) & 1, dead);
         ptx::tc_fence_after();
         const uint32_t d = tmem + acc * BN;
         for (int ks = 0; ks < kstages; ++ks, ++n) {
           const int s = n % STAGES;
-          ptx::mbar_wait(&full[s], (n / STAGES) & 1, dead);
+          ptx::mbar_wait_warp(&full[s], (n / STAGES) & 1, dead);
           ptx::tc_fence_after();
           const uint32_t a = ptx::smem_u32(tiles + s * S::STAGE_BYTES);
+          if (ptx::elect_one()) {
 #pragma unroll
-          for (int c = 0; c < KCH; ++c) {
-            if (ks * KCH + c < kchunks) {
-              const uint64_t ad = ptx::smem_desc_sw128(a + c * (128 * 128));
-              const uint64_t bd = ptx::smem_desc_sw128(a + S::A_BYTES + c * (BN * 128));
+            for (int c = 0; c < KCH; ++c) {
+              if (ks * KCH + c < kchunks) {
+                const uint64_t ad = ptx::smem_desc_sw128(a + c * (128 * 128));
+                const uint64_t bd = ptx::smem_desc_sw128(a + S::A_BYTES + c * (BN * 128));
 #pragma unroll
-              for (int kk = 0; kk < 4; ++kk) ptx::mma_bf16(d, ad + 2 * kk, bd + 2 * kk, idesc, (ks | c | kk) != 0);
+                for (int kk = 0; kk < 4; ++kk) ptx::mma_bf16(d, ad + 2 * kk, bd + 2 * kk, idesc, (ks | c | kk) != 0);
+              }
             }
+            ptx::mma_commit(&empty[s]);
+            if (ks + 1 == kstages) ptx::mma_commit(&tmem_full[acc]);
           }
-          ptx::mma_commit(&empty[s]);
+          __syncwarp();
         }
-        ptx::mma_commit(&tmem_full[acc]);
       }
     }
   } else {
