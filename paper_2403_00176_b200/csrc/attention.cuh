@@ -17,7 +17,7 @@
 namespace sod2 {
 namespace k {
 
-constexpr int ATTN_MAX_REQ = 32;
+constexpr int ATTN_MAX_REQ = 64;
 struct AttnReq {
   long long q_off, k_off, v_off, o_off;  // element offsets of this request's views
   int L;

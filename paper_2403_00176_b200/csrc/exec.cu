@@ -840,7 +840,7 @@ struct Builder : BuildState {
             tp.status = reinterpret_cast<int*>(x.arena);
             static bool once = (cudaFuncSetAttribute(k::attention_tcgen05_bf16, cudaFuncAttributeMaxDynamicSharedMemorySize, k::ATC_SMEM), true);
             (void)once;
-            launch_pdl(k::attention_tcgen05_bf16, dim3(static_cast<unsigned>(tiles128) * tp.H), dim3(k::ATC_THREADS), k::ATC_SMEM, x.stream,
+            launch_pdl(k::attention_tcgen05_bf16, dim3(static_cast<unsigned>(std::min(tiles128 * tp.H, 2 * x.plan->sm_count))), dim3(k::ATC_THREADS), k::ATC_SMEM, x.stream,
                        cache->tq, cache->tk, cache->tv, tp);
             return cudaGetLastError();
           });

@@ -76,3 +76,20 @@ def test_conv_strips_segments_and_ring(shapes):
     p.run()
     for a, b in zip(outs, p.outputs()):
         assert all(np.array_equal(a[n], b[n]) for n in a)
+
+
+@pytest.mark.parametrize("lens", [[1], [33, 64], [129, 640], list(range(1, 129, 3)) + [129, 191, 192, 193, 255, 256, 257, 300, 383, 385, 511, 512, 513, 577] + [200] * 8])
+def test_attention_blocks_items_and_tables(lens):
+    # blocks of 64 keys and tiles of 128 rows at their edges, warps without a live row, a CTA's first, second and third
+    # item (the last list: 65 requests, two tables, more than two items per CTA in the first)
+    wl = WL.cfg2(layers=1, D=384, H=6, F=384, n_requests=1, lmin=1, lmax=640)
+    rng = np.random.default_rng(43)
+    reqs = [Request({"L": n}, {"x": bf16_round(rng.standard_normal((1, n, 384)).astype(np.float32))}) for n in lens]
+    s, p, outs = run_batch(wl, reqs, opt_flags=B.OPT_NO_REUSE)
+    for r in range(0, len(reqs), 4 if len(reqs) > 8 else 1):
+        errs = lockstep(wl, s, p, outs, r, BF16_TOL)
+        bad = {k: v for k, v in errs.items() if not (isinstance(v, float) and v <= BF16_TOL)}
+        assert errs and not bad, (reqs[r].syms, bad)
+    p.run()
+    for a, b in zip(outs, p.outputs()):
+        assert np.array_equal(a["y"], b["y"])
