@@ -180,7 +180,7 @@ attention_tcgen05_bf16(const __grid_constant__ CUtensorMap tmQ, const __grid_con
       const AtcReq R = reqs[it.ri];
       if (is_k) {
         const int qs = i & 1;
-        if (i >= 2) ptx::mbar_wait_warp(&q_free[qs], ((i >> 1) - 1) & 1, dead);
+        if (i >= 2) ptx::mbar_wait_elect(&q_free[qs], ((i >> 1) - 1) & 1, dead);
         if (ptx::elect_one()) {
           ptx::mbar_expect_tx(&q_full[qs], ATC_Q_BYTES);
           ptx::tma_load_2d(sQ + qs * ATC_Q_BYTES, &tmQ, p.q_col + it.head * p.q_hs, R.q_row + it.q0, &q_full[qs]);
@@ -194,7 +194,7 @@ attention_tcgen05_bf16(const __grid_constant__ CUtensorMap tmQ, const __grid_con
       const int col = is_k ? p.k_col + it.head * p.k_hs : p.v_col + it.head * p.v_hs, row = is_k ? R.k_row : R.v_row;
       for (int j = 0; j < it.nkv; ++j, ++n) {
         const int b = n % ATC_ST;
-        if (n >= ATC_ST) ptx::mbar_wait_warp(&free_[b], ((n / ATC_ST) - 1) & 1, dead);
+        if (n >= ATC_ST) ptx::mbar_wait_elect(&free_[b], ((n / ATC_ST) - 1) & 1, dead);
         if (ptx::elect_one()) {
           ptx::mbar_expect_tx(&full[b], ATC_KV_BYTES);
           ptx::tma_load_2d(dst + b * ATC_KV_BYTES, tm, col, row + j * ATC_KB, &full[b]);
@@ -213,8 +213,8 @@ attention_tcgen05_bf16(const __grid_constant__ CUtensorMap tmQ, const __grid_con
       ptx::mbar_wait_warp(&q_full[i & 1], (i >> 1) & 1, dead);
       for (int j = 0; j < it.nkv; ++j, ++n) {
         const uint64_t dK = ptx::smem_desc_sw128(ptx::smem_u32(sK + (n % ATC_ST) * ATC_KV_BYTES));
-        ptx::mbar_wait_warp(&k_full[n % ATC_ST], (n / ATC_ST) & 1, dead);
-        if (n >= 2) ptx::mbar_wait_warp(&s_free[n & 1], ((n >> 1) - 1) & 1, dead);
+        ptx::mbar_wait_elect(&k_full[n % ATC_ST], (n / ATC_ST) & 1, dead);
+        if (n >= 2) ptx::mbar_wait_elect(&s_free[n & 1], ((n >> 1) - 1) & 1, dead);
         ptx::tc_fence_after();
         if (ptx::elect_one()) {
 #pragma unroll
@@ -236,8 +236,8 @@ attention_tcgen05_bf16(const __grid_constant__ CUtensorMap tmQ, const __grid_con
       for (int j = 0; j < it.nkv; ++j, ++n) {
         const int steps = (it.L - j * ATC_KB + 15) >> 4;       // keys past the request are left out
         const uint32_t aV = ptx::smem_u32(sV + (n % ATC_ST) * ATC_KV_BYTES);
-        ptx::mbar_wait_warp(&v_full[n % ATC_ST], (n / ATC_ST) & 1, dead);
-        ptx::mbar_wait_warp(&p_full[n & 1], (n >> 1) & 1, dead);
+        ptx::mbar_wait_elect(&v_full[n % ATC_ST], (n / ATC_ST) & 1, dead);
+        ptx::mbar_wait_elect(&p_full[n & 1], (n >> 1) & 1, dead);
         ptx::tc_fence_after();
         if (ptx::elect_one()) {
           // 16 keys per step: 8 packed columns of P in tensor memory, 16 rows (2048 B) down V

@@ -145,7 +145,7 @@ conv3x3_strip_bf16_tcgen05(const __grid_constant__ Conv3Batch B, const __grid_co
   };
 
   if (warp == 0) {
-    if (lane == 0) {
+    {
       // ---- input rows: a segment's L output rows need the L + 2 rows around them
       int n = 0;
       for (int t = begin; t < end;) {
@@ -155,9 +155,12 @@ conv3x3_strip_bf16_tcgen05(const __grid_constant__ Conv3Batch B, const __grid_co
         if (p.in_ids) img = p.in_ids[img];
         for (int i = row - 1; i <= row + len; ++i, ++n) {
           const int s = n % ST;
-          if (n >= ST) ptx::mbar_wait_parked(&empty[s], ((n / ST) - 1) & 1, dead);
-          ptx::mbar_expect_tx(&full[s], C3_A_BYTES);
-          ptx::tma_load_4d(rows + s * C3_A_SLOT, &B.tx[rq], 0, w0 - 1, i, img, &full[s]);
+          if (n >= ST) ptx::mbar_wait_elect(&empty[s], ((n / ST) - 1) & 1, dead);
+          if (ptx::elect_one()) {
+            ptx::mbar_expect_tx(&full[s], C3_A_BYTES);
+            ptx::tma_load_4d(rows + s * C3_A_SLOT, &B.tx[rq], 0, w0 - 1, i, img, &full[s]);
+          }
+          __syncwarp();
         }
         t += len;
       }
@@ -173,7 +176,7 @@ conv3x3_strip_bf16_tcgen05(const __grid_constant__ Conv3Batch B, const __grid_co
       // Output row o of the segment accumulates in block (j + o) % 8; input row ii (counted from the
       // row above the segment) gives to the output rows ii - 2 (dy = 2), ii - 1 and ii, as far as they belong to the
       // segment.  Row ii is touched for the first time: its very first instruction does not accumulate.
-      ptx::mbar_wait_warp(w_full, 0, dead);
+      ptx::mbar_wait_elect(w_full, 0, dead);
       const uint64_t wdesc = ptx::smem_desc_sw128(ptx::smem_u32(wres));
       const int me = warp == 1 ? 0 : 1;
       int n = 0, j = 0;
@@ -190,9 +193,9 @@ conv3x3_strip_bf16_tcgen05(const __grid_constant__ Conv3Batch B, const __grid_co
           const int c1 = min(cnt, NB - b0), c2 = cnt - c1;            // blocks before and behind the ring's end
           const uint64_t wb = wdesc + (lo - (ii - 2)) * (STRIP_TAP >> 4);
           const uint32_t d1 = tmem + b0 * 64;
-          if (fresh && j + ii >= NB) ptx::mbar_wait_warp(&tmem_empty[(j + ii) % NB], (((j + ii) / NB) - 1) & 1, dead);
-          ptx::mbar_wait_warp(&full[s], (n / ST) & 1, dead);
-          if (n > 0) ptx::mbar_wait_warp(&turn[me], me ? (n >> 1) & 1 : ((n >> 1) - 1) & 1, dead);
+          if (fresh && j + ii >= NB) ptx::mbar_wait_elect(&tmem_empty[(j + ii) % NB], (((j + ii) / NB) - 1) & 1, dead);
+          ptx::mbar_wait_elect(&full[s], (n / ST) & 1, dead);
+          if (n > 0) ptx::mbar_wait_elect(&turn[me], me ? (n >> 1) & 1 : ((n >> 1) - 1) & 1, dead);
           ptx::tc_fence_after();
           const uint64_t ad = ptx::smem_desc_sw128(ptx::smem_u32(rows + s * C3_A_SLOT));
           const uint32_t a_lo = static_cast<uint32_t>(ad), b_lo = static_cast<uint32_t>(wb);
@@ -221,7 +224,7 @@ conv3x3_strip_bf16_tcgen05(const __grid_constant__ Conv3Batch B, const __grid_co
       }
     }
   } else if (warp == 2) {
-    if (lane == 0) {
+    {
       // ---- staging agent: unit u = this CTA's u-th tile, in buffer u % NSB.  prepare(u) hands the buffer to the
       // epilogue warps: with a residual it is TMA-loaded into the buffer (updated in place), otherwise a plain arrive.
       // The buffer of unit u - 1 is free for unit u + NSB - 1 once its store, issued one unit ago, has read it.
@@ -245,27 +248,31 @@ conv3x3_strip_bf16_tcgen05(const __grid_constant__ Conv3Batch B, const __grid_co
       if (HASRES) open(in, p.res_ids);
       open(out, p.out_ids);
       auto prepare = [&](int bsel) {
-        if (HASRES) {
-          ptx::mbar_expect_tx(&res_full[bsel], CONV_STAGE_OUT);
-          ptx::tma_load_4d(out_stage + bsel * CONV_STAGE_OUT, &B.tr[in.rq], 0, in.w0, in.row, in.img, &res_full[bsel]);
-          next(in, p.res_ids);
-        } else {
-          ptx::mbar_arrive(&res_full[bsel]);
+        if (ptx::elect_one()) {
+          if (HASRES) {
+            ptx::mbar_expect_tx(&res_full[bsel], CONV_STAGE_OUT);
+            ptx::tma_load_4d(out_stage + bsel * CONV_STAGE_OUT, &B.tr[in.rq], 0, in.w0, in.row, in.img, &res_full[bsel]);
+          } else {
+            ptx::mbar_arrive(&res_full[bsel]);
+          }
         }
+        __syncwarp();
+        if (HASRES) next(in, p.res_ids);
       };
       for (int u = 0; u < NSB && u < U; ++u) prepare(u);
       for (int u = 0; u < U; ++u) {
         const int bsel = u % NSB;
-        ptx::mbar_wait_parked(&stage_ready[bsel], (u / NSB) & 1, dead);
-        tma_store_4d(&B.to[out.rq], out_stage + bsel * CONV_STAGE_OUT, 0, out.w0, out.row, out.img);
-        bulk_commit();
-        if (u >= 1 && u + NSB - 1 < U) {
-          asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
-          prepare((u + NSB - 1) % NSB);
+        ptx::mbar_wait_elect(&stage_ready[bsel], (u / NSB) & 1, dead);
+        if (ptx::elect_one()) {        // (always the same lane: bulk groups belong to a thread)
+          tma_store_4d(&B.to[out.rq], out_stage + bsel * CONV_STAGE_OUT, 0, out.w0, out.row, out.img);
+          bulk_commit();
+          if (u >= 1 && u + NSB - 1 < U) asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
         }
+        __syncwarp();
+        if (u >= 1 && u + NSB - 1 < U) prepare((u + NSB - 1) % NSB);
         next(out, p.out_ids);
       }
-      bulk_wait0();
+      if (ptx::elect_one()) bulk_wait0();
     }
   } else if (warp >= 4) {
     // ---- epilogue: group g (eight warps) takes the tiles j = g, g + 2, ...; warp (q, half) of a group owns TMEM lanes
@@ -279,8 +286,7 @@ conv3x3_strip_bf16_tcgen05(const __grid_constant__ Conv3Batch B, const __grid_co
     const float4* bp4 = reinterpret_cast<const float4*>(bias_s + half * 32);
     for (int j = g; j < end - begin; j += 2) {
       const int blk = j % NB, bsel = j % NSB;
-      if (e == 0) { if (lane == 0) ptx::mbar_wait_parked(&tmem_full[blk], (j / NB) & 1, dead); __syncwarp(); }   // one polling warp, the others park at the barrier
-      group_bar();
+      ptx::mbar_wait_warp(&tmem_full[blk], (j / NB) & 1, dead);
       ptx::tc_fence_after();
       uint32_t r[32];
       ptx::tmem_ld32(tmem + (static_cast<uint32_t>(q * 32) << 16) + blk * 64 + half * 32, r);

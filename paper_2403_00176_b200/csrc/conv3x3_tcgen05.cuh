@@ -111,35 +111,37 @@ conv3x3_rows_bf16_tcgen05(const __grid_constant__ Conv3Batch B, const __grid_con
   };
 
   if (warp == 0) {
-    if (lane == 0) {
-      // ---- A producer: one halo row segment per stage
-      int n = 0;
-      for (int t = blockIdx.x; t < num_tiles; t += gridDim.x) {
-        int n0, img, h0, w0;
-        const int rq = decode(t, &n0, &img, &h0, &w0);
-        if (p.in_ids) img = p.in_ids[img];
-        for (int ks = 0; ks < kstages; ++ks, ++n) {
-          const int s = n % STAGES;
-          if (n >= STAGES) ptx::mbar_wait(&empty[s], ((n / STAGES) - 1) & 1, dead);
-          const int dy = ks / cchunks, cc = ks % cchunks;
+    // ---- A producer: one halo row segment per stage
+    int n = 0;
+    for (int t = blockIdx.x; t < num_tiles; t += gridDim.x) {
+      int n0, img, h0, w0;
+      const int rq = decode(t, &n0, &img, &h0, &w0);
+      if (p.in_ids) img = p.in_ids[img];
+      for (int ks = 0; ks < kstages; ++ks, ++n) {
+        const int s = n % STAGES;
+        if (n >= STAGES) ptx::mbar_wait_elect(&empty[s], ((n / STAGES) - 1) & 1, dead);
+        const int dy = ks / cchunks, cc = ks % cchunks;
+        if (ptx::elect_one()) {
           SOD2_TRACE(0, 100 + ks)
           ptx::mbar_expect_tx(&full[s], C3_A_BYTES);
           ptx::tma_load_4d(tiles + s * S::STAGE_BYTES, &B.tx[rq], cc * 64, w0 - 1, h0 + dy - 1, img, &full[s]);
         }
+        __syncwarp();
       }
     }
   } else if (warp == 1) {
-    if (lane == 0) {
-      // ---- B producer: the three dx taps of (dy, chunk) are consecutive k-chunks
-      int n = 0;
-      for (int t = blockIdx.x; t < num_tiles; t += gridDim.x) {
-        const int n0 = (t / tiles_px) * BN;
-        for (int ks = 0; ks < kstages; ++ks, ++n) {
-          const int s = n % STAGES;
-          if (n >= STAGES) ptx::mbar_wait(&empty[s], ((n / STAGES) - 1) & 1, dead);
+    // ---- B producer: the three dx taps of (dy, chunk) are consecutive k-chunks
+    int n = 0;
+    for (int t = blockIdx.x; t < num_tiles; t += gridDim.x) {
+      const int n0 = (t / tiles_px) * BN;
+      for (int ks = 0; ks < kstages; ++ks, ++n) {
+        const int s = n % STAGES;
+        if (n >= STAGES) ptx::mbar_wait_elect(&empty[s], ((n / STAGES) - 1) & 1, dead);
+        if (ptx::elect_one()) {
           ptx::mbar_expect_tx(&full[s], 3 * BN * 128);
           ptx::tma_load_3d(tiles + s * S::STAGE_BYTES + C3_A_SLOT, &tmW, 0, n0, ks * 3, &full[s]);
         }
+        __syncwarp();
       }
     }
   } else if (warp == 3 || warp == 12) {
@@ -158,13 +160,13 @@ conv3x3_rows_bf16_tcgen05(const __grid_constant__ Conv3Batch B, const __grid_con
         const int acc = j & 1;
         const bool mine = acc == me;
         if (mine) {
-          if (j >= 2) ptx::mbar_wait_warp(&tmem_empty[acc], ((j >> 1) - 1) & 1, dead);
+          if (j >= 2) ptx::mbar_wait_elect(&tmem_empty[acc], ((j >> 1) - 1) & 1, dead);
           ptx::tc_fence_after();
         }
         const uint32_t d = tmem + acc * BN;
         for (int ks = 0; ks < kstages; ++ks, ++n) {
           const int s = n % STAGES;
-          ptx::mbar_wait_warp(&full[s], (n / STAGES) & 1, dead);
+          ptx::mbar_wait_elect(&full[s], (n / STAGES) & 1, dead);
           if (!mine) continue;
           ptx::tc_fence_after();
           if (me == 0) { SOD2_TRACE(1, 200 + ks) }
@@ -187,37 +189,36 @@ conv3x3_rows_bf16_tcgen05(const __grid_constant__ Conv3Batch B, const __grid_con
       }
     }
   } else if (warp == 2) {
-    if (lane == 0) {
-      // ---- staging agent: owns the staging buffers' traffic so that no epilogue thread waits on a TMA
-      // round trip.  A unit is one 64-channel pass of one tile; unit u uses buffer u % NSB.  prepare(u)
-      // hands the buffer to the epilogue warps: with a residual it is TMA-loaded into the buffer (the
-      // epilogue updates it in place), otherwise a plain arrive.  After the epilogue warps have filled
-      // the buffer the agent stores it and, once the store has read the buffer, prepares unit u + NSB.
-      int my_tiles = 0;
-      for (int t = blockIdx.x; t < num_tiles; t += gridDim.x) ++my_tiles;
-      const int U = my_tiles * PASSES;
-      auto prepare = [&](int u) {
-        const int t = blockIdx.x + (u / PASSES) * gridDim.x;
-        int n0, img, h0, w0;
-        const int rq = decode(t, &n0, &img, &h0, &w0);
-        const int np = n0 + (u % PASSES) * 64;
-        const int bsel = u % NSB;
-        if (HASRES && np < p.Cout) {
-          ptx::mbar_expect_tx(&res_full[bsel], CONV_STAGE_OUT);
-          ptx::tma_load_4d(out_stage + bsel * CONV_STAGE_OUT, &B.tr[rq], np, w0, h0, p.res_ids ? p.res_ids[img] : img, &res_full[bsel]);
-        } else {
-          ptx::mbar_arrive(&res_full[bsel]);
-        }
-      };
-      for (int u = 0; u < NSB && u < U; ++u) prepare(u);
-      for (int u = 0; u < U; ++u) {
-        const int bsel = u % NSB;
-        ptx::mbar_wait(&stage_ready[bsel], (u / NSB) & 1, dead);
-        SOD2_TRACE(2, 300)
-        const int t = blockIdx.x + (u / PASSES) * gridDim.x;
-        int n0, img, h0, w0;
-        const int rq = decode(t, &n0, &img, &h0, &w0);
-        const int np = n0 + (u % PASSES) * 64;
+    // ---- staging agent: owns the staging buffers' traffic so that no epilogue thread waits on a TMA
+    // round trip.  A unit is one 64-channel pass of one tile; unit u uses buffer u % NSB.  prepare(u)
+    // hands the buffer to the epilogue warps: with a residual it is TMA-loaded into the buffer (the
+    // epilogue updates it in place), otherwise a plain arrive.  After the epilogue warps have filled
+    // the buffer the agent stores it and, once the store has read the buffer, prepares unit u + NSB.
+    int my_tiles = 0;
+    for (int t = blockIdx.x; t < num_tiles; t += gridDim.x) ++my_tiles;
+    const int U = my_tiles * PASSES;
+    auto prepare = [&](int u) {
+      const int t = blockIdx.x + (u / PASSES) * gridDim.x;
+      int n0, img, h0, w0;
+      const int rq = decode(t, &n0, &img, &h0, &w0);
+      const int np = n0 + (u % PASSES) * 64;
+      const int bsel = u % NSB;
+      if (HASRES && np < p.Cout) {
+        ptx::mbar_expect_tx(&res_full[bsel], CONV_STAGE_OUT);
+        ptx::tma_load_4d(out_stage + bsel * CONV_STAGE_OUT, &B.tr[rq], np, w0, h0, p.res_ids ? p.res_ids[img] : img, &res_full[bsel]);
+      } else {
+        ptx::mbar_arrive(&res_full[bsel]);
+      }
+    };
+    if (ptx::elect_one()) { for (int u = 0; u < NSB && u < U; ++u) prepare(u); }
+    for (int u = 0; u < U; ++u) {
+      const int bsel = u % NSB;
+      ptx::mbar_wait_elect(&stage_ready[bsel], (u / NSB) & 1, dead);
+      const int t = blockIdx.x + (u / PASSES) * gridDim.x;
+      int n0, img, h0, w0;
+      const int rq = decode(t, &n0, &img, &h0, &w0);
+      const int np = n0 + (u % PASSES) * 64;
+      if (ptx::elect_one()) {      // (always the same lane: bulk groups belong to a thread)
         if (np < p.Cout) {
           tma_store_4d(&B.to[rq], out_stage + bsel * CONV_STAGE_OUT, np, w0, h0, p.out_ids ? p.out_ids[img] : img);
           bulk_commit();
@@ -228,8 +229,9 @@ conv3x3_rows_bf16_tcgen05(const __grid_constant__ Conv3Batch B, const __grid_con
           prepare(u + NSB);
         }
       }
-      bulk_wait0();
+      __syncwarp();
     }
+    if (ptx::elect_one()) bulk_wait0();
   } else if (warp >= 4 && warp < 12) {
     // ---- epilogue warps 4..11: TMEM -> +bias -> act -> (+residual, act2) -> bf16 -> swizzled staging
     const int e = warp - 4;
@@ -250,8 +252,8 @@ conv3x3_rows_bf16_tcgen05(const __grid_constant__ Conv3Batch B, const __grid_con
       float* bias_t = bias_s + (j & 1) * 256;
       bias_t[et] = bias_next;
       bias_next = load_bias(t + gridDim.x);
-      if (warp == 4) ptx::mbar_wait_warp(&tmem_full[acc], (j >> 1) & 1, dead);   // one polling warp, the others park at the barrier
-      conv_epi_bar();
+      conv_epi_bar();                              // the bias of this tile is written
+      ptx::mbar_wait_warp(&tmem_full[acc], (j >> 1) & 1, dead);
       ptx::tc_fence_after();
       if (et == 0) { SOD2_TRACE(3, 400) }
 #pragma unroll 1

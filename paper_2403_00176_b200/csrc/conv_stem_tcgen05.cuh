@@ -251,14 +251,14 @@ conv_stem_bf16_tcgen05(const __grid_constant__ CUtensorMap tmW, const __grid_con
     {
       // ---- MMA issuer
       constexpr uint32_t idesc = ptx::idesc_bf16(128, 64);
-      ptx::mbar_wait_warp(w_full, 0, dead);
+      ptx::mbar_wait_elect(w_full, 0, dead);
       const uint32_t aW = ptx::smem_u32(sW);
       int it = 0;
       for (int t = blockIdx.x; t < n_tiles; t += gridDim.x, ++it) {
         const int b = it & 1;
-        ptx::mbar_wait_warp(&a_full[b], (it >> 1) & 1, dead);
+        ptx::mbar_wait_elect(&a_full[b], (it >> 1) & 1, dead);
         SOD2_TRACE(1, 40)
-        if (it >= 2) ptx::mbar_wait_warp(&acc_free[b], ((it >> 1) - 1) & 1, dead);
+        if (it >= 2) ptx::mbar_wait_elect(&acc_free[b], ((it >> 1) - 1) & 1, dead);
         SOD2_TRACE(1, 41)
         ptx::tc_fence_after();
         const uint32_t aA = ptx::smem_u32(sA + b * STEM_A_BYTES);

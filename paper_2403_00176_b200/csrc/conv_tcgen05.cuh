@@ -152,16 +152,16 @@ conv_igemm_bf16_tcgen05(const __grid_constant__ CUtensorMap tmX, const __grid_co
   };
 
   if (warp < 2) {
-    if (lane == 0) {
-      // ---- A producers: warp 0 loads the even chunks of every stage, warp 1 the odd ones
-      int n = 0;
-      for (int t = blockIdx.x; t < num_tiles; t += gridDim.x) {
-        int n0, img, ho0, wo0;
-        decode(t, &n0, &img, &ho0, &wo0);
-        if (p.in_ids) img = p.in_ids[img];
-        for (int ks = 0; ks < kstages; ++ks, ++n) {
-          const int s = n % STAGES;
-          if (n >= STAGES) ptx::mbar_wait(&empty[s], ((n / STAGES) - 1) & 1, dead);
+    // ---- A producers: warp 0 loads the even chunks of every stage, warp 1 the odd ones
+    int n = 0;
+    for (int t = blockIdx.x; t < num_tiles; t += gridDim.x) {
+      int n0, img, ho0, wo0;
+      decode(t, &n0, &img, &ho0, &wo0);
+      if (p.in_ids) img = p.in_ids[img];
+      for (int ks = 0; ks < kstages; ++ks, ++n) {
+        const int s = n % STAGES;
+        if (n >= STAGES) ptx::mbar_wait_elect(&empty[s], ((n / STAGES) - 1) & 1, dead);
+        if (ptx::elect_one()) {
           int mine = 0;
           for (int c = warp; c < KCH; c += 2) ++mine;
           ptx::mbar_expect_tx(&full[s], mine * 128 * 128);
@@ -175,20 +175,22 @@ conv_igemm_bf16_tcgen05(const __grid_constant__ CUtensorMap tmX, const __grid_co
             ptx::tma_load_4d(tiles + s * S::STAGE_BYTES + c * (128 * 128), &tmX, cc * 64, wo0 * p.stride + dx - p.pad, hi, img, &full[s]);
           }
         }
+        __syncwarp();
       }
     }
   } else if (warp == 2) {
-    if (lane == 0) {
-      // ---- B producer
-      int n = 0;
-      for (int t = blockIdx.x; t < num_tiles; t += gridDim.x) {
-        const int n0 = (t / tiles_px) * BN;
-        for (int ks = 0; ks < kstages; ++ks, ++n) {
-          const int s = n % STAGES;
-          if (n >= STAGES) ptx::mbar_wait(&empty[s], ((n / STAGES) - 1) & 1, dead);
+    // ---- B producer
+    int n = 0;
+    for (int t = blockIdx.x; t < num_tiles; t += gridDim.x) {
+      const int n0 = (t / tiles_px) * BN;
+      for (int ks = 0; ks < kstages; ++ks, ++n) {
+        const int s = n % STAGES;
+        if (n >= STAGES) ptx::mbar_wait_elect(&empty[s], ((n / STAGES) - 1) & 1, dead);
+        if (ptx::elect_one()) {
           ptx::mbar_expect_tx(&full[s], S::B_BYTES);
           ptx::tma_load_3d(tiles + s * S::STAGE_BYTES + S::A_BYTES, &tmW, 0, n0, ks * KCH, &full[s]);
         }
+        __syncwarp();
       }
     }
   } else if (warp == 3) {
@@ -198,12 +200,12 @@ conv_igemm_bf16_tcgen05(const __grid_constant__ CUtensorMap tmX, const __grid_co
       int n = 0, j = 0;
       for (int t = blockIdx.x; t < num_tiles; t += gridDim.x, ++j) {
         const int acc = j & 1;
-        if (j >= 2) ptx::mbar_wait_warp(&tmem_empty[acc], ((j >> 1) - 1) & 1, dead);
+        if (j >= 2) ptx::mbar_wait_elect(&tmem_empty[acc], ((j >> 1) - 1) & 1, dead);
         ptx::tc_fence_after();
         const uint32_t d = tmem + acc * BN;
         for (int ks = 0; ks < kstages; ++ks, ++n) {
           const int s = n % STAGES;
-          ptx::mbar_wait_warp(&full[s], (n / STAGES) & 1, dead);
+          ptx::mbar_wait_elect(&full[s], (n / STAGES) & 1, dead);
           ptx::tc_fence_after();
           const uint32_t a = ptx::smem_u32(tiles + s * S::STAGE_BYTES);
           if (ptx::elect_one()) {
@@ -245,8 +247,8 @@ conv_igemm_bf16_tcgen05(const __grid_constant__ CUtensorMap tmX, const __grid_co
       float* bias_t = bias_s + (j & 1) * 256;
       bias_t[et] = bias_next;
       bias_next = load_bias(t + gridDim.x);
-      if (warp == 4) ptx::mbar_wait_warp(&tmem_full[acc], (j >> 1) & 1, dead);   // one polling warp, the others park at the barrier
-      conv_epi_bar();
+      conv_epi_bar();                              // the bias of this tile is written
+      ptx::mbar_wait_warp(&tmem_full[acc], (j >> 1) & 1, dead);
       ptx::tc_fence_after();
 #pragma unroll 1
       for (int ps = 0; ps < PASSES; ++ps) {

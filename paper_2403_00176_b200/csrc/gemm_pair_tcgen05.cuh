@@ -152,94 +152,99 @@ gemm_pair_bf16_tcgen05(const __grid_constant__ CUtensorMap tmA, const __grid_con
   if (threadIdx.x == 96) { SOD2_PAIR_TRACE(2, 1) }
 
   if (warp == 0) {
-    if (lane == 0) {
-      // ---- TMA producer: this CTA's A rows; completion on the leader's barrier
-      ptx::pdl_wait();
-      int n = 0;
-      for (int w = first; w < num_tiles; w += step) {
-        const int m0 = ((w % tiles_m2) * 2 + static_cast<int>(rank)) * GEMM_BM;
-        for (int ks = 0; ks < kstages; ++ks, ++n) {
-          const int s = n % STAGES;
-          if (n >= STAGES) ptx::mbar_wait(&empty[s], ((n / STAGES) - 1) & 1, dead);
+    // ---- TMA producer: this CTA's A rows; completion on the leader's barrier
+    ptx::pdl_wait();
+    int n = 0;
+    for (int w = first; w < num_tiles; w += step) {
+      const int m0 = ((w % tiles_m2) * 2 + static_cast<int>(rank)) * GEMM_BM;
+      for (int ks = 0; ks < kstages; ++ks, ++n) {
+        const int s = n % STAGES;
+        if (n >= STAGES) ptx::mbar_wait_elect(&empty[s], ((n / STAGES) - 1) & 1, dead);
+        if (ptx::elect_one()) {
           SOD2_PAIR_TRACE(0, n)
           if (leader) ptx::mbar_expect_tx(&full[s], 2 * S::A_BYTES);
           tma_load_3d_pair(tiles + s * S::STAGE_BYTES, &tmA, 0, m0, ks * KCH, map_to_cta(ptx::smem_u32(&full[s]), 0));
         }
+        __syncwarp();
       }
     }
   } else if (warp == 1) {
-    if (lane == 0) {
-      // ---- TMA producer: this CTA's half of the weight tile (constants: no wait for the previous kernel)
-      int n = 0;
-      for (int w = first; w < num_tiles; w += step) {
-        const int n0 = (w / tiles_m2) * BN + static_cast<int>(rank) * (BN / 2);
-        for (int ks = 0; ks < kstages; ++ks, ++n) {
-          const int s = n % STAGES;
-          if (n >= STAGES) ptx::mbar_wait(&empty[s], ((n / STAGES) - 1) & 1, dead);
+    // ---- TMA producer: this CTA's half of the weight tile (constants: no wait for the previous kernel)
+    int n = 0;
+    for (int w = first; w < num_tiles; w += step) {
+      const int n0 = (w / tiles_m2) * BN + static_cast<int>(rank) * (BN / 2);
+      for (int ks = 0; ks < kstages; ++ks, ++n) {
+        const int s = n % STAGES;
+        if (n >= STAGES) ptx::mbar_wait_elect(&empty[s], ((n / STAGES) - 1) & 1, dead);
+        if (ptx::elect_one()) {
           if (leader) ptx::mbar_expect_tx(&full[s], 2 * S::B_BYTES);
           tma_load_3d_pair(tiles + s * S::STAGE_BYTES + S::A_BYTES, &tmB, 0, n0, ks * KCH, map_to_cta(ptx::smem_u32(&full[s]), 0));
         }
+        __syncwarp();
       }
     }
   } else if (warp == 2) {
-    if (lane == 0 && leader) {
+    if (leader) {
       // ---- MMA issuer (leader only): 256 x BN x 16 per instruction over both CTAs
       constexpr uint32_t idesc = ptx::idesc_bf16(2 * GEMM_BM, BN);
       int n = 0, j = 0;
       for (int w = first; w < num_tiles; w += step, ++j) {
         const int acc = j & 1;
-        if (j >= 2) ptx::mbar_wait(&tmem_empty[acc], ((j >> 1) - 1) & 1, dead);
+        if (j >= 2) ptx::mbar_wait_elect(&tmem_empty[acc], ((j >> 1) - 1) & 1, dead);
         ptx::tc_fence_after();
         const uint32_t d = tmem + acc * BN;
         for (int ks = 0; ks < kstages; ++ks, ++n) {
           const int s = n % STAGES;
-          ptx::mbar_wait(&full[s], (n / STAGES) & 1, dead);
+          ptx::mbar_wait_elect(&full[s], (n / STAGES) & 1, dead);
           ptx::tc_fence_after();
-          SOD2_PAIR_TRACE(1, n)
-          const uint32_t a = ptx::smem_u32(tiles + s * S::STAGE_BYTES);
+          if (ptx::elect_one()) {
+            SOD2_PAIR_TRACE(1, n)
+            const uint32_t a = ptx::smem_u32(tiles + s * S::STAGE_BYTES);
 #pragma unroll
-          for (int c = 0; c < KCH; ++c) {
-            if (ks * KCH + c < kchunks) {
-              const uint64_t ad = ptx::smem_desc_sw128(a + c * (GEMM_BM * 128));
-              const uint64_t bd = ptx::smem_desc_sw128(a + S::A_BYTES + c * ((BN / 2) * 128));
+            for (int c = 0; c < KCH; ++c) {
+              if (ks * KCH + c < kchunks) {
+                const uint64_t ad = ptx::smem_desc_sw128(a + c * (GEMM_BM * 128));
+                const uint64_t bd = ptx::smem_desc_sw128(a + S::A_BYTES + c * ((BN / 2) * 128));
 #pragma unroll
-              for (int kk = 0; kk < 4; ++kk) mma_bf16_pair(d, ad + 2 * kk, bd + 2 * kk, idesc, (ks > 0) || c != 0 || kk != 0);
+                for (int kk = 0; kk < 4; ++kk) mma_bf16_pair(d, ad + 2 * kk, bd + 2 * kk, idesc, (ks > 0) || c != 0 || kk != 0);
+              }
             }
+            mma_commit_pair(&empty[s]);     // frees the stage in both CTAs
+            if (ks + 1 == kstages) mma_commit_pair(&tmem_full[acc]);
           }
-          mma_commit_pair(&empty[s]);     // frees the stage in both CTAs
+          __syncwarp();
         }
-        mma_commit_pair(&tmem_full[acc]);
       }
     }
   } else if (warp == 11) {
-    if (lane == 0) {
-      // ---- staging agent (as in the single-CTA kernel): this CTA's 128 rows
-      ptx::pdl_wait();
-      int my_tiles = 0;
-      for (int t = first; t < num_tiles; t += step) ++my_tiles;
-      const int U = my_tiles * PASSES;
-      auto coords = [&](int u, int* m0, int* np) {
-        const int w = first + (u / PASSES) * step;
-        *m0 = ((w % tiles_m2) * 2 + static_cast<int>(rank)) * GEMM_BM;
-        *np = (w / tiles_m2) * BN + (u % PASSES) * GEMM_PASS_COLS;
-      };
-      auto prepare = [&](int u) {
-        int m0, np;
-        coords(u, &m0, &np);
-        const int bsel = u % NSB;
-        if (RES && np < N && m0 < M) {
-          ptx::mbar_expect_tx(&buf_ready[bsel], GEMM_STAGE_OUT);
-          ptx::tma_load_2d(out_stage + bsel * GEMM_STAGE_OUT, &tmRes, np, m0, &buf_ready[bsel]);
-        } else {
-          ptx::mbar_arrive(&buf_ready[bsel]);
-        }
-      };
-      for (int u = 0; u < NSB && u < U; ++u) prepare(u);
-      for (int u = 0; u < U; ++u) {
-        const int bsel = u % NSB;
-        ptx::mbar_wait(&buf_filled[bsel], (u / NSB) & 1, dead);
-        int m0, np;
-        coords(u, &m0, &np);
+    // ---- staging agent (as in the single-CTA kernel): this CTA's 128 rows
+    ptx::pdl_wait();
+    int my_tiles = 0;
+    for (int t = first; t < num_tiles; t += step) ++my_tiles;
+    const int U = my_tiles * PASSES;
+    auto coords = [&](int u, int* m0, int* np) {
+      const int w = first + (u / PASSES) * step;
+      *m0 = ((w % tiles_m2) * 2 + static_cast<int>(rank)) * GEMM_BM;
+      *np = (w / tiles_m2) * BN + (u % PASSES) * GEMM_PASS_COLS;
+    };
+    auto prepare = [&](int u) {
+      int m0, np;
+      coords(u, &m0, &np);
+      const int bsel = u % NSB;
+      if (RES && np < N && m0 < M) {
+        ptx::mbar_expect_tx(&buf_ready[bsel], GEMM_STAGE_OUT);
+        ptx::tma_load_2d(out_stage + bsel * GEMM_STAGE_OUT, &tmRes, np, m0, &buf_ready[bsel]);
+      } else {
+        ptx::mbar_arrive(&buf_ready[bsel]);
+      }
+    };
+    if (ptx::elect_one()) { for (int u = 0; u < NSB && u < U; ++u) prepare(u); }
+    for (int u = 0; u < U; ++u) {
+      const int bsel = u % NSB;
+      ptx::mbar_wait_elect(&buf_filled[bsel], (u / NSB) & 1, dead);
+      int m0, np;
+      coords(u, &m0, &np);
+      if (ptx::elect_one()) {
         if (np < N && m0 < M) {
           tma_store_2d(&tmOut, out_stage + bsel * GEMM_STAGE_OUT, np, m0);
           bulk_commit();
@@ -249,8 +254,9 @@ gemm_pair_bf16_tcgen05(const __grid_constant__ CUtensorMap tmA, const __grid_con
           prepare(u + NSB);
         }
       }
-      bulk_wait_read0();
+      __syncwarp();
     }
+    if (ptx::elect_one()) bulk_wait_read0();
   } else {
     // ---- epilogue warps 3..10 of each CTA: its own TMEM lanes (its 128 rows)
     const int e = warp - 3;
@@ -271,8 +277,8 @@ gemm_pair_bf16_tcgen05(const __grid_constant__ CUtensorMap tmA, const __grid_con
       float* bias_t = bias_s + (j & 1) * 256;
       bias_t[et] = bias_next;
       bias_next = load_bias(w + step);
-      if (warp == 3) ptx::mbar_wait_warp(&tmem_full[acc], (j >> 1) & 1, dead);
-      epi_bar_sync();
+      epi_bar_sync();                              // the bias of this tile is written
+      ptx::mbar_wait_warp(&tmem_full[acc], (j >> 1) & 1, dead);
       ptx::tc_fence_after();
       if (et == 0) { SOD2_PAIR_TRACE(2, 100 + j) }
       const uint32_t taddr = tmem + (static_cast<uint32_t>(q * 32) << 16) + acc * BN + half * 32;

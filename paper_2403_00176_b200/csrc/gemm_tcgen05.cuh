@@ -208,113 +208,113 @@ gemm_bf16_tcgen05(const __grid_constant__ CUtensorMap tmA, const __grid_constant
   ptx::pdl_launch();
 
   if (warp == 0) {
-    if (lane == 0) {
-      // ---- TMA producer: A stages
-      ptx::pdl_wait();
-      SOD2_TRACE(0, 2)
-      int n = 0;
-      for (int w = blockIdx.x; w < num_tiles; w += gridDim.x) {
-        const int t = SPLITK ? w % out_tiles : w;
-        const int m0 = (t % tiles_m) * GEMM_BM;
-        int ks0, ks1;
-        k_range(w, &ks0, &ks1);
-        for (int ks = ks0; ks < ks1; ++ks, ++n) {
-          const int s = n % STAGES;
-          if (n >= STAGES) ptx::mbar_wait(&empty[s], ((n / STAGES) - 1) & 1, dead);
+    // ---- TMA producer: A stages
+    ptx::pdl_wait();
+    int n = 0;
+    for (int w = blockIdx.x; w < num_tiles; w += gridDim.x) {
+      const int t = SPLITK ? w % out_tiles : w;
+      const int m0 = (t % tiles_m) * GEMM_BM;
+      int ks0, ks1;
+      k_range(w, &ks0, &ks1);
+      for (int ks = ks0; ks < ks1; ++ks, ++n) {
+        const int s = n % STAGES;
+        if (n >= STAGES) ptx::mbar_wait_elect(&empty[s], ((n / STAGES) - 1) & 1, dead);
+        if (ptx::elect_one()) {
+          if (n == 0) { SOD2_TRACE(0, 2) }
           ptx::mbar_expect_tx(&full[s], S::A_BYTES);
           ptx::tma_load_3d(tiles + s * S::STAGE_BYTES, &tmA, 0, m0, ks * KCH, &full[s]);
         }
+        __syncwarp();
       }
     }
   } else if (warp == 1) {
-    if (lane == 0) {
-      // ---- TMA producer: B stages
-      int n = 0;
-      for (int w = blockIdx.x; w < num_tiles; w += gridDim.x) {
-        const int t = SPLITK ? w % out_tiles : w;
-        const int n0 = (t / tiles_m) * BN;
-        int ks0, ks1;
-        k_range(w, &ks0, &ks1);
-        for (int ks = ks0; ks < ks1; ++ks, ++n) {
-          const int s = n % STAGES;
-          if (n >= STAGES) ptx::mbar_wait(&empty[s], ((n / STAGES) - 1) & 1, dead);
+    // ---- TMA producer: B stages
+    int n = 0;
+    for (int w = blockIdx.x; w < num_tiles; w += gridDim.x) {
+      const int t = SPLITK ? w % out_tiles : w;
+      const int n0 = (t / tiles_m) * BN;
+      int ks0, ks1;
+      k_range(w, &ks0, &ks1);
+      for (int ks = ks0; ks < ks1; ++ks, ++n) {
+        const int s = n % STAGES;
+        if (n >= STAGES) ptx::mbar_wait_elect(&empty[s], ((n / STAGES) - 1) & 1, dead);
+        if (ptx::elect_one()) {
           ptx::mbar_expect_tx(&full[s], S::B_BYTES);
           ptx::tma_load_3d(tiles + s * S::STAGE_BYTES + S::A_BYTES, &tmB, 0, n0, ks * KCH, &full[s]);
         }
+        __syncwarp();
       }
     }
   } else if (warp == 2) {
-    // ---- MMA issuer.  Up to 128 columns the whole warp goes in step and one lane issues (ptx::elect_one): an MMA takes 64
-    // cycles of the pipe then, less than issuing it under lane == 0 costs.  At 256 columns (128 cycles) one thread keeps
-    // up, and its barrier waits are the shorter ones (QKV at 12.7 k rows: 44.6 us against 46.3).
-    constexpr bool STEP = BN <= 128;
-    auto wait = [&](uint64_t* bar, uint32_t parity) { if constexpr (STEP) ptx::mbar_wait_warp(bar, parity, dead); else ptx::mbar_wait(bar, parity, dead); };
-    if (STEP || lane == 0) {
-      constexpr uint32_t idesc = ptx::idesc_bf16(GEMM_BM, BN);
-      int n = 0, j = 0;
-      for (int w = blockIdx.x; w < num_tiles; w += gridDim.x, ++j) {
-        const int acc = j & 1;
-        if (j >= 2) wait(&tmem_empty[acc], ((j >> 1) - 1) & 1);
+    // ---- MMA issuer: the warp goes in step and one lane issues (ptx::elect_one), as in the roles above.  Under lane == 0 an
+    // MMA costs 56 to 97 cycles to issue (the pipe takes 64 at 128 columns) and a wait twice as long: with the roles in
+    // step the 12.7 k row GEMMs of the encoder went 45 -> 42.4 us (QKV), 66 -> 59.6 (FFN1, GELU), 71.5 -> 70 (FFN2).
+    constexpr uint32_t idesc = ptx::idesc_bf16(GEMM_BM, BN);
+    int n = 0, j = 0;
+    for (int w = blockIdx.x; w < num_tiles; w += gridDim.x, ++j) {
+      const int acc = j & 1;
+      if (j >= 2) ptx::mbar_wait_elect(&tmem_empty[acc], ((j >> 1) - 1) & 1, dead);
+      ptx::tc_fence_after();
+      const uint32_t d = tmem + acc * BN;
+      int ks0, ks1;
+      k_range(w, &ks0, &ks1);
+      for (int ks = ks0; ks < ks1; ++ks, ++n) {
+        const int s = n % STAGES;
+        ptx::mbar_wait_elect(&full[s], (n / STAGES) & 1, dead);
         ptx::tc_fence_after();
-        const uint32_t d = tmem + acc * BN;
-        int ks0, ks1;
-        k_range(w, &ks0, &ks1);
-        for (int ks = ks0; ks < ks1; ++ks, ++n) {
-          const int s = n % STAGES;
-          wait(&full[s], (n / STAGES) & 1);
-          ptx::tc_fence_after();
+        const uint32_t a = ptx::smem_u32(tiles + s * S::STAGE_BYTES);
+        if (ptx::elect_one()) {
           if (ks == 0) { SOD2_TRACE(1, 10 + j) }
-          const uint32_t a = ptx::smem_u32(tiles + s * S::STAGE_BYTES);
-          if (!STEP || ptx::elect_one()) {
 #pragma unroll
-            for (int c = 0; c < KCH; ++c) {
-              if (ks * KCH + c < kchunks) {
-                const uint64_t ad = ptx::smem_desc_sw128(a + c * (GEMM_BM * 128));
-                const uint64_t bd = ptx::smem_desc_sw128(a + S::A_BYTES + c * (BN * 128));
+          for (int c = 0; c < KCH; ++c) {
+            if (ks * KCH + c < kchunks) {
+              const uint64_t ad = ptx::smem_desc_sw128(a + c * (GEMM_BM * 128));
+              const uint64_t bd = ptx::smem_desc_sw128(a + S::A_BYTES + c * (BN * 128));
 #pragma unroll
-                for (int kk = 0; kk < 4; ++kk) ptx::mma_bf16(d, ad + 2 * kk, bd + 2 * kk, idesc, (ks > ks0) || c != 0 || kk != 0);
-              }
+              for (int kk = 0; kk < 4; ++kk) ptx::mma_bf16(d, ad + 2 * kk, bd + 2 * kk, idesc, (ks > ks0) || c != 0 || kk != 0);
             }
-            ptx::mma_commit(&empty[s]);  // frees the stage once these MMAs have read it
-            if (ks + 1 == ks1) ptx::mma_commit(&tmem_full[acc]);
           }
-          if constexpr (STEP) __syncwarp();
+          ptx::mma_commit(&empty[s]);  // frees the stage once these MMAs have read it
+          if (ks + 1 == ks1) {
+            ptx::mma_commit(&tmem_full[acc]);
+            SOD2_TRACE(1, 20 + j)
+          }
         }
-        SOD2_TRACE(1, 20 + j)
+        __syncwarp();
       }
     }
   } else if (warp == 11) {
-    if (lane == 0) {
-      // ---- staging agent: owns the staging buffers' TMA traffic so that no epilogue thread waits on a
-      // TMA round trip.  A unit is one 64-column pass of one tile; unit u uses buffer u % NSB.
-      // prepare(u) hands the buffer to the epilogue warps: with a residual it is TMA-loaded into the
-      // buffer (the epilogue updates it in place), otherwise a plain arrive.  Once the epilogue warps
-      // have filled the buffer the agent stores it and, after the store has read the buffer, prepares
-      // unit u + NSB.  The kernel may end once the last store has read shared memory.
-      ptx::pdl_wait();
-      int my_tiles = 0;
-      for (int t = blockIdx.x; t < num_tiles; t += gridDim.x) ++my_tiles;
-      const int U = my_tiles * PASSES;
-      constexpr int PASS_COLS = SPLITK ? 32 : GEMM_PASS_COLS;
-      auto prepare = [&](int u) {
-        const int w = blockIdx.x + (u / PASSES) * gridDim.x;
-        const int t = SPLITK ? w % out_tiles : w;
-        const int m0 = (t % tiles_m) * GEMM_BM, np = (t / tiles_m) * BN + (u % PASSES) * PASS_COLS;
-        const int bsel = u % NSB;
-        if (!SPLITK && RES && np < N) {
-          ptx::mbar_expect_tx(&buf_ready[bsel], GEMM_STAGE_OUT);
-          ptx::tma_load_2d(out_stage + bsel * GEMM_STAGE_OUT, &tmRes, np, m0, &buf_ready[bsel]);
-        } else {
-          ptx::mbar_arrive(&buf_ready[bsel]);
-        }
-      };
-      if (SPLITK || RES) { for (int u = 0; u < NSB && u < U; ++u) prepare(u); }   // else: done at barrier initialisation
-      for (int u = 0; u < U; ++u) {
-        const int bsel = u % NSB;
-        ptx::mbar_wait(&buf_filled[bsel], (u / NSB) & 1, dead);
-        const int w = blockIdx.x + (u / PASSES) * gridDim.x;
-        const int t = SPLITK ? w % out_tiles : w;
-        const int m0 = (t % tiles_m) * GEMM_BM, np = (t / tiles_m) * BN + (u % PASSES) * PASS_COLS;
+    // ---- staging agent: owns the staging buffers' TMA traffic so that no epilogue thread waits on a
+    // TMA round trip.  A unit is one 64-column pass of one tile; unit u uses buffer u % NSB.
+    // prepare(u) hands the buffer to the epilogue warps: with a residual it is TMA-loaded into the
+    // buffer (the epilogue updates it in place), otherwise a plain arrive.  Once the epilogue warps
+    // have filled the buffer the agent stores it and, after the store has read the buffer, prepares
+    // unit u + NSB.  The kernel may end once the last store has read shared memory.
+    ptx::pdl_wait();
+    int my_tiles = 0;
+    for (int t = blockIdx.x; t < num_tiles; t += gridDim.x) ++my_tiles;
+    const int U = my_tiles * PASSES;
+    constexpr int PASS_COLS = SPLITK ? 32 : GEMM_PASS_COLS;
+    auto prepare = [&](int u) {
+      const int w = blockIdx.x + (u / PASSES) * gridDim.x;
+      const int t = SPLITK ? w % out_tiles : w;
+      const int m0 = (t % tiles_m) * GEMM_BM, np = (t / tiles_m) * BN + (u % PASSES) * PASS_COLS;
+      const int bsel = u % NSB;
+      if (!SPLITK && RES && np < N) {
+        ptx::mbar_expect_tx(&buf_ready[bsel], GEMM_STAGE_OUT);
+        ptx::tma_load_2d(out_stage + bsel * GEMM_STAGE_OUT, &tmRes, np, m0, &buf_ready[bsel]);
+      } else {
+        ptx::mbar_arrive(&buf_ready[bsel]);
+      }
+    };
+    if ((SPLITK || RES) && ptx::elect_one()) { for (int u = 0; u < NSB && u < U; ++u) prepare(u); }   // else: done at barrier initialisation
+    for (int u = 0; u < U; ++u) {
+      const int bsel = u % NSB;
+      ptx::mbar_wait_elect(&buf_filled[bsel], (u / NSB) & 1, dead);
+      const int w = blockIdx.x + (u / PASSES) * gridDim.x;
+      const int t = SPLITK ? w % out_tiles : w;
+      const int m0 = (t % tiles_m) * GEMM_BM, np = (t / tiles_m) * BN + (u % PASSES) * PASS_COLS;
+      if (ptx::elect_one()) {      // (always the same lane: bulk groups belong to a thread)
         if (np < N) {
           if (SPLITK) tma_store_3d(&tmOut, out_stage + bsel * GEMM_STAGE_OUT, np, m0, w / out_tiles);
           else tma_store_2d(&tmOut, out_stage + bsel * GEMM_STAGE_OUT, np, m0);
@@ -325,6 +325,9 @@ gemm_bf16_tcgen05(const __grid_constant__ CUtensorMap tmA, const __grid_constant
           prepare(u + NSB);
         }
       }
+      __syncwarp();
+    }
+    if (ptx::elect_one()) {
       SOD2_TRACE(2, 40)
       bulk_wait_read0();
       SOD2_TRACE(2, 41)
@@ -423,10 +426,8 @@ gemm_bf16_tcgen05(const __grid_constant__ CUtensorMap tmA, const __grid_constant
         if (grow < M) ln_merge_stats(ep.ln_stats + grow, ep.ln_pitch, ep.ln_slots, ep.ln_cols, ep.ln_eps, &ln_mean, &ln_rstd);
       }
       float em_n = 0.f, em_mean = 0.f, em_m2 = 0.f;    // EMIT: running statistics of this thread's columns of the row
-      // one warp polls for the accumulator, the others park at the hardware barrier: seven more polling
-      // lanes cost the main loop 3-4 % of its issue slots
-      if (warp == 3) ptx::mbar_wait_warp(&tmem_full[acc], (j >> 1) & 1, dead);
-      epi_bar_sync();
+      epi_bar_sync();                              // the vectors of this tile are written
+      ptx::mbar_wait_warp(&tmem_full[acc], (j >> 1) & 1, dead);
       ptx::tc_fence_after();
       if (et == 0) { SOD2_TRACE(2, 30 + j) }
       const uint32_t taddr = tmem + (static_cast<uint32_t>(q * 32) << 16) + acc * BN + half * 32;

@@ -88,32 +88,25 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volati
   return mbar_wait_limited(bar, parity, dead, SOD2_SPIN_LIMIT);
 }
 
-// The same for a single thread whose waits are long: after the first test the thread is suspended by the hardware
-// (try_wait) instead of polling.
-__device__ __forceinline__ bool mbar_wait_parked(uint64_t* bar, uint32_t parity, volatile int* dead) {
-  if (mbar_test_wait(bar, parity)) return true;
-#pragma unroll 1
-  for (uint32_t i = 0; i < SOD2_SPIN_LIMIT / 16; ++i) {
-    if (mbar_try_wait(bar, parity)) return true;
-    if ((i & 63u) == 63u && *dead) return false;
-  }
-  *dead = 1;
-  return false;
-}
-
 // The same wait for a whole warp in step.  All 32 lanes test and park together: the access is uniform, and the warp never
 // diverges.  Measured on B200 (ping-pong between two warps, cycles per hand-over): 125, against 231 where a role runs
 // under lane == 0 and 266 where lane 0 polls and the warp joins it; through tcgen05.commit 133 against 365 and 244.  Must
 // be called by all 32 lanes.
-__device__ __forceinline__ void mbar_wait_warp(uint64_t* bar, uint32_t parity, volatile int* dead) {
-  bool ok = mbar_test_wait(bar, parity);
+// Lanes may in principle see the phase end at different tests.  `mbar_wait_elect` is for a warp whose next step is
+// elect_one(), which brings the lanes together; `mbar_wait_warp` does it itself, for what wants a warp in step at once
+// (tcgen05.ld and .st).  A __syncwarp in each wait of the producers and issuers cost a 64-token GEMM 0.2 us (of 7.5).
+__device__ __forceinline__ void mbar_wait_elect(uint64_t* bar, uint32_t parity, volatile int* dead) {
+  if (__builtin_expect(mbar_test_wait(bar, parity), 1)) return;
 #pragma unroll 1
-  for (uint32_t i = 0; !ok && i < SOD2_SPIN_LIMIT / 16; ++i) {
-    ok = mbar_try_wait(bar, parity);
-    if ((i & 63u) == 63u && *dead) ok = true;
+  for (uint32_t i = 0; i < SOD2_SPIN_LIMIT / 16; ++i) {
+    if (mbar_try_wait(bar, parity)) return;
+    if ((i & 63u) == 63u && *dead) return;
   }
-  if (!ok) *dead = 1;
-  __syncwarp();     // lanes may see the phase end at different tests
+  *dead = 1;
+}
+__device__ __forceinline__ void mbar_wait_warp(uint64_t* bar, uint32_t parity, volatile int* dead) {
+  mbar_wait_elect(bar, parity, dead);
+  __syncwarp();
 }
 // One arrival for a warp in step, without a branch around it.
 __device__ __forceinline__ void mbar_arrive_warp(uint64_t* bar) {
