@@ -155,24 +155,23 @@ cudaError_t gemm_dispatch(int act, bool res, int ln, bool emit, dim3 grid, cudaS
   return cudaErrorInvalidValue;
 }
 
-template <int BN, int KCH, int ST, int ACT, bool RES>
-cudaError_t launch_gemm_pair_variant(dim3 grid, cudaStream_t st, const CUtensorMap& ta, const CUtensorMap& tb, const CUtensorMap& to,
-                                     const CUtensorMap& tr, int M, int N, int K, const k::GemmEpilogue& ep) {
-  constexpr int smem = k::GemmPairSmem<BN, KCH, ST>::TOTAL;
-  static bool once = (cudaFuncSetAttribute(k::gemm_pair_bf16_tcgen05<BN, KCH, ST, ACT, RES>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem), true);
+template <int ACT, bool RES>
+cudaError_t launch_gemm_pair_variant(dim3 grid, cudaStream_t st, const CUtensorMap& ta, const k::GemmPairMaps& tb, const CUtensorMap& to,
+                                     const CUtensorMap& tr, int M, int N, int K, const k::GemmEpilogue& ep, const k::PairSplit& sp) {
+  constexpr int smem = k::GemmPairSmem::TOTAL;
+  static bool once = (cudaFuncSetAttribute(k::gemm_pair_bf16_tcgen05<ACT, RES>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem), true);
   (void)once;
-  return launch_pdl_pair(k::gemm_pair_bf16_tcgen05<BN, KCH, ST, ACT, RES>, grid, dim3(k::GEMM_THREADS), smem, st, ta, tb, to, tr, M, N, K, ep);
+  return launch_pdl_pair(k::gemm_pair_bf16_tcgen05<ACT, RES>, grid, dim3(k::GEMM_THREADS), smem, st, ta, tb, to, tr, M, N, K, ep, sp);
 }
-template <int BN, int KCH, int ST>
-cudaError_t gemm_pair_dispatch(int act, bool res, dim3 grid, cudaStream_t st, const CUtensorMap& ta, const CUtensorMap& tb, const CUtensorMap& to,
-                               const CUtensorMap& tr, int M, int N, int K, const k::GemmEpilogue& ep) {
+cudaError_t gemm_pair_dispatch(int act, bool res, dim3 grid, cudaStream_t st, const CUtensorMap& ta, const k::GemmPairMaps& tb, const CUtensorMap& to,
+                               const CUtensorMap& tr, int M, int N, int K, const k::GemmEpilogue& ep, const k::PairSplit& sp) {
   switch (act * 2 + (res ? 1 : 0)) {
-    case 0: return launch_gemm_pair_variant<BN, KCH, ST, 0, false>(grid, st, ta, tb, to, tr, M, N, K, ep);
-    case 1: return launch_gemm_pair_variant<BN, KCH, ST, 0, true>(grid, st, ta, tb, to, tr, M, N, K, ep);
-    case 2: return launch_gemm_pair_variant<BN, KCH, ST, 1, false>(grid, st, ta, tb, to, tr, M, N, K, ep);
-    case 3: return launch_gemm_pair_variant<BN, KCH, ST, 1, true>(grid, st, ta, tb, to, tr, M, N, K, ep);
-    case 4: return launch_gemm_pair_variant<BN, KCH, ST, 2, false>(grid, st, ta, tb, to, tr, M, N, K, ep);
-    default: return launch_gemm_pair_variant<BN, KCH, ST, 2, true>(grid, st, ta, tb, to, tr, M, N, K, ep);
+    case 0: return launch_gemm_pair_variant<0, false>(grid, st, ta, tb, to, tr, M, N, K, ep, sp);
+    case 1: return launch_gemm_pair_variant<0, true>(grid, st, ta, tb, to, tr, M, N, K, ep, sp);
+    case 2: return launch_gemm_pair_variant<1, false>(grid, st, ta, tb, to, tr, M, N, K, ep, sp);
+    case 3: return launch_gemm_pair_variant<1, true>(grid, st, ta, tb, to, tr, M, N, K, ep, sp);
+    case 4: return launch_gemm_pair_variant<2, false>(grid, st, ta, tb, to, tr, M, N, K, ep, sp);
+    default: return launch_gemm_pair_variant<2, true>(grid, st, ta, tb, to, tr, M, N, K, ep, sp);
   }
 }
 
@@ -429,20 +428,37 @@ struct Builder : BuildState {
         bn_group = bn;
         p.stats_layout[G.out] = {static_cast<int>(N / bn) * 2, bn / 2};
       }
-      // CTA pairs (tcgen05.mma.cta_group::2, 256 x BN tiles): each CTA loads its own A rows and half of the weight tile,
-      // a third to a half fewer operand bytes per flop.  Same makespan estimate, per 64-wide k-chunk and pair of SMs.
-      int pair_bn = 0;
-      if ((c.flags & OPT_GEMM_PAIR) && !lna && !lnr && !emit && G.act2 == 0 && tiles_m >= 2 && N >= 128) {
-        auto pair_span = [&](int bn_) {
-          const double pairs = std::ceil(tiles_m / 2.0) * ((N + bn_ - 1) / bn_);
-          const double waves = std::ceil(pairs / (sms / 2));
-          const double mma = 4 * (bn_ / 2.0), tma = (128 + bn_ / 2) * 128.0 / 70.0;
-          return waves * std::ceil(K / 64.0) * std::max(mma, tma);
+      // CTA pairs (tcgen05.mma.cta_group::2): each CTA loads its own A rows and half of the weight tile, a third to a half
+      // fewer operand bytes per flop, in tiles of 256 rows x 256, 192 or 128 columns whose last wave may be cut in two.
+      // Both kernels are estimated as (waves of tiles) x (64-wide k-chunks) x (time of a chunk) + the epilogue of the
+      // last tile; the times (ns, from sweeps of 700 to 14 k rows at the four encoder shapes) say which wins: pairs cost
+      // 1.6 us more to start (cluster launch, two cluster barriers), so they take over at a few thousand rows, e.g. K =
+      // 3072, N = 768: 23.2 -> 19.3 us at 4224 rows, 38.9 -> 29.5 at 7168, 65.7 -> 54 at 14072; 0.4 us more must be gained.
+      // Below 12 chunks the epilogue bounds both kernels and the pairs' start is never earned back.
+      bool pair = false;
+      k::PairSplit split{4, 0, 1, 1};
+      if (!lna && !lnr && !emit && G.act2 == 0 && tiles_m >= 2 && N >= 128) {
+        const int pairs = sms / 2, tiles_m2 = (tiles_m + 1) / 2, units_n = static_cast<int>((N + 63) / 64);
+        const double kst = K / 64.0, chunk_ns[5] = {0, 235, 255, 305, 355}, unit_ns = 570;   // by units of 64 columns
+        double best = 1e30;
+        auto offer = [&](int bw, int parts) {
+          const int tiles_n = (units_n + bw - 1) / bw, tiles = tiles_m2 * tiles_n, rest = tiles % pairs, waves = tiles / pairs;
+          const int last = (bw + parts - 1) / parts;
+          if (parts > 1 && (rest == 0 || waves == 0 || rest * parts > pairs)) return;
+          const double t = waves * kst * chunk_ns[bw] + (rest ? kst * chunk_ns[last] : 0.0) + unit_ns * (rest ? last : bw) + (parts > 1 ? 700.0 : 0.0);
+          if (t >= best) return;
+          best = t;
+          // Row tiles are walked in bands one wave high where A does not stay in half of L2 while all its column tiles
+          // pass (14072 x 3072: 55.5 -> 53.4 us); otherwise all of them, which reads each weight tile in one go
+          const bool big = static_cast<int64_t>(M) * K * 2 > (int64_t(64) << 20);
+          split = {bw, parts > 1 ? tiles - rest : tiles, parts, big ? std::min(tiles_m2, (pairs + tiles_n - 1) / tiles_n) : tiles_m2};
         };
-        const double single = bn == 256 ? makespan(256, 1) : makespan(128, 2);
-        const int pb = (N >= 256 && pair_span(256) <= pair_span(128)) ? 256 : 128;
+        if (units_n >= 4) { offer(4, 1); offer(4, 2); }
+        if (units_n >= 3) offer(3, 1);
+        offer(2, 1);
+        const double single = std::ceil(static_cast<double>(tiles_m) * ((N + bn - 1) / bn) / sms) * kst * (bn == 256 ? 386.0 : 263.0) + unit_ns * (bn / 64);
         static const bool force_pair = getenv("SOD2_GEMM_PAIR_FORCE") != nullptr;   // tests: the pair kernel wherever it is eligible
-        if (pair_span(pb) < single || force_pair) pair_bn = pb;
+        pair = (c.flags & OPT_GEMM_PAIR) ? (best < single || force_pair) : (K >= 12 * 64 && best + 2000.0 < single);
       }
       const bool hb = G.bias >= 0, hr = G.res >= 0;
       const int act = G.act;
@@ -461,7 +477,7 @@ struct Builder : BuildState {
       }
       if (emit && !stats_ptr(G.out, sg.r0, N, &ps_out, &pitch_out)) return fail(E_INTERNAL, "row statistics of " + g.tensors[G.out].name + " are not planned");
       const float ln_eps = G.ln_eps;
-      struct Cache { const void* a = nullptr; const void* w = nullptr; const void* o = nullptr; const void* r = nullptr; CUtensorMap ta, tb, to, tr; };
+      struct Cache { const void* a = nullptr; const void* w = nullptr; const void* o = nullptr; const void* r = nullptr; CUtensorMap ta, tb, to, tr; k::GemmPairMaps pb; };
       auto cache = std::make_shared<Cache>();
       add(gi, 1, [=](const RunCtx& x) {
         const void* A = x.resolve(pa);
@@ -469,10 +485,12 @@ struct Builder : BuildState {
         void* O = x.resolve(po);
         const void* R = hr ? x.resolve(pr) : O;
         if (cache->a != A || cache->w != Wt || cache->o != O || cache->r != R) {
-          const int kch = pair_bn ? (pair_bn == 256 ? 1 : 2) : (bn == 256 ? 1 : 2);
-          const int brows = pair_bn ? pair_bn / 2 : bn;      // a CTA of a pair loads half of the weight tile
-          if (!encode_bf16_kchunks(&cache->ta, A, M, K, lda, 128, kch) || !encode_bf16_kchunks(&cache->tb, Wt, N, K, K, brows, kch) ||
-              !encode_bf16_2d(&cache->to, O, M, N, ldo, 128) || !encode_bf16_2d(&cache->tr, R, M, N, hr ? ldr : ldo, 128))
+          const int kch = pair || bn == 256 ? 1 : 2;
+          bool ok = encode_bf16_kchunks(&cache->ta, A, M, K, lda, 128, kch) && encode_bf16_2d(&cache->to, O, M, N, ldo, 128) &&
+                    encode_bf16_2d(&cache->tr, R, M, N, hr ? ldr : ldo, 128);
+          if (!pair) ok = ok && encode_bf16_kchunks(&cache->tb, Wt, N, K, K, bn, kch);
+          else for (int w = 0; w < 4; ++w) ok = ok && encode_bf16_kchunks(&cache->pb.b[w], Wt, N, K, K, 32 * (w + 1), 1);
+          if (!ok)
             return cudaErrorInvalidValue;
           cache->a = A; cache->w = Wt; cache->o = O; cache->r = R;
         }
@@ -500,11 +518,10 @@ struct Builder : BuildState {
           ep.emit_pitch = pitch_out;
         }
         const int Ni = static_cast<int>(N), Ki = static_cast<int>(K);
-        if (pair_bn) {
-          const int pairs = ((tiles_m + 1) / 2) * static_cast<int>((N + pair_bn - 1) / pair_bn);
-          const dim3 gp(2 * std::max(1, std::min(pairs, x.plan->sm_count / 2)));
-          const cudaError_t ep2 = pair_bn == 256 ? gemm_pair_dispatch<256, 1, 6>(act, hr, gp, x.stream, cache->ta, cache->tb, cache->to, cache->tr, M, Ni, Ki, ep)
-                                                 : gemm_pair_dispatch<128, 2, 4>(act, hr, gp, x.stream, cache->ta, cache->tb, cache->to, cache->tr, M, Ni, Ki, ep);
+        if (pair) {
+          const int tiles = ((tiles_m + 1) / 2) * static_cast<int>(((N + 63) / 64 + split.bw - 1) / split.bw);
+          const int items = split.n_full + (tiles - split.n_full) * split.parts;
+          const cudaError_t ep2 = gemm_pair_dispatch(act, hr, dim3(2 * std::min(items, x.plan->sm_count / 2)), x.stream, cache->ta, cache->pb, cache->to, cache->tr, M, Ni, Ki, ep, split);
           return ep2 != cudaSuccess ? ep2 : cudaGetLastError();
         }
         const int tiles = tiles_m * static_cast<int>((N + bn - 1) / bn);

@@ -16,12 +16,14 @@
 //     kernel and arrive on the LEADER's accumulator-empty barrier (a remote mbarrier arrive for the odd CTA);
 //   - tensor memory is allocated and freed by one warp of EACH CTA with the cta_group::2 forms; a cluster barrier after
 //     the barrier initialisation and one before the release keep both CTAs alive while the other can still reach them.
-// Every wait is bounded (ptx.cuh).  Launch: cluster dimension 2, grid = 2 x min(pairs of tiles, SM count / 2).
-// Measured: the pair's MMA instructions run at the single-CTA rate (128 cycles per 256 x 256 x 16, 74 per 256 x 128 x 16,
-// issue-rate probe), and kernel time against K has the same slope as the single-CTA kernel's (0.30 us per 64-wide k-stage
-// at N = 2304): the single-CTA main loop does not wait for operands at a few thousand rows, so loading fewer of them
-// gains nothing, and the cluster launch, the two cluster barriers and the paired tensor-memory allocation add 0.5 - 1.5 us
-// per kernel.  The planner uses this kernel only on request.
+// Every wait is bounded (ptx.cuh).  Launch: cluster dimension 2, grid = 2 x min(items, SM count / 2).
+// What bounds it: at 14 k rows the board's power (its SM clock falls to 1.3 - 1.4 GHz; 1300 - 1350 TFLOP/s at N = 2304),
+// where fewer operand bytes through L2 are clock won; below that the L2 -> shared memory path, 702 cycles per k-chunk of
+// a 128 x 256 tile against 512 of MMA, which the pair's 32 KB fit under.  Waves of 256 x 256 tiles fit 74 pairs badly
+// at N = 768 (3 column tiles), so the width is chosen per launch and the last wave's tiles may be cut.  Dealing the
+// columns out evenly in 64-wide units instead was slower (narrow MMAs: 43 us against 39.5 at N = 2304).  Measured at
+// 14072 rows against the single-CTA kernel: N = 2304 K = 768 40.3 -> 37.2 us, 768 x 768 20.2 -> 18.2, 3072 x 768 (GELU)
+// 58.2 -> 55.4, 768 x 3072 65.7 -> 54.
 #pragma once
 #include "gemm_tcgen05.cuh"
 
@@ -79,25 +81,63 @@ __device__ __forceinline__ void mma_commit_pair(uint64_t* bar) {
                ::"r"(ptx::smem_u32(bar)), "h"(static_cast<uint16_t>(3)) : "memory");
 }
 
-template <int BN, int KCH, int STAGES>
+// Weight tiles of 1 to 4 units of 64 columns: box b[w - 1] is the CTA's half, 32 w rows, of a 64-wide k-chunk.
+struct GemmPairMaps { CUtensorMap b[4]; };
+
+constexpr int PAIR_STAGES = 6;
 struct GemmPairSmem {
-  static constexpr int A_BYTES = KCH * GEMM_BM * 128;          // this CTA's 128 rows
-  static constexpr int B_BYTES = KCH * (BN / 2) * 128;         // this CTA's half of the weight tile
+  static constexpr int A_BYTES = GEMM_BM * 128;            // this CTA's 128 rows of a 64-wide k-chunk
+  static constexpr int B_BYTES = 128 * 128;                // this CTA's half of the widest weight tile
   static constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
-  static constexpr int USED = STAGES * STAGE_BYTES + GEMM_NSB * GEMM_STAGE_OUT + 2048 /*bias*/ + 8 * (2 * STAGES + 4 + 2 * GEMM_NSB) + 16;
+  static constexpr int USED = PAIR_STAGES * STAGE_BYTES + GEMM_NSB * GEMM_STAGE_OUT + 2048 /*bias*/ + 8 * (2 * PAIR_STAGES + 4 + 2 * GEMM_NSB) + 16;
   // plus the pad that brings the tiles to a 1024-byte boundary (the kernel checks what it really needs)
   static constexpr int TOTAL = USED + 848;
 };
 
-// tmA: {64, rows, K/64} box {64, 128, KCH}; tmB: the same view of the K-major weights, box {64, BN/2, KCH}.
-template <int BN, int KCH, int STAGES, int ACT, bool RES>
+// How the output is dealt out: tiles of 256 rows x `bw` units, in bands of `band` row tiles, row tiles fastest inside a
+// band; the first `n_full` tiles round robin over the pairs, each of the rest cut into `parts` so that the last, partly
+// filled wave is short.
+struct PairSplit { int bw, n_full, parts, band; };
+struct PairWalk {
+  int i, step, items, tiles_m2, tiles_n, units_n;
+  PairSplit sp;
+  int m, n0, w;          // the item: row tile, first column, width in units
+  __device__ __forceinline__ PairWalk(int M, int N, const PairSplit& split)
+      : i(static_cast<int>(cluster_id_x())), step(static_cast<int>(cluster_count_x())), tiles_m2((M + 2 * GEMM_BM - 1) / (2 * GEMM_BM)),
+        units_n((N + 63) / 64), sp(split), m(0), n0(0), w(0) {
+    tiles_n = (units_n + sp.bw - 1) / sp.bw;
+    items = sp.n_full + (tiles_m2 * tiles_n - sp.n_full) * sp.parts;
+  }
+  __device__ __forceinline__ bool next() {
+    while (i < items) {
+      int t = i, first = 0, width = sp.bw;
+      if (i >= sp.n_full) {
+        const int e = i - sp.n_full;
+        width = (sp.bw + sp.parts - 1) / sp.parts;
+        t = sp.n_full + e / sp.parts;
+        first = (e % sp.parts) * width;
+        width = min(width, sp.bw - first);
+      }
+      i += step;
+      const int b0 = t / (sp.band * tiles_n) * sp.band, rows = min(sp.band, tiles_m2 - b0), r = t - b0 * tiles_n;
+      const int nt = r / rows, u = nt * sp.bw + first;
+      m = b0 + r - nt * rows;
+      n0 = u * 64;
+      w = min(width, units_n - u);
+      if (w > 0) return true;
+    }
+    return false;
+  }
+};
+
+// tmA: {64, rows, K/64} box {64, 128, 1}; maps.b: the same view of the K-major weights.
+template <int ACT, bool RES>
 __global__ void __launch_bounds__(GEMM_THREADS, 1)
-gemm_pair_bf16_tcgen05(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
+gemm_pair_bf16_tcgen05(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ GemmPairMaps maps,
                        const __grid_constant__ CUtensorMap tmOut, const __grid_constant__ CUtensorMap tmRes,
-                       int M, int N, int K, GemmEpilogue ep) {
-  using S = GemmPairSmem<BN, KCH, STAGES>;
-  constexpr int PASSES = BN / GEMM_PASS_COLS;
-  constexpr int NSB = GEMM_NSB;
+                       int M, int N, int K, GemmEpilogue ep, PairSplit split) {
+  using S = GemmPairSmem;
+  constexpr int STAGES = PAIR_STAGES, BN = 256, NSB = GEMM_NSB;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* tiles = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint8_t* out_stage = tiles + STAGES * S::STAGE_BYTES;
@@ -123,11 +163,8 @@ gemm_pair_bf16_tcgen05(const __grid_constant__ CUtensorMap tmA, const __grid_con
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t rank = cluster_ctarank();          // 0 = leader
   const bool leader = rank == 0;
-  const int tiles_m2 = (M + 2 * GEMM_BM - 1) / (2 * GEMM_BM), tiles_n = (N + BN - 1) / BN;
-  const int kchunks = K / 64;
-  const int kstages = (kchunks + KCH - 1) / KCH;
-  const int num_tiles = tiles_m2 * tiles_n;          // pair tiles of 256 x BN
-  const int first = static_cast<int>(cluster_id_x()), step = static_cast<int>(cluster_count_x());
+  const int kstages = K / 64;
+  const PairWalk share(M, N, split);
   constexpr uint32_t TMEM_COLS = 2 * BN;
 
   if (threadIdx.x == 0) {
@@ -138,7 +175,7 @@ gemm_pair_bf16_tcgen05(const __grid_constant__ CUtensorMap tmA, const __grid_con
     ptx::fence_barrier_init();
     ptx::fence_proxy_async();
     ptx::prefetch_tmap(&tmA);
-    ptx::prefetch_tmap(&tmB);
+    for (int w = 0; w < 4; ++w) ptx::prefetch_tmap(&maps.b[w]);
     ptx::prefetch_tmap(&tmOut);
     if (RES) ptx::prefetch_tmap(&tmRes);
   }
@@ -155,15 +192,15 @@ gemm_pair_bf16_tcgen05(const __grid_constant__ CUtensorMap tmA, const __grid_con
     // ---- TMA producer: this CTA's A rows; completion on the leader's barrier
     ptx::pdl_wait();
     int n = 0;
-    for (int w = first; w < num_tiles; w += step) {
-      const int m0 = ((w % tiles_m2) * 2 + static_cast<int>(rank)) * GEMM_BM;
+    for (PairWalk wk = share; wk.next();) {
+      const int m0 = (wk.m * 2 + static_cast<int>(rank)) * GEMM_BM;
       for (int ks = 0; ks < kstages; ++ks, ++n) {
         const int s = n % STAGES;
         if (n >= STAGES) ptx::mbar_wait_elect(&empty[s], ((n / STAGES) - 1) & 1, dead);
         if (ptx::elect_one()) {
           SOD2_PAIR_TRACE(0, n)
           if (leader) ptx::mbar_expect_tx(&full[s], 2 * S::A_BYTES);
-          tma_load_3d_pair(tiles + s * S::STAGE_BYTES, &tmA, 0, m0, ks * KCH, map_to_cta(ptx::smem_u32(&full[s]), 0));
+          tma_load_3d_pair(tiles + s * S::STAGE_BYTES, &tmA, 0, m0, ks, map_to_cta(ptx::smem_u32(&full[s]), 0));
         }
         __syncwarp();
       }
@@ -171,25 +208,26 @@ gemm_pair_bf16_tcgen05(const __grid_constant__ CUtensorMap tmA, const __grid_con
   } else if (warp == 1) {
     // ---- TMA producer: this CTA's half of the weight tile (constants: no wait for the previous kernel)
     int n = 0;
-    for (int w = first; w < num_tiles; w += step) {
-      const int n0 = (w / tiles_m2) * BN + static_cast<int>(rank) * (BN / 2);
+    for (PairWalk wk = share; wk.next();) {
+      const int n0 = wk.n0 + static_cast<int>(rank) * wk.w * 32;
+      const CUtensorMap* tmB = &maps.b[wk.w - 1];
       for (int ks = 0; ks < kstages; ++ks, ++n) {
         const int s = n % STAGES;
         if (n >= STAGES) ptx::mbar_wait_elect(&empty[s], ((n / STAGES) - 1) & 1, dead);
         if (ptx::elect_one()) {
-          if (leader) ptx::mbar_expect_tx(&full[s], 2 * S::B_BYTES);
-          tma_load_3d_pair(tiles + s * S::STAGE_BYTES + S::A_BYTES, &tmB, 0, n0, ks * KCH, map_to_cta(ptx::smem_u32(&full[s]), 0));
+          if (leader) ptx::mbar_expect_tx(&full[s], 2 * wk.w * (32 * 128));
+          tma_load_3d_pair(tiles + s * S::STAGE_BYTES + S::A_BYTES, tmB, 0, n0, ks, map_to_cta(ptx::smem_u32(&full[s]), 0));
         }
         __syncwarp();
       }
     }
   } else if (warp == 2) {
     if (leader) {
-      // ---- MMA issuer (leader only): 256 x BN x 16 per instruction over both CTAs
-      constexpr uint32_t idesc = ptx::idesc_bf16(2 * GEMM_BM, BN);
+      // ---- MMA issuer (leader only): 256 x 64w x 16 per instruction over both CTAs
       int n = 0, j = 0;
-      for (int w = first; w < num_tiles; w += step, ++j) {
+      for (PairWalk wk = share; wk.next(); ++j) {
         const int acc = j & 1;
+        const uint32_t idesc = ptx::idesc_bf16(2 * GEMM_BM, 64 * wk.w);
         if (j >= 2) ptx::mbar_wait_elect(&tmem_empty[acc], ((j >> 1) - 1) & 1, dead);
         ptx::tc_fence_after();
         const uint32_t d = tmem + acc * BN;
@@ -197,18 +235,12 @@ gemm_pair_bf16_tcgen05(const __grid_constant__ CUtensorMap tmA, const __grid_con
           const int s = n % STAGES;
           ptx::mbar_wait_elect(&full[s], (n / STAGES) & 1, dead);
           ptx::tc_fence_after();
+          const uint32_t a = ptx::smem_u32(tiles + s * S::STAGE_BYTES);
           if (ptx::elect_one()) {
             SOD2_PAIR_TRACE(1, n)
-            const uint32_t a = ptx::smem_u32(tiles + s * S::STAGE_BYTES);
+            const uint64_t ad = ptx::smem_desc_sw128(a), bd = ptx::smem_desc_sw128(a + S::A_BYTES);
 #pragma unroll
-            for (int c = 0; c < KCH; ++c) {
-              if (ks * KCH + c < kchunks) {
-                const uint64_t ad = ptx::smem_desc_sw128(a + c * (GEMM_BM * 128));
-                const uint64_t bd = ptx::smem_desc_sw128(a + S::A_BYTES + c * ((BN / 2) * 128));
-#pragma unroll
-                for (int kk = 0; kk < 4; ++kk) mma_bf16_pair(d, ad + 2 * kk, bd + 2 * kk, idesc, (ks > 0) || c != 0 || kk != 0);
-              }
-            }
+            for (int kk = 0; kk < 4; ++kk) mma_bf16_pair(d, ad + 2 * kk, bd + 2 * kk, idesc, (ks > 0) || kk != 0);
             mma_commit_pair(&empty[s]);     // frees the stage in both CTAs
             if (ks + 1 == kstages) mma_commit_pair(&tmem_full[acc]);
           }
@@ -217,44 +249,43 @@ gemm_pair_bf16_tcgen05(const __grid_constant__ CUtensorMap tmA, const __grid_con
       }
     }
   } else if (warp == 11) {
-    // ---- staging agent (as in the single-CTA kernel): this CTA's 128 rows
+    // ---- staging agent (as in the single-CTA kernel): this CTA's 128 rows, a unit of 64 columns per buffer
     ptx::pdl_wait();
-    int my_tiles = 0;
-    for (int t = first; t < num_tiles; t += step) ++my_tiles;
-    const int U = my_tiles * PASSES;
-    auto coords = [&](int u, int* m0, int* np) {
-      const int w = first + (u / PASSES) * step;
-      *m0 = ((w % tiles_m2) * 2 + static_cast<int>(rank)) * GEMM_BM;
-      *np = (w / tiles_m2) * BN + (u % PASSES) * GEMM_PASS_COLS;
+    struct Cursor {
+      PairWalk wk;
+      int ps;
+      bool live;
+      __device__ __forceinline__ explicit Cursor(const PairWalk& s) : wk(s), ps(0) { live = wk.next(); }
+      __device__ __forceinline__ void step() { if (++ps == wk.w) { ps = 0; live = wk.next(); } }
     };
-    auto prepare = [&](int u) {
-      int m0, np;
-      coords(u, &m0, &np);
-      const int bsel = u % NSB;
-      if (RES && np < N && m0 < M) {
-        ptx::mbar_expect_tx(&buf_ready[bsel], GEMM_STAGE_OUT);
-        ptx::tma_load_2d(out_stage + bsel * GEMM_STAGE_OUT, &tmRes, np, m0, &buf_ready[bsel]);
-      } else {
-        ptx::mbar_arrive(&buf_ready[bsel]);
-      }
-    };
-    if (ptx::elect_one()) { for (int u = 0; u < NSB && u < U; ++u) prepare(u); }
-    for (int u = 0; u < U; ++u) {
-      const int bsel = u % NSB;
-      ptx::mbar_wait_elect(&buf_filled[bsel], (u / NSB) & 1, dead);
-      int m0, np;
-      coords(u, &m0, &np);
+    Cursor in(share), out(share);
+    auto prepare = [&](int bsel) {
+      const int m0 = (in.wk.m * 2 + static_cast<int>(rank)) * GEMM_BM, np = in.wk.n0 + in.ps * GEMM_PASS_COLS;
       if (ptx::elect_one()) {
-        if (np < N && m0 < M) {
-          tma_store_2d(&tmOut, out_stage + bsel * GEMM_STAGE_OUT, np, m0);
-          bulk_commit();
-        }
-        if (u + NSB < U) {
-          bulk_wait_read0();
-          prepare(u + NSB);
+        if (RES && m0 < M) {
+          ptx::mbar_expect_tx(&buf_ready[bsel], GEMM_STAGE_OUT);
+          ptx::tma_load_2d(out_stage + bsel * GEMM_STAGE_OUT, &tmRes, np, m0, &buf_ready[bsel]);
+        } else {
+          ptx::mbar_arrive(&buf_ready[bsel]);
         }
       }
       __syncwarp();
+      in.step();
+    };
+    for (int u = 0; u < NSB && in.live; ++u) prepare(u);
+    for (int u = 0; out.live; ++u, out.step()) {
+      const int bsel = u % NSB;
+      const int m0 = (out.wk.m * 2 + static_cast<int>(rank)) * GEMM_BM, np = out.wk.n0 + out.ps * GEMM_PASS_COLS;
+      ptx::mbar_wait_elect(&buf_filled[bsel], (u / NSB) & 1, dead);
+      if (ptx::elect_one()) {        // (always the same lane: bulk groups belong to a thread)
+        if (m0 < M) {
+          tma_store_2d(&tmOut, out_stage + bsel * GEMM_STAGE_OUT, np, m0);
+          bulk_commit();
+        }
+        if (in.live) bulk_wait_read0();
+      }
+      __syncwarp();
+      if (in.live) prepare(bsel);
     }
     if (ptx::elect_one()) bulk_wait_read0();
   } else {
@@ -267,16 +298,19 @@ gemm_pair_bf16_tcgen05(const __grid_constant__ CUtensorMap tmA, const __grid_con
     ptx::pdl_wait();
     const uint32_t empty_leader[2] = {map_to_cta(ptx::smem_u32(&tmem_empty[0]), 0), map_to_cta(ptx::smem_u32(&tmem_empty[1]), 0)};
     int j = 0, u = 0;
-    auto load_bias = [&](int w) -> float {
-      const int idx = (w / tiles_m2) * BN + et;
-      return (ep.bias && et < BN && w < num_tiles && idx < N) ? __bfloat162float(ep.bias[idx]) : 0.0f;
+    PairWalk wk = share;
+    bool live = wk.next();
+    auto load_bias = [&]() -> float {
+      const int idx = wk.n0 + et;
+      return (ep.bias && live && et < 64 * wk.w && idx < N) ? __bfloat162float(ep.bias[idx]) : 0.0f;
     };
-    float bias_next = load_bias(first);
-    for (int w = first; w < num_tiles; w += step, ++j) {
-      const int acc = j & 1;
+    float bias_next = load_bias();
+    for (; live; ++j) {
+      const int acc = j & 1, units = wk.w;
       float* bias_t = bias_s + (j & 1) * 256;
       bias_t[et] = bias_next;
-      bias_next = load_bias(w + step);
+      live = wk.next();
+      bias_next = load_bias();
       epi_bar_sync();                              // the bias of this tile is written
       ptx::mbar_wait_warp(&tmem_full[acc], (j >> 1) & 1, dead);
       ptx::tc_fence_after();
@@ -285,11 +319,12 @@ gemm_pair_bf16_tcgen05(const __grid_constant__ CUtensorMap tmA, const __grid_con
       uint32_t r[2][32];
       ptx::tmem_ld32(taddr, r[0]);
 #pragma unroll
-      for (int ps = 0; ps < PASSES; ++ps, ++u) {
+      for (int ps = 0; ps < 4; ++ps) {
+        if (ps >= units) break;
         const int bsel = u % NSB;
         uint8_t* obase = out_stage + bsel * GEMM_STAGE_OUT + row * 128;
         ptx::tmem_ld_wait();
-        if (ps + 1 < PASSES) {
+        if (ps + 1 < units) {
           ptx::tmem_ld32(taddr + (ps + 1) * GEMM_PASS_COLS, r[(ps + 1) & 1]);
         } else {
           // every column of this warp's share has left TMEM: tell the leader's MMA thread
@@ -331,6 +366,7 @@ gemm_pair_bf16_tcgen05(const __grid_constant__ CUtensorMap tmA, const __grid_con
         ptx::fence_proxy_async();
         __syncwarp();
         if (lane == 0) ptx::mbar_arrive(&buf_filled[bsel]);
+        ++u;
       }
     }
   }

@@ -93,3 +93,24 @@ def test_attention_blocks_items_and_tables(lens):
     p.run()
     for a, b in zip(outs, p.outputs()):
         assert np.array_equal(a["y"], b["y"])
+
+
+@pytest.mark.parametrize("K,N,M,act,residual", [(768, 768, 7169, None, True), (768, 2312, 4224, "Gelu", False), (3072, 768, 4100, "Relu", True), (3072, 776, 11009, None, False), (768, 392, 12700, None, True)])
+def test_gemm_pairs_by_rule(K, N, M, act, residual):
+    # sizes at which the dispatch takes CTA pairs by itself: tiles of 192 and 256 columns, a ragged last column unit, the last
+    # wave's tiles cut in two, row tiles in bands, an odd number of 128-row tiles
+    ir = f"sym M 1 20000\ninput x bf16 [1,M,{K}]\n" + (f"input r bf16 [1,M,{N}]\n" if residual else "") + f"const W bf16 [{K},{N}]\nconst b bf16 [{N}]\nnode MatMul x W -> t0\nnode Add t0 b -> t1\n"
+    ir += (f"node {act} t1 -> t2\n" if act else "") + (f"node Add {'t2' if act else 't1'} r -> y\n" if residual else "")
+    y = "y" if residual else "t2" if act else "t1"
+    ir += f"output {y}\n"
+    rng = np.random.default_rng(47)
+    consts = {"W": bf16_round((rng.standard_normal((K, N)) / np.sqrt(K)).astype(np.float32)), "b": bf16_round(rng.standard_normal(N).astype(np.float32))}
+    ins = {"x": bf16_round(rng.standard_normal((1, M, K), dtype=np.float32))}
+    if residual:
+        ins["r"] = bf16_round(rng.standard_normal((1, M, N), dtype=np.float32))
+    reqs = [Request({"M": M}, ins)]
+    wl = WL.Workload("gemm_pair_rule", "bf16", ir, consts, ["M"], [y], {"batch_fn": lambda j: reqs})
+    _, p, outs = run_batch(wl, reqs)
+    assert O.rel_err(outs[0][y], O.run(ir, consts, ins)[y]) <= BF16_TOL
+    p.run()
+    assert np.array_equal(outs[0][y], p.outputs()[0][y])
