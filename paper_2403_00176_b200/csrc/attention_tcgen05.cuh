@@ -64,21 +64,6 @@ __device__ __forceinline__ float ex2_approx(float x) {
   return y;
 }
 
-// two fp32 lanes per instruction
-__device__ __forceinline__ float2 fma_x2(float2 a, float2 b, float2 c) {
-  float2 d;
-  asm("{\n\t.reg .b64 a, b, c, d;\n\tmov.b64 a, {%2, %3};\n\tmov.b64 b, {%4, %5};\n\tmov.b64 c, {%6, %7};\n\t"
-      "fma.rn.f32x2 d, a, b, c;\n\tmov.b64 {%0, %1}, d;\n\t}"
-      : "=f"(d.x), "=f"(d.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y), "f"(c.x), "f"(c.y));
-  return d;
-}
-__device__ __forceinline__ float2 add_x2(float2 a, float2 b) {
-  float2 d;
-  asm("{\n\t.reg .b64 a, b, d;\n\tmov.b64 a, {%2, %3};\n\tmov.b64 b, {%4, %5};\n\tadd.rn.f32x2 d, a, b;\n\tmov.b64 {%0, %1}, d;\n\t}"
-      : "=f"(d.x), "=f"(d.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
-  return d;
-}
-
 // maximum of 32 scores, three operands per instruction
 __device__ __forceinline__ float atc_max32(float mx, const uint32_t* s) {
   float mx0 = mx, mx1 = -INFINITY;
@@ -93,9 +78,9 @@ __device__ __forceinline__ float atc_max32(float mx, const uint32_t* s) {
 __device__ __forceinline__ void atc_exp32(const uint32_t* s, uint32_t* pk, float2 c2, float2 mc2, float2* l) {
 #pragma unroll
   for (int e = 0; e < 32; e += 2) {
-    const float2 t = fma_x2(make_float2(__uint_as_float(s[e]), __uint_as_float(s[e + 1])), c2, mc2);
+    const float2 t = ptx::fma_x2(make_float2(__uint_as_float(s[e]), __uint_as_float(s[e + 1])), c2, mc2);
     const float2 q = make_float2(ex2_approx(t.x), ex2_approx(t.y));
-    *l = add_x2(*l, q);
+    *l = ptx::add_x2(*l, q);
     const __nv_bfloat162 pb = __floats2bfloat162_rn(q.x, q.y);
     pk[e >> 1] = *reinterpret_cast<const uint32_t*>(&pb);
   }

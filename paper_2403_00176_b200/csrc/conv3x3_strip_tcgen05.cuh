@@ -283,7 +283,6 @@ conv3x3_strip_bf16_tcgen05(const __grid_constant__ Conv3Batch B, const __grid_co
     const int row = q * 32 + lane;
     const float relu2_floor = p.act2 == ACT_RELU ? 0.0f : -INFINITY;
     auto group_bar = [&]() { asm volatile("bar.sync %0, 256;" ::"r"(1 + g) : "memory"); };
-    const float4* bp4 = reinterpret_cast<const float4*>(bias_s + half * 32);
     for (int j = g; j < end - begin; j += 2) {
       const int blk = j % NB, bsel = j % NSB;
       ptx::mbar_wait_warp(&tmem_full[blk], (j / NB) & 1, dead);
@@ -295,14 +294,7 @@ conv3x3_strip_bf16_tcgen05(const __grid_constant__ Conv3Batch B, const __grid_co
       __syncwarp();
       if (lane == 0) ptx::mbar_arrive(&tmem_empty[blk]);
       float v[32];
-#pragma unroll
-      for (int i4 = 0; i4 < 8; ++i4) {
-        const float4 b4 = bp4[i4];
-        v[4 * i4] = apply_act<ACT>(__uint_as_float(r[4 * i4]) + b4.x);
-        v[4 * i4 + 1] = apply_act<ACT>(__uint_as_float(r[4 * i4 + 1]) + b4.y);
-        v[4 * i4 + 2] = apply_act<ACT>(__uint_as_float(r[4 * i4 + 2]) + b4.z);
-        v[4 * i4 + 3] = apply_act<ACT>(__uint_as_float(r[4 * i4 + 3]) + b4.w);
-      }
+      bias_act32<ACT>(v, r, bias_s + half * 32);
       uint8_t* obase = out_stage + bsel * CONV_STAGE_OUT + row * 128;
       uint4 rv[4];        // residual loads together, then the arithmetic, then the stores (never reordered by the compiler)
       ptx::mbar_wait_warp(&res_full[bsel], (j / NSB) & 1, dead);

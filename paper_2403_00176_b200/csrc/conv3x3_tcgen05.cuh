@@ -277,8 +277,7 @@ conv3x3_rows_bf16_tcgen05(const __grid_constant__ Conv3Batch B, const __grid_con
         const float* bp = bias_t + ps * 64 + half * 32;
         float v[32];
         if (live) {
-#pragma unroll
-          for (int i = 0; i < 32; ++i) v[i] = apply_act<ACT>(__uint_as_float(r[i]) + bp[i]);
+          bias_act32<ACT>(v, r, bp);
         }
         ptx::mbar_wait_warp(&res_full[bsel], (u / NSB) & 1, dead);
         if (et == 0) { SOD2_TRACE(3, 410) }

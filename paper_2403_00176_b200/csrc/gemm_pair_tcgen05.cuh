@@ -334,8 +334,7 @@ gemm_pair_bf16_tcgen05(const __grid_constant__ CUtensorMap tmA, const __grid_con
         }
         const float* bp = bias_t + ps * GEMM_PASS_COLS + half * 32;
         float v[32];
-#pragma unroll
-        for (int i = 0; i < 32; ++i) v[i] = apply_act<ACT>(__uint_as_float(r[ps & 1][i]) + bp[i]);
+        bias_act32<ACT>(v, r[ps & 1], bp);
         uint4 pk[4];
         if constexpr (!RES) {
 #pragma unroll

@@ -87,26 +87,47 @@ struct GemmSmem {
 };
 
 // GELU(x) = x * Phi(x) with Phi written as 0.5 * (1 + tanh(u(x))), u(x) = atanh(erf(x / sqrt 2)).
-// u is odd; x * (c0 + c1 x^2 + c2 x^4) fitted by least squares on [-8, 8] reproduces the erf form of
-// GELU to 3e-5 absolute, and the hardware tanh adds a relative 2^-11: both far inside the bf16 output
-// rounding.  x^2 is clamped where the quintic would turn over (|x| > 7; tanh is saturated there).
-// Eight instructions per element instead of seventeen for a polynomial erf: the epilogue of a
-// GELU GEMM is bound by instruction issue.
-__device__ __forceinline__ float gelu_erf(float x) {
-  const float x2 = fminf(x * x, 50.0f);
-  const float u = x * fmaf(x2, fmaf(x2, -0.00035873236f, 0.037050345f), 0.79745847f);
-  float t;
-  asm("tanh.approx.f32 %0, %1;" : "=f"(t) : "f"(u));
-  const float hx = 0.5f * x;
-  return fmaf(hx, t, hx);
+// u is odd; x * (c0 + c1 x^2 + c2 x^4 + c3 x^6), fitted (reweighted least squares, c3 > 0 fixed so that u rises for all
+// x) on [-9, 9], reproduces the erf form of GELU to 2.9e-5 absolute, and the hardware tanh adds a relative 2^-11: both
+// far inside the bf16 output rounding.  No clamp is needed, so all but the tanh goes two elements per instruction: with
+// the bias and the packing 11 instructions per pair, where a scalar quintic with its clamp took 19 and a polynomial erf
+// 35.  The epilogue of a GELU GEMM is bound by instruction issue: 14072 x 3072 x 768 57.5 -> 55.4 us,
+// 2176 rows 14.9 -> 13.9 us against the scalar form.
+__device__ __forceinline__ float2 gelu_x2(float2 x) {
+  const float2 t = ptx::mul_x2(x, x);
+  float2 p = ptx::fma_x2(t, make_float2(2.0e-6f, 2.0e-6f), make_float2(-0.0003754595f, -0.0003754595f));
+  p = ptx::fma_x2(t, p, make_float2(0.03707786f, 0.03707786f));
+  p = ptx::fma_x2(t, p, make_float2(0.79745764f, 0.79745764f));
+  const float2 u = ptx::mul_x2(x, p);
+  float2 th;
+  asm("tanh.approx.f32 %0, %1;" : "=f"(th.x) : "f"(u.x));
+  asm("tanh.approx.f32 %0, %1;" : "=f"(th.y) : "f"(u.y));
+  const float2 hx = ptx::mul_x2(x, make_float2(0.5f, 0.5f));
+  return ptx::fma_x2(hx, th, hx);
 }
 // The activation is a template parameter: a run-time switch inside the unrolled element loops
 // turns every element into its own basic block and serialises the dependent FMA / MUFU chains.
 template <int ACT>
-__device__ __forceinline__ float apply_act(float v) {
-  if constexpr (ACT == ACT_GELU) return gelu_erf(v);
-  else if constexpr (ACT == ACT_RELU) return fmaxf(v, 0.0f);
+__device__ __forceinline__ float2 apply_act_x2(float2 v) {
+  if constexpr (ACT == ACT_GELU) return gelu_x2(v);
+  else if constexpr (ACT == ACT_RELU) return make_float2(fmaxf(v.x, 0.0f), fmaxf(v.y, 0.0f));
   else return v;
+}
+template <int ACT>
+__device__ __forceinline__ float apply_act(float v) {
+  return apply_act_x2<ACT>(make_float2(v, 0.0f)).x;
+}
+// 32 accumulators + bias (128-byte aligned, the same for all lanes), activated
+template <int ACT>
+__device__ __forceinline__ void bias_act32(float* v, const uint32_t* r, const float* bias) {
+  const float4* b4 = reinterpret_cast<const float4*>(bias);      // eight 16-byte broadcast loads
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    const float4 b = b4[i];
+    const float2 lo = apply_act_x2<ACT>(ptx::add_x2(make_float2(__uint_as_float(r[4 * i]), __uint_as_float(r[4 * i + 1])), make_float2(b.x, b.y)));
+    const float2 hi = apply_act_x2<ACT>(ptx::add_x2(make_float2(__uint_as_float(r[4 * i + 2]), __uint_as_float(r[4 * i + 3])), make_float2(b.z, b.w)));
+    v[4 * i] = lo.x; v[4 * i + 1] = lo.y; v[4 * i + 2] = hi.x; v[4 * i + 3] = hi.y;
+  }
 }
 
 __device__ __forceinline__ void tma_store_2d(const void* tmap, const void* src, int x, int y) {
@@ -456,16 +477,7 @@ gemm_bf16_tcgen05(const __grid_constant__ CUtensorMap tmA, const __grid_constant
 #pragma unroll
           for (int i = 0; i < 32; ++i) v[i] = apply_act<ACT>(fmaf(ln_rstd, __uint_as_float(r[ps & 1][i]), fmaf(nmr, bp[BN + i], bp[i])));
         } else {
-          // the 32 bias values as eight 16-byte broadcast loads (the offset is a multiple of 128 bytes)
-          const float4* bp4 = reinterpret_cast<const float4*>(bp);
-#pragma unroll
-          for (int i4 = 0; i4 < 8; ++i4) {
-            const float4 b4 = bp4[i4];
-            v[4 * i4] = apply_act<ACT>(__uint_as_float(r[ps & 1][4 * i4]) + b4.x);
-            v[4 * i4 + 1] = apply_act<ACT>(__uint_as_float(r[ps & 1][4 * i4 + 1]) + b4.y);
-            v[4 * i4 + 2] = apply_act<ACT>(__uint_as_float(r[ps & 1][4 * i4 + 2]) + b4.z);
-            v[4 * i4 + 3] = apply_act<ACT>(__uint_as_float(r[ps & 1][4 * i4 + 3]) + b4.w);
-          }
+          bias_act32<ACT>(v, r[ps & 1], bp);
         }
         uint4 pk[4];
         if constexpr (!RES) {
