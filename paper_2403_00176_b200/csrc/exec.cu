@@ -19,6 +19,7 @@
 #include "gemm_tcgen05.cuh"
 #include "gemm_chain_tcgen05.cuh"
 #include "gemm_pair_tcgen05.cuh"
+#include "gemm_cluster_tcgen05.cuh"
 #include "kernels_compact.cuh"
 #include "kernels_rows.cuh"
 #include "kernels_unfused.cuh"
@@ -72,9 +73,9 @@ cudaError_t launch_pdl(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t sme
   return cudaLaunchKernelEx(&cfg, kern, std::forward<Args>(args)...);
 }
 
-// The same with a thread-block cluster of two CTAs along x (the CTA-pair GEMM).
+// The same with a thread-block cluster of `cluster` CTAs along x (the CTA-pair and the split-K GEMM).
 template <typename... KArgs, typename... Args>
-cudaError_t launch_pdl_pair(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args&&... args) {
+cudaError_t launch_pdl_cluster(int cluster, void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args&&... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = block;
@@ -84,7 +85,7 @@ cudaError_t launch_pdl_pair(void (*kern)(KArgs...), dim3 grid, dim3 block, size_
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   attr[1].id = cudaLaunchAttributeClusterDimension;
-  attr[1].val.clusterDim.x = 2;
+  attr[1].val.clusterDim.x = cluster;
   attr[1].val.clusterDim.y = 1;
   attr[1].val.clusterDim.z = 1;
   cfg.attrs = attr;
@@ -161,7 +162,7 @@ cudaError_t launch_gemm_pair_variant(dim3 grid, cudaStream_t st, const CUtensorM
   constexpr int smem = k::GemmPairSmem::TOTAL;
   static bool once = (cudaFuncSetAttribute(k::gemm_pair_bf16_tcgen05<ACT, RES>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem), true);
   (void)once;
-  return launch_pdl_pair(k::gemm_pair_bf16_tcgen05<ACT, RES>, grid, dim3(k::GEMM_THREADS), smem, st, ta, tb, to, tr, M, N, K, ep, sp);
+  return launch_pdl_cluster(2, k::gemm_pair_bf16_tcgen05<ACT, RES>, grid, dim3(k::GEMM_THREADS), smem, st, ta, tb, to, tr, M, N, K, ep, sp);
 }
 cudaError_t gemm_pair_dispatch(int act, bool res, dim3 grid, cudaStream_t st, const CUtensorMap& ta, const k::GemmPairMaps& tb, const CUtensorMap& to,
                                const CUtensorMap& tr, int M, int N, int K, const k::GemmEpilogue& ep, const k::PairSplit& sp) {
@@ -173,6 +174,19 @@ cudaError_t gemm_pair_dispatch(int act, bool res, dim3 grid, cudaStream_t st, co
     case 4: return launch_gemm_pair_variant<2, false>(grid, st, ta, tb, to, tr, M, N, K, ep, sp);
     default: return launch_gemm_pair_variant<2, true>(grid, st, ta, tb, to, tr, M, N, K, ep, sp);
   }
+}
+
+template <int S, int ACT>
+cudaError_t launch_gemm_cluster_variant(int tiles, cudaStream_t st, const CUtensorMap& ta, const CUtensorMap& tb, const k::GemmClusterParams& cp) {
+  constexpr int smem = k::GemmClusterSmem::TOTAL;
+  static bool once = (cudaFuncSetAttribute(k::gemm_cluster_bf16_tcgen05<S, ACT>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem), true);
+  (void)once;
+  return launch_pdl_cluster(S, k::gemm_cluster_bf16_tcgen05<S, ACT>, dim3(tiles * S), dim3(k::GCL_THREADS), smem, st, ta, tb, cp);
+}
+template <int S>
+cudaError_t gemm_cluster_act(int act, int tiles, cudaStream_t st, const CUtensorMap& ta, const CUtensorMap& tb, const k::GemmClusterParams& cp) {
+  if (act == 0) return launch_gemm_cluster_variant<S, 0>(tiles, st, ta, tb, cp);
+  return act == 1 ? launch_gemm_cluster_variant<S, 1>(tiles, st, ta, tb, cp) : launch_gemm_cluster_variant<S, 2>(tiles, st, ta, tb, cp);
 }
 
 struct Builder : BuildState {
@@ -460,6 +474,18 @@ struct Builder : BuildState {
         static const bool force_pair = getenv("SOD2_GEMM_PAIR_FORCE") != nullptr;   // tests: the pair kernel wherever it is eligible
         pair = (c.flags & OPT_GEMM_PAIR) ? (best < single || force_pair) : (K >= 12 * 64 && best + 2000.0 < single);
       }
+      // Few tiles and a long K: S CTAs of a cluster share a tile's K (gemm_cluster_tcgen05.cuh), as many as the chip can hold
+      // clusters for (measured with this kernel's shared memory: 15, 33 and 74 of 8, 4 and 2 CTAs; a second wave would cost
+      // more than the split gains).  The exchange takes about 1.2 us, a 64-wide chunk 0.16 us: 48 chunks gain from any S
+      // (64 rows: 11.8 -> 9.8, 7.2, 5.9 us with S = 2, 4, 8), 24 as well (7.5 -> 6.7, 5.7, 5.0), 12 chunks gain 10 % with
+      // S = 4, with S = 2 only while half of the tile's rows are empty; 6 chunks lose.
+      int ksplit = 0;
+      if (!pair && !lna && !lnr && !emit && bn == 64) {
+        const int tiles = tiles_m * static_cast<int>((N + 63) / 64), chunks = static_cast<int>(K / 64);
+        if (tiles <= 15 && chunks >= 24) ksplit = 8;
+        else if (tiles <= 33 && chunks >= 12) ksplit = 4;
+        else if (tiles <= 74 && (chunks >= 24 || (chunks >= 12 && M <= 64))) ksplit = 2;
+      }
       const bool hb = G.bias >= 0, hr = G.res >= 0;
       const int act = G.act;
       const int act2 = G.act2;
@@ -485,7 +511,7 @@ struct Builder : BuildState {
         void* O = x.resolve(po);
         const void* R = hr ? x.resolve(pr) : O;
         if (cache->a != A || cache->w != Wt || cache->o != O || cache->r != R) {
-          const int kch = pair || bn == 256 ? 1 : 2;
+          const int kch = pair || ksplit || bn == 256 ? 1 : 2;
           bool ok = encode_bf16_kchunks(&cache->ta, A, M, K, lda, 128, kch) && encode_bf16_2d(&cache->to, O, M, N, ldo, 128) &&
                     encode_bf16_2d(&cache->tr, R, M, N, hr ? ldr : ldo, 128);
           if (!pair) ok = ok && encode_bf16_kchunks(&cache->tb, Wt, N, K, K, bn, kch);
@@ -518,6 +544,20 @@ struct Builder : BuildState {
           ep.emit_pitch = pitch_out;
         }
         const int Ni = static_cast<int>(N), Ki = static_cast<int>(K);
+        if (ksplit) {
+          k::GemmClusterParams cp{};
+          cp.out = static_cast<__nv_bfloat16*>(O);
+          cp.res = hr ? static_cast<const __nv_bfloat16*>(R) : nullptr;
+          cp.bias = ep.bias;
+          cp.ldo = ldo; cp.ldr = ldr;
+          cp.M = M; cp.N = Ni; cp.K = Ki; cp.act2 = act2;
+          cp.status = ep.status;
+          const int tiles = tiles_m * ((Ni + 63) / 64);
+          const cudaError_t ec = ksplit == 8 ? gemm_cluster_act<8>(act, tiles, x.stream, cache->ta, cache->tb, cp)
+                               : ksplit == 4 ? gemm_cluster_act<4>(act, tiles, x.stream, cache->ta, cache->tb, cp)
+                                             : gemm_cluster_act<2>(act, tiles, x.stream, cache->ta, cache->tb, cp);
+          return ec != cudaSuccess ? ec : cudaGetLastError();
+        }
         if (pair) {
           const int tiles = ((tiles_m + 1) / 2) * static_cast<int>(((N + 63) / 64 + split.bw - 1) / split.bw);
           const int items = split.n_full + (tiles - split.n_full) * split.parts;

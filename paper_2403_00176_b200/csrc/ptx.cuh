@@ -14,6 +14,10 @@
 namespace sod2 {
 namespace ptx {
 
+// A parked wait (try_wait suspends the warp for a time the hardware chooses) is bounded by cycles instead: about half a second.
+#ifndef SOD2_WAIT_CYCLES
+#define SOD2_WAIT_CYCLES (1ll << 30)
+#endif
 #ifndef SOD2_SPIN_LIMIT
 #define SOD2_SPIN_LIMIT (1u << 24)
 #endif
@@ -97,12 +101,12 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volati
 // (tcgen05.ld and .st).  A __syncwarp in each wait of the producers and issuers cost a 64-token GEMM 0.2 us (of 7.5).
 __device__ __forceinline__ void mbar_wait_elect(uint64_t* bar, uint32_t parity, volatile int* dead) {
   if (__builtin_expect(mbar_test_wait(bar, parity), 1)) return;
+  const long long give_up = clock64() + SOD2_WAIT_CYCLES;
 #pragma unroll 1
-  for (uint32_t i = 0; i < SOD2_SPIN_LIMIT / 16; ++i) {
-    if (mbar_try_wait(bar, parity)) return;
-    if ((i & 63u) == 63u && *dead) return;
+  while (!mbar_try_wait(bar, parity)) {
+    if (*dead) return;
+    if (clock64() > give_up) { *dead = 1; return; }
   }
-  *dead = 1;
 }
 __device__ __forceinline__ void mbar_wait_warp(uint64_t* bar, uint32_t parity, volatile int* dead) {
   mbar_wait_elect(bar, parity, dead);

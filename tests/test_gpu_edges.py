@@ -114,3 +114,23 @@ def test_gemm_pairs_by_rule(K, N, M, act, residual):
     assert O.rel_err(outs[0][y], O.run(ir, consts, ins)[y]) <= BF16_TOL
     p.run()
     assert np.array_equal(outs[0][y], p.outputs()[0][y])
+
+
+@pytest.mark.parametrize("K,N,Ms", [(3072, 768, [1, 64, 97, 128]), (1536, 392, [129, 256, 300]), (1600, 776, [513, 640]), (768, 1000, [63, 64, 65]), (832, 2304, [33])])
+@pytest.mark.parametrize("act,residual", [("Gelu", False), (None, True)])
+def test_gemm_k_split_over_clusters(K, N, Ms, act, residual):
+    # clusters of 8, 4 and 2 CTAs: shares of rows with none left for the last ranks, a ragged last column tile, chunk counts the
+    # cluster does not divide (25, 13), the ReLU behind the residual, two row tiles with one row in the last
+    ir = f"sym M 1 1000\ninput x bf16 [1,M,{K}]\n" + (f"input r bf16 [1,M,{N}]\n" if residual else "") + f"const W bf16 [{K},{N}]\nconst b bf16 [{N}]\nnode MatMul x W -> t0\nnode Add t0 b -> t1\n"
+    ir += (f"node {act} t1 -> y\n" if act else "node Add t1 r -> t2\nnode Relu t2 -> y\n") + "output y\n"
+    rng = np.random.default_rng(53)
+    consts = {"W": bf16_round((rng.standard_normal((K, N)) / np.sqrt(K)).astype(np.float32)), "b": bf16_round(rng.standard_normal(N).astype(np.float32))}
+    wl = WL.Workload("gemm_cluster", "bf16", ir, consts, ["M"], ["y"], {"batch_fn": lambda j: []})
+    for M in Ms:
+        ins = {"x": bf16_round(rng.standard_normal((1, M, K)).astype(np.float32))}
+        if residual:
+            ins["r"] = bf16_round(rng.standard_normal((1, M, N)).astype(np.float32))
+        _, p, outs = run_batch(wl, [Request({"M": M}, ins)])
+        assert O.rel_err(outs[0]["y"], O.run(ir, consts, ins)["y"]) <= BF16_TOL, M
+        p.run()
+        assert np.array_equal(outs[0]["y"], p.outputs()[0]["y"])
