@@ -14,7 +14,8 @@
 // buffer to the softmax warps seeing it) is under way a whole block ahead -- 64 keys are what TMEM holds twice at two
 // CTAs per SM; no exchange between threads (with two threads per row, the scores read twice and the row maximum exchanged
 // through shared memory, 128 keys took 3600 cycles of an SM); two scores per instruction where the FMA pipe has the form.
-// The CTAs are persistent and take items round robin, longest request first; phases run on from item to item: the
+// The CTAs are persistent and take items back and forth, longest request first (16 requests of 238 to 780 tokens, 6 heads:
+// the busiest CTA has 23 blocks, round robin 26; at 0.7 of the tokens 11 against 15); phases run on from item to item: the
 // softmax warps go straight on to the next item's first block and write an item's output between that block's
 // exponentials and its P, by when the last product has landed.
 // Q, K, V are 2-D tensor maps over the packed [tokens, row stride] buffers; a tile that runs past a
@@ -118,6 +119,8 @@ attention_tcgen05_bf16(const __grid_constant__ CUtensorMap tmQ, const __grid_con
     starts[t] = t < p.n_req ? p.tile_start[t] : 0x7fffffff;
     if (t < p.n_req) reqs[t] = p.r[t];
   }
+  // the CTA's i-th item: rounds go back and forth, so that who has the longest item of one round has the shortest of the next
+  auto nth_item = [&](int i) { return i * static_cast<int>(gridDim.x) + static_cast<int>((i & 1) ? gridDim.x - 1 - blockIdx.x : blockIdx.x); };
   struct Item { int head, q0, L, nkv, ri; };
   auto locate = [&](int item) {
     Item it;
@@ -160,7 +163,7 @@ attention_tcgen05_bf16(const __grid_constant__ CUtensorMap tmQ, const __grid_con
     const bool is_k = warp == 4;
     ptx::pdl_wait();
     int n = 0, i = 0;
-    for (int item = blockIdx.x; item < items; item += gridDim.x, ++i) {
+    for (int item; (item = nth_item(i)) < items; ++i) {
       const Item it = locate(item);
       const AtcReq R = reqs[it.ri];
       if (is_k) {
@@ -192,7 +195,7 @@ attention_tcgen05_bf16(const __grid_constant__ CUtensorMap tmQ, const __grid_con
     // ---- S issuer: S_n once S_{n-2} is in registers
     constexpr uint32_t idesc_qk = ptx::idesc_bf16(128, ATC_KB);
     int n = 0, i = 0;
-    for (int item = blockIdx.x; item < items; item += gridDim.x, ++i) {
+    for (int item; (item = nth_item(i)) < items; ++i) {
       const Item it = locate(item);
       const uint64_t dQ = ptx::smem_desc_sw128(ptx::smem_u32(sQ + (i & 1) * ATC_Q_BYTES));
       ptx::mbar_wait_warp(&q_full[i & 1], (i >> 1) & 1, dead);
@@ -216,7 +219,7 @@ attention_tcgen05_bf16(const __grid_constant__ CUtensorMap tmQ, const __grid_con
     // before they hand over the next item's first P, so the accumulator needs no barrier of its own.
     constexpr uint32_t idesc_pv = ptx::idesc_bf16(128, 64) | (1u << 16);   // B (= V tile) is MN-major
     int n = 0;
-    for (int item = blockIdx.x; item < items; item += gridDim.x) {
+    for (int i = 0, item; (item = nth_item(i)) < items; ++i) {
       const Item it = locate(item);
       for (int j = 0; j < it.nkv; ++j, ++n) {
         const int steps = (it.L - j * ATC_KB + 15) >> 4;       // keys past the request are left out
@@ -290,7 +293,7 @@ attention_tcgen05_bf16(const __grid_constant__ CUtensorMap tmQ, const __grid_con
     };
     int n = 0, i = 0;
     bool s_seen = false;
-    for (int item = blockIdx.x; item < items; item += gridDim.x, ++i) {
+    for (int item; (item = nth_item(i)) < items; ++i) {
       const Item it = locate(item);
       const bool live = it.q0 + warp * 32 < it.L;    // a warp whose 32 rows are all past the request only keeps the barriers moving
       // Online softmax with a lazily updated reference: the exponent reference m only moves when a block's
