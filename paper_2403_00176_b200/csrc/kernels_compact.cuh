@@ -51,16 +51,18 @@ __global__ void __launch_bounds__(256) row_sumsq_f64(ScoreParams p) {
 }
 
 // ---------------------------------------------------------------------------------------------
-// Keep the k highest-scoring tokens of each request in ascending index order.
-//   rank_i = #{j : s_j > s_i} + #{j < i : s_j == s_i};  keep_i = rank_i < k
-//   pos_i  = exclusive scan of keep;  idx[pos_i] = i;  out[pos_i, :] = y[i, :]
-// Two kernels over the same grid, one CTA per chunk of 64 tokens of a request (so a batch of 16
-// requests spreads over about a hundred SMs instead of 16):
-//   topk_flags   the request's fp64 scores staged in shared memory; four threads share a token's
-//                ranking (a quarter of the comparisons each); writes keep_i as a byte
-//   topk_gather  counts the kept tokens before the chunk, scans the chunk's 64 flags with two ballots,
-//                writes the indices and copies the kept rows, one warp per row, 128-bit accesses
-constexpr int TOPK_CHUNK = 64;
+// Keep the k highest-scoring tokens of each request in ascending index order, ties by the lower index:
+//   keep_i = s_i > T, or s_i == T and fewer than `rem` equal scores before i;  pos_i = #{j < i : keep_j}
+//   idx[pos_i] = i;  out[pos_i, :] = y[i, :]
+// with T the k-th largest score and `rem` the number of scores equal to T that are kept.  One CTA per chunk of 32 tokens
+// (a single request of 577 tokens is 19 CTAs, 16 of 500 are 250); every CTA selects T for itself out of its request's
+// scores in shared memory, so nothing has to be exchanged between CTAs and one launch does: scores as 64-bit integers in
+// the order of the doubles, radix selection eight bits at a time from the highest bit in which any two scores differ,
+// until the digit found is kept whole (two or three passes for scores that differ).
+// Bound by latency: the wait for the scores, about 200 cycles per pass, the rows out.  With the score kernel, against a
+// kernel that ranked every token with all others in fp64 and one that copied (D = 384): 16 requests of 238 to 780 tokens
+// 28.4 -> 9.1 us, one of 577 tokens 9.7 -> 6.2 us.
+constexpr int TOPK_CHUNK = 32, TOPK_THREADS = 256;
 struct TopkReq {
   long long row0;      // first packed input row of the request
   long long out_row0;  // first packed output row
@@ -70,13 +72,12 @@ struct TopkReq {
 struct TopkParams {
   const __nv_bfloat16* y;
   const double* score;       // packed [rows] relative to the first request's row0
-  unsigned char* keep;       // packed [rows], same indexing as score
   __nv_bfloat16* out;
   long long* idx;            // packed [sum k] int64, per request k entries
   int D;
   int n_req;
-  long long first_row;       // row0 of the first request (score / keep are indexed from it)
-  int chunk_start[COMPACT_MAX_REQ + 1];   // prefix sum of ceil(n / 64)
+  long long first_row;       // row0 of the first request (scores are indexed from it)
+  int chunk_start[COMPACT_MAX_REQ + 1];   // prefix sum of ceil(n / TOPK_CHUNK)
   TopkReq r[COMPACT_MAX_REQ];
 };
 
@@ -87,80 +88,106 @@ __device__ __forceinline__ int topk_locate(const TopkParams& p, int cta, int* ch
   return ri;
 }
 
-__global__ void __launch_bounds__(256) topk_flags(const __grid_constant__ TopkParams p) {
-  extern __shared__ double s_score[];                  // [n]
-  int chunk;
-  const TopkReq R = p.r[topk_locate(p, blockIdx.x, &chunk)];
-  ptx::pdl_wait();
-  ptx::pdl_launch();
-  const int tid = threadIdx.x;
-  const double* sc = p.score + (R.row0 - p.first_row);
-  // a NaN score (an overflow upstream) compares false with everything and would be kept by every chunk: it ranks
-  // last instead, ties among NaNs by index, so that exactly k tokens are kept whatever the data
-  for (int i = tid; i < R.n; i += 256) { const double v = sc[i]; s_score[i] = v == v ? v : -INFINITY; }
-  __syncthreads();
-  const int i = chunk * TOPK_CHUNK + (tid >> 2), part = tid & 3;
-  int rank = 0;
-  if (i < R.n) {
-    const double si = s_score[i];
-    const int per = (R.n + 3) >> 2, j0 = part * per, j1 = min(R.n, j0 + per);
-    for (int j = j0; j < j1; ++j) {
-      const double sj = s_score[j];
-      rank += (sj > si) || (sj == si && j < i);
-    }
-  }
-  rank += __shfl_xor_sync(0xffffffffu, rank, 1);
-  rank += __shfl_xor_sync(0xffffffffu, rank, 2);
-  if (i < R.n && part == 0) p.keep[R.row0 - p.first_row + i] = rank < R.k;
-}
-
-__global__ void __launch_bounds__(256) topk_gather(const __grid_constant__ TopkParams p) {
-  __shared__ int warp_cnt[8];
-  __shared__ int s_pos[TOPK_CHUNK];
+__global__ void __launch_bounds__(TOPK_THREADS) topk_select_gather(const __grid_constant__ TopkParams p) {
+  extern __shared__ unsigned long long s_key[];        // [n]
+  __shared__ unsigned s_hist[256];
+  __shared__ unsigned s_diff[2];
+  __shared__ int s_found[3], s_before[2], s_pos[TOPK_CHUNK];
   int chunk;
   const TopkReq R = p.r[topk_locate(p, blockIdx.x, &chunk)];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int base = chunk * TOPK_CHUNK;
-  // The rows of the chunk are fetched before the dependency wait: they were written by the kernel before the
-  // score kernel, which had completed before the flag kernel (the one waited for here) let this one start, so
-  // only the flags are still in flight.  Whether a row is kept is not known yet: all rows of the chunk are read.
+  // The rows of the chunk are fetched before the dependency wait: they were written by the kernel before the score
+  // kernel, which had completed before any CTA of the score kernel let this one start, so only the scores are still in
+  // flight.  Whether a row is kept is not known yet: all rows of the chunk are read.
   const int vec = (p.D * 2) >> 4;  // 16-byte pieces per row (D % 8 == 0 checked on the host)
   const uint4* src = reinterpret_cast<const uint4*>(p.y + (R.row0 + base) * p.D);
   const int items = min(TOPK_CHUNK, R.n - base) * vec;
-  constexpr int PRE = 12;
+  constexpr int PRE = 6;
   uint4 pre[PRE];
 #pragma unroll
   for (int u = 0; u < PRE; ++u) {
-    const int it = tid + u * 256;
+    const int it = tid + u * TOPK_THREADS;
     if (it < items) pre[u] = src[it];
   }
+  s_hist[tid] = 0;
+  if (tid < 2) { s_diff[tid] = 0; s_before[tid] = 0; }
   ptx::pdl_wait();
   ptx::pdl_launch();
-  const unsigned char* kp = p.keep + (R.row0 - p.first_row);
-  // kept tokens before this chunk
-  int c = 0;
-  for (int j = tid; j < base; j += 256) c += kp[j];
-#pragma unroll
-  for (int o = 16; o; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
-  if (lane == 0) warp_cnt[warp] = c;
+  // Scores are sums of squares: as integers with the top bit set they keep their order.  A NaN score (an overflow
+  // upstream) becomes 0 and ranks last, ties among NaNs by index, so that exactly k tokens are kept whatever the data.
+  const double* sc = p.score + (R.row0 - p.first_row);
+  auto key_of = [&](int i) -> unsigned long long {
+    const double v = sc[i];
+    return v == v ? static_cast<unsigned long long>(__double_as_longlong(v)) | (1ull << 63) : 0ull;
+  };
+  const unsigned long long key0 = key_of(0);
+  unsigned long long diff = 0;
+  for (int i = tid; i < R.n; i += TOPK_THREADS) { const unsigned long long q = key_of(i); s_key[i] = q; diff |= q ^ key0; }
+  const unsigned d_hi = __reduce_or_sync(0xffffffffu, static_cast<unsigned>(diff >> 32)), d_lo = __reduce_or_sync(0xffffffffu, static_cast<unsigned>(diff));
   __syncthreads();
-  int carry = 0;
+  if (lane == 0) { if (d_hi) atomicOr(&s_diff[1], d_hi); if (d_lo) atomicOr(&s_diff[0], d_lo); }
+  __syncthreads();
+  diff = static_cast<unsigned long long>(s_diff[1]) << 32 | s_diff[0];
+  // T: keys above it are kept, and the first `rem` of those equal to it
+  unsigned long long T = key0;
+  int rem = R.k;
+  if (R.k >= R.n) { T = 0; rem = R.n; }
+  else if (R.k <= 0) { T = ~0ull; rem = 0; }
+  else if (diff) {
+    int top = 64 - __clzll(static_cast<long long>(diff));        // bits not decided yet; those above are the same in all keys
+    unsigned long long high = top < 64 ? key0 >> top : 0ull;
+    for (;;) {
+      const int width = min(8, top), low = top - width;
+      for (int i = tid; i < R.n; i += TOPK_THREADS) {
+        const unsigned long long q = s_key[i];
+        if ((top < 64 ? q >> top : 0ull) == high) atomicAdd(&s_hist[static_cast<unsigned>(q >> low) & ((1u << width) - 1)], 1u);
+      }
+      __syncthreads();
+      if (warp == 0) {
+        // eight digits per lane, from the largest
+        int h[8], c = 0;
 #pragma unroll
-  for (int w = 0; w < 8; ++w) carry += warp_cnt[w];
-  // the chunk's own 64 flags: warps 0 and 1 take 32 each
-  if (warp < 2) {
-    const int i = base + tid;
-    const int keep = i < R.n ? kp[i] : 0;
-    const unsigned bal = __ballot_sync(0xffffffffu, keep);
-    const int pre = __popc(bal & ((1u << lane) - 1));
-    if (lane == 0) warp_cnt[warp] = __popc(bal);
-    __syncwarp();
-    s_pos[tid] = keep ? pre : -1;
+        for (int u = 0; u < 8; ++u) { h[u] = static_cast<int>(s_hist[255 - lane * 8 - u]); c += h[u]; }
+        int incl = c;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) { const int t = __shfl_up_sync(0xffffffffu, incl, o); if (lane >= o) incl += t; }
+        int above = incl - c;
+        if (above < rem && rem <= incl) {
+#pragma unroll
+          for (int u = 0; u < 8; ++u) {
+            if (above < rem && rem <= above + h[u]) { s_found[0] = 255 - lane * 8 - u; s_found[1] = rem - above; s_found[2] = h[u]; }
+            above += h[u];
+          }
+        }
+      }
+      __syncthreads();
+      high = high << width | static_cast<unsigned>(s_found[0]);
+      rem = s_found[1];
+      top = low;
+      if (rem == s_found[2] || top == 0) break;
+      s_hist[tid] = 0;
+      __syncthreads();
+    }
+    T = high << top;
+    if (top > 0) { T -= 1; rem = 0; }      // the digit is kept whole: everything above T
   }
+  // scores above T and equal to it, before the chunk
+  int gt = 0, eq = 0;
+  for (int j = tid; j < base; j += TOPK_THREADS) { const unsigned long long q = s_key[j]; gt += q > T; eq += q == T; }
+  gt = __reduce_add_sync(0xffffffffu, gt);
+  eq = __reduce_add_sync(0xffffffffu, eq);
+  if (lane == 0 && (gt | eq)) { atomicAdd(&s_before[0], gt); atomicAdd(&s_before[1], eq); }
   __syncthreads();
-  if (tid < TOPK_CHUNK && s_pos[tid] >= 0) {
-    s_pos[tid] += carry + (tid >= 32 ? warp_cnt[0] : 0);
-    p.idx[R.idx0 + s_pos[tid]] = base + tid;
+  if (warp == 0) {
+    const int i = base + lane;
+    const unsigned long long q = i < R.n ? s_key[i] : 0ull;
+    const unsigned bg = __ballot_sync(0xffffffffu, i < R.n && q > T), be = __ballot_sync(0xffffffffu, i < R.n && q == T), lt = (1u << lane) - 1;
+    const int eq_before = s_before[1] + __popc(be & lt);
+    const bool keep = ((bg >> lane) & 1u) || (((be >> lane) & 1u) && eq_before < rem);
+    const int pos = s_before[0] + __popc(bg & lt) + min(eq_before, rem);
+    s_pos[lane] = keep ? pos : -1;
+    if (keep) p.idx[R.idx0 + pos] = i;
   }
   __syncthreads();
   // write the kept rows: (row, 16-byte piece) items spread over the whole CTA; the first PRE per thread are
@@ -168,7 +195,7 @@ __global__ void __launch_bounds__(256) topk_gather(const __grid_constant__ TopkP
   uint4* dst = reinterpret_cast<uint4*>(p.out + R.out_row0 * p.D);
 #pragma unroll
   for (int u = 0; u < PRE; ++u) {
-    const int it = tid + u * 256;
+    const int it = tid + u * TOPK_THREADS;
     if (it < items) {
       const int t = it / vec, c4 = it - t * vec;
       const int pos = s_pos[t];
@@ -176,7 +203,7 @@ __global__ void __launch_bounds__(256) topk_gather(const __grid_constant__ TopkP
     }
   }
 #pragma unroll 4
-  for (int it = tid + PRE * 256; it < items; it += 256) {
+  for (int it = tid + PRE * TOPK_THREADS; it < items; it += TOPK_THREADS) {
     const int t = it / vec, c4 = it - t * vec;
     const int pos = s_pos[t];
     if (pos >= 0) dst[static_cast<long long>(pos) * vec + c4] = src[it];

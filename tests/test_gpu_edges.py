@@ -134,3 +134,31 @@ def test_gemm_k_split_over_clusters(K, N, Ms, act, residual):
         assert O.rel_err(outs[0]["y"], O.run(ir, consts, ins)["y"]) <= BF16_TOL, M
         p.run()
         assert np.array_equal(outs[0]["y"], p.outputs()[0]["y"])
+
+
+@pytest.mark.parametrize("n,k,D", [(1, 1, 64), (31, 7, 64), (32, 32, 64), (33, 32, 768), (300, 211, 768), (1025, 40, 64), (7000, 4900, 64)])
+def test_topk_selection_digits_ties_and_chunks(n, k, D):
+    # the radix selection: all scores equal, two values, scores that differ only in their low bits, over the whole exponent
+    # range, distinct ones; chunks of 32 tokens at their edges, everything kept, more shared memory than the default, rows
+    # wider than the prefetch.  Sums of few squares of powers of two are exact in fp64 whatever their order
+    ir = (f"sym N 1 8000\ninput y bf16 [1,N,{D}]\niconst k i64 [1] = {k}\niconst i_m1 i64 [1] = -1\n"
+          "node ReduceSumSquare y -> sc {axis=-1 keepdims=0}\nnode TopK sc k -> tv idx {axis=-1 largest=1 order=index}\n"
+          "node Reshape idx i_m1 -> ix\nnode Gather y ix -> keep {axis=1}\noutput keep\noutput idx\n")
+    rng = np.random.default_rng(59)
+    ys = []
+    for kind in range(5):
+        y = np.zeros((1, n, D), np.float32)
+        y[..., 0] = 1.0
+        if kind == 1: y[0, :, 1] = rng.integers(0, 2, n)
+        if kind == 2: y[0, :, 1] = 2.0 ** -rng.integers(18, 25, n)
+        if kind == 3: y[0, :, 0] = 2.0 ** rng.integers(-60, 60, n)
+        if kind == 4: y = bf16_round(rng.standard_normal((1, n, D)).astype(np.float32))
+        ys.append(y)
+    reqs = [Request({"N": n}, {"y": y}) for y in ys]
+    wl = WL.Workload("topk_edges", "bf16", ir, {}, ["N"], ["keep", "idx"], {"batch_fn": lambda j: reqs})
+    _, p, outs = run_batch(wl, reqs)
+    for r, y in enumerate(ys):
+        sc = (y[0].astype(np.float64) ** 2).sum(-1)
+        want = np.sort(np.argsort(-sc, kind="stable")[:k])
+        assert np.array_equal(outs[r]["idx"][0], want), (r, n, k)
+        assert np.array_equal(outs[r]["keep"][0], y[0][want]), (r, n, k)
