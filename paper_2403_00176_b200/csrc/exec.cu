@@ -1439,11 +1439,13 @@ struct Builder : BuildState {
         B.n_seg = static_cast<int>(batch.size());
         B.C = C;
         int tiles = 0;
-        bool aligned = true;
+        bool aligned = true, any = false;
         for (int i = 0; i < B.n_seg; ++i) {
           B.in[i] = reinterpret_cast<const __nv_bfloat16*>(x.resolve(batch[i].pi));
           B.out[i] = reinterpret_cast<__nv_bfloat16*>(x.resolve(batch[i].po));
           B.HW[i] = batch[i].HW;
+          B.images[i] = batch[i].N;
+          any = any || batch[i].HW % 8 != 0;
           B.tile_start[i] = tiles;
           tiles += batch[i].N * static_cast<int>((batch[i].HW + 63) / 64);
           aligned = aligned && ((reinterpret_cast<uintptr_t>(B.in[i]) | reinterpret_cast<uintptr_t>(B.out[i])) & 15) == 0;
@@ -1451,8 +1453,8 @@ struct Builder : BuildState {
         B.tile_start[B.n_seg] = tiles;
         if (aligned) {
           const dim3 grid(static_cast<unsigned>(tiles), (C + 63) / 64, 1);
-          if (from) k::nhwc_to_nchw_bf16_v8<<<grid, 256, 0, x.stream>>>(B);
-          else k::nchw_to_nhwc_bf16_v8<<<grid, 256, 0, x.stream>>>(B);
+          if (from) (any ? k::nhwc_to_nchw_bf16_v8<true> : k::nhwc_to_nchw_bf16_v8<false>)<<<grid, 256, 0, x.stream>>>(B);
+          else (any ? k::nchw_to_nhwc_bf16_v8<true> : k::nchw_to_nhwc_bf16_v8<false>)<<<grid, 256, 0, x.stream>>>(B);
         } else {   // a caller buffer that is not 16-byte aligned: the element-wise kernels, one tensor at a time
           for (int i = 0; i < B.n_seg; ++i) {
             const dim3 grid(static_cast<unsigned>((B.HW[i] + 63) / 64), (C + 63) / 64, batch[i].N);
@@ -1480,7 +1482,7 @@ struct Builder : BuildState {
       if (!nchw.contiguous() || !is_channels_last(cl)) return fail(E_UNSUPPORTED_OP, "layout change between unexpected layouts");
       const int N = static_cast<int>(vi.dims[0]), C = static_cast<int>(vi.dims[1]);
       const long long HW = vi.dims[2] * vi.dims[3];
-      if (C % 8 == 0 && HW % 8 == 0 && N * ((HW + 63) / 64) < (1ll << 28)) {
+      if (C % 8 == 0 && N * ((HW + 63) / 64) < (1ll << 28)) {
         if (segC >= 0 && segC != C) flush();
         segC = C;
         segs.push_back(Seg{pi, po, HW, N});

@@ -162,3 +162,17 @@ def test_topk_selection_digits_ties_and_chunks(n, k, D):
         want = np.sort(np.argsort(-sc, kind="stable")[:k])
         assert np.array_equal(outs[r]["idx"][0], want), (r, n, k)
         assert np.array_equal(outs[r]["keep"][0], y[0][want]), (r, n, k)
+
+
+@pytest.mark.parametrize("C", [64, 192])
+def test_layout_changes_of_rows_that_start_anywhere(C):
+    # channels-last and back around an identity 1x1 convolution: image sizes of every remainder modulo 8, below and past a
+    # 64-pixel tile, mixed with aligned ones in one launch; exact
+    ir = f"sym H 1 64\nsym W 1 64\ninput x bf16 [1,{C},H,W]\nconst w bf16 [{C},{C},1,1]\nnode Conv x w -> y {{kernel=1 stride=1 pad=0}}\noutput y\n"
+    rng = np.random.default_rng(67)
+    shapes = [(1, 3), (5, 5), (7, 9), (1, 62), (13, 5), (11, 6), (3, 23), (9, 15), (8, 16), (31, 33), (1, 1)]
+    reqs = [Request({"H": h, "W": w}, {"x": bf16_round(rng.standard_normal((1, C, h, w)).astype(np.float32))}) for h, w in shapes]
+    wl = WL.Workload("layout_any", "bf16", ir, {"w": np.eye(C, dtype=np.float32).reshape(C, C, 1, 1)}, ["H", "W"], ["y"], {"batch_fn": lambda j: reqs})
+    _, p, outs = run_batch(wl, reqs)
+    for r, req in enumerate(reqs):
+        assert np.array_equal(outs[r]["y"], req.inputs["x"]), req.syms
