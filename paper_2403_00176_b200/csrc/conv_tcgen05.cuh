@@ -58,7 +58,7 @@ struct ConvSmem {
   static constexpr int A_BYTES = KCH * 128 * 128;
   static constexpr int B_BYTES = KCH * BN * 128;
   static constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
-  static constexpr int TOTAL = STAGES * STAGE_BYTES + CONV_STAGE_OUT + 896 + 2048 + 128;
+  static constexpr int TOTAL = STAGES * STAGE_BYTES + 2 * CONV_STAGE_OUT + 896 + 2048 + 128;
 };
 
 __device__ __forceinline__ void tma_store_4d(const void* tmap, const void* src, int c0, int c1, int c2, int c3) {
@@ -100,13 +100,13 @@ conv_igemm_bf16_tcgen05(const __grid_constant__ CUtensorMap tmX, const __grid_co
   extern __shared__ uint8_t smem_raw[];
   uint8_t* tiles = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint8_t* out_stage = tiles + STAGES * S::STAGE_BYTES;
-  float* bias_s = reinterpret_cast<float*>(out_stage + CONV_STAGE_OUT);  // [2][256]
+  float* bias_s = reinterpret_cast<float*>(out_stage + 2 * CONV_STAGE_OUT);  // [2][256]
   uint64_t* full = reinterpret_cast<uint64_t*>(bias_s + 512);
   uint64_t* empty = full + STAGES;
   uint64_t* tmem_full = empty + STAGES;
   uint64_t* tmem_empty = tmem_full + 2;
-  uint64_t* res_full = tmem_empty + 2;
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(res_full + 1);
+  uint64_t* res_full = tmem_empty + 2;    // [2]
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(res_full + 2);
   volatile int* dead = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -115,7 +115,7 @@ conv_igemm_bf16_tcgen05(const __grid_constant__ CUtensorMap tmX, const __grid_co
   if (threadIdx.x == 0) {
     for (int s = 0; s < STAGES; ++s) { ptx::mbar_init(&full[s], 3); ptx::mbar_init(&empty[s], 1); }
     for (int b = 0; b < 2; ++b) { ptx::mbar_init(&tmem_full[b], 1); ptx::mbar_init(&tmem_empty[b], 8); }
-    ptx::mbar_init(res_full, 1);
+    ptx::mbar_init(&res_full[0], 1); ptx::mbar_init(&res_full[1], 1);
     *dead = 0;
     ptx::fence_barrier_init();
     ptx::fence_proxy_async();
@@ -233,83 +233,97 @@ conv_igemm_bf16_tcgen05(const __grid_constant__ CUtensorMap tmX, const __grid_co
     const int et = threadIdx.x - 128; // 0..255
     const int row = q * 32 + lane;    // pixel inside the tile
     const float relu2_floor = p.act2 == ACT_RELU ? 0.0f : -INFINITY;
-    int j = 0, rp = 0;
+    // Pass u uses staging buffer u & 1.  Before the barrier that ends a pass, the store of the pass before has read its
+    // buffer; behind the barrier the next pass's residual is loaded into that buffer while this pass's store leaves, so the
+    // warps meet once per pass and wait for no TMA round trip.  (One buffer, its store and its residual load waited for in
+    // every pass: 1x1 shortcut convolutions of 32 images 12.9 -> 11.2 us and 6.3 -> 5.7 us, 3x3 ones with a residual -1 to -3 %.)
+    int j = 0, u = 0;
     auto load_bias = [&](int t) -> float {
       const int idx = (t / tiles_px) * BN + et;
       return (p.bias && et < BN && t < num_tiles && idx < p.Cout) ? __bfloat162float(p.bias[idx]) : 0.0f;
     };
+    auto load_res = [&](int v, int np, int ho0, int wo0, int img) {
+      ptx::mbar_expect_tx(&res_full[v & 1], CONV_STAGE_OUT);
+      ptx::tma_load_4d(out_stage + (v & 1) * CONV_STAGE_OUT, &tmRes, np, wo0, ho0, p.res_ids ? p.res_ids[img] : img, &res_full[v & 1]);
+    };
     float bias_next = load_bias(blockIdx.x);
+    if (HASRES && et == 0 && static_cast<int>(blockIdx.x) < num_tiles) {
+      int n0, img, ho0, wo0;
+      decode(blockIdx.x, &n0, &img, &ho0, &wo0);
+      load_res(0, n0, ho0, wo0, img);
+    }
     for (int t = blockIdx.x; t < num_tiles; t += gridDim.x, ++j) {
       const int acc = j & 1;
       int n0, img, ho0, wo0;
       decode(t, &n0, &img, &ho0, &wo0);
-      const int img_r = p.res_ids ? p.res_ids[img] : img, img_o = p.out_ids ? p.out_ids[img] : img;
+      const int img_o = p.out_ids ? p.out_ids[img] : img;
       float* bias_t = bias_s + (j & 1) * 256;
       bias_t[et] = bias_next;
       bias_next = load_bias(t + gridDim.x);
       conv_epi_bar();                              // the bias of this tile is written
       ptx::mbar_wait_warp(&tmem_full[acc], (j >> 1) & 1, dead);
       ptx::tc_fence_after();
+      const int passes = min(PASSES, (p.Cout - n0 + 63) >> 6);     // columns past Cout are left in tensor memory
 #pragma unroll 1
-      for (int ps = 0; ps < PASSES; ++ps) {
+      for (int ps = 0; ps < passes; ++ps, ++u) {
         const int np = n0 + ps * 64;
-        const bool live = np < p.Cout;
-        constexpr bool res_t = HASRES;
-        const bool res = res_t && live;
-        if (res) {
-          if (et == 0) {
-            bulk_wait_read0();
-            ptx::mbar_expect_tx(res_full, CONV_STAGE_OUT);
-            ptx::tma_load_4d(out_stage, &tmRes, np, wo0, ho0, img_r, res_full);
-          }
-          ptx::mbar_wait_warp(res_full, rp & 1, dead);
-          ++rp;
+        uint8_t* stage = out_stage + (u & 1) * CONV_STAGE_OUT;
+        uint8_t* obase = stage + row * 128;
+        uint32_t r[32];
+        ptx::tmem_ld32(tmem + (static_cast<uint32_t>(q * 32) << 16) + acc * BN + ps * 64 + half * 32, r);
+        ptx::tmem_ld_wait();
+        if (ps == passes - 1) {
+          ptx::tc_fence_before();
+          __syncwarp();
+          if (lane == 0) ptx::mbar_arrive(&tmem_empty[acc]);
         }
-        uint8_t* obase = out_stage + row * 128;
+        float v[32];
+        bias_act32<ACT>(v, r, bias_t + ps * 64 + half * 32);
         uint4 pk[4];
-        if (live) {
-          uint32_t r[32];
-          ptx::tmem_ld32(tmem + (static_cast<uint32_t>(q * 32) << 16) + acc * BN + ps * 64 + half * 32, r);
-          ptx::tmem_ld_wait();
-          const float* bp = bias_t + ps * 64 + half * 32;
+        if constexpr (HASRES) {
+          ptx::mbar_wait_warp(&res_full[u & 1], (u >> 1) & 1, dead);
+          uint4 rv[4];
+#pragma unroll
+          for (int g = 0; g < 4; ++g) rv[g] = *reinterpret_cast<const uint4*>(obase + (((half * 4 + g) ^ (row & 7)) << 4));
 #pragma unroll
           for (int g = 0; g < 4; ++g) {
-            float v[8];
-#pragma unroll
-            for (int i = 0; i < 8; ++i) v[i] = apply_act<ACT>(__uint_as_float(r[g * 8 + i]) + bp[g * 8 + i]);
-            if constexpr (HASRES) {
-              const uint4 rv = *reinterpret_cast<const uint4*>(obase + (((half * 4 + g) ^ (row & 7)) << 4));
-              const __nv_bfloat162* h = reinterpret_cast<const __nv_bfloat162*>(&rv);
-#pragma unroll
-              for (int i = 0; i < 4; ++i) { const float2 f = __bfloat1622float2(h[i]); v[2 * i] += f.x; v[2 * i + 1] += f.y; }
-#pragma unroll
-              for (int i = 0; i < 8; ++i) v[i] = fmaxf(v[i], relu2_floor);
-            }
+            const __nv_bfloat162* h = reinterpret_cast<const __nv_bfloat162*>(&rv[g]);
             __nv_bfloat162* oh = reinterpret_cast<__nv_bfloat162*>(&pk[g]);
 #pragma unroll
-            for (int i = 0; i < 4; ++i) oh[i] = __floats2bfloat162_rn(v[2 * i], v[2 * i + 1]);
+            for (int i = 0; i < 4; ++i) {
+              const float2 f = __bfloat1622float2(h[i]);
+              oh[i] = __floats2bfloat162_rn(fmaxf(v[g * 8 + 2 * i] + f.x, relu2_floor), fmaxf(v[g * 8 + 2 * i + 1] + f.y, relu2_floor));
+            }
+          }
+        } else {
+#pragma unroll
+          for (int g = 0; g < 4; ++g) {
+            __nv_bfloat162* oh = reinterpret_cast<__nv_bfloat162*>(&pk[g]);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) oh[i] = __floats2bfloat162_rn(v[g * 8 + 2 * i], v[g * 8 + 2 * i + 1]);
           }
         }
-        if (!res) {
-          if (et == 0) bulk_wait_read0();
-          conv_epi_bar();
-        }
-        if (live) {
 #pragma unroll
-          for (int g = 0; g < 4; ++g) *reinterpret_cast<uint4*>(obase + (((half * 4 + g) ^ (row & 7)) << 4)) = pk[g];
-        }
-        ptx::tc_fence_before();
+        for (int g = 0; g < 4; ++g) *reinterpret_cast<uint4*>(obase + (((half * 4 + g) ^ (row & 7)) << 4)) = pk[g];
         ptx::fence_proxy_async();
-        __syncwarp();
-        if (ps == PASSES - 1 && lane == 0) ptx::mbar_arrive(&tmem_empty[acc]);
+        if (et == 0) bulk_wait_read0();              // the pass before has left its buffer
         conv_epi_bar();
-        if (et == 0 && live) {
-          tma_store_4d(&tmOut, out_stage, np, wo0, ho0, img_o);
+        if (et == 0) {
+          if constexpr (HASRES) {
+            if (ps + 1 < passes) {
+              load_res(u + 1, np + 64, ho0, wo0, img);
+            } else if (t + static_cast<int>(gridDim.x) < num_tiles) {
+              int n1, img1, ho1, wo1;
+              decode(t + gridDim.x, &n1, &img1, &ho1, &wo1);
+              load_res(u + 1, n1, ho1, wo1, img1);
+            }
+          }
+          tma_store_4d(&tmOut, stage, np, wo0, ho0, img_o);
           bulk_commit();
         }
-        if (p.gap_sum && live) {
+        if (p.gap_sum) {
           const int tw_shift = __ffs(p.TW) - 1;      // TW * TH == 128: a power of two
-          gap_accumulate_tile(out_stage, et, p.gap_sum + static_cast<long long>(img_o) * p.Cout + np, [&](int px) {
+          gap_accumulate_tile(stage, et, p.gap_sum + static_cast<long long>(img_o) * p.Cout + np, [&](int px) {
             return ho0 + (px >> tw_shift) < p.Ho && wo0 + (px & (p.TW - 1)) < p.Wo;
           });
         }
