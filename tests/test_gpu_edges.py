@@ -176,3 +176,25 @@ def test_layout_changes_of_rows_that_start_anywhere(C):
     _, p, outs = run_batch(wl, reqs)
     for r, req in enumerate(reqs):
         assert np.array_equal(outs[r]["y"], req.inputs["x"]), req.syms
+
+
+def test_gelu_epilogue_in_the_negative_tail():
+    # pre-activations between -4.25 and -3, where GELU is small enough for bf16 to show the fit: per bin, rms error within what
+    # bf16 rounding gives (ulp / sqrt 12) and 2.2e-5: the fit's own error is at most 2.0e-5 there, the hardware tanh adds little
+    from math import erf
+    M = 2048
+    ir = "sym M 1 4096\ninput x bf16 [1,M,64]\nconst W bf16 [64,64]\nnode MatMul x W -> t\nnode Gelu t -> y\noutput y\n"
+    W = np.zeros((64, 64), np.float32)
+    W[0], W[1] = 1.0, np.arange(64) * 2.0 ** -12
+    x = np.zeros((1, M, 64), np.float32)
+    x[0, :, 0], x[0, :, 1] = bf16_round(np.linspace(-4.25, -3.0, M).astype(np.float32)), 1.0
+    wl = WL.Workload("gelu_tail", "bf16", ir, {"W": bf16_round(W)}, ["M"], ["y"], {"batch_fn": lambda j: []})
+    _, _, outs = run_batch(wl, [Request({"M": M}, {"x": x})])
+    pre = x[0, :, :1].astype(np.float64) + bf16_round(W)[1]
+    want = np.array([0.5 * v * (1 + erf(v / np.sqrt(2))) for v in pre.ravel()])
+    err = outs[0]["y"][0].astype(np.float64).ravel() - want
+    ulp = 2.0 ** (np.floor(np.log2(np.abs(want))) - 7)
+    for lo in np.arange(-4.25, -3.0, 0.25):
+        m = (pre.ravel() >= lo) & (pre.ravel() < lo + 0.25)
+        rms, rounding = np.sqrt((err[m] ** 2).mean()), np.sqrt((ulp[m] ** 2 / 12).mean())
+        assert rms <= np.hypot(rounding, 2.2e-5), (lo, rms, rounding)
