@@ -306,7 +306,7 @@ attention_tcgen05_bf16(const __grid_constant__ CUtensorMap tmQ, const __grid_con
         const int buf = n & 1;
         const uint32_t s_addr = tmem + lane_base + ATC_TMEM_S + buf * 64, p_addr = tmem + lane_base + ATC_TMEM_P + buf * 32;
         if (!s_seen) ptx::mbar_wait_warp(&s_full[buf], (n >> 1) & 1, dead);
-        const bool o_seen = ptx::mbar_test_wait(&o_full[buf], ((n >> 1) - 1) & 1);     // consumed below (n >= 2)
+        const bool o_seen = ptx::mbar_test_wait_warp(&o_full[buf], ((n >> 1) - 1) & 1);     // consumed below (n >= 2)
         ptx::tc_fence_after();
         if (tracer) { SOD2_TRACE(2, 300 + n) }
         if (__builtin_expect(!live, 0)) {
@@ -366,7 +366,7 @@ attention_tcgen05_bf16(const __grid_constant__ CUtensorMap tmQ, const __grid_con
         }
         if (tracer) { SOD2_TRACE(2, 400 + n) }
         if (__builtin_expect(j == 0 && i > 0, 0)) finish(i - 1, n);
-        s_seen = ptx::mbar_test_wait(&s_full[buf ^ 1], ((n + 1) >> 1) & 1);     // the next block's scores are usually there
+        s_seen = ptx::mbar_test_wait_warp(&s_full[buf ^ 1], ((n + 1) >> 1) & 1);     // the next block's scores are usually there
         ptx::tmem_st_wait();
         ptx::tc_fence_before();
         __syncwarp();

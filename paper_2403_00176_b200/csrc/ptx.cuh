@@ -112,6 +112,11 @@ __device__ __forceinline__ void mbar_wait_warp(uint64_t* bar, uint32_t parity, v
   mbar_wait_elect(bar, parity, dead);
   __syncwarp();
 }
+// Whether the phase has ended, the same answer in every lane: what a warp may branch on around a wait, a tcgen05.ld or a
+// __syncwarp.  (The lanes' own tests may disagree; a branch on them would leave part of the warp behind.)
+__device__ __forceinline__ bool mbar_test_wait_warp(uint64_t* bar, uint32_t parity) {
+  return __all_sync(0xffffffffu, mbar_test_wait(bar, parity));
+}
 // One arrival for a warp in step, without a branch around it.
 __device__ __forceinline__ void mbar_arrive_warp(uint64_t* bar) {
   asm volatile(

@@ -1,0 +1,21 @@
+"""Properties of the kernel sources that no run can show reliably: checked on the text."""
+import os
+import re
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2403_00176_b200", "csrc")
+
+
+def _sources():
+    for f in sorted(os.listdir(CSRC)):
+        if f.endswith((".cu", ".cuh")):
+            with open(os.path.join(CSRC, f)) as h:
+                yield f, re.sub(r"//[^\n]*", "", h.read())
+
+
+def test_kernels_branch_on_barrier_tests_only_through_a_vote():
+    # mbar_test_wait answers per lane, and the lanes of a warp may see a phase end at different tests: a kernel that branches
+    # on it around a warp-wide wait or tcgen05.ld could leave lanes behind.  Outside ptx.cuh only the voted form is used
+    users = [f for f, text in _sources() if f != "ptx.cuh" and re.search(r"\bmbar_test_wait\s*\(", text)]
+    assert users == []
+    ptx = dict(_sources())["ptx.cuh"]
+    assert re.search(r"bool mbar_test_wait_warp\([^)]*\) \{\s*return __all_sync\(0xffffffffu, mbar_test_wait\(", ptx)
