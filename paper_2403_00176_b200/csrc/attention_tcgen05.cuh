@@ -291,15 +291,31 @@ attention_tcgen05_bf16(const __grid_constant__ CUtensorMap tmQ, const __grid_con
       }
       if (tracer) { SOD2_TRACE(2, 700 + pi) }
     };
+    // maximum of the first `live_cols` scores of a tile in tensor memory (registers are few where this is needed)
+    auto max_ahead = [&](uint32_t addr, int live_cols) {
+      float mx = -INFINITY;
+#pragma unroll 1
+      for (int h = 0; h < ATC_KB && h < live_cols; h += 8) {
+        uint32_t r[8];
+        ptx::tmem_ld8(addr + h, r);
+        ptx::tmem_ld_wait();
+#pragma unroll
+        for (int e = 0; e < 8; ++e) if (h + e < live_cols) mx = fmaxf(mx, __uint_as_float(r[e]));
+      }
+      return mx;
+    };
     int n = 0, i = 0;
     bool s_seen = false;
     for (int item; (item = nth_item(i)) < items; ++i) {
       const Item it = locate(item);
       const bool live = it.q0 + warp * 32 < it.L;    // a warp whose 32 rows are all past the request only keeps the barriers moving
-      // Online softmax with a lazily updated reference: the exponent reference m only moves when a block's
-      // row maximum exceeds it by more than 2^8 after scaling, so p stays <= 256 (exact enough in bf16 and
-      // fp32) and the accumulator O in TMEM is rescaled only then -- for almost every block nothing is read
-      // back from TMEM.  l and O always refer to the same m, so O / l at the end is the softmax average.
+      // Online softmax with a lazily updated reference: the exponent reference m starts as the row maximum of the first
+      // 128 keys and then only moves when a block's row maximum exceeds it by more than 2^8 after scaling, so p stays
+      // <= 256 (exact enough in bf16 and fp32) and the accumulator O in TMEM is rescaled only then -- for almost every block
+      // nothing is read back from TMEM.  l and O always refer to the same m, so O / l at the end is the softmax average.
+      // References are chosen over pairs of blocks, the second block's scores looked at ahead: the largest p of those keys is
+      // then exactly 1, where bf16 does not round it.  (A reference out of 64 keys alone rounds the weight that dominates
+      // a row: against fp64, scores of standard deviation 2 and 128 keys, 1.17 times the error.)
       float m = -INFINITY;
       float2 l = make_float2(0.f, 0.f);
       for (int j = 0; j < it.nkv; ++j, ++n) {
@@ -320,8 +336,27 @@ attention_tcgen05_bf16(const __grid_constant__ CUtensorMap tmQ, const __grid_con
           continue;
         }
         const int valid = it.L - j * ATC_KB;     // keys of the block inside the request
+        const bool pair = !(j & 1) && valid > ATC_KB;
+        const uint32_t s_next = s_addr ^ 64;     // the other score tile
         uint32_t s[64];
-        ptx::tmem_ld32(s_addr, s);
+        if (__builtin_expect(j == 0 && pair, 0)) {
+          ptx::mbar_wait_warp(&s_full[buf ^ 1], ((n + 1) >> 1) & 1, dead);
+          ptx::tc_fence_after();
+          if (valid >= 2 * ATC_KB) {           // half a tile is reduced while the next half is under way
+            ptx::tmem_ld32(s_next, s);
+            ptx::tmem_ld_wait();
+            ptx::tmem_ld32(s_next + 32, s + 32);
+            m = atc_max32(m, s);
+            ptx::tmem_ld_wait();
+            ptx::tmem_ld32(s_addr, s);
+            m = atc_max32(m, s + 32);
+          } else {
+            m = max_ahead(s_next, valid - ATC_KB);
+            ptx::tmem_ld32(s_addr, s);
+          }
+        } else {
+          ptx::tmem_ld32(s_addr, s);
+        }
         ptx::tmem_ld32(s_addr + 32, s + 32);
         ptx::tmem_ld_wait();
         ptx::tc_fence_before();
@@ -335,9 +370,16 @@ attention_tcgen05_bf16(const __grid_constant__ CUtensorMap tmQ, const __grid_con
         if (tracer) { SOD2_TRACE(2, 600 + n) }
         // move the reference if the block asks for it
         const bool move = (mx - m) * c > 8.0f;
-        float corr = 1.f;
-        if (move) { corr = ex2_approx((m - mx) * c); m = mx; l.x *= corr; l.y *= corr; }
+        if (j == 0) m = fmaxf(m, mx);
         if (__builtin_expect(j > 0 && __any_sync(0xffffffffu, move), 0)) {
+          float ref = mx;
+          if (pair) {
+            ptx::mbar_wait_warp(&s_full[buf ^ 1], ((n + 1) >> 1) & 1, dead);
+            ptx::tc_fence_after();
+            ref = fmaxf(mx, max_ahead(s_next, valid - ATC_KB));
+          }
+          float corr = 1.f;
+          if (move) { corr = ex2_approx((m - ref) * c); m = ref; l.x *= corr; l.y *= corr; }
           // all products issued so far must have landed in O before it is scaled
           ptx::mbar_wait_warp(&o_full[(n - 1) & 1], ((n - 1) >> 1) & 1, dead);
           ptx::tc_fence_after();

@@ -198,3 +198,55 @@ def test_gelu_epilogue_in_the_negative_tail():
         m = (pre.ravel() >= lo) & (pre.ravel() < lo + 0.25)
         rms, rounding = np.sqrt((err[m] ** 2).mean()), np.sqrt((ulp[m] ** 2 / 12).mean())
         assert rms <= np.hypot(rounding, 2.2e-5), (lo, rms, rounding)
+
+
+def _attention_alone(D, H):
+    """softmax(Q K^T / 8) V out of a packed [L, 3 D] input, behind it a product with the identity (exact in bf16)."""
+    ir = WL._IR()
+    ir.add("sym L 1 1024")
+    ir.add(f"input x bf16 [1,L,{3 * D}]")
+    WL._attn_iconsts(ir, D, H)
+    ir.add(f"const I bf16 [{D},{D}]")
+    xs = ir.node("Shape", ["x"], ir.tmp())
+    bl = ir.node("Gather", [xs, "i_01"], ir.tmp(), axis=0)
+    s4, s3 = (ir.node("Concat", [bl, c], ir.tmp(), axis=0) for c in ("i_heads", "i_D"))
+    qkv = []
+    for i, perm in enumerate(("0,2,1,3", "0,2,3,1", "0,2,1,3")):
+        sl = ir.node("Slice", ["x", f"i_st{i}", f"i_en{i}", "i_ax2"], ir.tmp())
+        qkv.append(ir.node("Transpose", [ir.node("Reshape", [sl, s4], ir.tmp())], ir.tmp(), perm=perm))
+    s1 = ir.node("Mul", [ir.node("MatMul", qkv[:2], ir.tmp()), "f_scale"], ir.tmp())
+    o = ir.node("MatMul", [ir.node("Softmax", [s1], ir.tmp(), axis=-1), qkv[2]], ir.tmp())
+    y0 = ir.node("Reshape", [ir.node("Transpose", [o], ir.tmp(), perm="0,2,1,3"), s3], ir.tmp())
+    ir.node("MatMul", [y0, "I"], "y")
+    ir.add("output y")
+    return WL.Workload("attention_alone", "bf16", ir.text(), {"I": np.eye(D, dtype=np.float32)}, ["L"], ["y"], {"batch_fn": lambda j: []})
+
+
+def _softmax64(x, H):
+    L = x.shape[1]
+    q, k, v = x.astype(np.float64).reshape(L, 3, H, 64).transpose(1, 2, 0, 3)
+    s = q @ k.transpose(0, 2, 1) / 8
+    p = np.exp(s - s.max(-1, keepdims=True))
+    return ((p / p.sum(-1, keepdims=True)) @ v).transpose(1, 0, 2).reshape(L, H * 64)
+
+
+@pytest.mark.parametrize("L,top,base", [(128, 100, 10), (65, 64, 0), (300, 127, 63), (400, 384, 200), (300, 200, 130)])
+def test_attention_rows_dominated_by_one_key(L, top, base):
+    # every row has one heavy key, the next one powers of two below it: where the heavy key is among the first 128 (or moves
+    # the reference later on), its weight is exactly 1 and what is left is the output's rounding (1.66e-3 rms over normal values)
+    # and that of weights of a fifth or less; a heavy weight that is rounded to bf16 as well makes it 2.2e-3
+    H = 6
+    wl = _attention_alone(64 * H, H)
+    rng = np.random.default_rng(71)
+    x = np.zeros((1, L, 3, H, 64), np.float32)
+    # past the first 128 keys the gap is more than 2^8, so that the reference moves
+    x[0, :, 0, :, 0] = rng.uniform(*((24, 86) if top < 128 else (100, 400)), (L, H))
+    x[0, :, 1, :, 0] = -3.0
+    x[0, base, 1, :, 0], x[0, top, 1, :, 0] = 0.5, 1.0
+    x[0, :, 2] = rng.standard_normal((L, H, 64))
+    x = bf16_round(x.reshape(1, L, -1))
+    _, _, outs = run_batch(wl, [Request({"L": L}, {"x": x}), Request({"L": L}, {"x": x})])
+    want = _softmax64(x, H)
+    for o in outs:
+        err = o["y"][0].astype(np.float64) - want
+        assert np.linalg.norm(err) / np.linalg.norm(want) <= 1.85e-3
