@@ -300,6 +300,9 @@ struct BuildState {
   int gapsum_root = -1;
   size_t gapsum_aux = 0;
   std::map<int, size_t> gap_accum;    // convolution group -> offset of the table it accumulates into
+  // per tensor with row statistics: slots the producer's tile version really writes and columns per slot
+  struct StatsLayout { int slots = 0, cols = 0; };
+  std::vector<StatsLayout> stats_layout;
 };
 
 struct Plan {
@@ -319,9 +322,6 @@ struct Plan {
   bool sm_count_known = false;
   bool uses_header = true;                // false: no kernel of the plan writes the status word, a ticket or a count: nothing to clear or read
   std::vector<double> group_flops, group_bytes;   // algorithmic cost per group for the bound shapes
-  // per tensor with row statistics: slots the producer's tile version really writes and columns per slot
-  struct StatsLayout { int slots = 0, cols = 0; };
-  std::vector<StatsLayout> stats_layout;
   // Runs of consecutive GEMM groups that execute as one persistent kernel (gemm_chain_tcgen05.cuh): decided after
   // view resolution and before liveness, because the members run concurrently: everything a member reads stays
   // live, and everything a member writes is live, over the whole run.

@@ -394,7 +394,7 @@ struct Builder : BuildState {
     // folded LayerNorm: where the statistics of the normalised rows live, and where this group's own go
     if ((lna || lnr) && (lds[lna ? 0 : 2] != (lna ? K : N))) return fail(E_UNSUPPORTED_OP, "folded LayerNorm needs densely packed rows");
     if (emit && lds[1] != N) return fail(E_UNSUPPORTED_OP, "row statistics need densely packed output rows");
-    if (p.stats_layout.size() != g.tensors.size()) p.stats_layout.assign(g.tensors.size(), Plan::StatsLayout());
+    if (stats_layout.size() != g.tensors.size()) stats_layout.assign(g.tensors.size(), StatsLayout());
     auto stats_ptr = [&](int t, int r0, int64_t width, Ptr* out, int64_t* pitch) -> bool {
       const int root = p.root_of[t];
       const RootBuf& RR = p.roots[root];
@@ -440,7 +440,7 @@ struct Builder : BuildState {
         while (bn > 64 && N % bn) bn /= 2;
         if (N % bn) return fail(E_UNSUPPORTED_OP, "row statistics need an output width that is a multiple of 64");
         bn_group = bn;
-        p.stats_layout[G.out] = {static_cast<int>(N / bn) * 2, bn / 2};
+        stats_layout[G.out] = {static_cast<int>(N / bn) * 2, bn / 2};
       }
       // CTA pairs (tcgen05.mma.cta_group::2): each CTA loads its own A rows and half of the weight tile, a third to a half
       // fewer operand bytes per flop, in tiles of 256 rows x 256, 192 or 128 columns whose last wave may be cut in two.
@@ -492,10 +492,10 @@ struct Builder : BuildState {
       const int ln = lna ? 1 : lnr ? 2 : 0;
       Ptr ps_in, ps_out, pc1, pg, pbt;
       int64_t pitch_in = 0, pitch_out = 0;
-      Plan::StatsLayout lay;
+      StatsLayout lay;
       if (ln) {
         const int raw = lna ? G.ln_a : G.ln_res;
-        lay = p.stats_layout[raw];
+        lay = stats_layout[raw];
         if (!lay.slots || !stats_ptr(raw, sg.r0, lna ? K : N, &ps_in, &pitch_in)) return fail(E_INTERNAL, "row statistics of " + g.tensors[raw].name + " are not planned");
         if (static_cast<int64_t>(lay.slots) * lay.cols != (lna ? K : N)) return fail(E_INTERNAL, "row statistics layout of " + g.tensors[raw].name);
         if (lna) { pc1.where = 5; pc1.off = static_cast<int64_t>(pk + ((static_cast<size_t>(N) * K * 2 + 255) & ~size_t(255))); }
@@ -680,12 +680,12 @@ struct Builder : BuildState {
   Status build_gemm_chain(int ci) {
     const Plan::Chain& ch = p.chains[ci];
     const int n = static_cast<int>(ch.groups.size());
-    if (p.stats_layout.size() != g.tensors.size()) p.stats_layout.assign(g.tensors.size(), Plan::StatsLayout());
+    if (stats_layout.size() != g.tensors.size()) stats_layout.assign(g.tensors.size(), StatsLayout());
     struct Mem {
       ChainMember cm;
       Ptr pa, po, pr, pw, pb, pc1, pg, pbt, ps_in, ps_out;
       int64_t pitch_in = 0, pitch_out = 0;
-      Plan::StatsLayout lay;
+      StatsLayout lay;
       bool hb = false, hr = false, emit = false;
       int ln = 0, dep_a = -1, dep_r = -1;
       float eps = 1e-5f;
@@ -725,12 +725,12 @@ struct Builder : BuildState {
       if (!found) return fail(E_INTERNAL, "no prepacked copy of " + g.tensors[G.w].name);
       m.pw.where = 5; m.pw.off = static_cast<int64_t>(pk);
       if (m.emit) {
-        p.stats_layout[G.out] = {static_cast<int>(N / k::CHAIN_BN) * 2, k::CHAIN_BN / 2};
+        stats_layout[G.out] = {static_cast<int>(N / k::CHAIN_BN) * 2, k::CHAIN_BN / 2};
         if (!stats_ptr(G.out, N, &m.ps_out, &m.pitch_out)) return fail(E_INTERNAL, "row statistics of " + g.tensors[G.out].name + " are not planned");
       }
       if (m.ln) {
         const int raw = m.ln == 1 ? G.ln_a : G.ln_res;
-        m.lay = p.stats_layout[raw];
+        m.lay = stats_layout[raw];
         if (!m.lay.slots || !stats_ptr(raw, m.ln == 1 ? K : N, &m.ps_in, &m.pitch_in)) return fail(E_INTERNAL, "row statistics of " + g.tensors[raw].name + " are not planned");
         if (static_cast<int64_t>(m.lay.slots) * m.lay.cols != (m.ln == 1 ? K : N)) return fail(E_INTERNAL, "row statistics layout of " + g.tensors[raw].name);
         if (m.ln == 1) { m.pc1.where = 5; m.pc1.off = static_cast<int64_t>(pk + ((static_cast<size_t>(N) * K * 2 + 255) & ~size_t(255))); }

@@ -250,3 +250,31 @@ def test_attention_rows_dominated_by_one_key(L, top, base):
     for o in outs:
         err = o["y"][0].astype(np.float64) - want
         assert np.linalg.norm(err) / np.linalg.norm(want) <= 1.85e-3
+
+
+def test_exact_staging_with_a_folded_layernorm_across_stages():
+    # the GEMM that writes the row statistics of a folded LayerNorm runs in the first stage, the one that reads them (as its
+    # residual; its own operand is the gated network's pooled output) in the last: same bits as the bounded run
+    wl = WL.cfg5(B=6, side=32, widths=(64,), per_stage=2)
+    lines = wl.ir.splitlines()
+    head = [ln for ln in lines if not ln.startswith(("node", "output"))]
+    nodes = [ln for ln in lines if ln.startswith("node")]
+    rng = np.random.default_rng(73)
+    consts = {"W0": (64, 64), "b0": (64,), "g": (64,), "be": (64,), "W1": (64, 64), "b1": (64,)}
+    head += ["input z bf16 [1,6,64]", "iconst i_r3 i64 [3] = 1 6 64"] + [f"const lf.{n} bf16 [{','.join(map(str, s))}]" for n, s in consts.items()]
+    first = ["node MatMul z lf.W0 -> lf0", "node Add lf0 lf.b0 -> lf1", "node Add lf1 z -> lf2",
+             "node LayerNormalization lf2 lf.g lf.be -> lf3 {axis=-1 epsilon=1e-5}"]
+    last = ["node Reshape gap i_r3 -> gr", "node MatMul gr lf.W1 -> lf4", "node Add lf4 lf.b1 -> lf5", "node Add lf5 lf3 -> lfy"]
+    ir = "\n".join(head + first + nodes + last + [ln for ln in lines if ln.startswith("output")] + ["output lfy"]) + "\n"
+    wl2 = WL.Workload("gated_ln_fold", "bf16", ir, {**wl.consts, **{"lf." + n: bf16_round((rng.standard_normal(s) / 8).astype(np.float32)) for n, s in consts.items()}},
+                      wl.sym_names, wl.outputs + ["lfy"], wl.meta)
+    req = wl.batch(0)[0]
+    req = Request(req.syms, {**req.inputs, "z": bf16_round(rng.standard_normal((1, 6, 64)).astype(np.float32))})
+    s, p, ref = run_batch(wl2, [req], opt_flags=B.OPT_LN_FOLD)
+    kinds = [s.graph.group_info(i)["kind"] for i in range(s.graph.num_groups())]
+    assert "layernorm" not in kinds and kinds[0] == "gemm" and kinds.index("gate") < len(kinds) - 1 - kinds[::-1].index("gemm")
+    assert p.run_exact().reserved[2] == 3
+    p.check_device_status()
+    got = p.outputs()
+    for name in ref[0]:
+        assert np.array_equal(ref[0][name], got[0][name]), name
