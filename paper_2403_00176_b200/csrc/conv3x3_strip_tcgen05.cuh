@@ -4,10 +4,15 @@
 // instruction a 64-channel layer cannot pass half of the pipe's rate.  Here an instruction carries the three dy taps of
 // one dx: the operand B is [dy = 2 | dy = 1 | dy = 0] x 64 output channels, and the result is what input row i gives to
 // the output rows i - 1, i and i + 1, whose accumulators lie side by side in tensor memory (a ring of eight 64-column
-// blocks; where the three blocks wrap around its end the instruction is cut in two).  The dx taps are the same rows of
-// shared memory through descriptors whose start address is shifted by a pixel.  So a CTA walks down a column of tiles
-// of 128 pixels, every input row is loaded ONCE per strip (one box of 130 pixels, zero-filled outside the image = the
-// padding), and takes 12 instructions instead of 36.
+// blocks; where the three blocks wrap around its end the instruction is cut in two).  Tensor-core instructions are only
+// documented to take effect in the order of issue where accumulator and shape are the same.  Consecutive rows share two of
+// their three blocks, so a row's first instruction waits until the row before has completed (its commit passes the turn),
+// and within a row every block sees one shape only: no instruction starts a block from zero, the epilogue clears it when it
+// has read it (0 + x: the same bits).  This costs about 160 cycles per row against relying on the order of issue (4 images
+// 53.5 -> 57.5 us a layer).
+// The dx taps are the same rows of shared memory through descriptors whose start address is shifted by a pixel.  So a CTA
+// walks down a column of tiles of 128 pixels, every input row is loaded ONCE per strip (one box of 130 pixels, zero-filled
+// outside the image = the padding), and takes 12 instructions instead of 36.
 //
 // Work is the list of all (request, image, column tile, row) tiles in that order; CTA b takes an equal, contiguous
 // share, which it walks in segments that do not leave their column.  A segment of L rows costs L + 2 input rows.
@@ -15,9 +20,8 @@
 // Warps: 0 activation and weight TMA, 1 and 3 MMA issuers (alternate rows), 2 staging agent (residual prefetch + output
 // stores), 4..19 epilogue: two groups of eight that take alternate rows (a row's accumulator -> activation -> residual -> staging is a
 // chain of about 2000 cycles against 1300 of the main loop).
-// Measured on B200, 640x480 + 416x416 + 224x608 + 544x320 (6976 tiles): 92 us a layer with one tap per instruction, 60 here;
-// a row takes about 1500 cycles of which the MMAs are 1170 (1730 where the window wraps), the rest is the hand-over
-// between the issuers.
+// Measured on B200, 640x480 + 416x416 + 224x608 + 544x320 (6976 tiles): 92 us a layer with one tap per instruction, 58 here;
+// the MMAs of a row are 1170 cycles (1730 where the window wraps), the rest is the hand-over from row to row.
 #pragma once
 #include <cuda.h>
 #include <cuda_bf16.h>
@@ -37,36 +41,40 @@ constexpr int STRIP_SMEM = STRIP_W + STRIP_STAGES * C3_A_SLOT + STRIP_NSB * CONV
 
 // One MMA whose descriptors differ from the others' only in their start addresses (low words, in units of 16 bytes).
 template <int BLOCKS>
-__device__ __forceinline__ void strip_mma(uint32_t d, uint32_t a_lo, uint32_t b_lo, uint32_t accumulate) {
+__device__ __forceinline__ void strip_mma(uint32_t d, uint32_t a_lo, uint32_t b_lo) {
   constexpr uint32_t desc_hi = (1024u >> 4) | 1u << 14 | 2u << 29;      // ptx::smem_desc_sw128: row-group stride, version, 128-byte swizzle
   asm volatile(
-      "{\n\t.reg .pred p;\n\t.reg .b64 ad, bd;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "mov.b64 ad, {%1, %5};\n\t"
-      "mov.b64 bd, {%2, %5};\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], ad, bd, %3, p;\n\t}"
-      ::"r"(d), "r"(a_lo), "r"(b_lo), "n"(ptx::idesc_bf16(128, 64 * BLOCKS)), "r"(accumulate), "n"(desc_hi)
+      "{\n\t.reg .b64 ad, bd;\n\t"
+      "mov.b64 ad, {%1, %4};\n\t"
+      "mov.b64 bd, {%2, %4};\n\t"
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], ad, bd, %3, 1;\n\t}"
+      ::"r"(d), "r"(a_lo), "r"(b_lo), "n"(ptx::idesc_bf16(128, 64 * BLOCKS)), "n"(desc_hi)
       : "memory");
 }
-// One input row: three dx taps of 64 input channels onto C1 accumulator blocks from d1 and C2 behind the ring's end; the
-// last of them starts from zero (in its own block dn) if FRESH.  Everything but the start addresses is a constant: the
-// issuing thread has one MMA's time (96 cycles) for all its arithmetic, beside epilogue warps on its scheduler.
-template <int C1, int C2, bool FRESH>
-__device__ __forceinline__ void strip_row(uint32_t d1, uint32_t d2, uint32_t dn, uint32_t a_lo, uint32_t b_lo) {
+// One input row: three dx taps of 64 input channels onto C1 accumulator blocks from d1 and C2 behind the ring's end.
+// Everything but the start addresses is a constant: the issuing thread has one MMA's time (96 cycles) for all its
+// arithmetic, beside epilogue warps on its scheduler.
+template <int C1, int C2>
+__device__ __forceinline__ void strip_row(uint32_t d1, uint32_t d2, uint32_t a_lo, uint32_t b_lo) {
   constexpr uint32_t TAP = STRIP_TAP >> 4;
-  constexpr int OLD = C1 + C2 - 1, O1 = OLD < C1 ? OLD : C1, O2 = OLD - O1;
 #pragma unroll
   for (int q = 0; q < 12; ++q) {
     const uint32_t a = a_lo + (q >> 2) * 8 + 2 * (q & 3), b = b_lo + (q >> 2) * (3 * TAP) + 2 * (q & 3);
-    if (FRESH && q == 0) {
-      if constexpr (O1 > 0) strip_mma<O1>(d1, a, b, 1);
-      if constexpr (O2 > 0) strip_mma<O2>(d2, a, b + O1 * TAP, 1);
-      strip_mma<1>(dn, a, b + OLD * TAP, 0);
-    } else {
-      strip_mma<C1>(d1, a, b, 1);
-      if constexpr (C2 > 0) strip_mma<C2>(d2, a, b + C1 * TAP, 1);
-    }
+    strip_mma<C1>(d1, a, b);
+    if constexpr (C2 > 0) strip_mma<C2>(d2, a, b + C1 * TAP);
   }
+}
+
+// A warp's share of an accumulator block (32 lanes, 32 columns) becomes zero and is handed to the issuers.
+__device__ __forceinline__ void strip_hand_over(uint32_t tmem, int blk, int q, int half, int lane, uint64_t* bar) {
+  uint32_t zero[32];
+#pragma unroll
+  for (int i = 0; i < 32; ++i) zero[i] = 0u;
+  ptx::tmem_st32(tmem + (static_cast<uint32_t>(q * 32) << 16) + blk * 64 + half * 32, zero);
+  ptx::tmem_st_wait();
+  ptx::tc_fence_before();
+  __syncwarp();
+  if (lane == 0) ptx::mbar_arrive(bar);
 }
 
 // B.tx: {64, W, H, N}, box {64, 130, 1, 1};  tmW: k-chunk view {64, 64, 9} of the weights in (dy, dx, ci) order, box
@@ -120,6 +128,9 @@ conv3x3_strip_bf16_tcgen05(const __grid_constant__ Conv3Batch B, const __grid_co
     for (int dx = 0; dx < 3; ++dx)
       for (int dy = 2; dy >= 0; --dy) ptx::tma_load_3d(wres + (dx * 3 + 2 - dy) * STRIP_TAP, &tmW, 0, 0, dy * 3 + dx, w_full);
   }
+  // the accumulator ring starts from zero: each epilogue warp clears its share of its group's blocks
+  if (warp >= 4)
+    for (int blk = (warp - 4) >> 3; blk < NB; blk += 2) strip_hand_over(tmem, blk, warp & 3, ((warp - 4) & 7) >> 2, lane, &tmem_empty[blk]);
   ptx::pdl_wait();
   ptx::pdl_launch();
   int total = B.tile_start[B.n_req];
@@ -167,15 +178,13 @@ conv3x3_strip_bf16_tcgen05(const __grid_constant__ Conv3Batch B, const __grid_co
     }
   } else if (warp == 1 || warp == 3) {
     {
-      // ---- MMA issuers: rows alternate between two threads.  One thread's commits, address arithmetic and barrier
-      // waits between two rows leave the tensor pipe idle for about 300 cycles; here the next row's thread has done its
-      // waiting while this row's is issuing, and starts on its word (`turn`, passed on before the commits).  The rows
-      // stay in order, so sums do not depend on timing.  (A thread may wait on `full` and `tmem_empty` for its own rows
-      // only: its row n - 2 was issued after every earlier row had seen its barriers, so at row n each barrier is at most
-      // one phase away from the one waited for.)
-      // Output row o of the segment accumulates in block (j + o) % 8; input row ii (counted from the
-      // row above the segment) gives to the output rows ii - 2 (dy = 2), ii - 1 and ii, as far as they belong to the
-      // segment.  Row ii is touched for the first time: its very first instruction does not accumulate.
+      // ---- MMA issuers: rows alternate between two threads.  A row starts when the row before has completed: its issuer
+      // commits to this one's `turn`, so the commit of an output row also covers what the other thread issued for it.  The
+      // next row's thread has done its address arithmetic and its other waits by then.  (A thread may wait on `full` and
+      // `tmem_empty` for its own rows only: its row n - 2 was issued after every earlier row had seen its barriers, so at row
+      // n each barrier is at most one phase away from the one waited for.)
+      // Output row o of the segment accumulates in block (j + o) % 8; input row ii (counted from the row above the segment)
+      // gives to the output rows ii - 2 (dy = 2), ii - 1 and ii, as far as they belong to the segment.
       ptx::mbar_wait_elect(w_full, 0, dead);
       const uint64_t wdesc = ptx::smem_desc_sw128(ptx::smem_u32(wres));
       const int me = warp == 1 ? 0 : 1;
@@ -193,27 +202,22 @@ conv3x3_strip_bf16_tcgen05(const __grid_constant__ Conv3Batch B, const __grid_co
           const int c1 = min(cnt, NB - b0), c2 = cnt - c1;            // blocks before and behind the ring's end
           const uint64_t wb = wdesc + (lo - (ii - 2)) * (STRIP_TAP >> 4);
           const uint32_t d1 = tmem + b0 * 64;
-          if (fresh && j + ii >= NB) ptx::mbar_wait_elect(&tmem_empty[(j + ii) % NB], (((j + ii) / NB) - 1) & 1, dead);
+          if (fresh) ptx::mbar_wait_elect(&tmem_empty[(j + ii) % NB], ((j + ii) / NB) & 1, dead);
           ptx::mbar_wait_elect(&full[s], (n / ST) & 1, dead);
           if (n > 0) ptx::mbar_wait_elect(&turn[me], me ? (n >> 1) & 1 : ((n >> 1) - 1) & 1, dead);
           ptx::tc_fence_after();
           const uint64_t ad = ptx::smem_desc_sw128(ptx::smem_u32(rows + s * C3_A_SLOT));
           const uint32_t a_lo = static_cast<uint32_t>(ad), b_lo = static_cast<uint32_t>(wb);
-          const uint32_t dn = tmem + ((j + ii) % NB) * 64;
           if (ptx::elect_one()) {
-            switch (c1 * 8 + c2 * 2 + (fresh ? 1 : 0)) {
-#define SOD2_STRIP_ROW(C1_, C2_) case C1_ * 8 + C2_ * 2: strip_row<C1_, C2_, false>(d1, tmem, dn, a_lo, b_lo); break; \
-                                   case C1_ * 8 + C2_ * 2 + 1: strip_row<C1_, C2_, true>(d1, tmem, dn, a_lo, b_lo); break;
-              SOD2_STRIP_ROW(3, 0)
-              SOD2_STRIP_ROW(2, 1)
-              SOD2_STRIP_ROW(1, 2)
-              SOD2_STRIP_ROW(2, 0)
-              SOD2_STRIP_ROW(1, 1)
-              SOD2_STRIP_ROW(1, 0)
-#undef SOD2_STRIP_ROW
+            switch (c1 * 4 + c2) {
+              case 12: strip_row<3, 0>(d1, tmem, a_lo, b_lo); break;
+              case 9: strip_row<2, 1>(d1, tmem, a_lo, b_lo); break;
+              case 6: strip_row<1, 2>(d1, tmem, a_lo, b_lo); break;
+              case 8: strip_row<2, 0>(d1, tmem, a_lo, b_lo); break;
+              case 5: strip_row<1, 1>(d1, tmem, a_lo, b_lo); break;
+              case 4: strip_row<1, 0>(d1, tmem, a_lo, b_lo); break;
             }
-            ptx::tc_fence_before();
-            ptx::mbar_arrive(&turn[me ^ 1]);
+            ptx::mma_commit(&turn[me ^ 1]);
             ptx::mma_commit(&empty[s]);
             if (ii >= 2) ptx::mma_commit(&tmem_full[(j + ii - 2) % NB]);
           }
@@ -290,9 +294,7 @@ conv3x3_strip_bf16_tcgen05(const __grid_constant__ Conv3Batch B, const __grid_co
       uint32_t r[32];
       ptx::tmem_ld32(tmem + (static_cast<uint32_t>(q * 32) << 16) + blk * 64 + half * 32, r);
       ptx::tmem_ld_wait();
-      ptx::tc_fence_before();
-      __syncwarp();
-      if (lane == 0) ptx::mbar_arrive(&tmem_empty[blk]);
+      strip_hand_over(tmem, blk, q, half, lane, &tmem_empty[blk]);
       float v[32];
       bias_act32<ACT>(v, r, bias_s + half * 32);
       uint8_t* obase = out_stage + bsel * CONV_STAGE_OUT + row * 128;

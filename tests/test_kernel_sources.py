@@ -19,3 +19,11 @@ def test_kernels_branch_on_barrier_tests_only_through_a_vote():
     assert users == []
     ptx = dict(_sources())["ptx.cuh"]
     assert re.search(r"bool mbar_test_wait_warp\([^)]*\) \{\s*return __all_sync\(0xffffffffu, mbar_test_wait\(", ptx)
+
+
+def test_strip_convolution_orders_rows_by_completion():
+    # consecutive input rows accumulate into overlapping blocks with instructions of different shapes, which have no documented
+    # order of their own: a row is issued on the commit of the row before, and no instruction overwrites its accumulator
+    text = dict(_sources())["conv3x3_strip_tcgen05.cuh"]
+    assert "mma_commit(&turn[me ^ 1])" in text and not re.search(r"mbar_arrive\w*\(&turn", text)
+    assert re.search(r"tcgen05\.mma\.[^;]*%3, 1;", text) and len(re.findall(r"tcgen05\.mma\.", text)) == 1
