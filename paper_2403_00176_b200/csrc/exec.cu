@@ -2495,6 +2495,8 @@ Status read_counts(Plan* p, const void* arena, void* stream) {
 
 // Second streams (with their fork and join events) are parked between plans: a plan is made per batch, and creating
 // and destroying the three cost 55 + 60 us of host time, more than planning and launching a convolution stage.
+// A caller may capture a run and drop its plan before the capture ends: the parked stream then still belongs to that
+// capture, and nobody takes it before it has left it.
 namespace {
 struct SideSet { int device; void *stream, *fork, *join; };
 constexpr size_t SIDE_MAX = 8;
@@ -2519,7 +2521,13 @@ Plan::~Plan() {
   }
 }
 
-// The second stream and the two events of a plan with side groups (taken outside any stream capture).
+static bool in_capture(void* stream) {
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(static_cast<cudaStream_t>(stream), &cap) != cudaSuccess) { cudaGetLastError(); return true; }
+  return cap != cudaStreamCaptureStatusNone;
+}
+
+// The second stream and the two events of a plan with side groups, in no capture when they are taken.
 static bool ensure_side_stream(Plan* p) {
   bool any = false;
   for (char c : p->side_group) any = any || c;
@@ -2530,7 +2538,7 @@ static bool ensure_side_stream(Plan* p) {
     SidePool& P = side_pool();
     std::lock_guard<std::mutex> lk(P.mu);
     for (size_t i = 0; i < P.parked.size(); ++i)
-      if (P.parked[i].device == dev) {
+      if (P.parked[i].device == dev && !in_capture(P.parked[i].stream)) {
         const SideSet q = P.parked[i];
         P.parked.erase(P.parked.begin() + i);
         p->side_device = dev; p->side_stream = q.stream; p->ev_fork = q.fork; p->ev_join = q.join;

@@ -278,3 +278,34 @@ def test_exact_staging_with_a_folded_layernorm_across_stages():
     got = p.outputs()
     for name in ref[0]:
         assert np.array_equal(ref[0][name], got[0][name]), name
+
+
+def test_plan_dropped_inside_a_callers_capture():
+    # the second stream of a plan that a caller has captured and dropped belongs to the capture until it ends: another plan that
+    # wants a second stream meanwhile, on another stream, gets one of its own; both give the eager run's bits
+    wl = WL.cfg4(blocks=1)
+    rng = np.random.default_rng(79)
+    reqs = [Request({"H": 24, "W": 70}, {"x": bf16_round(rng.uniform(-1, 1, (1, 64, 24, 70)).astype(np.float32))})]
+    s, p, ref = run_batch(wl, reqs)
+    assert any(p.plan.group_on_side_stream(i) for i in range(s.graph.num_groups()))
+    args = [t.data_ptr() for t in p.in_dev], [t.data_ptr() for t in p.out_dev], p.arena.data_ptr(), p.arena.numel()
+    q = s.prepare(reqs)
+    mine, other = torch.cuda.Stream(), torch.cuda.Stream()
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.stream(mine):
+        graph.capture_begin(capture_error_mode="relaxed")
+        plan = s.graph.bind_dims(wl.sym_names, [[24, 70]]).plan()
+        plan.run(*args, mine.cuda_stream)
+        del plan
+        q.plan.run([t.data_ptr() for t in q.in_dev], [t.data_ptr() for t in q.out_dev], q.arena.data_ptr(), q.arena.numel(), other.cuda_stream)
+        graph.capture_end()
+    torch.cuda.synchronize()
+    got = q.outputs()
+    for t in p.out_dev:
+        t.zero_()
+    graph.replay()
+    torch.cuda.synchronize()
+    again = p.outputs()
+    for name in ref[0]:
+        assert np.array_equal(got[0][name], ref[0][name]) and np.array_equal(again[0][name], ref[0][name])
