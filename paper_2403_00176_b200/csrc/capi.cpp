@@ -247,7 +247,7 @@ sod2_status sod2_run_exact(sod2_plan_t* p, const void* const* inputs, void* cons
   }
   int64_t inf[8] = {0};
   std::string err;
-  ++p->p.run_epoch;
+  note_run(&p->p, stream);
   Status s = run_exact(&p->g->c, p->p.b, &p->p, inputs, outputs, arena, arena_bytes, stream, inf, &err);
   if (s != OK) p->h.err = err;
   if (info) {
@@ -459,9 +459,7 @@ sod2_status sod2_run_output_shape(sod2_plan_t* p, const void* arena, void* strea
   for (auto& d : T.S.dims) if (d.known() && e_has_runtime(G.cx, d.e)) need = true;
   if (need) {
     if (!arena) return SOD2_E_INVALID_ARG;
-    if (read_counts(&p->p, arena, stream) != OK) return SOD2_E_CUDA;
-    for (size_t a = 0; a < G.cx.atoms.size(); ++a)
-      if (G.cx.atoms[a].kind == AtomKind::SYM && G.cx.atoms[a].runtime) vals[a] = p->p.counts[a * p->p.n_req + r];
+    if (read_counts(&p->p, arena, stream, r, &vals) != OK) return SOD2_E_CUDA;
   }
   if (rank) *rank = T.S.rank;
   for (int i = 0; i < T.S.rank; ++i) {

@@ -3,6 +3,7 @@
 #include <initializer_list>
 #include <map>
 #include <memory>
+#include <mutex>
 #include <new>
 #include <set>
 #include <string>
@@ -363,12 +364,14 @@ struct Plan {
   void* ev_join = nullptr;                // cudaEvent_t
   std::vector<const void*> graph_key;     // inputs, outputs, arena the graph was captured with
   // Run-time counts of the last run, read back by the first sod2_run_output_shape after it (read_counts).  They are kept
-  // only while the library can tell that no other run has happened: a run that a caller captured into a graph of its own
-  // may be replayed without a call, so such a plan reads the counts every time.
+  // only while the library can tell that they are that run's: read through the stream of the run, and no run since.  A run
+  // that a caller captured into a graph of its own may be replayed without a call, so such a plan reads the counts every time.
   uint64_t run_epoch = 1, counts_epoch = 0;
+  void* run_stream = nullptr;             // cudaStream_t of the last run
   const void* counts_arena = nullptr;
   bool captured_by_caller = false;
   std::vector<long long> counts;          // [atom][request], as in the arena header
+  std::mutex counts_mu;                   // output shapes may be asked for by several threads
   Plan() = default;
   Plan(const Plan&) = delete;
   Plan& operator=(const Plan&) = delete;
@@ -380,8 +383,10 @@ Status make_plan(const Compiled* c, const Binding* b, Plan* p);
 // pointer differs from the captured ones, then replayed on `stream`.  info[3] = 1 if this call captured.
 Status run_plan_graph(Plan* p, const void* const* inputs, void* const* outputs, void* arena, size_t arena_bytes, void* stream,
                       int64_t* info);
-// The counts in the arena header -> Plan::counts (synchronises `stream`).
-Status read_counts(Plan* p, const void* arena, void* stream);
+// A run of `p` is about to be enqueued on `stream`: the counts read so far are those of another run.
+void note_run(Plan* p, void* stream);
+// The run-time symbols among `vals` <- their counts for request r in the arena header (synchronises `stream`).
+Status read_counts(Plan* p, const void* arena, void* stream, int r, std::vector<int64_t>* vals);
 Status build_launches(Plan* p);   // exec.cu
 Status detect_chains(Plan* p);    // exec.cu: fills Plan::chains / chain_of from the resolved views
 // step_lo..step_hi: only these groups (positions in execution order) are enqueued (all by default); the arena header

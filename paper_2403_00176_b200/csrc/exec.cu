@@ -2422,7 +2422,7 @@ Status run_plan_timed(Plan* p, const void* const* inputs, void* const* outputs, 
   if (reinterpret_cast<uintptr_t>(arena) & 255) { p->err = "arena must be 256-byte aligned"; return E_MISALIGNED; }
   RunCtx x{inputs, outputs, static_cast<char*>(arena), static_cast<char*>(p->c->packed_ws), static_cast<cudaStream_t>(stream), p};
   const size_t n = p->launches.size();
-  ++p->run_epoch;
+  note_run(p, stream);
   std::vector<cudaEvent_t> ev(2 * n);
   for (auto& e : ev) if (cudaEventCreate(&e) != cudaSuccess) { p->err = "cudaEventCreate failed"; return E_CUDA; }
   if (p->uses_header) cudaMemsetAsync(arena, 0, p->header_clear_bytes, x.stream);
@@ -2482,14 +2482,38 @@ bool read_back(void* dst, const void* src, size_t bytes, cudaStream_t st) {
 }
 }  // namespace
 
-Status read_counts(Plan* p, const void* arena, void* stream) {
+static bool in_capture(void* stream) {
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(static_cast<cudaStream_t>(stream), &cap) != cudaSuccess) { cudaGetLastError(); return true; }
+  return cap != cudaStreamCaptureStatusNone;
+}
+
+void note_run(Plan* p, void* stream) {
+  ++p->run_epoch;
+  p->run_stream = stream;
+  if (p->captured_by_caller) return;
+  for (auto& syms : p->rt_syms_after)
+    if (!syms.empty()) { p->captured_by_caller = in_capture(stream); break; }
+}
+
+Status read_counts(Plan* p, const void* arena, void* stream, int r, std::vector<int64_t>* vals) {
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  if (!p->captured_by_caller && p->counts_epoch == p->run_epoch && p->counts_arena == arena)
-    return cudaStreamSynchronize(st) == cudaSuccess ? OK : E_CUDA;
-  p->counts.resize(p->c->g.cx.atoms.size() * static_cast<size_t>(p->n_req));
-  if (!read_back(p->counts.data(), static_cast<const char*>(arena) + 256, p->counts.size() * 8, st)) return E_CUDA;
-  p->counts_epoch = p->run_epoch;
-  p->counts_arena = arena;
+  const char* src = static_cast<const char*>(arena) + 256;
+  std::lock_guard<std::mutex> lk(p->counts_mu);
+  const bool own = stream == p->run_stream && !p->captured_by_caller;
+  if (own && p->counts_epoch == p->run_epoch && p->counts_arena == arena) {
+    if (cudaStreamSynchronize(st) != cudaSuccess) return E_CUDA;
+  } else {
+    p->counts.resize(p->c->g.cx.atoms.size() * static_cast<size_t>(p->n_req));
+    const size_t bytes = p->counts.size() * 8;
+    // through another stream than the run's the caller has ordered the two, or relies on the default stream's order
+    if (own ? !read_back(p->counts.data(), src, bytes, st)
+            : cudaStreamSynchronize(st) != cudaSuccess || cudaMemcpy(p->counts.data(), src, bytes, cudaMemcpyDeviceToHost) != cudaSuccess) return E_CUDA;
+    p->counts_epoch = own ? p->run_epoch : 0;
+    p->counts_arena = arena;
+  }
+  for (size_t a = 0; a < p->c->g.cx.atoms.size(); ++a)
+    if (p->c->g.cx.atoms[a].kind == AtomKind::SYM && p->c->g.cx.atoms[a].runtime) (*vals)[a] = p->counts[a * p->n_req + r];
   return OK;
 }
 
@@ -2519,12 +2543,6 @@ Plan::~Plan() {
       cudaEventDestroy(static_cast<cudaEvent_t>(ev_join));
     }
   }
-}
-
-static bool in_capture(void* stream) {
-  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-  if (cudaStreamIsCapturing(static_cast<cudaStream_t>(stream), &cap) != cudaSuccess) { cudaGetLastError(); return true; }
-  return cap != cudaStreamCaptureStatusNone;
 }
 
 // The second stream and the two events of a plan with side groups, in no capture when they are taken.
@@ -2589,7 +2607,7 @@ Status run_plan_graph(Plan* p, const void* const* inputs, void* const* outputs, 
   } else {
     if (arena_bytes < p->arena_bytes) { p->err = "arena too small"; return E_ARENA_TOO_SMALL; }
   }
-  ++p->run_epoch;
+  note_run(p, stream);
   const cudaError_t el = cudaGraphLaunch(static_cast<cudaGraphExec_t>(p->graph_exec), static_cast<cudaStream_t>(stream));
   if (el != cudaSuccess) { p->err = std::string("graph launch failed: ") + cudaGetErrorString(el); return E_CUDA; }
   if (info) {
@@ -2607,16 +2625,7 @@ Status run_plan(Plan* p, const void* const* inputs, void* const* outputs, void* 
   if (reinterpret_cast<uintptr_t>(arena) & 255) { p->err = "arena must be 256-byte aligned"; return E_MISALIGNED; }
   if (p->c->packed_bytes && !p->c->packed_ws) { p->err = "weights are not prepacked"; return E_INVALID_ARG; }
   auto t0 = std::chrono::steady_clock::now();
-  ++p->run_epoch;
-  if (!p->captured_by_caller && stream != p->capture_stream) {
-    for (auto& syms : p->rt_syms_after)
-      if (!syms.empty()) {
-        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-        if (cudaStreamIsCapturing(static_cast<cudaStream_t>(stream), &cap) != cudaSuccess) cudaGetLastError();
-        if (cap != cudaStreamCaptureStatusNone) p->captured_by_caller = true;
-        break;
-      }
-  }
+  if (stream != p->capture_stream || !stream) note_run(p, stream);     // (the library's own capture: run_plan_graph)
   if (!p->sm_count_known) {
     int dev = 0, n = 0;
     if (cudaGetDevice(&dev) == cudaSuccess && cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && n > 0) p->sm_count = n;

@@ -309,3 +309,45 @@ def test_plan_dropped_inside_a_callers_capture():
     again = p.outputs()
     for name in ref[0]:
         assert np.array_equal(got[0][name], ref[0][name]) and np.array_equal(again[0][name], ref[0][name])
+
+
+def test_counts_are_those_of_the_last_run():
+    # the counts behind an output shape are read once per run, and must not outlive it: a shape asked for through another
+    # stream while the run is still waiting, several threads asking at once, replays of a caller's graph that holds the run
+    import threading
+    ir = "sym A 0 100000\ninput x f32 [A]\nnode NonZero x -> nz\noutput nz\n"
+    wl = WL.Workload("counts", "f32", ir, {}, ["A"], ["nz"], {"batch_fn": lambda j: []})
+    reqs = [Request({"A": n}, {"x": np.ones(n, np.float32)}) for n in (1000, 5000)]
+    s, p, _ = run_batch(wl, reqs)
+    args = [t.data_ptr() for t in p.in_dev], [t.data_ptr() for t in p.out_dev], p.arena.data_ptr(), p.arena.numel()
+    shapes = lambda stream: [p.plan.output_shape(p.arena.data_ptr(), stream, r, 0) for r in range(2)]
+    full, none = [[1, 1000], [1, 5000]], [[1, 0], [1, 0]]
+    # another stream asks while the run waits behind a long kernel
+    mine, other = torch.cuda.Stream(), torch.cuda.Stream()
+    p.in_dev[0].zero_()
+    torch.cuda.synchronize()
+    with torch.cuda.stream(mine):
+        torch.cuda._sleep(200_000_000)
+    p.plan.run(*args, mine.cuda_stream)
+    shapes(other.cuda_stream)                            # whatever it is, it is not kept
+    mine.synchronize()
+    assert shapes(mine.cuda_stream) == none and shapes(other.cuda_stream) == none
+    # threads
+    p.in_dev[0].copy_(torch.from_numpy(p.in_host[0]))
+    torch.cuda.synchronize()
+    p.plan.run(*args, mine.cuda_stream)
+    bad = []
+    threads = [threading.Thread(target=lambda: bad.extend(i for i in range(200) if shapes(mine.cuda_stream) != full)) for _ in range(4)]
+    for t in threads: t.start()
+    for t in threads: t.join()
+    assert not bad
+    # a run inside a graph of the caller's
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.stream(mine):
+        graph.capture_begin(capture_error_mode="relaxed")
+        p.plan.run(*args, mine.cuda_stream)
+        graph.capture_end()
+        for data, want in ((p.in_host[0], full), (np.zeros_like(p.in_host[0]), none), (p.in_host[0], full)):
+            p.in_dev[0].copy_(torch.from_numpy(data))
+            graph.replay()
+            assert shapes(mine.cuda_stream) == want
