@@ -1060,8 +1060,8 @@ struct Builder : BuildState {
       Ptr pout = ptr_of(G.out, r);
       const int64_t total = numel(ov.dims);
       const long long items = red ? od[0] * od[1] * od[2] : (total + tile - 1) / tile;
-      // flat indices are 32-bit, and a tile may reach past the last element
-      if ((red ? items : total + tile) >= (int64_t(1) << 31)) return fail(E_UNSUPPORTED_OP, "chain request above 2^31 elements");
+      // flat indices are 32-bit
+      if ((red ? items : total) >= (int64_t(1) << 31)) return fail(E_UNSUPPORTED_OP, "chain request above 2^31 elements");
       // does it fit the open table?
       bool fits = cur.cb.n_req < k::CHAIN_MAX_REQ && (red || cur.cb.total + items < (1ll << 31));
       if (fits && cur.cb.n_req) {

@@ -545,21 +545,23 @@ __global__ void __launch_bounds__(256, 4) chain_elementwise(const __grid_constan
     chain_split_row(R, row, &i0, &i1, &i2);
     chain_store1(p, R.out_off + e, chain_eval(p, R, i0, i1, i2, e - row * inner));
   };
+  // (a request may have up to 2^31 - 1 elements: its last tile must not be added to)
+  const int rest = R.numel - e0;
   if (!(p.vec_ok && R.fast)) {
-    for (int e = e0 + threadIdx.x; e < min(e0 + TILE, R.numel); e += 256) by_element(e);
+    for (int d = threadIdx.x; d < min(TILE, rest); d += 256) by_element(e0 + d);
     return;
   }
   const int row0 = static_cast<int>(static_cast<unsigned>(e0) / static_cast<unsigned>(inner));
   const int col0 = e0 - row0 * inner;
   const int d = threadIdx.x * E;
-  if (col0 + TILE <= inner) {
+  if (TILE <= inner - col0) {
     chain_eval_vec<BF16, true>(p, R, e0 + d, row0, col0 + d, CHAIN_NV);
     return;
   }
-  const int whole = R.numel / E * E;                     // the tail behind the last whole vector: one element per thread
-  const int left = whole - (e0 + d);
+  const int whole = rest / E * E;                        // the tail behind the last whole vector: one element per thread
+  const int left = whole - d;
   if (left > 0) chain_eval_vec<BF16, false>(p, R, e0 + d, 0, 0, min(CHAIN_NV, (left + 256 * E - 1) / (256 * E)));
-  if (whole >= e0 && whole < e0 + TILE && whole + static_cast<int>(threadIdx.x) < R.numel) by_element(whole + threadIdx.x);
+  if (whole < TILE && whole + static_cast<int>(threadIdx.x) < rest) by_element(e0 + whole + threadIdx.x);
 }
 
 __device__ __forceinline__ void chain_row_index(const ChainReq& R, long long row, int* i0, int* i1, int* i2) {

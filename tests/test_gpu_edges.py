@@ -351,3 +351,38 @@ def test_counts_are_those_of_the_last_run():
             p.in_dev[0].copy_(torch.from_numpy(data))
             graph.replay()
             assert shapes(mine.cuda_stream) == want
+
+
+def _relu_chain():
+    return B.Graph("sym A 1 4000000000\ninput x bf16 [A]\nnode Relu x -> y\noutput y\n", 0)
+
+
+def _run_relu(x, out):
+    g = _relu_chain()
+    plan = g.bind_dims(["A"], [[x.numel()]]).plan()
+    arena = torch.empty(max(plan.arena_bytes, 256), dtype=torch.uint8, device="cuda")
+    plan.run([x.data_ptr()], [out.data_ptr()], arena.data_ptr(), arena.numel(), torch.cuda.current_stream().cuda_stream)
+    torch.cuda.synchronize()
+
+
+@pytest.mark.parametrize("n", [2 ** 31 - 1, 2 ** 31 - 8192])
+def test_chain_up_to_the_last_32_bit_index(n):
+    # the largest requests that 32-bit flat indices hold, whose last tile reaches past them; the words behind stay as they are
+    x = torch.empty(n + 9, dtype=torch.bfloat16, device="cuda")[:n]
+    x.normal_()
+    buf = torch.full((n + 9,), 7.0, dtype=torch.bfloat16, device="cuda")
+    _run_relu(x, buf[:n])
+    for lo in range(0, n, 1 << 28):
+        hi = min(n, lo + (1 << 28))
+        assert torch.equal(buf[lo:hi], torch.relu(x[lo:hi]))
+    assert bool((buf[n:] == 7.0).all())
+
+
+@pytest.mark.parametrize("n,dx,dy", [(100003, 1, 0), (8192, 0, 1), (8193, 3, 5), (5, 1, 1)])
+def test_chain_buffers_off_16_bytes(n, dx, dy):
+    # a caller's buffers that start on an odd element are read and written one element at a time
+    x = torch.randn(n + 8, device="cuda").to(torch.bfloat16)[dx:dx + n]
+    buf = torch.full((n + 16,), 7.0, dtype=torch.bfloat16, device="cuda")
+    _run_relu(x, buf[dy:dy + n])
+    assert torch.equal(buf[dy:dy + n], torch.relu(x))
+    assert bool((buf[:dy] == 7.0).all()) and bool((buf[dy + n:] == 7.0).all())

@@ -127,3 +127,13 @@ def test_plan_vs_exhaustive_optimum_on_small_graphs():
         assert tensors_top >= opt >= mem["peak_live_bytes"] * 0 and opt >= max(i[0] for i in items)
         ratios.append(tensors_top / opt)
     assert ratios and max(ratios) <= 1.25 and float(np.mean(ratios)) <= 1.06, ratios
+
+
+def test_elementwise_chains_are_planned_up_to_the_last_32_bit_index():
+    # flat indices of a chain request are 32-bit: 2^31 - 1 elements are planned, 2^31 are refused
+    ir = "sym A 1 4000000000\ninput x bf16 [A]\nnode Relu x -> y\noutput y\n"
+    g = B.Graph(ir, 0)
+    for n in (2 ** 31 - 8193, 2 ** 31 - 8192, 2 ** 31 - 1):
+        g.bind_dims(["A"], [[n]]).plan()
+    with pytest.raises(B.Sod2Error, match="2\\^31"):
+        g.bind_dims(["A"], [[2 ** 31]]).plan()
