@@ -223,6 +223,8 @@ sod2_status sod2_plan_memory(const sod2_plan_t* p, size_t* arena_bytes, size_t* 
  * HBM-bound groups) and bytes = every external input and output once, constants once, nothing for
  * tensors that stay inside the group. */
 sod2_status sod2_plan_group_cost(const sod2_plan_t* p, int group, double* flops, double* bytes);
+/* Number of addresses that a run of this plan reads from `inputs` and `outputs` (graph declaration order). */
+sod2_status sod2_plan_io_counts(const sod2_plan_t* p, int* inputs, int* outputs);
 /* *on_side = 1 if the group's kernels run on the plan's second stream beside the previous group (Section 4.3 orders
  * the groups; two consecutive groups overlap only where neither reads what the other writes AND both read the same
  * tensor, so that the memory plan, which knows liveness by step, cannot hand one of them a slot the other still

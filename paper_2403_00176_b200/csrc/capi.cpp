@@ -202,6 +202,13 @@ sod2_status sod2_plan_cached(sod2_graph* g, int n_req, int n_syms, const char* c
   return SOD2_OK;
 }
 
+sod2_status sod2_plan_io_counts(const sod2_plan_t* p, int* inputs, int* outputs) {
+  if (!p) return SOD2_E_INVALID_ARG;
+  if (inputs) *inputs = static_cast<int>(p->g->c.g.inputs.size());
+  if (outputs) *outputs = static_cast<int>(p->g->c.g.outputs.size());
+  return SOD2_OK;
+}
+
 sod2_status sod2_run(sod2_plan_t* p, const void* const* inputs, void* const* outputs, void* arena, size_t arena_bytes,
                      void* stream, sod2_run_info* info) {
   if (!p || !inputs || !outputs) return SOD2_E_INVALID_ARG;

@@ -12,14 +12,14 @@
 
 namespace {
 
-// Small argument arrays live on the stack.
+// Small argument arrays live on the stack.  They start out as zeros: a missing address is a null address.
 template <class T, int N>
 struct Buf {
-  T local[N];
+  T local[N] = {};
   T* p = local;
   bool reserve(Py_ssize_t n) {
     if (n <= N) return true;
-    p = new (std::nothrow) T[n];
+    p = new (std::nothrow) T[n]();
     if (!p) { p = local; PyErr_NoMemory(); return false; }
     return true;
   }
@@ -43,14 +43,27 @@ bool as_ptr(PyObject* o, void** out) {
   *out = PyLong_AsVoidPtr(o);
   return !(*out == nullptr && PyErr_Occurred());
 }
+// An entry of a list of addresses may also be a ctypes.c_void_p.
+bool as_entry(PyObject* o, void** out) {
+  if (o == Py_None || PyLong_Check(o)) return as_ptr(o, out);
+  PyObject* v = PyObject_GetAttrString(o, "value");
+  if (!v) {
+    PyErr_Format(PyExc_TypeError, "an address is wanted, got %.100s", Py_TYPE(o)->tp_name);
+    return false;
+  }
+  const bool ok = as_ptr(v, out);
+  Py_DECREF(v);
+  return ok;
+}
 
+// At least `least` entries: what the list lacks is null, and refused by the call.
 template <int N>
-bool as_ptrs(PyObject* seq, Buf<void*, N>* out, Py_ssize_t* n) {
+bool as_ptrs(PyObject* seq, Buf<void*, N>* out, Py_ssize_t least) {
   PyObject* f = PySequence_Fast(seq, "a sequence of addresses is wanted");
   if (!f) return false;
-  *n = PySequence_Fast_GET_SIZE(f);
-  bool ok = out->reserve(*n);
-  for (Py_ssize_t i = 0; ok && i < *n; ++i) ok = as_ptr(PySequence_Fast_GET_ITEM(f, i), &out->p[i]);
+  const Py_ssize_t n = PySequence_Fast_GET_SIZE(f);
+  bool ok = out->reserve(n > least ? n : least);
+  for (Py_ssize_t i = 0; ok && i < n; ++i) ok = as_entry(PySequence_Fast_GET_ITEM(f, i), &out->p[i]);
   Py_DECREF(f);
   return ok;
 }
@@ -118,8 +131,10 @@ PyObject* py_run(PyObject*, PyObject* const* a, Py_ssize_t n) {
   int64_t how, bytes;
   void *p, *arena, *stream;
   Buf<void*, 64> in, out;
-  Py_ssize_t ni, no;
-  if (!as_i64(a[0], &how) || !as_ptr(a[1], &p) || !as_ptrs(a[2], &in, &ni) || !as_ptrs(a[3], &out, &no) || !as_ptr(a[4], &arena) ||
+  int n_in = 0, n_out = 0;
+  if (!as_i64(a[0], &how) || !as_ptr(a[1], &p)) return nullptr;
+  sod2_plan_io_counts(static_cast<sod2_plan_t*>(p), &n_in, &n_out);
+  if (!as_ptrs(a[2], &in, n_in) || !as_ptrs(a[3], &out, n_out) || !as_ptr(a[4], &arena) ||
       !as_i64(a[5], &bytes) || !as_ptr(a[6], &stream))
     return nullptr;
   Py_buffer info;
