@@ -244,6 +244,11 @@ sod2_status sod2_run_graph(sod2_plan_t* p, const void* const* inputs, void* cons
 sod2_status sod2_run_exact(sod2_plan_t* p, const void* const* inputs, void* const* outputs, void* arena, size_t arena_bytes,
                            void* stream, sod2_run_info* info) {
   if (!p || !inputs || !outputs || !arena) return SOD2_E_INVALID_ARG;
+  const Graph& G = p->g->c.g;
+  for (size_t i = 0; i < G.inputs.size(); ++i) if (!inputs[i]) { p->h.err = "null input"; return SOD2_E_INVALID_ARG; }
+  for (size_t i = 0; i < G.outputs.size(); ++i) if (!outputs[i]) { p->h.err = "null output"; return SOD2_E_INVALID_ARG; }
+  for (int c : p->g->c.used_consts)
+    if (!G.tensors[c].dev_ptr) { p->h.err = "constant " + G.tensors[c].name + " has no device data"; return SOD2_E_INVALID_ARG; }
   if (arena_bytes < p->p.arena_bytes) { p->h.err = "arena too small"; return SOD2_E_ARENA_TOO_SMALL; }
   if (reinterpret_cast<uintptr_t>(arena) & 255) { p->h.err = "arena must be 256-byte aligned"; return SOD2_E_MISALIGNED; }
   if (p->g->c.packed_bytes && !p->g->c.packed_ws) { p->h.err = "weights are not prepacked"; return SOD2_E_INVALID_ARG; }

@@ -14,7 +14,7 @@ def _plan(ir=IR, names=("A",), values=((5,),)):
 
 @pytest.mark.parametrize("ins,outs", [([], [256]), ([256], [256]), ([256, None], [256]), ([256, 512], []), ([256, 512], [None]), ([256, 0], [256]),
                                       ([C.c_void_p(256), C.c_void_p(None)], [256])])
-@pytest.mark.parametrize("how", ["run", "run_graph"])
+@pytest.mark.parametrize("how", ["run", "run_graph", "run_exact"])
 def test_missing_and_null_buffers_are_refused(how, ins, outs):
     # a list that lacks a buffer is a list with a null buffer, whatever the stack holds behind it
     p = _plan()
