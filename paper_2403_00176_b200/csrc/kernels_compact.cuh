@@ -243,12 +243,13 @@ __device__ __forceinline__ const NonZeroReq& nz_find(const NonZeroBatch& p) {
   while (ri + 1 < p.n_req && static_cast<int>(blockIdx.x) >= p.r[ri + 1].first) ++ri;
   return p.r[ri];
 }
-__device__ __forceinline__ int nz_block_sum(int v, int* warp_sums) {
+template <class T>
+__device__ __forceinline__ T nz_block_sum(T v, T* warp_sums) {
 #pragma unroll
   for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   if ((threadIdx.x & 31) == 0) warp_sums[threadIdx.x >> 5] = v;
   __syncthreads();
-  int t = 0;
+  T t = 0;
 #pragma unroll
   for (int w = 0; w < NZ_THREADS / 32; ++w) t += warp_sums[w];
   return t;
@@ -311,17 +312,18 @@ __global__ void __launch_bounds__(NZ_THREADS) nonzero_mask(const __grid_constant
   if (tid == 0) R.count[chunk] = total;
 }
 __global__ void __launch_bounds__(NZ_THREADS) nonzero_write(const __grid_constant__ NonZeroBatch p) {
-  __shared__ int sums[3][NZ_THREADS / 32];
+  __shared__ long long totals[2][NZ_THREADS / 32];       // (a request may hold more than 2^31 non-zero elements)
+  __shared__ int sums[NZ_THREADS / 32];
   __shared__ unsigned short list[NZ_SUB];
   const NonZeroReq& R = nz_find(p);
   const int chunk = blockIdx.x - R.first, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const long long lo = chunk * R.chunk, hi = min(R.numel, lo + R.chunk);
   ptx::pdl_wait();
   ptx::pdl_launch();
-  int before = 0, all = 0;
+  long long before = 0, all = 0;
   for (int j = tid; j < R.chunks; j += NZ_THREADS) { const int c = R.count[j]; all += c; before += j < chunk ? c : 0; }
-  before = nz_block_sum(before, sums[0]);
-  const long long nnz = nz_block_sum(all, sums[1]);
+  before = nz_block_sum(before, totals[0]);
+  const long long nnz = nz_block_sum(all, totals[1]);
   if (chunk == 0 && tid == 0) *R.count_out = nnz;
   long long off = before;
   for (long long base = lo; base < hi; base += NZ_SUB) {
@@ -331,11 +333,11 @@ __global__ void __launch_bounds__(NZ_THREADS) nonzero_write(const __grid_constan
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) { const int t = __shfl_up_sync(0xffffffffu, inc, o); if (lane >= o) inc += t; }
     __syncthreads();                     // the previous piece's list and sums have been read
-    if (lane == 31) sums[2][warp] = inc;
+    if (lane == 31) sums[warp] = inc;
     __syncthreads();
     int at = inc - mine, cnt = 0;
 #pragma unroll
-    for (int w = 0; w < NZ_THREADS / 32; ++w) { const int t = sums[2][w]; at += w < warp ? t : 0; cnt += t; }
+    for (int w = 0; w < NZ_THREADS / 32; ++w) { const int t = sums[w]; at += w < warp ? t : 0; cnt += t; }
     while (m) {
       const int b = __ffs(m) - 1;
       m &= m - 1;

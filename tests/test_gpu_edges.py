@@ -386,3 +386,48 @@ def test_chain_buffers_off_16_bytes(n, dx, dy):
     _run_relu(x, buf[dy:dy + n])
     assert torch.equal(buf[dy:dy + n], torch.relu(x))
     assert bool((buf[:dy] == 7.0).all()) and bool((buf[dy + n:] == 7.0).all())
+
+
+def _nonzero(x, dims, out):
+    """NonZero of a tensor on the GPU into `out`; returns the number of elements found."""
+    names = ["A", "B", "C", "D"][:len(dims)]
+    ir = "".join(f"sym {n} 0 8000000000\n" for n in names) + f"input x {'bf16' if x.dtype == torch.bfloat16 else 'f32'} [{','.join(names)}]\nnode NonZero x -> nz\noutput nz\n"
+    plan = B.Graph(ir, 0).bind_dims(names, [list(dims)]).plan()
+    arena = torch.empty(max(plan.arena_bytes, 256), dtype=torch.uint8, device="cuda")
+    stream = torch.cuda.current_stream().cuda_stream
+    plan.run([x.data_ptr()], [out.data_ptr()], arena.data_ptr(), arena.numel(), stream)
+    return plan.output_shape(arena.data_ptr(), stream, 0, 0)[1]
+
+
+def test_nonzero_finds_more_than_32_bits_count():
+    # every element non-zero, more of them than an int holds: offsets and the count itself
+    n = 2 ** 31 + 4099
+    x = torch.ones(n, dtype=torch.bfloat16, device="cuda")
+    out = torch.empty(n, dtype=torch.int64, device="cuda")
+    assert _nonzero(x, (n,), out) == n
+    for lo in range(0, n, 1 << 28):
+        hi = min(n, lo + (1 << 28))
+        assert torch.equal(out[lo:hi], torch.arange(lo, hi, device="cuda"))
+
+
+@pytest.mark.parametrize("rows,cols", [(4099, 4097), (2 ** 20 + 1, 4097)])
+def test_nonzero_chunks_of_several_pieces(rows, cols):
+    # above 2048 x 8192 elements a chunk has several pieces, above 2^32 the coordinates are worked out in 64 bits
+    n = rows * cols
+    x = torch.zeros(n, dtype=torch.bfloat16, device="cuda")
+    at = torch.tensor(sorted({0, 1, 8191, 8192, cols - 1, cols, n // 2, n // 2 + 1, n - cols, n - 8193, n - 2, n - 1}), device="cuda")
+    x[at] = 1.0
+    k = at.numel()
+    out = torch.full((2 * k,), -1, dtype=torch.int64, device="cuda")
+    assert _nonzero(x, (rows, cols), out) == k
+    assert torch.equal(out[:k], at // cols) and torch.equal(out[k:], at % cols)
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("n", [5, 8193, 40001])
+def test_nonzero_of_a_buffer_off_16_bytes(dtype, n):
+    x = (torch.randn(n + 1, device="cuda") * (torch.rand(n + 1, device="cuda") < 0.5)).to(dtype)[1:]
+    want = torch.nonzero(x).flatten()
+    out = torch.empty(n, dtype=torch.int64, device="cuda")
+    assert _nonzero(x, (n,), out) == want.numel()
+    assert torch.equal(out[:want.numel()], want)
