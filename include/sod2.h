@@ -48,7 +48,7 @@ typedef enum {
 #define SOD2_OPT_NO_SEP 32u /* groups run in their default topological order: no static execution planning (Section 4.3) */
 #define SOD2_OPT_LN_FOLD 128u /* a LayerNorm between bf16 GEMMs is folded into its neighbours (Section 4.2: fusion removes the materialised intermediate): the producing GEMM writes per-row statistics, the consuming GEMMs read the raw rows and normalise in their epilogues, the normalised tensor is never stored.  Opt-in: measured slower on the encoder workloads, where the LayerNorm kernel runs beside the next GEMM's pipeline fill */
 #define SOD2_OPT_GUARD_BANDS 512u /* debugging aid: every arena tensor gets a slot of its own (a band another tensor may cover at another time proves nothing) with 256 bytes behind it, also behind the scratch regions (sod2_plan_poison_arena / sod2_plan_check_guards) */
-#define SOD2_OPT_GEMM_PAIR 1024u /* the CTA-pair GEMM (two CTAs of a cluster share a 256 x N tile, each loading its own rows and half of the weight tile: tcgen05.mma.cta_group::2) wherever its main loop is estimated shorter; without the flag it is taken where the estimate also covers its longer start, from a few thousand rows on (Section 4.4.2: one more code version).  Results equal the single-CTA kernel's */
+#define SOD2_OPT_GEMM_PAIR 1024u /* the CTA-pair GEMM (two CTAs of a cluster share a 256 x N tile, each loading its own rows and half of the weight tile: tcgen05.mma.cta_group::2) wherever its main loop is estimated shorter; without the flag it is taken where the estimate also covers its longer start, from 1500 to 6300 rows on at the encoder's shapes (Section 4.4.2: one more code version).  Results equal the single-CTA kernel's */
 #define SOD2_OPT_GEMM_CHAIN 256u /* consecutive GEMM groups that depend on each other row block by row block run as one persistent kernel with per-row-block dependency counters in the arena header (their operands stay live over the whole chain).  Opt-in: measured slower than one launch per GEMM at a few thousand rows */
 #define SOD2_OPT_SPLITK_LN 4u /* bf16 GEMM (+bias, +residual) -> LayerNorm as one group: split-K GEMM into fp32 slabs + finishing kernel */
 
@@ -230,6 +230,9 @@ sod2_status sod2_plan_io_counts(const sod2_plan_t* p, int* inputs, int* outputs)
  * tensor, so that the memory plan, which knows liveness by step, cannot hand one of them a slot the other still
  * reads), else 0. */
 sod2_status sod2_plan_group_on_side_stream(const sod2_plan_t* p, int group, int* on_side);
+/* Which form of its kernel a group takes for the bound shapes: GEMM "tile 64", "tile 128", "tile 256", "pair", "cluster 2",
+ * "cluster 4" or "cluster 8"; attention "tcgen05" or "mma.sync"; "mixed" where launches of one group differ, empty otherwise. */
+sod2_status sod2_plan_group_form(const sod2_plan_t* p, int group, char* buf, size_t len);
 /* True shape of an output after a run (execution-determined extents are read back from the device;
  * synchronises cuda_stream). */
 sod2_status sod2_run_output_shape(sod2_plan_t* p, const void* arena, void* cuda_stream, int request, int output,

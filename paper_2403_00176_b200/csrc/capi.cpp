@@ -452,6 +452,12 @@ sod2_status sod2_plan_group_on_side_stream(const sod2_plan_t* p, int group, int*
   return SOD2_OK;
 }
 
+sod2_status sod2_plan_group_form(const sod2_plan_t* p, int group, char* buf, size_t len) {
+  if (!p || !buf || group < 0 || group >= static_cast<int>(p->p.group_form.size())) return SOD2_E_INVALID_ARG;
+  copy_str(p->p.group_form[group] ? p->p.group_form[group] : "", buf, len);
+  return SOD2_OK;
+}
+
 sod2_status sod2_plan_memory(const sod2_plan_t* p, size_t* arena, size_t* peak, size_t* sum) {
   if (!p) return SOD2_E_INVALID_ARG;
   if (arena) *arena = p->p.arena_bytes;

@@ -269,6 +269,11 @@ struct Builder : BuildState {
     p.launches.push_back(L);
   }
 
+  void form(int gi, const char* name) {
+    const char*& f = p.group_form[gi];
+    f = !f || !std::strcmp(f, name) ? name : "mixed";
+  }
+
   // ------------------------------------------------------------------------------ GEMM
   Status build_gemm(int gi, const Group& G) {
     const Tensor& W = g.tensors[G.w];
@@ -445,10 +450,12 @@ struct Builder : BuildState {
       // CTA pairs (tcgen05.mma.cta_group::2): each CTA loads its own A rows and half of the weight tile, a third to a half
       // fewer operand bytes per flop, in tiles of 256 rows x 256, 192 or 128 columns whose last wave may be cut in two.
       // Both kernels are estimated as (waves of tiles) x (64-wide k-chunks) x (time of a chunk) + the epilogue of the
-      // last tile; the times (ns, from sweeps of 700 to 14 k rows at the four encoder shapes) say which wins: pairs cost
-      // 1.6 us more to start (cluster launch, two cluster barriers), so they take over at a few thousand rows, e.g. K =
-      // 3072, N = 768: 23.2 -> 19.3 us at 4224 rows, 38.9 -> 29.5 at 7168, 65.7 -> 54 at 14072; 0.4 us more must be gained.
-      // Below 12 chunks the epilogue bounds both kernels and the pairs' start is never earned back.
+      // last tile; pairs cost 1.6 us more to start (cluster launch, two cluster barriers), and 0.4 us more must be gained.
+      // The times (ns) are from sweeps of 700 to 14 k rows at K x N = 768 x 768, 768 x 2304, 768 x 3072 and 3072 x 768; they
+      // depend on the operand bytes of a chunk, not on K or N, and outside of these shapes they have not been checked.  Pairs
+      // win where their waves are fuller: at 768 x 3072 from 1537 rows on, 768 x 2304 from 2049, 3072 x 768 from 3073, 768 x
+      // 768 from 6273, with gaps between.  K = 3072, N = 768: 23.2 -> 19.3 us at 4224 rows, 38.9 -> 29.5 at 7168, 65.7 -> 54 at
+      // 14072.  Below 12 chunks the epilogue bounds both kernels and the pairs' start is never earned back.
       bool pair = false;
       k::PairSplit split{4, 0, 1, 1};
       if (!lna && !lnr && !emit && G.act2 == 0 && tiles_m >= 2 && N >= 128) {
@@ -475,10 +482,11 @@ struct Builder : BuildState {
         pair = (c.flags & OPT_GEMM_PAIR) ? (best < single || force_pair) : (K >= 12 * 64 && best + 2000.0 < single);
       }
       // Few tiles and a long K: S CTAs of a cluster share a tile's K (gemm_cluster_tcgen05.cuh), as many as the chip can hold
-      // clusters for (measured with this kernel's shared memory: 15, 33 and 74 of 8, 4 and 2 CTAs; a second wave would cost
-      // more than the split gains).  The exchange takes about 1.2 us, a 64-wide chunk 0.16 us: 48 chunks gain from any S
-      // (64 rows: 11.8 -> 9.8, 7.2, 5.9 us with S = 2, 4, 8), 24 as well (7.5 -> 6.7, 5.7, 5.0), 12 chunks gain 10 % with
-      // S = 4, with S = 2 only while half of the tile's rows are empty; 6 chunks lose.
+      // clusters for (measured on B200 with this kernel's shared memory: 15, 33 and 74 of 8, 4 and 2 CTAs; a second wave
+      // would cost more than the split gains).  The exchange takes about 1.2 us, a 64-wide chunk 0.16 us: 48 chunks gain
+      // from any S (64 rows: 11.8 -> 9.8, 7.2, 5.9 us with S = 2, 4, 8), 24 as well (7.5 -> 6.7, 5.7, 5.0), 12 chunks gain
+      // 10 % with S = 4; with S = 2 only one shape of 12 chunks was measured to gain, with half of the tile's rows empty
+      // (M <= 64); 6 chunks lose.
       int ksplit = 0;
       if (!pair && !lna && !lnr && !emit && bn == 64) {
         const int tiles = tiles_m * static_cast<int>((N + 63) / 64), chunks = static_cast<int>(K / 64);
@@ -486,6 +494,7 @@ struct Builder : BuildState {
         else if (tiles <= 33 && chunks >= 12) ksplit = 4;
         else if (tiles <= 74 && (chunks >= 24 || (chunks >= 12 && M <= 64))) ksplit = 2;
       }
+      form(gi, pair ? "pair" : ksplit == 8 ? "cluster 8" : ksplit == 4 ? "cluster 4" : ksplit == 2 ? "cluster 2" : bn == 256 ? "tile 256" : bn == 128 ? "tile 128" : "tile 64");
       const bool hb = G.bias >= 0, hr = G.res >= 0;
       const int act = G.act;
       const int act2 = G.act2;
@@ -876,6 +885,7 @@ struct Builder : BuildState {
         if (ok && (tp.q_col + (H - 1) * R0.q_hs + 64 > R0.q_ts || tp.k_col + (H - 1) * R0.k_hs + 64 > R0.k_ts || tp.v_col + (H - 1) * R0.v_hs + 64 > R0.v_ts ||
                    (tp.q_col | tp.k_col | tp.v_col) % 8 || bo.off % 16 || !(G.scale > 0.f)))
           ok = false;
+        form(gi, ok ? "tcgen05" : "mma.sync");
         if (ok) {
           tp.n_req = nr; tp.H = H;
           tp.q_hs = R0.q_hs; tp.k_hs = R0.k_hs; tp.v_hs = R0.v_hs; tp.o_ts = R0.o_ts; tp.o_hs = R0.o_hs;
@@ -2205,6 +2215,7 @@ struct Builder : BuildState {
     p.launches.clear();
     p.group_flops.clear();
     p.group_bytes.clear();
+    p.group_form.assign(c.groups.size(), nullptr);
     p.gpu_launches = 0;
     p.rt_syms_after.assign(c.groups.size(), {});
     // a pooling group right after a layout change of the SAME tensor: neither reads what the other writes, and the

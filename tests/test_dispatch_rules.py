@@ -1,0 +1,34 @@
+"""Which form of the GEMM and attention kernels a bound shape takes: the ends of the dispatch rules, on the CPU."""
+import pytest
+
+from paper_2403_00176_b200 import binding as B
+from paper_2403_00176_b200 import workloads as WL
+
+
+def _gemm(K, N, M):
+    g = B.Graph(f"sym M 1 40000\ninput x bf16 [1,M,{K}]\nconst W bf16 [{K},{N}]\nnode MatMul x W -> y\noutput y\n", 0)
+    return g.bind_dims(["M"], [[M]]).plan().group_form(0)
+
+
+@pytest.mark.parametrize("K,N,M,form", [
+    # K split over clusters: 8 CTAs up to 15 tiles, 4 up to 33, 2 up to 74, from 24 (4 CTAs: 12) chunks of 64 on
+    (3072, 768, 1, "cluster 8"), (3072, 768, 128, "cluster 8"), (3072, 768, 129, "cluster 4"), (3072, 768, 257, "cluster 2"), (3072, 768, 769, "tile 64"),
+    (1536, 384, 256, "cluster 8"), (1472, 384, 256, "cluster 4"), (704, 768, 64, "tile 64"), (768, 768, 64, "cluster 4"), (768, 2304, 64, "cluster 2"),
+    (768, 2304, 65, "tile 64"), (768, 768, 257, "tile 64"),
+    # one wave of 64-column tiles, then 128 or 256 columns by waves
+    (768, 768, 1536, "tile 64"), (768, 768, 1537, "tile 128"), (768, 3072, 769, "tile 256"),
+    # pairs where their estimate is 2 us below the single CTA's; never below 12 chunks
+    (768, 3072, 1806, "pair"), (768, 3072, 2305, "tile 256"), (768, 2304, 2049, "pair"), (3072, 768, 3073, "pair"), (3072, 768, 14072, "pair"),
+    (384, 1536, 8228, "tile 256"), (704, 3072, 1806, "tile 256")])
+def test_gemm_forms(K, N, M, form):
+    assert _gemm(K, N, M) == form
+
+
+def test_attention_forms():
+    g = B.Graph(WL.cfg2(layers=1).ir, 0)
+    at = [g.group_info(i)["kind"] for i in range(g.num_groups())].index("attention")
+    form = lambda lens, graph=g: graph.bind_dims(["L"], [[n] for n in lens]).plan().group_form(at)
+    assert form([2]) == form([512, 16, 127]) == form([1]) == "tcgen05"
+    assert form([1, 64]) == "mma.sync"                     # the views of a single token have other strides
+    assert form([64] * 64 + [1, 2]) == "mixed"             # a table of 64 requests and one of two
+    assert form([64], B.Graph(WL.cfg2(layers=1).ir, B.OPT_LEGACY_ATTENTION)) == "mma.sync"

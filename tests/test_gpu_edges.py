@@ -78,14 +78,18 @@ def test_conv_strips_segments_and_ring(shapes):
         assert all(np.array_equal(a[n], b[n]) for n in a)
 
 
-@pytest.mark.parametrize("lens", [[1], [33, 64], [129, 640], list(range(1, 129, 3)) + [129, 191, 192, 193, 255, 256, 257, 300, 383, 385, 511, 512, 513, 577] + [200] * 8])
+@pytest.mark.parametrize("lens", [[1], [33, 64], [129, 640], list(range(1, 129, 3)) + [129, 191, 192, 193, 255, 256, 257, 300, 383, 385, 511, 512, 513, 577] + [200] * 8,
+                                  list(range(2, 130, 3)) + [128, 129, 191, 192, 193, 255, 256, 257, 300, 383, 385, 511, 512, 513, 577] + [200] * 7])
 def test_attention_blocks_items_and_tables(lens):
     # blocks of 64 keys and tiles of 128 rows at their edges, warps without a live row, a CTA's first, second and third
-    # item (the last list: 65 requests, two tables, more than two items per CTA in the first)
+    # item (the last list: 65 requests, two tables, more than two items per CTA in the first; the list before it has a request of
+    # one token among others, whose table goes to the mma.sync kernel)
     wl = WL.cfg2(layers=1, D=384, H=6, F=384, n_requests=1, lmin=1, lmax=640)
     rng = np.random.default_rng(43)
     reqs = [Request({"L": n}, {"x": bf16_round(rng.standard_normal((1, n, 384)).astype(np.float32))}) for n in lens]
     s, p, outs = run_batch(wl, reqs, opt_flags=B.OPT_NO_REUSE)
+    form = [p.plan.group_form(i) for i in range(s.graph.num_groups()) if s.graph.group_info(i)["kind"] == "attention"]
+    assert form == ["mixed" if 1 in lens and len(lens) == 65 else "tcgen05"], form
     for r in range(0, len(reqs), 4 if len(reqs) > 8 else 1):
         errs = lockstep(wl, s, p, outs, r, BF16_TOL)
         bad = {k: v for k, v in errs.items() if not (isinstance(v, float) and v <= BF16_TOL)}
@@ -111,6 +115,7 @@ def test_gemm_pairs_by_rule(K, N, M, act, residual):
     reqs = [Request({"M": M}, ins)]
     wl = WL.Workload("gemm_pair_rule", "bf16", ir, consts, ["M"], [y], {"batch_fn": lambda j: reqs})
     _, p, outs = run_batch(wl, reqs)
+    assert p.plan.group_form(0) == "pair"
     assert O.rel_err(outs[0][y], O.run(ir, consts, ins)[y]) <= BF16_TOL
     p.run()
     assert np.array_equal(outs[0][y], p.outputs()[0][y])
@@ -131,6 +136,7 @@ def test_gemm_k_split_over_clusters(K, N, Ms, act, residual):
         if residual:
             ins["r"] = bf16_round(rng.standard_normal((1, M, N)).astype(np.float32))
         _, p, outs = run_batch(wl, [Request({"M": M}, ins)])
+        assert p.plan.group_form(0) == f"cluster {8 if K == 3072 or (K == 1536 and M <= 256) else 4 if K in (768, 1536) else 2}", M
         assert O.rel_err(outs[0]["y"], O.run(ir, consts, ins)["y"]) <= BF16_TOL, M
         p.run()
         assert np.array_equal(outs[0]["y"], p.outputs()[0]["y"])
