@@ -12,6 +12,7 @@
 #include "attention.cuh"
 #include "attention_tcgen05.cuh"
 #include "conv_tcgen05.cuh"
+#include "conv3x3_halo_tcgen05.cuh"
 #include "conv3x3_strip_tcgen05.cuh"
 #include "conv3x3_tcgen05.cuh"
 #include "conv_stem_tcgen05.cuh"
@@ -1775,6 +1776,21 @@ struct Builder : BuildState {
       const int padded_w = ((cp.Wo + 127) / 128) * 128;
       const bool rows = ks == 3 && G.stride == 1 && G.pad == 1 && (strip ? padded_w <= cp.Wo * 2 : cp.Wo >= 96 && padded_w * 4 <= cp.Wo * 5);
       if (rows) { cp.TW = 128; cp.TH = 1; }
+      // other 3x3 / stride 1 / pad 1 layers of 128-column tiles: patches fetched once per 64 channels with their halo.  A tile
+      // takes 0.62 of the implicit GEMM's time where the main loop is long, so up to 1.4 times as many of them pay
+      bool halo = false;
+      if (ks == 3 && G.stride == 1 && G.pad == 1 && bn == 128 && !rows) {
+        const long long igemm_tiles = best / 128;
+        long long fewest = -1;
+        int tw_best = 0, th_best = 0;
+        for (int tw = 1; tw + 2 <= k::HALO_MAX_P && tw <= cp.Wo; ++tw) {
+          const int th = std::min((128 - tw) / (tw + 2) + 1, cp.Ho);
+          const long long n = static_cast<long long>((cp.Wo + tw - 1) / tw) * ((cp.Ho + th - 1) / th);
+          if (fewest < 0 || n <= fewest) { fewest = n; tw_best = tw; th_best = th; }
+        }
+        halo = fewest * 5 <= igemm_tiles * 7;
+        if (halo) { cp.TW = tw_best; cp.TH = th_best; }
+      }
       if (cp.TW * G.stride > 256 || cp.TH * G.stride > 256) return fail(E_UNSUPPORTED_OP, "convolution stride too large for the TMA box");
       const int H = static_cast<int>(vx.dims[2]), Wd = static_cast<int>(vx.dims[3]);
       Ptr px = ptr_of(G.a, r), po = ptr_of(G.out, r), pr = G.res >= 0 ? ptr_of(G.res, r) : Ptr();
@@ -1791,12 +1807,14 @@ struct Builder : BuildState {
       if (rows) {
         RowsReq q{px, po, pr, H, Wd, cp.Ho, cp.Wo, cp.n_img, n_in_map, n_out_map, n_res_map, cp, rt, rt_slot, ids_in, ids_res, ids_out};
         // a run-time image count or id lists belong to one request: such a request is launched alone
+        form(gi, strip ? "strip" : "rows");
         const bool solo = rt || ids_in >= 0 || ids_res >= 0 || ids_out >= 0;
         if (solo) { emit_rows({q}); continue; }
         rows_reqs.push_back(q);
         if (rows_reqs.size() == static_cast<size_t>(k::C3_MAX_REQ)) { emit_rows(rows_reqs); rows_reqs.clear(); }
         continue;
       }
+      form(gi, halo ? "halo" : "implicit GEMM");
       struct Cache { const void* a = nullptr; const void* w = nullptr; const void* o = nullptr; const void* r = nullptr; CUtensorMap tx, tw, to, tr; };
       auto cache = std::make_shared<Cache>();
       add(gi, 1, [=](const RunCtx& x) mutable {
@@ -1805,8 +1823,8 @@ struct Builder : BuildState {
         void* O = x.resolve(po);
         const void* R = hr ? x.resolve(pr) : O;
         if (cache->a != X || cache->w != Wp || cache->o != O || cache->r != R) {
-          if (!encode_bf16_nhwc(&cache->tx, X, n_in_map, H, Wd, Cin, cp.TW, cp.TH, stride) ||
-              !encode_bf16_kchunks(&cache->tw, Wp, Cout, K, K, bn, kch) ||
+          if (!encode_bf16_nhwc(&cache->tx, X, n_in_map, H, Wd, Cin, cp.TW + (halo ? 2 : 0), cp.TH + (halo ? 2 : 0), stride) ||
+              !encode_bf16_kchunks(&cache->tw, Wp, Cout, K, K, bn, halo ? 3 : kch) ||
               !encode_bf16_nhwc(&cache->to, O, n_out_map, cp.Ho, cp.Wo, Cout, cp.TW, cp.TH, 1) ||
               !encode_bf16_nhwc(&cache->tr, R, hr ? n_res_map : n_out_map, cp.Ho, cp.Wo, Cout, cp.TW, cp.TH, 1))
             return cudaErrorInvalidValue;
@@ -1821,6 +1839,18 @@ struct Builder : BuildState {
         cp.out_ids = ids_out >= 0 ? reinterpret_cast<const int*>(auxb + ids_out) : nullptr;
         cp.gap_sum = gap_table != SIZE_MAX ? reinterpret_cast<double*>(const_cast<char*>(auxb) + gap_table) : nullptr;
         const dim3 gd(static_cast<unsigned>(std::min<long long>(tiles, x.plan->sm_count))), bd(k::CONV_THREADS);
+        if (halo) {
+#define SOD2_HALO(ACT_, HR_)                                                                                                             \
+          {                                                                                                                              \
+            static bool once = (cudaFuncSetAttribute(k::conv3x3_halo_bf16_tcgen05<ACT_, HR_>, cudaFuncAttributeMaxDynamicSharedMemorySize, \
+                                                     k::HALO_SMEM), true);                                                               \
+            (void)once;                                                                                                                  \
+            return launch_pdl(k::conv3x3_halo_bf16_tcgen05<ACT_, HR_>, gd, bd, k::HALO_SMEM, x.stream, cache->tx, cache->tw, cache->to, cache->tr, cp); \
+          }
+          if (act == 2) { if (hr) SOD2_HALO(2, true) else SOD2_HALO(2, false) }
+          else { if (hr) SOD2_HALO(0, true) else SOD2_HALO(0, false) }
+#undef SOD2_HALO
+        }
         const int variant = ((bn == 128 ? 2 : 0) + (act == 2 ? 1 : 0)) * 2 + (hr ? 1 : 0);
 #define SOD2_CONV_CASE(V, BN_, KCH_, ST_, ACT_, HR_)                                                                     \
         case V: {                                                                                                        \

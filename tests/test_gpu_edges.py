@@ -78,6 +78,24 @@ def test_conv_strips_segments_and_ring(shapes):
         assert all(np.array_equal(a[n], b[n]) for n in a)
 
 
+@pytest.mark.parametrize("C,shapes", [(128, [(14, 14), (28, 28), (56, 56), (5, 29), (31, 30), (1, 1)]), (256, [(7, 7), (17, 43), (33, 64)]), (384, [(2, 15)])])
+def test_conv_halo_patches(C, shapes):
+    # patches that fill their 128 rows and that do not, lines of the widest pitch (29 pixels), images smaller than a patch and a
+    # pixel larger, two and three channel tiles, tiles in a CTA's second round
+    wl = WL.cfg4(blocks=2, C=C)
+    rng = np.random.default_rng(61)
+    reqs = [Request({"H": h, "W": w}, {"x": bf16_round(rng.uniform(-1, 1, (1, C, h, w)).astype(np.float32))}) for h, w in shapes]
+    s, p, outs = run_batch(wl, reqs, opt_flags=B.OPT_NO_REUSE)
+    forms = {p.plan.group_form(i) for i in range(s.graph.num_groups()) if s.graph.group_info(i)["kind"] == "conv"}
+    assert forms == {"halo"}, forms
+    for r, req in enumerate(reqs):
+        errs = lockstep(wl, s, p, outs, r, BF16_TOL)
+        assert max(errs.values()) <= BF16_TOL, (req.syms, errs)
+    p.run()
+    for a, b in zip(outs, p.outputs()):
+        assert all(np.array_equal(a[n], b[n]) for n in a)
+
+
 @pytest.mark.parametrize("lens", [[1], [33, 64], [129, 640], list(range(1, 129, 3)) + [129, 191, 192, 193, 255, 256, 257, 300, 383, 385, 511, 512, 513, 577] + [200] * 8,
                                   list(range(2, 130, 3)) + [128, 129, 191, 192, 193, 255, 256, 257, 300, 383, 385, 511, 512, 513, 577] + [200] * 7])
 def test_attention_blocks_items_and_tables(lens):
