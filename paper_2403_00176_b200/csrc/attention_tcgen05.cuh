@@ -161,6 +161,7 @@ attention_tcgen05_bf16(const __grid_constant__ CUtensorMap tmQ, const __grid_con
   if (warp == 4 || warp == 7) {
     // ---- TMA producers: warp 4 Q and K, warp 7 V
     const bool is_k = warp == 4;
+    const ptx::Leader one = ptx::elect_leader();
     ptx::pdl_wait();
     int n = 0, i = 0;
     for (int item; (item = nth_item(i)) < items; ++i) {
@@ -169,11 +170,8 @@ attention_tcgen05_bf16(const __grid_constant__ CUtensorMap tmQ, const __grid_con
       if (is_k) {
         const int qs = i & 1;
         if (i >= 2) ptx::mbar_wait_elect(&q_free[qs], ((i >> 1) - 1) & 1, dead);
-        if (ptx::elect_one()) {
-          ptx::mbar_expect_tx(&q_full[qs], ATC_Q_BYTES);
-          ptx::tma_load_2d(sQ + qs * ATC_Q_BYTES, &tmQ, p.q_col + it.head * p.q_hs, R.q_row + it.q0, &q_full[qs]);
-        }
-        __syncwarp();
+        ptx::mbar_expect_tx(one, &q_full[qs], ATC_Q_BYTES);
+        ptx::tma_load_2d(one, sQ + qs * ATC_Q_BYTES, &tmQ, p.q_col + it.head * p.q_hs, R.q_row + it.q0, &q_full[qs]);
       }
       uint64_t* full = is_k ? k_full : v_full;
       uint64_t* free_ = is_k ? k_free : v_free;
@@ -183,17 +181,15 @@ attention_tcgen05_bf16(const __grid_constant__ CUtensorMap tmQ, const __grid_con
       for (int j = 0; j < it.nkv; ++j, ++n) {
         const int b = n % ATC_ST;
         if (n >= ATC_ST) ptx::mbar_wait_elect(&free_[b], ((n / ATC_ST) - 1) & 1, dead);
-        if (ptx::elect_one()) {
-          ptx::mbar_expect_tx(&full[b], ATC_KV_BYTES);
-          ptx::tma_load_2d(dst + b * ATC_KV_BYTES, tm, col, row + j * ATC_KB, &full[b]);
-          SOD2_TRACE(0, (is_k ? 800 : 840) + n)
-        }
-        __syncwarp();
+        ptx::mbar_expect_tx(one, &full[b], ATC_KV_BYTES);
+        ptx::tma_load_2d(one, dst + b * ATC_KV_BYTES, tm, col, row + j * ATC_KB, &full[b]);
+        SOD2_TRACE(0, (is_k ? 800 : 840) + n)
       }
     }
   } else if (warp == 5) {
     // ---- S issuer: S_n once S_{n-2} is in registers
     constexpr uint32_t idesc_qk = ptx::idesc_bf16(128, ATC_KB);
+    const ptx::Leader one = ptx::elect_leader();
     int n = 0, i = 0;
     for (int item; (item = nth_item(i)) < items; ++i) {
       const Item it = locate(item);
@@ -204,13 +200,10 @@ attention_tcgen05_bf16(const __grid_constant__ CUtensorMap tmQ, const __grid_con
         ptx::mbar_wait_elect(&k_full[n % ATC_ST], (n / ATC_ST) & 1, dead);
         if (n >= 2) ptx::mbar_wait_elect(&s_free[n & 1], ((n >> 1) - 1) & 1, dead);
         ptx::tc_fence_after();
-        if (ptx::elect_one()) {
 #pragma unroll
-          for (int kk = 0; kk < 4; ++kk) ptx::mma_bf16(tmem + ATC_TMEM_S + (n & 1) * 64, dQ + 2 * kk, dK + 2 * kk, idesc_qk, kk != 0);
-          ptx::mma_commit(&s_full[n & 1]);
-          ptx::mma_commit(&k_free[n % ATC_ST]);
-        }
-        __syncwarp();
+        for (int kk = 0; kk < 4; ++kk) ptx::mma_bf16(one, tmem + ATC_TMEM_S + (n & 1) * 64, dQ + 2 * kk, dK + 2 * kk, idesc_qk, kk != 0);
+        ptx::mma_commit(one, &s_full[n & 1]);
+        ptx::mma_commit(one, &k_free[n % ATC_ST]);
         if (lane == 0) { SOD2_TRACE(1, 100 + n) }
       }
     }
@@ -218,6 +211,7 @@ attention_tcgen05_bf16(const __grid_constant__ CUtensorMap tmQ, const __grid_con
     // ---- O issuer: O += P_n V_n.  The softmax warps rescale O (rarely) before they hand over P_n, and read an item's O
     // before they hand over the next item's first P, so the accumulator needs no barrier of its own.
     constexpr uint32_t idesc_pv = ptx::idesc_bf16(128, 64) | (1u << 16);   // B (= V tile) is MN-major
+    const ptx::Leader one = ptx::elect_leader();
     int n = 0;
     for (int i = 0, item; (item = nth_item(i)) < items; ++i) {
       const Item it = locate(item);
@@ -227,15 +221,12 @@ attention_tcgen05_bf16(const __grid_constant__ CUtensorMap tmQ, const __grid_con
         ptx::mbar_wait_elect(&v_full[n % ATC_ST], (n / ATC_ST) & 1, dead);
         ptx::mbar_wait_elect(&p_full[n & 1], (n >> 1) & 1, dead);
         ptx::tc_fence_after();
-        if (ptx::elect_one()) {
-          // 16 keys per step: 8 packed columns of P in tensor memory, 16 rows (2048 B) down V
+        // 16 keys per step: 8 packed columns of P in tensor memory, 16 rows (2048 B) down V
 #pragma unroll
-          for (int kk = 0; kk < ATC_KB / 16; ++kk)
-            if (kk < steps) ptx::mma_bf16_a_tmem(tmem + ATC_TMEM_O, tmem + ATC_TMEM_P + (n & 1) * 32 + kk * 8, ptx::smem_desc_sw128(aV + kk * 2048), idesc_pv, (j | kk) != 0);
-          ptx::mma_commit(&o_full[n & 1]);
-          ptx::mma_commit(&v_free[n % ATC_ST]);
-        }
-        __syncwarp();
+        for (int kk = 0; kk < ATC_KB / 16; ++kk)
+          if (kk < steps) ptx::mma_bf16_a_tmem(one, tmem + ATC_TMEM_O, tmem + ATC_TMEM_P + (n & 1) * 32 + kk * 8, ptx::smem_desc_sw128(aV + kk * 2048), idesc_pv, (j | kk) != 0);
+        ptx::mma_commit(one, &o_full[n & 1]);
+        ptx::mma_commit(one, &v_free[n % ATC_ST]);
         if (lane == 0) { SOD2_TRACE(1, 200 + n) }
       }
     }
@@ -421,6 +412,7 @@ attention_tcgen05_bf16(const __grid_constant__ CUtensorMap tmQ, const __grid_con
     }
     if (i > 0) finish(i - 1, n);
   }
+  __syncwarp();
   ptx::tc_fence_before();
   __syncthreads();
   if (warp == 5) ptx::tmem_dealloc(tmem, 256);

@@ -80,15 +80,14 @@ conv3x3_halo_bf16_tcgen05(const __grid_constant__ CUtensorMap tmX, const __grid_
   const int cchunks = p.Cin / 64;
   const int groups = 3 * cchunks;                    // weight stages per tile
   const int tiles_w = (p.Wo + p.TW - 1) / p.TW, tiles_h = (p.Ho + p.TH - 1) / p.TH;
-  auto weight_box = [&](int s, int n0, int gq) {     // group gq of a tile = (chunk gq / 3, kernel row gq % 3)
-    ptx::mbar_expect_tx(&b_full[s], HALO_B_STAGE);
-    ptx::tma_load_3d(weights + s * HALO_B_STAGE, &tmW, 0, n0, ((gq % 3) * cchunks + gq / 3) * 3, &b_full[s]);
+  auto weight_box = [&](ptx::Leader one, int s, int n0, int gq) {     // group gq of a tile = (chunk gq / 3, kernel row gq % 3)
+    ptx::mbar_expect_tx(one, &b_full[s], HALO_B_STAGE);
+    ptx::tma_load_3d(one, weights + s * HALO_B_STAGE, &tmW, 0, n0, ((gq % 3) * cchunks + gq / 3) * 3, &b_full[s]);
   };
   // the first weight stages do not depend on the previous kernel
   if (warp == 1) {
-    if (ptx::elect_one())
-      for (int gq = 0; gq < BS; ++gq) weight_box(gq, (static_cast<int>(blockIdx.x) % tiles_n) * BN, gq);   // groups >= 3 = BS
-    __syncwarp();
+    const ptx::Leader one = ptx::elect_leader();
+    for (int gq = 0; gq < BS; ++gq) weight_box(one, gq, (static_cast<int>(blockIdx.x) % tiles_n) * BN, gq);   // groups >= 3 = BS
   }
   ptx::pdl_wait();
   int n_img = p.n_img;
@@ -106,6 +105,7 @@ conv3x3_halo_bf16_tcgen05(const __grid_constant__ CUtensorMap tmX, const __grid_
   if (warp == 0) {
     // ---- activation patches
     const uint32_t bytes = P * (p.TH + 2) * 128;
+    const ptx::Leader one = ptx::elect_leader();
     int n = 0;
     for (int t = blockIdx.x; t < num_tiles; t += gridDim.x) {
       int n0, img, ho0, wo0;
@@ -114,11 +114,8 @@ conv3x3_halo_bf16_tcgen05(const __grid_constant__ CUtensorMap tmX, const __grid_
       for (int cc = 0; cc < cchunks; ++cc, ++n) {
         const int s = n % AS;
         if (n >= AS) ptx::mbar_wait_elect(&a_empty[s], ((n / AS) - 1) & 1, dead);
-        if (ptx::elect_one()) {
-          ptx::mbar_expect_tx(&a_full[s], bytes);
-          ptx::tma_load_4d(patches + s * HALO_A_SLOT, &tmX, cc * 64, wo0 - 1, ho0 - 1, img, &a_full[s]);
-        }
-        __syncwarp();
+        ptx::mbar_expect_tx(one, &a_full[s], bytes);
+        ptx::tma_load_4d(one, patches + s * HALO_A_SLOT, &tmX, cc * 64, wo0 - 1, ho0 - 1, img, &a_full[s]);
       }
     }
   } else if (warp == 1) {
@@ -126,6 +123,7 @@ conv3x3_halo_bf16_tcgen05(const __grid_constant__ CUtensorMap tmX, const __grid_
     if (static_cast<int>(blockIdx.x) >= num_tiles) {
       for (int s = 0; s < BS; ++s) ptx::mbar_wait_elect(&b_full[s], 0, dead);    // nothing may land after the CTA has gone
     }
+    const ptx::Leader one = ptx::elect_leader();
     int n = 0;
     for (int t = blockIdx.x; t < num_tiles; t += gridDim.x) {
       const int n0 = (t % tiles_n) * BN;
@@ -133,42 +131,41 @@ conv3x3_halo_bf16_tcgen05(const __grid_constant__ CUtensorMap tmX, const __grid_
         if (n < BS) continue;
         const int s = n % BS;
         ptx::mbar_wait_elect(&b_empty[s], ((n / BS) - 1) & 1, dead);
-        if (ptx::elect_one()) weight_box(s, n0, gq);
-        __syncwarp();
+        weight_box(one, s, n0, gq);
       }
     }
   } else if (warp == 3) {
-    // ---- MMA issuer: the whole warp in step, one lane issues (ptx::elect_one)
+    // ---- MMA issuer: the whole warp in step, one lane issues (ptx::Leader)
     constexpr uint32_t idesc = ptx::idesc_bf16(128, BN);
-    int na = 0, nb = 0, j = 0;
+    const ptx::Leader one = ptx::elect_leader();
+    // (weight stage dy holds kernel row dy of every chunk: BS == 3.  Straight-line code with the descriptors at hand: with
+    // the three rows as a loop the issuer took 82 cycles per MMA, 67 like this; the pipe takes 64)
+    static_assert(BS == 3 && AS == 2, "one weight stage per kernel row, patches in turn");
+    const uint64_t a0 = ptx::smem_desc_sw128(ptx::smem_u32(patches)), b0 = ptx::smem_desc_sw128(ptx::smem_u32(weights));
+    const uint32_t line = P * 8;             // a patch line in descriptor units of 16 bytes
+    int na = 0, j = 0;
     for (int t = blockIdx.x; t < num_tiles; t += gridDim.x, ++j) {
       const int acc = j & 1;
       if (j >= 2) ptx::mbar_wait_elect(&tmem_empty[acc], ((j >> 1) - 1) & 1, dead);
       const uint32_t d = tmem + acc * BN;
       for (int cc = 0; cc < cchunks; ++cc, ++na) {
-        const int sa = na % AS;
-        ptx::mbar_wait_elect(&a_full[sa], (na / AS) & 1, dead);
-#pragma unroll 1
-        for (int dy = 0; dy < 3; ++dy, ++nb) {
-          const int sb = nb % BS;
-          ptx::mbar_wait_elect(&b_full[sb], (nb / BS) & 1, dead);
+        const int sa = na & 1;
+        const uint64_t as = a0 + sa * (HALO_A_SLOT >> 4);
+        ptx::mbar_wait_elect(&a_full[sa], (na >> 1) & 1, dead);
+#pragma unroll
+        for (int dy = 0; dy < 3; ++dy) {
+          ptx::mbar_wait_elect(&b_full[dy], na & 1, dead);
           ptx::tc_fence_after();
-          if (ptx::elect_one()) {
-            const uint64_t ad = ptx::smem_desc_sw128(ptx::smem_u32(patches + sa * HALO_A_SLOT + dy * P * 128));
-            const uint64_t bd = ptx::smem_desc_sw128(ptx::smem_u32(weights + sb * HALO_B_STAGE));
+          const uint64_t ad = as + dy * line, bd = b0 + dy * (HALO_B_STAGE >> 4);
 #pragma unroll
-            for (int dx = 0; dx < 3; ++dx)
+          for (int dx = 0; dx < 3; ++dx)
 #pragma unroll
-              for (int kk = 0; kk < 4; ++kk) ptx::mma_bf16(d, ad + 8 * dx + 2 * kk, bd + dx * (BN * 128 / 16) + 2 * kk, idesc, (cc | dy | dx | kk) != 0);
-            ptx::mma_commit(&b_empty[sb]);
-            if (dy == 2) {
-              ptx::mma_commit(&a_empty[sa]);
-              if (cc + 1 == cchunks) ptx::mma_commit(&tmem_full[acc]);
-            }
-          }
-          __syncwarp();
+            for (int kk = 0; kk < 4; ++kk) ptx::mma_bf16(one, d, ad + 8 * dx + 2 * kk, bd + dx * (BN * 128 / 16) + 2 * kk, idesc, (cc | dy | dx | kk) != 0);
+          ptx::mma_commit(one, &b_empty[dy]);
         }
+        ptx::mma_commit(one, &a_empty[sa]);
       }
+      ptx::mma_commit(one, &tmem_full[acc]);
     }
   } else if (warp >= 4) {
     // ---- epilogue warps 4..11: passes of 64 channels through two staging buffers (conv_tcgen05.cuh)
@@ -277,6 +274,7 @@ conv3x3_halo_bf16_tcgen05(const __grid_constant__ CUtensorMap tmX, const __grid_
     }
     if (et == 0) bulk_wait0();
   }
+  __syncwarp();
   ptx::tc_fence_before();
   __syncthreads();
   if (warp == 3) ptx::tmem_dealloc(tmem, 2 * BN);

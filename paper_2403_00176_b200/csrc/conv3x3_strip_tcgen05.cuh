@@ -337,6 +337,7 @@ conv3x3_strip_bf16_tcgen05(const __grid_constant__ Conv3Batch B, const __grid_co
       if (lane == 0) ptx::mbar_arrive(&stage_ready[bsel]);
     }
   }
+  __syncwarp();
   ptx::tc_fence_before();
   __syncthreads();
   if (warp == 3) ptx::tmem_dealloc(tmem, 512);

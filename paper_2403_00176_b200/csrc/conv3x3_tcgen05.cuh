@@ -112,6 +112,7 @@ conv3x3_rows_bf16_tcgen05(const __grid_constant__ Conv3Batch B, const __grid_con
 
   if (warp == 0) {
     // ---- A producer: one halo row segment per stage
+    const ptx::Leader one = ptx::elect_leader();
     int n = 0;
     for (int t = blockIdx.x; t < num_tiles; t += gridDim.x) {
       int n0, img, h0, w0;
@@ -121,27 +122,22 @@ conv3x3_rows_bf16_tcgen05(const __grid_constant__ Conv3Batch B, const __grid_con
         const int s = n % STAGES;
         if (n >= STAGES) ptx::mbar_wait_elect(&empty[s], ((n / STAGES) - 1) & 1, dead);
         const int dy = ks / cchunks, cc = ks % cchunks;
-        if (ptx::elect_one()) {
-          SOD2_TRACE(0, 100 + ks)
-          ptx::mbar_expect_tx(&full[s], C3_A_BYTES);
-          ptx::tma_load_4d(tiles + s * S::STAGE_BYTES, &B.tx[rq], cc * 64, w0 - 1, h0 + dy - 1, img, &full[s]);
-        }
-        __syncwarp();
+        SOD2_TRACE(0, 100 + ks)
+        ptx::mbar_expect_tx(one, &full[s], C3_A_BYTES);
+        ptx::tma_load_4d(one, tiles + s * S::STAGE_BYTES, &B.tx[rq], cc * 64, w0 - 1, h0 + dy - 1, img, &full[s]);
       }
     }
   } else if (warp == 1) {
     // ---- B producer: the three dx taps of (dy, chunk) are consecutive k-chunks
+    const ptx::Leader one = ptx::elect_leader();
     int n = 0;
     for (int t = blockIdx.x; t < num_tiles; t += gridDim.x) {
       const int n0 = (t / tiles_px) * BN;
       for (int ks = 0; ks < kstages; ++ks, ++n) {
         const int s = n % STAGES;
         if (n >= STAGES) ptx::mbar_wait_elect(&empty[s], ((n / STAGES) - 1) & 1, dead);
-        if (ptx::elect_one()) {
-          ptx::mbar_expect_tx(&full[s], 3 * BN * 128);
-          ptx::tma_load_3d(tiles + s * S::STAGE_BYTES + C3_A_SLOT, &tmW, 0, n0, ks * 3, &full[s]);
-        }
-        __syncwarp();
+        ptx::mbar_expect_tx(one, &full[s], 3 * BN * 128);
+        ptx::tma_load_3d(one, tiles + s * S::STAGE_BYTES + C3_A_SLOT, &tmW, 0, n0, ks * 3, &full[s]);
       }
     }
   } else if (warp == 3 || warp == 12) {
@@ -154,6 +150,7 @@ conv3x3_rows_bf16_tcgen05(const __grid_constant__ Conv3Batch B, const __grid_con
       // the barrier's previous phase, and walking all stages keeps each issuer exactly in step (the
       // in-order producer cannot refill a slot twice while an issuer still owns an earlier stage).
       constexpr uint32_t idesc = ptx::idesc_bf16(128, BN);
+      const ptx::Leader one = ptx::elect_leader();
       const int me = warp == 3 ? 0 : 1;
       int n = 0, j = 0;
       for (int t = blockIdx.x; t < num_tiles; t += gridDim.x, ++j) {
@@ -172,18 +169,15 @@ conv3x3_rows_bf16_tcgen05(const __grid_constant__ Conv3Batch B, const __grid_con
           if (me == 0) { SOD2_TRACE(1, 200 + ks) }
           const uint32_t a = ptx::smem_u32(tiles + s * S::STAGE_BYTES);
           const uint32_t b = a + C3_A_SLOT;
-          if (ptx::elect_one()) {
 #pragma unroll
-            for (int dx = 0; dx < 3; ++dx) {
-              const uint64_t ad = ptx::smem_desc_sw128(a + dx * 128);     // rows shifted by dx pixels
-              const uint64_t bd = ptx::smem_desc_sw128(b + dx * (BN * 128));
+          for (int dx = 0; dx < 3; ++dx) {
+            const uint64_t ad = ptx::smem_desc_sw128(a + dx * 128);     // rows shifted by dx pixels
+            const uint64_t bd = ptx::smem_desc_sw128(b + dx * (BN * 128));
 #pragma unroll
-              for (int kk = 0; kk < 4; ++kk) ptx::mma_bf16(d, ad + 2 * kk, bd + 2 * kk, idesc, (ks | dx | kk) != 0);
-            }
-            ptx::mma_commit(&empty[s]);
-            if (ks + 1 == kstages) ptx::mma_commit(&tmem_full[acc]);
+            for (int kk = 0; kk < 4; ++kk) ptx::mma_bf16(one, d, ad + 2 * kk, bd + 2 * kk, idesc, (ks | dx | kk) != 0);
           }
-          __syncwarp();
+          ptx::mma_commit(one, &empty[s]);
+          if (ks + 1 == kstages) ptx::mma_commit(one, &tmem_full[acc]);
         }
         if (mine && me == 0) { SOD2_TRACE(1, 210) }
       }
@@ -326,6 +320,7 @@ conv3x3_rows_bf16_tcgen05(const __grid_constant__ Conv3Batch B, const __grid_con
       }
     }
   }
+  __syncwarp();
   ptx::tc_fence_before();
   __syncthreads();
   if (warp == 3) ptx::tmem_dealloc(tmem, TMEM_COLS);

@@ -251,6 +251,7 @@ conv_stem_bf16_tcgen05(const __grid_constant__ CUtensorMap tmW, const __grid_con
     {
       // ---- MMA issuer
       constexpr uint32_t idesc = ptx::idesc_bf16(128, 64);
+      const ptx::Leader one = ptx::elect_leader();
       ptx::mbar_wait_elect(w_full, 0, dead);
       const uint32_t aW = ptx::smem_u32(sW);
       int it = 0;
@@ -262,17 +263,14 @@ conv_stem_bf16_tcgen05(const __grid_constant__ CUtensorMap tmW, const __grid_con
         SOD2_TRACE(1, 41)
         ptx::tc_fence_after();
         const uint32_t aA = ptx::smem_u32(sA + b * STEM_A_BYTES);
-        if (ptx::elect_one()) {
 #pragma unroll
-          for (int c = 0; c < 3; ++c) {
-            const uint64_t ad = ptx::smem_desc_sw128(aA + c * (128 * 128)), bd = ptx::smem_desc_sw128(aW + c * (64 * 128));
+        for (int c = 0; c < 3; ++c) {
+          const uint64_t ad = ptx::smem_desc_sw128(aA + c * (128 * 128)), bd = ptx::smem_desc_sw128(aW + c * (64 * 128));
 #pragma unroll
-            for (int kk = 0; kk < 4; ++kk) ptx::mma_bf16(tmem + b * 64, ad + 2 * kk, bd + 2 * kk, idesc, (c | kk) != 0);
-          }
-          ptx::mma_commit(&a_free[b]);
-          ptx::mma_commit(&acc_full[b]);
+          for (int kk = 0; kk < 4; ++kk) ptx::mma_bf16(one, tmem + b * 64, ad + 2 * kk, bd + 2 * kk, idesc, (c | kk) != 0);
         }
-        __syncwarp();
+        ptx::mma_commit(one, &a_free[b]);
+        ptx::mma_commit(one, &acc_full[b]);
         SOD2_TRACE(1, 42)
       }
     }
@@ -329,6 +327,7 @@ conv_stem_bf16_tcgen05(const __grid_constant__ CUtensorMap tmW, const __grid_con
     }
     if (leader) bulk_wait_read0();
   }
+  __syncwarp();
   ptx::tc_fence_before();
   __syncthreads();
   if (warp == 13) ptx::tmem_dealloc(tmem, 128);

@@ -153,6 +153,7 @@ conv_igemm_bf16_tcgen05(const __grid_constant__ CUtensorMap tmX, const __grid_co
 
   if (warp < 2) {
     // ---- A producers: warp 0 loads the even chunks of every stage, warp 1 the odd ones
+    const ptx::Leader one = ptx::elect_leader();
     int n = 0;
     for (int t = blockIdx.x; t < num_tiles; t += gridDim.x) {
       int n0, img, ho0, wo0;
@@ -161,68 +162,64 @@ conv_igemm_bf16_tcgen05(const __grid_constant__ CUtensorMap tmX, const __grid_co
       for (int ks = 0; ks < kstages; ++ks, ++n) {
         const int s = n % STAGES;
         if (n >= STAGES) ptx::mbar_wait_elect(&empty[s], ((n / STAGES) - 1) & 1, dead);
-        if (ptx::elect_one()) {
-          int mine = 0;
-          for (int c = warp; c < KCH; c += 2) ++mine;
-          ptx::mbar_expect_tx(&full[s], mine * 128 * 128);
-          for (int c = warp; c < KCH; c += 2) {
-            const int q = ks * KCH + c;          // k-chunk: tap-major, then 64-channel chunk
-            int dy, dx, cc;
-            if (p.korder) { dy = q / (3 * cchunks); cc = (q / 3) % cchunks; dx = q % 3; }
-            else { const int tap = q / cchunks; cc = q % cchunks; dy = tap / p.ksize; dx = tap % p.ksize; }
-            // chunks past the end (K tail of the last stage) are loaded far out of range: zero fill
-            const int hi = q < kchunks ? ho0 * p.stride + dy - p.pad : -100000;
-            ptx::tma_load_4d(tiles + s * S::STAGE_BYTES + c * (128 * 128), &tmX, cc * 64, wo0 * p.stride + dx - p.pad, hi, img, &full[s]);
-          }
+        int mine = 0;
+        for (int c = warp; c < KCH; c += 2) ++mine;
+        ptx::mbar_expect_tx(one, &full[s], mine * 128 * 128);
+        for (int c = warp; c < KCH; c += 2) {
+          const int q = ks * KCH + c;          // k-chunk: tap-major, then 64-channel chunk
+          int dy, dx, cc;
+          if (p.korder) { dy = q / (3 * cchunks); cc = (q / 3) % cchunks; dx = q % 3; }
+          else { const int tap = q / cchunks; cc = q % cchunks; dy = tap / p.ksize; dx = tap % p.ksize; }
+          // chunks past the end (K tail of the last stage) are loaded far out of range: zero fill
+          const int hi = q < kchunks ? ho0 * p.stride + dy - p.pad : -100000;
+          ptx::tma_load_4d(one, tiles + s * S::STAGE_BYTES + c * (128 * 128), &tmX, cc * 64, wo0 * p.stride + dx - p.pad, hi, img, &full[s]);
         }
-        __syncwarp();
       }
     }
   } else if (warp == 2) {
     // ---- B producer
+    const ptx::Leader one = ptx::elect_leader();
     int n = 0;
     for (int t = blockIdx.x; t < num_tiles; t += gridDim.x) {
       const int n0 = (t / tiles_px) * BN;
       for (int ks = 0; ks < kstages; ++ks, ++n) {
         const int s = n % STAGES;
         if (n >= STAGES) ptx::mbar_wait_elect(&empty[s], ((n / STAGES) - 1) & 1, dead);
-        if (ptx::elect_one()) {
-          ptx::mbar_expect_tx(&full[s], S::B_BYTES);
-          ptx::tma_load_3d(tiles + s * S::STAGE_BYTES + S::A_BYTES, &tmW, 0, n0, ks * KCH, &full[s]);
-        }
-        __syncwarp();
+        ptx::mbar_expect_tx(one, &full[s], S::B_BYTES);
+        ptx::tma_load_3d(one, tiles + s * S::STAGE_BYTES + S::A_BYTES, &tmW, 0, n0, ks * KCH, &full[s]);
       }
     }
   } else if (warp == 3) {
     {
-      // ---- MMA issuer: the whole warp in step, one lane issues (ptx::elect_one)
+      // ---- MMA issuer: the whole warp in step, one lane issues (ptx::Leader)
       constexpr uint32_t idesc = ptx::idesc_bf16(128, BN);
-      int n = 0, j = 0;
+      const ptx::Leader one = ptx::elect_leader();
+      // (stage and parity counted along, descriptors as sums: see the GEMM's issuer)
+      static_assert(KCH <= 2, "the issuer leaves out one chunk at most");
+      const uint64_t a0 = ptx::smem_desc_sw128(ptx::smem_u32(tiles)), b0 = ptx::smem_desc_sw128(ptx::smem_u32(tiles + S::A_BYTES));
+      uint32_t s = 0, par = 0;
+      int j = 0;
       for (int t = blockIdx.x; t < num_tiles; t += gridDim.x, ++j) {
         const int acc = j & 1;
         if (j >= 2) ptx::mbar_wait_elect(&tmem_empty[acc], ((j >> 1) - 1) & 1, dead);
         ptx::tc_fence_after();
         const uint32_t d = tmem + acc * BN;
-        for (int ks = 0; ks < kstages; ++ks, ++n) {
-          const int s = n % STAGES;
-          ptx::mbar_wait_elect(&full[s], (n / STAGES) & 1, dead);
+        for (int ks = 0; ks < kstages; ++ks) {
+          ptx::mbar_wait_elect(&full[s], par, dead);
           ptx::tc_fence_after();
-          const uint32_t a = ptx::smem_u32(tiles + s * S::STAGE_BYTES);
-          if (ptx::elect_one()) {
+          const uint64_t ad = a0 + s * (S::STAGE_BYTES >> 4), bd = b0 + s * (S::STAGE_BYTES >> 4);
 #pragma unroll
-            for (int c = 0; c < KCH; ++c) {
-              if (ks * KCH + c < kchunks) {
-                const uint64_t ad = ptx::smem_desc_sw128(a + c * (128 * 128));
-                const uint64_t bd = ptx::smem_desc_sw128(a + S::A_BYTES + c * (BN * 128));
+          for (int kk = 0; kk < 4; ++kk) ptx::mma_bf16(one, d, ad + 2 * kk, bd + 2 * kk, idesc, (ks | kk) != 0);
+          if (KCH == 1 || (ks + 1) * KCH <= kchunks) {
 #pragma unroll
-                for (int kk = 0; kk < 4; ++kk) ptx::mma_bf16(d, ad + 2 * kk, bd + 2 * kk, idesc, (ks | c | kk) != 0);
-              }
-            }
-            ptx::mma_commit(&empty[s]);
-            if (ks + 1 == kstages) ptx::mma_commit(&tmem_full[acc]);
+            for (int c = 1; c < KCH; ++c)
+#pragma unroll
+              for (int kk = 0; kk < 4; ++kk) ptx::mma_bf16(one, d, ad + c * (128 * 8) + 2 * kk, bd + c * (BN * 8) + 2 * kk, idesc, 1);
           }
-          __syncwarp();
+          ptx::mma_commit(one, &empty[s]);
+          if (++s == STAGES) { s = 0; par ^= 1; }
         }
+        ptx::mma_commit(one, &tmem_full[acc]);
       }
     }
   } else {
@@ -331,6 +328,7 @@ conv_igemm_bf16_tcgen05(const __grid_constant__ CUtensorMap tmX, const __grid_co
     }
     if (et == 0) bulk_wait0();
   }
+  __syncwarp();
   ptx::tc_fence_before();
   __syncthreads();
   if (warp == 3) ptx::tmem_dealloc(tmem, TMEM_COLS);

@@ -84,34 +84,33 @@ gemm_cluster_bf16_tcgen05(const __grid_constant__ CUtensorMap tmA, const __grid_
   if (warp == 0 || warp == 1) {
     // ---- TMA producers: warp 0 A, warp 1 the weights (constants: no wait for the previous kernel)
     if (warp == 0) ptx::pdl_wait();
+    const ptx::Leader one = ptx::elect_leader();
     for (int n = 0; n < kn; ++n) {
       const int s = n % STAGES;
       if (n >= STAGES) ptx::mbar_wait_elect(&empty[s], ((n / STAGES) - 1) & 1, dead);
-      if (ptx::elect_one()) {
-        uint8_t* st = tiles + s * L::STAGE_BYTES;
-        ptx::mbar_expect_tx(&full[s], warp == 0 ? L::A_BYTES : L::B_BYTES);
-        if (warp == 0) ptx::tma_load_3d(st, &tmA, 0, m0, k0 + n, &full[s]);
-        else ptx::tma_load_3d(st + L::A_BYTES, &tmB, 0, n0, k0 + n, &full[s]);
-      }
-      __syncwarp();
+      uint8_t* st = tiles + s * L::STAGE_BYTES;
+      ptx::mbar_expect_tx(one, &full[s], warp == 0 ? L::A_BYTES : L::B_BYTES);
+      if (warp == 0) ptx::tma_load_3d(one, st, &tmA, 0, m0, k0 + n, &full[s]);
+      else ptx::tma_load_3d(one, st + L::A_BYTES, &tmB, 0, n0, k0 + n, &full[s]);
     }
+    __syncwarp();
   } else if (warp == 2) {
     // ---- MMA issuer
     constexpr uint32_t idesc = ptx::idesc_bf16(GEMM_BM, 64);
+    const ptx::Leader one = ptx::elect_leader();
+    const uint64_t a0 = ptx::smem_desc_sw128(ptx::smem_u32(tiles)), b0 = ptx::smem_desc_sw128(ptx::smem_u32(tiles + L::A_BYTES));
+    uint32_t s = 0, par = 0;
     for (int n = 0; n < kn; ++n) {
-      const int s = n % STAGES;
-      ptx::mbar_wait_elect(&full[s], (n / STAGES) & 1, dead);
+      ptx::mbar_wait_elect(&full[s], par, dead);
       ptx::tc_fence_after();
-      const uint32_t a = ptx::smem_u32(tiles + s * L::STAGE_BYTES);
-      if (ptx::elect_one()) {
-        const uint64_t ad = ptx::smem_desc_sw128(a), bd = ptx::smem_desc_sw128(a + L::A_BYTES);
+      const uint64_t ad = a0 + s * (L::STAGE_BYTES >> 4), bd = b0 + s * (L::STAGE_BYTES >> 4);
 #pragma unroll
-        for (int kk = 0; kk < 4; ++kk) ptx::mma_bf16(tmem, ad + 2 * kk, bd + 2 * kk, idesc, n != 0 || kk != 0);
-        ptx::mma_commit(&empty[s]);
-        if (n + 1 == kn) ptx::mma_commit(acc_full);
-      }
-      __syncwarp();
+      for (int kk = 0; kk < 4; ++kk) ptx::mma_bf16(one, tmem, ad + 2 * kk, bd + 2 * kk, idesc, n != 0 || kk != 0);
+      ptx::mma_commit(one, &empty[s]);
+      if (++s == STAGES) { s = 0; par ^= 1; }
     }
+    ptx::mma_commit(one, acc_full);
+    __syncwarp();
   }
   ptx::pdl_wait();        // residual and output belong to the previous kernels
   // ---- this thread's share of the reduction: pieces of four columns, rows [r0, r0 + rows) of the tile; its residual and

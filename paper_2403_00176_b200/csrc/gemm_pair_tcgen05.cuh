@@ -53,10 +53,11 @@ __device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_addr) {
 }
 // 3-D tiled TMA load into this CTA's shared memory whose completion is signalled on a barrier given by its
 // shared::cluster address (the leader's): the cta_group::2 form, no multicast
-__device__ __forceinline__ void tma_load_3d_pair(void* dst, const void* tmap, int x, int y, int z, uint32_t bar_cluster_addr) {
+__device__ __forceinline__ void tma_load_3d_pair(ptx::Leader l, void* dst, const void* tmap, int x, int y, int z, uint32_t bar_cluster_addr) {
   asm volatile(
-      "cp.async.bulk.tensor.3d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];"
-      ::"r"(ptx::smem_u32(dst)), "l"(tmap), "r"(x), "r"(y), "r"(z), "r"(bar_cluster_addr)
+      "{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %6, 0;\n\t"
+      "@q cp.async.bulk.tensor.3d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];\n\t}"
+      ::"r"(ptx::smem_u32(dst)), "l"(tmap), "r"(x), "r"(y), "r"(z), "r"(bar_cluster_addr), "r"(l.on)
       : "memory");
 }
 __device__ __forceinline__ void tmem_alloc_pair(uint32_t* dst_smem, uint32_t ncols) {
@@ -67,6 +68,12 @@ __device__ __forceinline__ void tmem_dealloc_pair(uint32_t taddr, uint32_t ncols
   asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols) : "memory");
 }
 // D[tmem of both CTAs] (+)= A[smem of both CTAs] * B[smem of both CTAs]; issued by one thread of the leader
+__device__ __forceinline__ void mma_bf16_pair(ptx::Leader l, uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t accumulate) {
+  asm volatile(
+      "{\n\t.reg .pred p, q;\n\tsetp.ne.b32 q, %5, 0;\n\tsetp.ne.b32 p, %4, 0;\n\t"
+      "@q tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}"
+      ::"r"(d_tmem), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate), "r"(l.on) : "memory");
+}
 __device__ __forceinline__ void mma_bf16_pair(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t accumulate) {
   asm volatile(
       "{\n\t.reg .pred p;\n\t"
@@ -79,6 +86,11 @@ __device__ __forceinline__ void mma_bf16_pair(uint32_t d_tmem, uint64_t adesc, u
 __device__ __forceinline__ void mma_commit_pair(uint64_t* bar) {
   asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;"
                ::"r"(ptx::smem_u32(bar)), "h"(static_cast<uint16_t>(3)) : "memory");
+}
+__device__ __forceinline__ void mma_commit_pair(ptx::Leader l, uint64_t* bar) {
+  asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %2, 0;\n\t"
+               "@q tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;\n\t}"
+               ::"r"(ptx::smem_u32(bar)), "h"(static_cast<uint16_t>(3)), "r"(l.on) : "memory");
 }
 
 // Weight tiles of 1 to 4 units of 64 columns: box b[w - 1] is the CTA's half, 32 w rows, of a 64-wide k-chunk.
@@ -191,22 +203,21 @@ gemm_pair_bf16_tcgen05(const __grid_constant__ CUtensorMap tmA, const __grid_con
   if (warp == 0) {
     // ---- TMA producer: this CTA's A rows; completion on the leader's barrier
     ptx::pdl_wait();
+    const ptx::Leader one = ptx::elect_leader();
     int n = 0;
     for (PairWalk wk = share; wk.next();) {
       const int m0 = (wk.m * 2 + static_cast<int>(rank)) * GEMM_BM;
       for (int ks = 0; ks < kstages; ++ks, ++n) {
         const int s = n % STAGES;
         if (n >= STAGES) ptx::mbar_wait_elect(&empty[s], ((n / STAGES) - 1) & 1, dead);
-        if (ptx::elect_one()) {
-          SOD2_PAIR_TRACE(0, n)
-          if (leader) ptx::mbar_expect_tx(&full[s], 2 * S::A_BYTES);
-          tma_load_3d_pair(tiles + s * S::STAGE_BYTES, &tmA, 0, m0, ks, map_to_cta(ptx::smem_u32(&full[s]), 0));
-        }
-        __syncwarp();
+        SOD2_PAIR_TRACE(0, n)
+        if (leader) ptx::mbar_expect_tx(one, &full[s], 2 * S::A_BYTES);
+        tma_load_3d_pair(one, tiles + s * S::STAGE_BYTES, &tmA, 0, m0, ks, map_to_cta(ptx::smem_u32(&full[s]), 0));
       }
     }
   } else if (warp == 1) {
     // ---- TMA producer: this CTA's half of the weight tile (constants: no wait for the previous kernel)
+    const ptx::Leader one = ptx::elect_leader();
     int n = 0;
     for (PairWalk wk = share; wk.next();) {
       const int n0 = wk.n0 + static_cast<int>(rank) * wk.w * 32;
@@ -214,38 +225,34 @@ gemm_pair_bf16_tcgen05(const __grid_constant__ CUtensorMap tmA, const __grid_con
       for (int ks = 0; ks < kstages; ++ks, ++n) {
         const int s = n % STAGES;
         if (n >= STAGES) ptx::mbar_wait_elect(&empty[s], ((n / STAGES) - 1) & 1, dead);
-        if (ptx::elect_one()) {
-          if (leader) ptx::mbar_expect_tx(&full[s], 2 * wk.w * (32 * 128));
-          tma_load_3d_pair(tiles + s * S::STAGE_BYTES + S::A_BYTES, tmB, 0, n0, ks, map_to_cta(ptx::smem_u32(&full[s]), 0));
-        }
-        __syncwarp();
+        if (leader) ptx::mbar_expect_tx(one, &full[s], 2 * wk.w * (32 * 128));
+        tma_load_3d_pair(one, tiles + s * S::STAGE_BYTES + S::A_BYTES, tmB, 0, n0, ks, map_to_cta(ptx::smem_u32(&full[s]), 0));
       }
     }
   } else if (warp == 2) {
     if (leader) {
       // ---- MMA issuer (leader only): 256 x 64w x 16 per instruction over both CTAs
-      int n = 0, j = 0;
+      const ptx::Leader one = ptx::elect_leader();
+      const uint64_t a0 = ptx::smem_desc_sw128(ptx::smem_u32(tiles)), b0 = ptx::smem_desc_sw128(ptx::smem_u32(tiles + S::A_BYTES));
+      uint32_t s = 0, par = 0;
+      int j = 0;
       for (PairWalk wk = share; wk.next(); ++j) {
         const int acc = j & 1;
         const uint32_t idesc = ptx::idesc_bf16(2 * GEMM_BM, 64 * wk.w);
         if (j >= 2) ptx::mbar_wait_elect(&tmem_empty[acc], ((j >> 1) - 1) & 1, dead);
         ptx::tc_fence_after();
         const uint32_t d = tmem + acc * BN;
-        for (int ks = 0; ks < kstages; ++ks, ++n) {
-          const int s = n % STAGES;
-          ptx::mbar_wait_elect(&full[s], (n / STAGES) & 1, dead);
+        for (int ks = 0; ks < kstages; ++ks) {
+          ptx::mbar_wait_elect(&full[s], par, dead);
           ptx::tc_fence_after();
-          const uint32_t a = ptx::smem_u32(tiles + s * S::STAGE_BYTES);
-          if (ptx::elect_one()) {
-            SOD2_PAIR_TRACE(1, n)
-            const uint64_t ad = ptx::smem_desc_sw128(a), bd = ptx::smem_desc_sw128(a + S::A_BYTES);
+          SOD2_PAIR_TRACE(1, ks)
+          const uint64_t ad = a0 + s * (S::STAGE_BYTES >> 4), bd = b0 + s * (S::STAGE_BYTES >> 4);
 #pragma unroll
-            for (int kk = 0; kk < 4; ++kk) mma_bf16_pair(d, ad + 2 * kk, bd + 2 * kk, idesc, (ks > 0) || kk != 0);
-            mma_commit_pair(&empty[s]);     // frees the stage in both CTAs
-            if (ks + 1 == kstages) mma_commit_pair(&tmem_full[acc]);
-          }
-          __syncwarp();
+          for (int kk = 0; kk < 4; ++kk) mma_bf16_pair(one, d, ad + 2 * kk, bd + 2 * kk, idesc, (ks > 0) || kk != 0);
+          mma_commit_pair(one, &empty[s]);     // frees the stage in both CTAs
+          if (++s == STAGES) { s = 0; par ^= 1; }
         }
+        mma_commit_pair(one, &tmem_full[acc]);
       }
     }
   } else if (warp == 11) {
@@ -370,6 +377,7 @@ gemm_pair_bf16_tcgen05(const __grid_constant__ CUtensorMap tmA, const __grid_con
     }
   }
   if (threadIdx.x == 96) { SOD2_PAIR_TRACE(2, 999) }
+  __syncwarp();
   ptx::tc_fence_before();
   __syncthreads();
   cluster_sync_all();               // neither CTA leaves (or frees tensor memory) while the other can still reach it

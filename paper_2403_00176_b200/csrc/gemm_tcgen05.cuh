@@ -167,6 +167,7 @@ gemm_bf16_tcgen05(const __grid_constant__ CUtensorMap tmA, const __grid_constant
                   const __grid_constant__ CUtensorMap tmOut, const __grid_constant__ CUtensorMap tmRes,
                   int M, int N, int K, GemmEpilogue ep) {
   using S = GemmSmem<BN, KCH, STAGES>;
+  static_assert(KCH <= 2, "the issuer leaves out one chunk at most");
   constexpr int PASSES = SPLITK ? BN / 32 : BN / GEMM_PASS_COLS;   // split-K passes are 32 fp32 columns (128-byte rows)
   constexpr int NSB = GEMM_NSB;
   extern __shared__ uint8_t smem_raw[];
@@ -232,6 +233,7 @@ gemm_bf16_tcgen05(const __grid_constant__ CUtensorMap tmA, const __grid_constant
   if (warp == 0) {
     // ---- TMA producer: A stages
     ptx::pdl_wait();
+    const ptx::Leader one = ptx::elect_leader();
     int n = 0;
     for (int w = blockIdx.x; w < num_tiles; w += gridDim.x) {
       const int t = SPLITK ? w % out_tiles : w;
@@ -241,16 +243,14 @@ gemm_bf16_tcgen05(const __grid_constant__ CUtensorMap tmA, const __grid_constant
       for (int ks = ks0; ks < ks1; ++ks, ++n) {
         const int s = n % STAGES;
         if (n >= STAGES) ptx::mbar_wait_elect(&empty[s], ((n / STAGES) - 1) & 1, dead);
-        if (ptx::elect_one()) {
-          if (n == 0) { SOD2_TRACE(0, 2) }
-          ptx::mbar_expect_tx(&full[s], S::A_BYTES);
-          ptx::tma_load_3d(tiles + s * S::STAGE_BYTES, &tmA, 0, m0, ks * KCH, &full[s]);
-        }
-        __syncwarp();
+        if (n == 0) { SOD2_TRACE(0, 2) }
+        ptx::mbar_expect_tx(one, &full[s], S::A_BYTES);
+        ptx::tma_load_3d(one, tiles + s * S::STAGE_BYTES, &tmA, 0, m0, ks * KCH, &full[s]);
       }
     }
   } else if (warp == 1) {
     // ---- TMA producer: B stages
+    const ptx::Leader one = ptx::elect_leader();
     int n = 0;
     for (int w = blockIdx.x; w < num_tiles; w += gridDim.x) {
       const int t = SPLITK ? w % out_tiles : w;
@@ -260,19 +260,21 @@ gemm_bf16_tcgen05(const __grid_constant__ CUtensorMap tmA, const __grid_constant
       for (int ks = ks0; ks < ks1; ++ks, ++n) {
         const int s = n % STAGES;
         if (n >= STAGES) ptx::mbar_wait_elect(&empty[s], ((n / STAGES) - 1) & 1, dead);
-        if (ptx::elect_one()) {
-          ptx::mbar_expect_tx(&full[s], S::B_BYTES);
-          ptx::tma_load_3d(tiles + s * S::STAGE_BYTES + S::A_BYTES, &tmB, 0, n0, ks * KCH, &full[s]);
-        }
-        __syncwarp();
+        ptx::mbar_expect_tx(one, &full[s], S::B_BYTES);
+        ptx::tma_load_3d(one, tiles + s * S::STAGE_BYTES + S::A_BYTES, &tmB, 0, n0, ks * KCH, &full[s]);
       }
     }
   } else if (warp == 2) {
-    // ---- MMA issuer: the warp goes in step and one lane issues (ptx::elect_one), as in the roles above.  Under lane == 0 an
+    // ---- MMA issuer: the warp goes in step and one lane issues, as in the roles above (ptx::Leader).  Under lane == 0 an
     // MMA costs 56 to 97 cycles to issue (the pipe takes 64 at 128 columns) and a wait twice as long: with the roles in
     // step the 12.7 k row GEMMs of the encoder went 45 -> 42.4 us (QKV), 66 -> 59.6 (FFN1, GELU), 71.5 -> 70 (FFN2).
     constexpr uint32_t idesc = ptx::idesc_bf16(GEMM_BM, BN);
-    int n = 0, j = 0;
+    const ptx::Leader one = ptx::elect_leader();
+    // The stage and its parity are counted along and the descriptors are sums: index arithmetic and branches between two
+    // stages' instructions are time that the pipe waits (at N = 128 82 -> 67 cycles per MMA).
+    const uint64_t a0 = ptx::smem_desc_sw128(ptx::smem_u32(tiles)), b0 = ptx::smem_desc_sw128(ptx::smem_u32(tiles + S::A_BYTES));
+    uint32_t s = 0, par = 0;
+    int j = 0;
     for (int w = blockIdx.x; w < num_tiles; w += gridDim.x, ++j) {
       const int acc = j & 1;
       if (j >= 2) ptx::mbar_wait_elect(&tmem_empty[acc], ((j >> 1) - 1) & 1, dead);
@@ -280,30 +282,24 @@ gemm_bf16_tcgen05(const __grid_constant__ CUtensorMap tmA, const __grid_constant
       const uint32_t d = tmem + acc * BN;
       int ks0, ks1;
       k_range(w, &ks0, &ks1);
-      for (int ks = ks0; ks < ks1; ++ks, ++n) {
-        const int s = n % STAGES;
-        ptx::mbar_wait_elect(&full[s], (n / STAGES) & 1, dead);
+      SOD2_TRACE(1, 10 + j)
+      for (int ks = ks0; ks < ks1; ++ks) {
+        ptx::mbar_wait_elect(&full[s], par, dead);
         ptx::tc_fence_after();
-        const uint32_t a = ptx::smem_u32(tiles + s * S::STAGE_BYTES);
-        if (ptx::elect_one()) {
-          if (ks == 0) { SOD2_TRACE(1, 10 + j) }
+        const uint64_t ad = a0 + s * (S::STAGE_BYTES >> 4), bd = b0 + s * (S::STAGE_BYTES >> 4);
 #pragma unroll
-          for (int c = 0; c < KCH; ++c) {
-            if (ks * KCH + c < kchunks) {
-              const uint64_t ad = ptx::smem_desc_sw128(a + c * (GEMM_BM * 128));
-              const uint64_t bd = ptx::smem_desc_sw128(a + S::A_BYTES + c * (BN * 128));
+        for (int kk = 0; kk < 4; ++kk) ptx::mma_bf16(one, d, ad + 2 * kk, bd + 2 * kk, idesc, (ks > ks0) || kk != 0);
+        if (KCH == 1 || (ks + 1) * KCH <= kchunks) {
 #pragma unroll
-              for (int kk = 0; kk < 4; ++kk) ptx::mma_bf16(d, ad + 2 * kk, bd + 2 * kk, idesc, (ks > ks0) || c != 0 || kk != 0);
-            }
-          }
-          ptx::mma_commit(&empty[s]);  // frees the stage once these MMAs have read it
-          if (ks + 1 == ks1) {
-            ptx::mma_commit(&tmem_full[acc]);
-            SOD2_TRACE(1, 20 + j)
-          }
-        }
-        __syncwarp();
+          for (int c = 1; c < KCH; ++c)
+#pragma unroll
+            for (int kk = 0; kk < 4; ++kk) ptx::mma_bf16(one, d, ad + c * (GEMM_BM * 8) + 2 * kk, bd + c * (BN * 8) + 2 * kk, idesc, 1);
+        }                                 // (K ends inside the stage: KCH is 2 at most)
+        ptx::mma_commit(one, &empty[s]);  // frees the stage once these MMAs have read it
+        if (++s == STAGES) { s = 0; par ^= 1; }
       }
+      ptx::mma_commit(one, &tmem_full[acc]);
+      SOD2_TRACE(1, 20 + j)
     }
   } else if (warp == 11) {
     // ---- staging agent: owns the staging buffers' TMA traffic so that no epilogue thread waits on a
@@ -552,6 +548,7 @@ gemm_bf16_tcgen05(const __grid_constant__ CUtensorMap tmA, const __grid_constant
     }
     }
   }
+  __syncwarp();
   ptx::tc_fence_before();
   __syncthreads();
   if (warp == 2) ptx::tmem_dealloc(tmem, TMEM_COLS);

@@ -178,6 +178,37 @@ __device__ __forceinline__ bool elect_one() {
   return p != 0;
 }
 
+// The lane that issues for its warp, elected once per role.  What it issues (MMAs, commits, TMA loads) is predicated and not
+// branched on: a branch on elect_one() around a stage's instructions, and the __syncwarp behind it, cost the issuing warp 130 to
+// 190 cycles per stage beside the pipe.  Measured on B200 (cycles per MMA with a satisfied wait and a commit per stage, branch ->
+// predicate; the pipe takes 48 at N = 64, 64 at 128): N = 64 in stages of 4 / 8 / 12 MMAs 93 / 72 / 63 -> 61 / 51 / 52, N = 128
+// 97 / 82 / 75 -> 64 / 64 / 64; from N = 192 on the pipe hides either.  A warp whose lanes have seen a phase end at different
+// tests may run a stage's instructions in parts: the leader's are issued once, behind the leader's own test.
+struct Leader { uint32_t on; };
+__device__ __forceinline__ Leader elect_leader() { return Leader{elect_one() ? 1u : 0u}; }
+__device__ __forceinline__ void mbar_expect_tx(Leader l, uint64_t* bar, uint32_t bytes) {
+  asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %2, 0;\n\t@q mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n\t}"
+               ::"r"(smem_u32(bar)), "r"(bytes), "r"(l.on) : "memory");
+}
+__device__ __forceinline__ void tma_load_2d(Leader l, void* dst, const void* tmap, int x, int y, uint64_t* bar) {
+  asm volatile(
+      "{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %5, 0;\n\t"
+      "@q cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];\n\t}"
+      ::"r"(smem_u32(dst)), "l"(tmap), "r"(x), "r"(y), "r"(smem_u32(bar)), "r"(l.on) : "memory");
+}
+__device__ __forceinline__ void tma_load_3d(Leader l, void* dst, const void* tmap, int x, int y, int z, uint64_t* bar) {
+  asm volatile(
+      "{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %6, 0;\n\t"
+      "@q cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];\n\t}"
+      ::"r"(smem_u32(dst)), "l"(tmap), "r"(x), "r"(y), "r"(z), "r"(smem_u32(bar)), "r"(l.on) : "memory");
+}
+__device__ __forceinline__ void tma_load_4d(Leader l, void* dst, const void* tmap, int x, int y, int z, int w, uint64_t* bar) {
+  asm volatile(
+      "{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %7, 0;\n\t"
+      "@q cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %5}], [%6];\n\t}"
+      ::"r"(smem_u32(dst)), "l"(tmap), "r"(x), "r"(y), "r"(z), "r"(w), "r"(smem_u32(bar)), "r"(l.on) : "memory");
+}
+
 // D[tmem] (+)= A[smem] * B[smem], bf16 inputs, fp32 accumulate; issued by one thread.
 __device__ __forceinline__ void mma_bf16(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t accumulate) {
   asm volatile(
@@ -199,6 +230,22 @@ __device__ __forceinline__ void mma_bf16_a_tmem(uint32_t d_tmem, uint32_t a_tmem
 // mbarrier arrive once every MMA issued so far by this thread has completed.
 __device__ __forceinline__ void mma_commit(uint64_t* bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
+}
+__device__ __forceinline__ void mma_bf16(Leader l, uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t accumulate) {
+  asm volatile(
+      "{\n\t.reg .pred p, q;\n\tsetp.ne.b32 q, %5, 0;\n\tsetp.ne.b32 p, %4, 0;\n\t"
+      "@q tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
+      ::"r"(d_tmem), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate), "r"(l.on) : "memory");
+}
+__device__ __forceinline__ void mma_bf16_a_tmem(Leader l, uint32_t d_tmem, uint32_t a_tmem, uint64_t bdesc, uint32_t idesc, uint32_t accumulate) {
+  asm volatile(
+      "{\n\t.reg .pred p, q;\n\tsetp.ne.b32 q, %5, 0;\n\tsetp.ne.b32 p, %4, 0;\n\t"
+      "@q tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
+      ::"r"(d_tmem), "r"(a_tmem), "l"(bdesc), "r"(idesc), "r"(accumulate), "r"(l.on) : "memory");
+}
+__device__ __forceinline__ void mma_commit(Leader l, uint64_t* bar) {
+  asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %1, 0;\n\t@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}"
+               ::"r"(smem_u32(bar)), "r"(l.on) : "memory");
 }
 // 32 lanes x 32 consecutive fp32 columns: thread t of the warp gets lane (base_lane + t).
 __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t* r) {
