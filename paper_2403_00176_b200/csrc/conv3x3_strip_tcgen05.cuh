@@ -41,27 +41,28 @@ constexpr int STRIP_SMEM = STRIP_W + STRIP_STAGES * C3_A_SLOT + STRIP_NSB * CONV
 
 // One MMA whose descriptors differ from the others' only in their start addresses (low words, in units of 16 bytes).
 template <int BLOCKS>
-__device__ __forceinline__ void strip_mma(uint32_t d, uint32_t a_lo, uint32_t b_lo) {
+__device__ __forceinline__ void strip_mma(ptx::Leader one, uint32_t d, uint32_t a_lo, uint32_t b_lo) {
   constexpr uint32_t desc_hi = (1024u >> 4) | 1u << 14 | 2u << 29;      // ptx::smem_desc_sw128: row-group stride, version, 128-byte swizzle
   asm volatile(
-      "{\n\t.reg .b64 ad, bd;\n\t"
+      "{\n\t.reg .pred q;\n\t.reg .b64 ad, bd;\n\t"
+      "setp.ne.b32 q, %5, 0;\n\t"
       "mov.b64 ad, {%1, %4};\n\t"
       "mov.b64 bd, {%2, %4};\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], ad, bd, %3, 1;\n\t}"
-      ::"r"(d), "r"(a_lo), "r"(b_lo), "n"(ptx::idesc_bf16(128, 64 * BLOCKS)), "n"(desc_hi)
+      "@q tcgen05.mma.cta_group::1.kind::f16 [%0], ad, bd, %3, 1;\n\t}"
+      ::"r"(d), "r"(a_lo), "r"(b_lo), "n"(ptx::idesc_bf16(128, 64 * BLOCKS)), "n"(desc_hi), "r"(one.on)
       : "memory");
 }
 // One input row: three dx taps of 64 input channels onto C1 accumulator blocks from d1 and C2 behind the ring's end.
 // Everything but the start addresses is a constant: the issuing thread has one MMA's time (96 cycles) for all its
 // arithmetic, beside epilogue warps on its scheduler.
 template <int C1, int C2>
-__device__ __forceinline__ void strip_row(uint32_t d1, uint32_t d2, uint32_t a_lo, uint32_t b_lo) {
+__device__ __forceinline__ void strip_row(ptx::Leader one, uint32_t d1, uint32_t d2, uint32_t a_lo, uint32_t b_lo) {
   constexpr uint32_t TAP = STRIP_TAP >> 4;
 #pragma unroll
   for (int q = 0; q < 12; ++q) {
     const uint32_t a = a_lo + (q >> 2) * 8 + 2 * (q & 3), b = b_lo + (q >> 2) * (3 * TAP) + 2 * (q & 3);
-    strip_mma<C1>(d1, a, b);
-    if constexpr (C2 > 0) strip_mma<C2>(d2, a, b + C1 * TAP);
+    strip_mma<C1>(one, d1, a, b);
+    if constexpr (C2 > 0) strip_mma<C2>(one, d2, a, b + C1 * TAP);
   }
 }
 
@@ -123,10 +124,11 @@ conv3x3_strip_bf16_tcgen05(const __grid_constant__ Conv3Batch B, const __grid_co
   ptx::tc_fence_after();
   const uint32_t tmem = *tmem_slot;
   // the weights do not depend on the previous kernel; tap (dy, dx) goes to slot dx * 3 + 2 - dy
-  if (warp == 0 && lane == 0) {
-    ptx::mbar_expect_tx(w_full, STRIP_W);
+  if (warp == 0) {
+    const ptx::Leader one = ptx::elect_leader();
+    ptx::mbar_expect_tx(one, w_full, STRIP_W);
     for (int dx = 0; dx < 3; ++dx)
-      for (int dy = 2; dy >= 0; --dy) ptx::tma_load_3d(wres + (dx * 3 + 2 - dy) * STRIP_TAP, &tmW, 0, 0, dy * 3 + dx, w_full);
+      for (int dy = 2; dy >= 0; --dy) ptx::tma_load_3d(one, wres + (dx * 3 + 2 - dy) * STRIP_TAP, &tmW, 0, 0, dy * 3 + dx, w_full);
   }
   // the accumulator ring starts from zero: each epilogue warp clears its share of its group's blocks
   if (warp >= 4)
@@ -158,6 +160,7 @@ conv3x3_strip_bf16_tcgen05(const __grid_constant__ Conv3Batch B, const __grid_co
   if (warp == 0) {
     {
       // ---- input rows: a segment's L output rows need the L + 2 rows around them
+      const ptx::Leader one = ptx::elect_leader();
       int n = 0;
       for (int t = begin; t < end;) {
         int img, row, w0;
@@ -167,11 +170,8 @@ conv3x3_strip_bf16_tcgen05(const __grid_constant__ Conv3Batch B, const __grid_co
         for (int i = row - 1; i <= row + len; ++i, ++n) {
           const int s = n % ST;
           if (n >= ST) ptx::mbar_wait_elect(&empty[s], ((n / ST) - 1) & 1, dead);
-          if (ptx::elect_one()) {
-            ptx::mbar_expect_tx(&full[s], C3_A_BYTES);
-            ptx::tma_load_4d(rows + s * C3_A_SLOT, &B.tx[rq], 0, w0 - 1, i, img, &full[s]);
-          }
-          __syncwarp();
+          ptx::mbar_expect_tx(one, &full[s], C3_A_BYTES);
+          ptx::tma_load_4d(one, rows + s * C3_A_SLOT, &B.tx[rq], 0, w0 - 1, i, img, &full[s]);
         }
         t += len;
       }
@@ -187,6 +187,8 @@ conv3x3_strip_bf16_tcgen05(const __grid_constant__ Conv3Batch B, const __grid_co
       // gives to the output rows ii - 2 (dy = 2), ii - 1 and ii, as far as they belong to the segment.
       ptx::mbar_wait_elect(w_full, 0, dead);
       const uint64_t wdesc = ptx::smem_desc_sw128(ptx::smem_u32(wres));
+      const ptx::Leader one = ptx::elect_leader();
+      const auto mma_commit = [&](uint64_t* bar) { ptx::mma_commit(one, bar); };
       const int me = warp == 1 ? 0 : 1;
       int n = 0, j = 0;
       for (int t = begin; t < end;) {
@@ -204,24 +206,23 @@ conv3x3_strip_bf16_tcgen05(const __grid_constant__ Conv3Batch B, const __grid_co
           const uint32_t d1 = tmem + b0 * 64;
           if (fresh) ptx::mbar_wait_elect(&tmem_empty[(j + ii) % NB], ((j + ii) / NB) & 1, dead);
           ptx::mbar_wait_elect(&full[s], (n / ST) & 1, dead);
-          if (n > 0) ptx::mbar_wait_elect(&turn[me], me ? (n >> 1) & 1 : ((n >> 1) - 1) & 1, dead);
-          ptx::tc_fence_after();
           const uint64_t ad = ptx::smem_desc_sw128(ptx::smem_u32(rows + s * C3_A_SLOT));
           const uint32_t a_lo = static_cast<uint32_t>(ad), b_lo = static_cast<uint32_t>(wb);
-          if (ptx::elect_one()) {
+          uint64_t* const done = &tmem_full[(j + ii + NB - 2) % NB];
+          if (n > 0) ptx::mbar_wait_elect(&turn[me], me ? (n >> 1) & 1 : ((n >> 1) - 1) & 1, dead);
+          ptx::tc_fence_after();
+          if (c1 == 3) strip_row<3, 0>(one, d1, tmem, a_lo, b_lo);
+          else
             switch (c1 * 4 + c2) {
-              case 12: strip_row<3, 0>(d1, tmem, a_lo, b_lo); break;
-              case 9: strip_row<2, 1>(d1, tmem, a_lo, b_lo); break;
-              case 6: strip_row<1, 2>(d1, tmem, a_lo, b_lo); break;
-              case 8: strip_row<2, 0>(d1, tmem, a_lo, b_lo); break;
-              case 5: strip_row<1, 1>(d1, tmem, a_lo, b_lo); break;
-              case 4: strip_row<1, 0>(d1, tmem, a_lo, b_lo); break;
+              case 9: strip_row<2, 1>(one, d1, tmem, a_lo, b_lo); break;
+              case 6: strip_row<1, 2>(one, d1, tmem, a_lo, b_lo); break;
+              case 8: strip_row<2, 0>(one, d1, tmem, a_lo, b_lo); break;
+              case 5: strip_row<1, 1>(one, d1, tmem, a_lo, b_lo); break;
+              case 4: strip_row<1, 0>(one, d1, tmem, a_lo, b_lo); break;
             }
-            ptx::mma_commit(&turn[me ^ 1]);
-            ptx::mma_commit(&empty[s]);
-            if (ii >= 2) ptx::mma_commit(&tmem_full[(j + ii - 2) % NB]);
-          }
-          __syncwarp();
+          mma_commit(&turn[me ^ 1]);
+          mma_commit(&empty[s]);
+          if (ii >= 2) mma_commit(done);
         }
         j += len;
         t += len;
