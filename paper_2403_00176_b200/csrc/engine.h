@@ -330,6 +330,9 @@ struct Plan {
   struct Chain { std::vector<int> groups; int rows = 0; size_t counter_word = 0; };
   std::vector<Chain> chains;
   std::vector<int> chain_of;              // [group] index into chains, -1 = a launch of its own
+  // [group] 1: a top-k keep whose launch also runs the LayerNorm group behind it.  Decided with the chains, for the same
+  // reason: what the launch reads stays live until the normalised rows are written, and they are live from its step on.
+  std::vector<char> takes_ln;
   size_t chain_counter_off = 0;           // byte offset in the arena header of the chains' row-block counters
   size_t chain_counter_words = 0;
   size_t header_clear_bytes = 256;        // what a run zeroes at the start of the arena (status word, tickets, chain counters)
@@ -389,7 +392,7 @@ void note_run(Plan* p, void* stream);
 // The run-time symbols among `vals` <- their counts for request r in the arena header (synchronises `stream`).
 Status read_counts(Plan* p, const void* arena, void* stream, int r, std::vector<int64_t>* vals);
 Status build_launches(Plan* p);   // exec.cu
-Status detect_chains(Plan* p);    // exec.cu: fills Plan::chains / chain_of from the resolved views
+Status detect_chains(Plan* p);    // exec.cu: fills Plan::chains / chain_of / takes_ln from the resolved views
 // step_lo..step_hi: only these groups (positions in execution order) are enqueued (all by default); the arena header
 // is cleared only by a run that starts at group 0.
 Status run_plan(Plan* p, const void* const* inputs, void* const* outputs, void* arena, size_t arena_bytes, void* stream,

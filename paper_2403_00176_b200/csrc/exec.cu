@@ -1315,14 +1315,36 @@ struct Builder : BuildState {
     return OK;
   }
 
-  // ------------------------------------------------------------------------------ top-k keep
-  Status build_topk(int gi, const Group& G) {
+  // ------------------------------------------------------------------------------ top-k keep (+ LayerNorm)
+  // Selections whose kept rows the next group normalises: rows of at most 512 columns (a warp holds four of them), packed alike in
+  // both outputs.
+  void find_topk_ln() {
+    const size_t n = c.groups.size();
+    p.takes_ln.assign(n, 0);
+    if (c.flags & OPT_NO_FUSION) return;
+    for (size_t gi = 0; gi + 1 < n; ++gi) {
+      const Group &G = c.groups[gi], &L = c.groups[gi + 1];
+      if (G.kind != GKind::TOPK_KEEP || L.kind != GKind::LAYERNORM || L.a != G.out) continue;
+      if (g.tensors[G.a].dtype != DType::BF16 || g.tensors[L.out].dtype != DType::BF16 || g.tensors[L.gamma].kind != TKind::CONST || g.tensors[L.beta].kind != TKind::CONST) continue;
+      bool ok = p.root_of[L.out] != p.root_of[G.out] && p.root_of[L.out] != p.root_of[G.a] && p.root_of[L.out] != p.root_of[G.out2];
+      const Ptr bo = ptr_of(G.out, 0), bl = ptr_of(L.out, 0);
+      for (int r = 0; r < p.n_req && ok; ++r) {
+        const View &o = p.views[G.out][r], &l = p.views[L.out][r];
+        const Ptr po = ptr_of(G.out, r), pl = ptr_of(L.out, r);
+        ok = !o.dims.empty() && o.contiguous() && l.contiguous() && o.dims.back() == l.dims.back() && o.dims.back() <= 512 && o.dims.back() % 8 == 0 &&
+             numel(o.dims) == numel(l.dims) && same_base(po, bo) && same_base(pl, bl) && po.off - bo.off == pl.off - bl.off;
+      }
+      p.takes_ln[gi] = ok;
+    }
+  }
+  Status build_topk(int gi, const Group& G, const Group* L = nullptr) {
     if (g.tensors[G.a].dtype != DType::BF16) return fail(E_UNSUPPORTED_OP, "top-k keep is bf16 only");
     for (int r0 = 0; r0 < p.n_req; r0 += k::COMPACT_MAX_REQ) {
       const int nr = std::min(k::COMPACT_MAX_REQ, p.n_req - r0);
       k::TopkParams tp{};
       tp.n_req = nr;
       Ptr by = ptr_of(G.a, r0), bo = ptr_of(G.out, r0), bi = ptr_of(G.out2, r0);
+      const Ptr bl = L ? ptr_of(L->out, r0) : Ptr(), pg = L ? ptr_of(L->gamma, 0) : Ptr(), pb = L ? ptr_of(L->beta, 0) : Ptr();
       int64_t D = -1, total_rows = 0, first_row = 0;
       int nmax = 0;
       for (int i = 0; i < nr; ++i) {
@@ -1351,6 +1373,8 @@ struct Builder : BuildState {
       const size_t sc_bytes = (static_cast<size_t>(total_rows) * 8 + 15) & ~size_t(15);
       scratch_need = std::max(scratch_need, sc_bytes);
       const long long rows = total_rows;
+      const int ln = !L ? 0 : D <= 256 ? 1 : 2;
+      if (L) tp.eps = L->eps;
       const size_t smem = static_cast<size_t>(nmax) * 8;
       if (smem > 200 * 1024) return fail(E_UNSUPPORTED_OP, "top-k keep: too many tokens per request for the shared-memory score table");
       add(gi, 2, [=](const RunCtx& x) mutable {
@@ -1363,11 +1387,18 @@ struct Builder : BuildState {
         k::ScoreParams sp{tp.y + first_row * tp.D, score, rows, tp.D};
         if (rows) launch_pdl(k::row_sumsq_f64, dim3(static_cast<unsigned>((rows + 7) / 8)), dim3(256), 0, x.stream, sp);
         if (chunks) {
-          if (smem > 40 * 1024) cudaFuncSetAttribute(k::topk_select_gather, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-          launch_pdl(k::topk_select_gather, dim3(chunks), dim3(k::TOPK_THREADS), smem, x.stream, tp);
+          auto kern = ln == 2 ? k::topk_select_gather<2> : ln == 1 ? k::topk_select_gather<1> : k::topk_select_gather<0>;
+          if (ln) {
+            tp.normed = reinterpret_cast<__nv_bfloat16*>(x.resolve(bl));
+            tp.gamma = reinterpret_cast<const __nv_bfloat16*>(x.resolve(pg));
+            tp.beta = reinterpret_cast<const __nv_bfloat16*>(x.resolve(pb));
+          }
+          if (smem > 40 * 1024) cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+          launch_pdl(kern, dim3(chunks), dim3(k::TOPK_THREADS), smem, x.stream, tp);
         }
         return cudaGetLastError();
       });
+      if (L) p.launches.back()->share = {{gi, 0.8}, {gi + 1, 0.2}};     // about the bytes of the two
     }
     return OK;
   }
@@ -2293,6 +2324,13 @@ struct Builder : BuildState {
         if (!p.stage_of) cost(G);
         continue;
       }
+      if (p.takes_ln[gi] && gi + 1 < end_group) {
+        s = build_topk(static_cast<int>(gi), G, &c.groups[gi + 1]);
+        if (s != OK) return s;
+        if (!p.stage_of) { cost(G); cost(c.groups[gi + 1]); }
+        ++gi;
+        continue;
+      }
       switch (G.kind) {
         case GKind::GEMM: s = build_gemm(static_cast<int>(gi), G); break;
         case GKind::ATTENTION: s = build_attention(static_cast<int>(gi), G); break;
@@ -2397,6 +2435,7 @@ Status build_launches(Plan* p) {
 
 Status detect_chains(Plan* p) {
   Builder b(*p);
+  b.find_topk_ln();
   return b.find_chains();
 }
 

@@ -62,6 +62,10 @@ __global__ void __launch_bounds__(256) row_sumsq_f64(ScoreParams p) {
 // Bound by latency: the wait for the scores, about 200 cycles per pass, the rows out.  With the score kernel, against a
 // kernel that ranked every token with all others in fp64 and one that copied (D = 384): 16 requests of 238 to 780 tokens
 // 28.4 -> 9.1 us, one of 577 tokens 9.7 -> 6.2 us.
+// LN > 0: the kept rows also leave normalised (the LayerNorm group behind the selection; D <= 256 * LN).  A warp then holds four
+// rows of the chunk and has their statistics before it waits for the scores, so that the LayerNorm costs its stores and no
+// launch.  The arithmetic is layernorm_bf16's, lane by lane: the same bits.  (One request of 577 tokens through 12 layers 367 -> 359 us,
+// 16 requests 541 -> 530 us.)
 constexpr int TOPK_CHUNK = 32, TOPK_THREADS = 256;
 struct TopkReq {
   long long row0;      // first packed input row of the request
@@ -79,6 +83,10 @@ struct TopkParams {
   long long first_row;       // row0 of the first request (scores are indexed from it)
   int chunk_start[COMPACT_MAX_REQ + 1];   // prefix sum of ceil(n / TOPK_CHUNK)
   TopkReq r[COMPACT_MAX_REQ];
+  // LN > 0: constants of the graph, and the normalised rows, packed like `out`
+  const __nv_bfloat16 *gamma, *beta;
+  __nv_bfloat16* normed;
+  float eps;
 };
 
 __device__ __forceinline__ int topk_locate(const TopkParams& p, int cta, int* chunk) {
@@ -88,6 +96,7 @@ __device__ __forceinline__ int topk_locate(const TopkParams& p, int cta, int* ch
   return ri;
 }
 
+template <int LN>
 __global__ void __launch_bounds__(TOPK_THREADS) topk_select_gather(const __grid_constant__ TopkParams p) {
   extern __shared__ unsigned long long s_key[];        // [n]
   __shared__ unsigned s_hist[256];
@@ -103,15 +112,59 @@ __global__ void __launch_bounds__(TOPK_THREADS) topk_select_gather(const __grid_
   const int vec = (p.D * 2) >> 4;  // 16-byte pieces per row (D % 8 == 0 checked on the host)
   const uint4* src = reinterpret_cast<const uint4*>(p.y + (R.row0 + base) * p.D);
   const int items = min(TOPK_CHUNK, R.n - base) * vec;
-  constexpr int PRE = 6;
-  uint4 pre[PRE];
+  constexpr int PRE = LN ? 4 * LN : 6;
+  uint4 pre[PRE];                // LN: row warp + 8 u of the chunk, vectors lane + 32 c, in pre[u * LN + c]
+  [[maybe_unused]] uint4 g4[LN ? LN : 1], b4[LN ? LN : 1];
+  [[maybe_unused]] float mu[4], rstd[4];
+  if constexpr (LN > 0) {
 #pragma unroll
-  for (int u = 0; u < PRE; ++u) {
-    const int it = tid + u * TOPK_THREADS;
-    if (it < items) pre[u] = src[it];
+    for (int u = 0; u < 4; ++u)
+#pragma unroll
+      for (int c = 0; c < LN; ++c) pre[u * LN + c] = src[min(warp + 8 * u, items / vec - 1) * vec + min(c * 32 + lane, vec - 1)];
+#pragma unroll
+    for (int c = 0; c < LN; ++c) {
+      g4[c] = reinterpret_cast<const uint4*>(p.gamma)[min(c * 32 + lane, vec - 1)];
+      b4[c] = reinterpret_cast<const uint4*>(p.beta)[min(c * 32 + lane, vec - 1)];
+    }
+  } else {
+#pragma unroll
+    for (int u = 0; u < PRE; ++u) {
+      const int it = tid + u * TOPK_THREADS;
+      if (it < items) pre[u] = src[it];
+    }
   }
   s_hist[tid] = 0;
   if (tid < 2) { s_diff[tid] = 0; s_before[tid] = 0; }
+  if constexpr (LN > 0) {
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      float s = 0.f, q = 0.f;
+#pragma unroll
+      for (int c = 0; c < LN; ++c) {
+        const bool in = c * 32 + lane < vec;
+        const __nv_bfloat162* h = reinterpret_cast<const __nv_bfloat162*>(&pre[u * LN + c]);
+#pragma unroll
+        for (int t = 0; t < 4; ++t) { const float2 f = __bfloat1622float2(h[t]); s += in ? f.x + f.y : 0.f; }
+      }
+#pragma unroll
+      for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+      mu[u] = s / p.D;
+#pragma unroll
+      for (int c = 0; c < LN; ++c)
+        if (c * 32 + lane < vec) {
+          const __nv_bfloat162* h = reinterpret_cast<const __nv_bfloat162*>(&pre[u * LN + c]);
+#pragma unroll
+          for (int t = 0; t < 4; ++t) {
+            const float2 f = __bfloat1622float2(h[t]);
+            float d = f.x - mu[u]; q += d * d;
+            d = f.y - mu[u]; q += d * d;
+          }
+        }
+#pragma unroll
+      for (int o = 16; o; o >>= 1) q += __shfl_xor_sync(0xffffffffu, q, o);
+      rstd[u] = rsqrtf(q / p.D + p.eps);
+    }
+  }
   ptx::pdl_wait();
   ptx::pdl_launch();
   // Scores are sums of squares: as integers with the top bit set they keep their order.  A NaN score (an overflow
@@ -193,6 +246,30 @@ __global__ void __launch_bounds__(TOPK_THREADS) topk_select_gather(const __grid_
   // write the kept rows: (row, 16-byte piece) items spread over the whole CTA; the first PRE per thread are
   // already in registers, wider rows load the rest now
   uint4* dst = reinterpret_cast<uint4*>(p.out + R.out_row0 * p.D);
+  if constexpr (LN > 0) {
+    uint4* nrm = reinterpret_cast<uint4*>(p.normed + R.out_row0 * p.D);
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int pos = s_pos[warp + 8 * u];
+      if (pos < 0) continue;
+#pragma unroll
+      for (int c = 0; c < LN; ++c)
+        if (c * 32 + lane < vec) {
+          const uint4 x = pre[u * LN + c];
+          uint4 y;
+          const __nv_bfloat162 *h = reinterpret_cast<const __nv_bfloat162*>(&x), *gh = reinterpret_cast<const __nv_bfloat162*>(&g4[c]), *bh = reinterpret_cast<const __nv_bfloat162*>(&b4[c]);
+          __nv_bfloat162* oh = reinterpret_cast<__nv_bfloat162*>(&y);
+#pragma unroll
+          for (int t = 0; t < 4; ++t) {
+            const float2 f = __bfloat1622float2(h[t]), gf = __bfloat1622float2(gh[t]), bf = __bfloat1622float2(bh[t]);
+            oh[t] = __floats2bfloat162_rn((f.x - mu[u]) * rstd[u] * gf.x + bf.x, (f.y - mu[u]) * rstd[u] * gf.y + bf.y);
+          }
+          dst[static_cast<long long>(pos) * vec + c * 32 + lane] = x;
+          nrm[static_cast<long long>(pos) * vec + c * 32 + lane] = y;
+        }
+    }
+    return;
+  }
 #pragma unroll
   for (int u = 0; u < PRE; ++u) {
     const int it = tid + u * TOPK_THREADS;

@@ -437,6 +437,8 @@ struct Planner {
         lo = ch.groups.front();
         hi = ch.groups.back();
       }
+      if (p.takes_ln[s]) hi = s + 1;
+      if (s > 0 && p.takes_ln[s - 1]) lo = s - 1;
       auto touch = [&](int t, bool def) {
         if (c.storage[t].kind == Storage::FOLDED || !resolved[t]) return;
         int root = p.root_of[t];
@@ -476,6 +478,7 @@ struct Planner {
     }
     p.chain_of = B.chain_of;
     p.chains = B.chains;
+    p.takes_ln = B.takes_ln;
     p.chain_counter_words = B.chain_counter_words;
     return plan_arena(static_cast<int>(c.groups.size()));
   }

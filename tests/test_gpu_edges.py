@@ -8,6 +8,7 @@ from paper_2403_00176_b200 import binding as B
 from paper_2403_00176_b200 import workloads as WL
 from paper_2403_00176_b200.workloads import Request, bf16_round
 from tests.gpu_harness import lockstep, run_batch
+from tests.test_gpu_parity import _check_topk_lockstep
 
 pytestmark = pytest.mark.gpu
 
@@ -115,6 +116,19 @@ def test_attention_blocks_items_and_tables(lens):
     p.run()
     for a, b in zip(outs, p.outputs()):
         assert np.array_equal(a["y"], b["y"])
+
+
+@pytest.mark.parametrize("D,H", [(64, 1), (256, 4), (320, 5), (512, 8), (576, 9)])
+def test_topk_keep_with_the_layernorm_behind_it(D, H):
+    # the kept rows of the first layer leave normalised for the second, in the launch that selects them: rows of one and two
+    # vectors a lane, whole and ragged, and rows too wide for that (576); chunks of 32 tokens at their edges, a request of one
+    # token, one of more tokens than a CTA has threads
+    lens = [1, 2, 31, 32, 33, 64, 65, 300]
+    wl = WL.cfg3(layers=2, D=D, H=H, F=2 * D)
+    rng = np.random.default_rng(67)
+    name, sym = wl.ir.split("input ")[1].split()[0], wl.sym_names[0]
+    reqs = [Request({sym: n}, {name: bf16_round((rng.standard_normal((1, n, D)) * rng.uniform(0.5, 2.0, (1, n, 1)) + rng.standard_normal((1, n, 1))).astype(np.float32))}) for n in lens]
+    _check_topk_lockstep(wl, reqs, 2)
 
 
 @pytest.mark.parametrize("K,N,M,act,residual", [(768, 768, 7169, None, True), (768, 2312, 4224, "Gelu", False), (3072, 768, 4100, "Relu", True), (3072, 776, 11009, None, False), (768, 392, 12700, None, True)])
