@@ -434,7 +434,23 @@ struct Builder : BuildState {
         const double tma = kch * (128 + bn_) * 128.0 / 70.0;   // empirical: stage cost grows with the operand bytes of a stage (measured 585 / 840 cycles)
         return waves * stages * std::max(std::max(mma, floor_cycles), tma);
       };
-      int bn = (N > 128 && makespan(256, 1) <= makespan(128, 2)) ? 256 : 128;
+      // With a GELU epilogue, a residual and fewer than 24 chunks, or a K of at most 8 chunks, the epilogue of a tile (e_ns) takes about as long as its main
+      // loop and bounds the waves behind the first (a longer K is bound by operand bytes, as above); there the two versions are compared by a launch's measured times instead:
+      // start and end + the first wave's main loop + for each further wave the longer of main loop and epilogue.  From a sweep of
+      // 500 to 12700 rows at eight K x N (128 against 256 columns, us): 1800 x 3072 x 768 with GELU 11.7 and 12.8 (14 to 15 in
+      // pairs), 2900 14.8 and 13.3; 4500 x 1152 x 384 8.0 and 9.0, 12700 x 1536 x 384 with GELU 24.1 and 22.5; 3600 x 768 x 768 with a
+      // residual 8.7 and 9.5.
+      const bool gelu = G.act == 1;
+      const double chunks64 = K / 64.0;
+      auto launch_ns = [&](int bn_) {
+        const double waves = std::ceil(static_cast<double>(tiles_m) * ((N + bn_ - 1) / bn_) / sms);
+        const double start_ns = bn_ == 256 ? 5500 : 4000, first_ns = bn_ == 256 ? 290 : 185, chunk_ns = bn_ == 256 ? 365 : 215;
+        const double e_ns = bn_ == 256 ? 3500 : gelu ? 2300 : 1900;
+        return start_ns + chunks64 * first_ns + (waves - 1) * std::max(chunks64 * chunk_ns, e_ns);
+      };
+      const bool by_launch = gelu || (G.res >= 0 && chunks64 < 24) || chunks64 <= 8;
+      const int bn_mainloop = (N > 128 && makespan(256, 1) <= makespan(128, 2)) ? 256 : 128;
+      int bn = !by_launch ? bn_mainloop : (N > 128 && launch_ns(256) <= launch_ns(128)) ? 256 : 128;
       // Small problems: while 128x64 tiles still fit one wave, a CTA's time is pipeline fill + main loop +
       // epilogue of ONE tile, and both of the latter shrink with the tile (the epilogue is 0.6 us per 64 columns).
       if (bn == 128 && N > 64 && static_cast<int64_t>(tiles_m) * ((N + 63) / 64) <= sms) bn = 64;
@@ -478,9 +494,21 @@ struct Builder : BuildState {
         if (units_n >= 4) { offer(4, 1); offer(4, 2); }
         if (units_n >= 3) offer(3, 1);
         offer(2, 1);
-        const double single = std::ceil(static_cast<double>(tiles_m) * ((N + bn - 1) / bn) / sms) * kst * (bn == 256 ? 386.0 : 263.0) + unit_ns * (bn / 64);
+        // (the single-CTA kernel as its main loop alone would choose it, but for problems of one wave of 64 columns)
+        const int bs = bn == 64 && bn_mainloop == 128 ? 64 : bn_mainloop;
+        const double single = std::ceil(static_cast<double>(tiles_m) * ((N + bs - 1) / bs) / sms) * kst * (bs == 256 ? 386.0 : 263.0) + unit_ns * (bs / 64);
         static const bool force_pair = getenv("SOD2_GEMM_PAIR_FORCE") != nullptr;   // tests: the pair kernel wherever it is eligible
         pair = (c.flags & OPT_GEMM_PAIR) ? (best < single || force_pair) : (K >= 12 * 64 && best + 2000.0 < single);
+        if (pair && gelu && !(c.flags & OPT_GEMM_PAIR)) {
+          // GELU: the epilogue of a pair's wider tiles bounds its waves too, and its start is longer by it.  Same sweep, one tile per
+          // CTA against the best pairs: 1800 x 3072 x 768 11.7 and 13.8 us, 2300 rows 12.1 and 14.2, 12700 rows 49.2 and 49.4; where the
+          // two are within an eighth the pairs stay (fewer operand bytes where the board's power is what bounds)
+          const double e_ns[5] = {0, 0, 3200, 4200, 4900}, first_ns[5] = {0, 0, 200, 265, 320}, start_ns[5] = {0, 0, 6000, 6600, 7000};
+          const int bw = split.bw, last = (bw + split.parts - 1) / split.parts, tiles = tiles_m2 * ((units_n + bw - 1) / bw);
+          double t = start_ns[bw] + kst * first_ns[bw] + (std::ceil(static_cast<double>(split.n_full ? split.n_full : tiles) / pairs) - 1) * std::max(kst * chunk_ns[bw], e_ns[bw]);
+          if (split.n_full < tiles) t += std::max(kst * chunk_ns[last], e_ns[last]) + 700.0;
+          pair = t < 1.125 * std::min(launch_ns(128), launch_ns(256));
+        }
       }
       // Few tiles and a long K: S CTAs of a cluster share a tile's K (gemm_cluster_tcgen05.cuh), as many as the chip can hold
       // clusters for (measured on B200 with this kernel's shared memory: 15, 33 and 74 of 8, 4 and 2 CTAs; a second wave

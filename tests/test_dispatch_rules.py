@@ -32,3 +32,17 @@ def test_attention_forms():
     assert form([1, 64]) == "mma.sync"                     # the views of a single token have other strides
     assert form([64] * 64 + [1, 2]) == "mixed"             # a table of 64 requests and one of two
     assert form([64], B.Graph(WL.cfg2(layers=1).ir, B.OPT_LEGACY_ATTENTION)) == "mma.sync"
+
+
+@pytest.mark.parametrize("K,N,M,tail,form", [
+    # GELU: a launch's time, main loop or epilogue, whichever bounds a wave; pairs only where they are within an eighth
+    (768, 3072, 1000, "gelu", "tile 128"), (768, 3072, 1806, "gelu", "tile 128"), (768, 3072, 2900, "gelu", "tile 256"), (768, 3072, 12700, "gelu", "pair"),
+    (384, 1536, 3600, "gelu", "tile 128"), (384, 1536, 6000, "gelu", "tile 256"),
+    # a residual and fewer than 24 chunks; 24 and more by the main loop
+    (768, 768, 3600, "residual", "tile 128"), (1472, 768, 2400, "residual", "tile 128"), (1536, 768, 2400, "residual", "tile 128"), (768, 768, 7169, "residual", "pair"),
+    # up to 8 chunks whatever the tail
+    (512, 1152, 4500, "", "tile 128"), (576, 1152, 4500, "", "tile 256")])
+def test_gemm_forms_by_epilogue(K, N, M, tail, form):
+    ir = f"sym M 1 40000\ninput x bf16 [1,M,{K}]\n" + (f"input r bf16 [1,M,{N}]\n" if tail == "residual" else "") + f"const W bf16 [{K},{N}]\nnode MatMul x W -> y\n"
+    ir += {"gelu": "node Gelu y -> z\noutput z\n", "residual": "node Add y r -> z\noutput z\n", "": "output y\n"}[tail]
+    assert B.Graph(ir, 0).bind_dims(["M"], [[M]]).plan().group_form(0) == form
