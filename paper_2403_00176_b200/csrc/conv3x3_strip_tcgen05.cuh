@@ -80,7 +80,9 @@ __device__ __forceinline__ void strip_hand_over(uint32_t tmem, int blk, int q, i
 
 // B.tx: {64, W, H, N}, box {64, 130, 1, 1};  tmW: k-chunk view {64, 64, 9} of the weights in (dy, dx, ci) order, box
 // {64, 64, 1};  B.to / B.tr: {64, W, H, N}, box {64, 128, 1, 1}.  B.tile_start as for the row-halo kernel.
-template <int ACT, bool HASRES>
+// GAP: p.gap_sum receives the channel sums (the code for it costs the kernel registers: one image of 227 x 341 111.2 -> 113.0 us with
+// it everywhere).  The additions fit under the main loop: the gated network of 32 images pools three tensors of 51 MB less, 785 -> 757 us.
+template <int ACT, bool HASRES, bool GAP>
 __global__ void __launch_bounds__(STRIP_THREADS, 1)
 conv3x3_strip_bf16_tcgen05(const __grid_constant__ Conv3Batch B, const __grid_constant__ CUtensorMap tmW, ConvParams p) {
   constexpr int NSB = STRIP_NSB, NB = STRIP_BLOCKS, ST = STRIP_STAGES;
@@ -287,6 +289,9 @@ conv3x3_strip_bf16_tcgen05(const __grid_constant__ Conv3Batch B, const __grid_co
     const int et = threadIdx.x - 128 - g * 256;
     const int row = q * 32 + lane;
     const float relu2_floor = p.act2 == ACT_RELU ? 0.0f : -INFINITY;
+    // sums of the stored values of one image (p.gap_sum): kept by the threads while the CTA's tiles stay in it
+    [[maybe_unused]] double gap0 = 0.0, gap1 = 0.0;
+    [[maybe_unused]] int gap_img = -1;
     auto group_bar = [&]() { asm volatile("bar.sync %0, 256;" ::"r"(1 + g) : "memory"); };
     for (int j = g; j < end - begin; j += 2) {
       const int blk = j % NB, bsel = j % NSB;
@@ -325,17 +330,24 @@ conv3x3_strip_bf16_tcgen05(const __grid_constant__ Conv3Batch B, const __grid_co
       }
 #pragma unroll
       for (int u = 0; u < 4; ++u) *reinterpret_cast<uint4*>(obase + (((half * 4 + u) ^ (row & 7)) << 4)) = pk[u];
-      if (p.gap_sum) {
+      if constexpr (GAP) {
         group_bar();                               // every row of the tile is in the staging buffer
         int img, trow, w0;
         const int rq = decode(begin + j, &img, &trow, &w0);
-        const int img_o = p.out_ids ? p.out_ids[img] : img;
         const int wo = B.Wo[rq];
-        gap_accumulate_tile(out_stage + bsel * CONV_STAGE_OUT, et, p.gap_sum + static_cast<long long>(img_o) * 64, [&](int px) { return w0 + px < wo; });
+        if (img != gap_img) {
+          if (gap_img >= 0) gap_flush(gap0, gap1, et, p.gap_sum + static_cast<long long>(p.out_ids ? p.out_ids[gap_img] : gap_img) * 64);
+          gap_img = img;
+          gap0 = gap1 = 0.0;
+        }
+        gap_add_tile(out_stage + bsel * CONV_STAGE_OUT, et, &gap0, &gap1, [&](int px) { return w0 + px < wo; });
       }
       ptx::fence_proxy_async();
       __syncwarp();
       if (lane == 0) ptx::mbar_arrive(&stage_ready[bsel]);
+    }
+    if constexpr (GAP) {
+      if (gap_img >= 0) gap_flush(gap0, gap1, et, p.gap_sum + static_cast<long long>(p.out_ids ? p.out_ids[gap_img] : gap_img) * 64);
     }
   }
   __syncwarp();

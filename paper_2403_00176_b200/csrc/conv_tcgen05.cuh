@@ -74,8 +74,9 @@ __device__ __forceinline__ void conv_epi_bar() { asm volatile("bar.sync 1, 256;"
 // bank conflicts; the eight lanes of a channel pair add up by shuffles and the tile costs one atomic per channel.  (Sixteen
 // neighbouring pixels per thread and eight atomics per channel: 280 tiles of 128 channels, two a CTA, took 20.0 us with the sums
 // and 11.8 without; here 14.1.  What is left is the conversions: about 9 cycles per warp and scheduler each.)
+// gap_add_tile adds this thread's share of a tile to its two sums, gap_flush adds the CTA's sums to the table row.
 template <typename Valid>
-__device__ __forceinline__ void gap_accumulate_tile(const uint8_t* stage, int et, double* dst_row, Valid valid) {
+__device__ __forceinline__ void gap_add_tile(const uint8_t* stage, int et, double* s0, double* s1, Valid valid) {
   const int g = et >> 5, pair = et & 3, sub = (et & 31) >> 2;
   const uint8_t* src = stage + sub * 128 + ((g ^ sub) << 4) + pair * 4;
   double a0 = 0.0, a1 = 0.0, b0 = 0.0, b1 = 0.0;
@@ -86,17 +87,25 @@ __device__ __forceinline__ void gap_accumulate_tile(const uint8_t* stage, int et
     a0 += static_cast<double>(__uint_as_float(w0 << 16)); a1 += static_cast<double>(__uint_as_float(w0 & 0xffff0000u));
     b0 += static_cast<double>(__uint_as_float(w1 << 16)); b1 += static_cast<double>(__uint_as_float(w1 & 0xffff0000u));
   }
-  a0 += b0;
-  a1 += b1;
+  *s0 += a0 + b0;
+  *s1 += a1 + b1;
+}
+__device__ __forceinline__ void gap_flush(double a0, double a1, int et, double* dst_row) {
 #pragma unroll
   for (int o = 4; o <= 16; o <<= 1) {
     a0 += __shfl_xor_sync(0xffffffffu, a0, o);
     a1 += __shfl_xor_sync(0xffffffffu, a1, o);
   }
-  if (sub == 0) {
-    atomicAdd(dst_row + g * 8 + pair * 2, a0);
-    atomicAdd(dst_row + g * 8 + pair * 2 + 1, a1);
+  if ((et & 31) < 4) {
+    atomicAdd(dst_row + (et >> 5) * 8 + (et & 3) * 2, a0);
+    atomicAdd(dst_row + (et >> 5) * 8 + (et & 3) * 2 + 1, a1);
   }
+}
+template <typename Valid>
+__device__ __forceinline__ void gap_accumulate_tile(const uint8_t* stage, int et, double* dst_row, Valid valid) {
+  double s0 = 0.0, s1 = 0.0;
+  gap_add_tile(stage, et, &s0, &s1, valid);
+  gap_flush(s0, s1, et, dst_row);
 }
 
 // tmX: {Cin, W, H, N} bf16, box {64, TW, TH, 1}, element strides {1, s, s, 1}

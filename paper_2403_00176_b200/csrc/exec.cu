@@ -1686,6 +1686,8 @@ struct Builder : BuildState {
   }
 
   // ------------------------------------------------------------------------------ convolution
+  // rows the strip kernel takes: its column tiles of 128 pixels at least half full
+  static bool strip_width(int64_t w) { return (w + 127) / 128 * 128 <= 2 * w; }
   Status build_conv(int gi, const Group& G) {
     const Tensor& W = g.tensors[G.w];
     if (W.dtype != DType::BF16) return fail(E_UNSUPPORTED_OP, "convolution is bf16 only");
@@ -1756,15 +1758,19 @@ struct Builder : BuildState {
         cp.gap_sum = (gap_table != SIZE_MAX && batch.size() == 1) ? reinterpret_cast<double*>(const_cast<char*>(auxb) + gap_table) : nullptr;
         const dim3 gd(static_cast<unsigned>(std::min<long long>(tiles, x.plan->sm_count)));
         if (strip) {
-#define SOD2_STRIP(ACT_, HR_)                                                                                                            \
+#define SOD2_STRIP(ACT_, HR_, GAP_)                                                                                                      \
           {                                                                                                                              \
-            static bool once = (cudaFuncSetAttribute(k::conv3x3_strip_bf16_tcgen05<ACT_, HR_>, cudaFuncAttributeMaxDynamicSharedMemorySize, \
+            static bool once = (cudaFuncSetAttribute(k::conv3x3_strip_bf16_tcgen05<ACT_, HR_, GAP_>, cudaFuncAttributeMaxDynamicSharedMemorySize, \
                                                      k::STRIP_SMEM), true);                                                              \
             (void)once;                                                                                                                  \
-            return launch_pdl(k::conv3x3_strip_bf16_tcgen05<ACT_, HR_>, gd, dim3(k::STRIP_THREADS), k::STRIP_SMEM, x.stream, cache->B, cache->tw, cp); \
+            return launch_pdl(k::conv3x3_strip_bf16_tcgen05<ACT_, HR_, GAP_>, gd, dim3(k::STRIP_THREADS), k::STRIP_SMEM, x.stream, cache->B, cache->tw, cp); \
           }
-          if (act == 2) { if (hr) SOD2_STRIP(2, true) else SOD2_STRIP(2, false) }
-          else { if (hr) SOD2_STRIP(0, true) else SOD2_STRIP(0, false) }
+          if (cp.gap_sum) {
+            if (act == 2) { if (hr) SOD2_STRIP(2, true, true) else SOD2_STRIP(2, false, true) }
+            else { if (hr) SOD2_STRIP(0, true, true) else SOD2_STRIP(0, false, true) }
+          }
+          if (act == 2) { if (hr) SOD2_STRIP(2, true, false) else SOD2_STRIP(2, false, false) }
+          else { if (hr) SOD2_STRIP(0, true, false) else SOD2_STRIP(0, false, false) }
 #undef SOD2_STRIP
         }
         const int variant = ((bn == 128 ? 2 : 0) + (act == 2 ? 1 : 0)) * 2 + (hr ? 1 : 0);
@@ -1833,7 +1839,7 @@ struct Builder : BuildState {
       // wide images with a 3x3 / stride 1 / pad 1 kernel: row-halo kernel (a tile is 128 pixels of one row)
       // (the strip kernel's tiles are the same, at less than half of the cost of any other: from half-full tiles on)
       const int padded_w = ((cp.Wo + 127) / 128) * 128;
-      const bool rows = ks == 3 && G.stride == 1 && G.pad == 1 && (strip ? padded_w <= cp.Wo * 2 : cp.Wo >= 96 && padded_w * 4 <= cp.Wo * 5);
+      const bool rows = ks == 3 && G.stride == 1 && G.pad == 1 && (strip ? strip_width(cp.Wo) : cp.Wo >= 96 && padded_w * 4 <= cp.Wo * 5);
       if (rows) { cp.TW = 128; cp.TH = 1; }
       // other 3x3 / stride 1 / pad 1 layers of 128-column tiles: patches fetched once per 64 channels with their halo.  A tile
       // takes 0.62 of the implicit GEMM's time where the main loop is long, so up to 1.4 times as many of them pay
@@ -2045,8 +2051,15 @@ struct Builder : BuildState {
           }
         }
         // accumulating in the convolution's epilogue costs about as much per byte as the pooling pass it
-        // replaces; what it saves is the pass's two launches, which only outweighs it on the smaller tensors
-        if (writer >= 0 && static_cast<double>(N) * gp.C * static_cast<double>(gp.HW) * 2.0 > 32e6) writer = -1;
+        // replaces; what it saves is the pass's two launches, which only outweighs it on the smaller tensors.  The strip
+        // kernel's epilogue has the time (it waits 1500 cycles a row for the main loop): any size (32 x 64 x 112 x 112: 785 -> 757 us
+        // for the gated network)
+        if (writer >= 0) {
+          const Group& Wg = c.groups[writer];
+          const auto& wd = g.tensors[Wg.w].S.dims;
+          const bool strip = gp.C == 64 && wd[1].e.const_value() == 64 && wd[2].e.const_value() == 3 && Wg.stride == 1 && Wg.pad == 1 && strip_width(vx.dims[3]);
+          if (!strip && static_cast<double>(N) * gp.C * static_cast<double>(gp.HW) * 2.0 > 32e6) writer = -1;
+        }
         if (writer >= 0) { gap_accum[writer] = table; keep_table = true; }
         gapsum_root = (in_place && writer < 0) ? -1 : xroot;   // overwritten without the sums being kept: the table goes stale
         gapsum_aux = table;
