@@ -82,8 +82,8 @@ struct Group {
 // How a tensor's storage relates to others (decided once, at graph creation).
 struct Storage {
   // INDIRECT_IN: an output of a Switch that is never copied: the samples of the Switch input selected
-  // by the executed / skipped id list.  INDIRECT_OUT: the executed operand of a Combine, written by its
-  // producer straight into the Combine output at the executed ids.
+  // by the executed / skipped id list.  INDIRECT_OUT: the executed operand of a Combine (and the skipped one, where a
+  // convolution produces it), written by its producer straight into the Combine output at those ids.
   // ALIAS: the tensor lives in the storage of `other` (same extents): the output of a Combine whose
   // skipped samples are already where they belong, because the executed ones are written in place.
   enum Kind { ROOT, VIEW_OF_INPUT, VIEW_OF_OUTPUT, FOLDED, INDIRECT_IN, INDIRECT_OUT, ALIAS } kind = ROOT;

@@ -560,7 +560,9 @@ struct Fuser {
     // convolutions (as input or residual), the skipped branch only by the matching Combine, and the
     // Combine's executed operand is a convolution output, nothing is copied at the Switch: the
     // convolutions read the Switch input through the executed-id list and the last one writes into the
-    // Combine output at those ids; the Combine only moves the skipped samples.
+    // Combine output at those ids; the Combine only moves the skipped samples.  Where the skipped branch is one convolution
+    // too (a projection shortcut), it reads the Switch input through the skipped-id list and writes into the Combine output at
+    // those ids, and nothing is copied at all.
     if (!(c.flags & (OPT_COPY_REGROUP | OPT_NO_FUSION))) {
       auto conv_ok = [&](const Group& G) {
         if (G.kind != GKind::CONV) return false;
@@ -573,12 +575,23 @@ struct Fuser {
         if (S.kind != GKind::SWITCH || S.out2 < 0) continue;
         const int e = S.out, sk = S.out2, x = S.a;
         if (g.tensors[e].is_output || g.tensors[sk].is_output) continue;
+        const std::vector<int> sc = data_consumers(sk);
+        if (sc.size() != 1 || assigned[sc[0]] < 0) continue;
+        const int skip_group = assigned[sc[0]];
+        const bool projected = c.groups[skip_group].kind == GKind::CONV;
+        const int ys = projected ? c.groups[skip_group].out : sk;      // the Combine's skipped operand
         int cb = -1;
         for (size_t ci = 0; ci < c.groups.size(); ++ci)
-          if (c.groups[ci].kind == GKind::COMBINE && c.groups[ci].gate == S.gate && c.groups[ci].res == sk) cb = static_cast<int>(ci);
+          if (c.groups[ci].kind == GKind::COMBINE && c.groups[ci].gate == S.gate && c.groups[ci].res == ys) cb = static_cast<int>(ci);
         if (cb < 0) continue;
         const Group& C = c.groups[cb];
         bool ok = true;
+        if (projected) {
+          const Group& P = c.groups[skip_group];
+          if (!conv_ok(P) || P.a != sk || g.nodes[P.nodes[0]].ins[0] != sk || P.res >= 0 || P.bias == sk || P.w == sk) ok = false;
+          const std::vector<int> pc = data_consumers(ys);
+          if (pc.size() != 1 || assigned[pc[0]] != cb || g.tensors[ys].is_output || c.storage[ys].kind != Storage::ROOT || ys == C.a) ok = false;
+        }
         for (int cn : data_consumers(e)) {
           const int gi = assigned[cn];
           if (gi < 0 || !conv_ok(c.groups[gi])) { ok = false; break; }
@@ -586,8 +599,7 @@ struct Fuser {
           if (!((G.a == e && g.nodes[G.nodes[0]].ins[0] == e) || G.res == e)) { ok = false; break; }
           if (G.bias == e || G.w == e) { ok = false; break; }
         }
-        std::vector<int> sc = data_consumers(sk);
-        if (sc.size() != 1 || assigned[sc[0]] != cb) ok = false;
+        if (!projected && skip_group != cb) ok = false;
         const int ye = C.a;
         const int yp = g.tensors[ye].producer;
         if (yp < 0 || assigned[yp] < 0 || !conv_ok(c.groups[assigned[yp]]) || c.groups[assigned[yp]].out != ye) ok = false;
@@ -598,6 +610,7 @@ struct Fuser {
         c.storage[e] = Storage{Storage::INDIRECT_IN, S.nodes[0], x, S.gate, 0};
         c.storage[sk] = Storage{Storage::INDIRECT_IN, S.nodes[0], x, S.gate, 1};
         c.storage[ye] = Storage{Storage::INDIRECT_OUT, C.nodes[0], C.out, S.gate, 0};
+        if (projected) { c.storage[ys] = Storage{Storage::INDIRECT_OUT, C.nodes[0], C.out, S.gate, 1}; continue; }
         // In place: if nothing else reads the Switch input (besides the gate that decided the Switch and
         // the Switch itself), the Combine output takes over its storage; the skipped samples then never
         // move and the executed ones are overwritten by the block's last convolution, which reads its
@@ -636,7 +649,8 @@ struct Fuser {
       maxsub = std::max(maxsub, s);
     }
     c.n_subgraphs = maxsub + 1;
-    // 5. execution order of groups: topological, ties by first node
+    // 5. execution order of groups: topological, ties by first node; a convolution that writes the skipped samples into a
+    // Combine output goes when nothing else is ready (that output need not live while the executed branch runs)
     size_t G = c.groups.size();
     std::vector<std::set<int>> deps(G);
     for (size_t gi = 0; gi < G; ++gi) {
@@ -657,12 +671,16 @@ struct Fuser {
     std::vector<int> orderg, done(G, 0);
     for (size_t it = 0; it < G; ++it) {
       int pick = -1;
-      for (size_t gi = 0; gi < G && pick < 0; ++gi) {
-        if (done[gi]) continue;
-        bool ready = true;
-        for (int d : deps[gi]) if (!done[d]) ready = false;
-        if (ready) pick = static_cast<int>(gi);
-      }
+      for (int last = 0; last < 2 && pick < 0; ++last)
+        for (size_t gi = 0; gi < G && pick < 0; ++gi) {
+          if (done[gi]) continue;
+          const Group& Q = c.groups[gi];
+          const bool skipped = Q.kind == GKind::CONV && Q.out >= 0 && c.storage[Q.out].kind == Storage::INDIRECT_OUT && c.storage[Q.out].list == 1;
+          if (skipped != (last == 1)) continue;
+          bool ready = true;
+          for (int d : deps[gi]) if (!done[d]) ready = false;
+          if (ready) pick = static_cast<int>(gi);
+        }
       if (pick < 0) { c.err = "cyclic group dependencies"; return E_INTERNAL; }
       done[pick] = 1;
       orderg.push_back(pick);

@@ -46,3 +46,16 @@ def test_gemm_forms_by_epilogue(K, N, M, tail, form):
     ir = f"sym M 1 40000\ninput x bf16 [1,M,{K}]\n" + (f"input r bf16 [1,M,{N}]\n" if tail == "residual" else "") + f"const W bf16 [{K},{N}]\nnode MatMul x W -> y\n"
     ir += {"gelu": "node Gelu y -> z\noutput z\n", "residual": "node Add y r -> z\noutput z\n", "": "output y\n"}[tail]
     assert B.Graph(ir, 0).bind_dims(["M"], [[M]]).plan().group_form(0) == form
+
+
+def test_projection_blocks_copy_no_samples():
+    # the executed and the skipped branch of a projection block are convolutions: both read the Switch input and write the Combine
+    # output through the id lists, so the groups around them launch nothing; with copies asked for, they do
+    wl = WL.cfg5()
+    launches = []
+    for flags in (0, B.OPT_COPY_REGROUP):
+        g = B.Graph(wl.ir, flags)
+        p = g.bind_dims([], [[]]).plan()
+        kinds = [g.group_info(i)["kind"] for i in range(g.num_groups())]
+        launches.append(sum(p.group_cost(i)[1] for i, k in enumerate(kinds) if k == "combine"))
+    assert launches[0] == 0 and launches[1] > 0
