@@ -9,8 +9,9 @@
 // line with x >= TW are computed and dropped (P <= 31: at most an eighth of the tile at 14, 28 and 56 pixels, where patches
 // of 14 x 8, 28 x 4 and 28 x 4 pixels give as many tiles as any shape of 128 pixels does).
 // What is left to fetch per tap is the weights (one box of three dx taps per 12 MMAs) and a ninth of the patch.
-// Measured on B200: without any load but the first the main loop takes the same time, so the MMA issue bounds it.  The gated
-// network of 32 images 890 -> 833 us with the 21 layers that take this form (512 channels at 14 x 14: 20 -> 18 us a layer).
+// Measured on B200: without any load but the first the main loop takes the same time, so the MMAs bound it (2470 cycles per 64
+// channels against 2304 of the pipe).  The gated network of 32 images 890 -> 833 us with the 21 layers that take this form; 512
+// channels at 14 x 14: 20 us a layer in the implicit GEMM, 15 to 17 here.
 //
 // Warps (384 threads, persistent, 1 CTA/SM): 0 activation TMA, 1 weight TMA (constant: starts before the previous kernel has
 // ended), 3 MMA issuer, 4..11 epilogue (as in conv_tcgen05.cuh; the staging tile is packed to TW pixels per line).

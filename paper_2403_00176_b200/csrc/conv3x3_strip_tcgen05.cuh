@@ -8,8 +8,7 @@
 // documented to take effect in the order of issue where accumulator and shape are the same.  Consecutive rows share two of
 // their three blocks, so a row's first instruction waits until the row before has completed (its commit passes the turn),
 // and within a row every block sees one shape only: no instruction starts a block from zero, the epilogue clears it when it
-// has read it (0 + x: the same bits).  This costs about 160 cycles per row against relying on the order of issue (4 images
-// 53.5 -> 57.5 us a layer).
+// has read it (0 + x: the same bits).  The hand-over costs a row about 200 cycles.
 // The dx taps are the same rows of shared memory through descriptors whose start address is shifted by a pixel.  So a CTA
 // walks down a column of tiles of 128 pixels, every input row is loaded ONCE per strip (one box of 130 pixels, zero-filled
 // outside the image = the padding), and takes 12 instructions instead of 36.
@@ -20,8 +19,10 @@
 // Warps: 0 activation and weight TMA, 1 and 3 MMA issuers (alternate rows), 2 staging agent (residual prefetch + output
 // stores), 4..19 epilogue: two groups of eight that take alternate rows (a row's accumulator -> activation -> residual -> staging is a
 // chain of about 2000 cycles against 1300 of the main loop).
-// Measured on B200, 640x480 + 416x416 + 224x608 + 544x320 (6976 tiles): 92 us a layer with one tap per instruction, 58 here;
-// the MMAs of a row are 1170 cycles (1730 where the window wraps), the rest is the hand-over from row to row.
+// Measured on B200, 640x480 + 416x416 + 224x608 + 544x320 (6976 tiles): 92 us a layer with one tap per instruction, 57 here, at an
+// SM clock of 1.4 GHz (power); one 640x480 image 22 us.  A row takes 1360 cycles (1900 where the window wraps), 1152 of MMAs;
+// behind a branch on elect.sync per row it was 1550.  With 192 accumulator columns per input row and the parts added up by the
+// epilogue, which needs no order, the epilogue bound (1500 cycles a row).
 #pragma once
 #include <cuda.h>
 #include <cuda_bf16.h>

@@ -5,9 +5,9 @@
 //
 // Persistent, warp-specialised, one CTA per SM.  Tile 128 x BN; one pipeline stage holds KCH
 // k-chunks of 64 (each chunk = one 128-byte swizzle atom per row).  Measured on B200: a
-// tcgen05.mma occupies the tensor pipe for max(~48, BN/2) cycles, and a barrier wait between MMAs
-// leaves the pipe idle for about 320 cycles unless the MMAs queued before it are long enough to
-// cover it, so a stage must carry >= 512 cycles of MMA work: (BN=256, KCH=1) or (BN=128, KCH=2).
+// tcgen05.mma occupies the tensor pipe for max(48, BN/2) cycles, and what the issuing warp does between
+// two stages is time the pipe waits (ptx::Leader): (BN=256, KCH=1) or (BN=128, KCH=2), and nothing but a
+// wait, the MMAs and a commit per stage.
 // An SM takes in about 70 bytes per clock from L2, which bounds the main loop of a 128 x 256 tile
 // at about 75 % of the tensor peak.
 //   warp 0      TMA producer for A (STAGES-deep mbarrier ring; one 3-D box per stage)

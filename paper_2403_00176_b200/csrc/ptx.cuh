@@ -163,8 +163,8 @@ __device__ __forceinline__ void tmem_dealloc(uint32_t taddr, uint32_t ncols) {
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
-// True in one lane of a warp whose 32 lanes are in step.  MMAs are issued under this and not under `lane == 0`, inside
-// loops that the whole warp runs: the operands of tcgen05.mma are uniform registers, and only behind elect.sync does the
+// True in one lane of a warp whose 32 lanes are in step.  MMAs are issued by this lane (see Leader) and not under `lane == 0`,
+// inside loops that the whole warp runs: the operands of tcgen05.mma are uniform registers, and only behind elect.sync does the
 // compiler keep the address arithmetic there instead of moving every operand over for every instruction.  Measured on
 // B200 (cycles per 128x64x16 MMA with changing addresses; the pipe takes 48): `lane == 0` 56 alone and 97 beside sixteen
 // busy warps, elect.sync 48 and 53.
