@@ -2740,6 +2740,15 @@ Status run_plan_graph(Plan* p, const void* const* inputs, void* const* outputs, 
   return OK;
 }
 
+// What a run zeroes at the start of the arena (a multiple of 256 bytes).  A kernel, so that the first kernel of the run, a
+// programmatic dependent of it, is set up while it runs: encoder, 1 request 188.2 -> 185.1 us, 8 requests 357.9 -> 354.7; graphs of
+// the gated and pruning networks 0.1 to 0.2 % shorter.
+__global__ void __launch_bounds__(128) clear_header(uint4* header, int n) {
+  ptx::pdl_launch();
+  ptx::pdl_wait();
+  for (int i = threadIdx.x; i < n; i += 128) header[i] = make_uint4(0u, 0u, 0u, 0u);
+}
+
 Status run_plan(Plan* p, const void* const* inputs, void* const* outputs, void* arena, size_t arena_bytes, void* stream, int64_t* info,
                 int step_lo, int step_hi) {
   if (!arena && p->arena_bytes) { p->err = "arena is null"; return E_INVALID_ARG; }
@@ -2754,7 +2763,13 @@ Status run_plan(Plan* p, const void* const* inputs, void* const* outputs, void* 
     p->sm_count_known = true;
   }
   RunCtx x{inputs, outputs, static_cast<char*>(arena), static_cast<char*>(p->c->packed_ws), static_cast<cudaStream_t>(stream), p};
-  if (p->uses_header && step_lo <= 0 && cudaMemsetAsync(arena, 0, p->header_clear_bytes, x.stream) != cudaSuccess) { p->err = "cannot clear the status word"; return E_CUDA; }
+  if (p->uses_header && step_lo <= 0) {
+    // (layout changes are plain launches, which wait for a kernel's end longer than for a memset: 109.2 against 110.1 us)
+    const bool plain_first = !p->launches.empty() && p->launches[0]->group >= 0 && p->c->groups[p->launches[0]->group].kind == GKind::LAYOUT;
+    const cudaError_t e = plain_first ? cudaMemsetAsync(arena, 0, p->header_clear_bytes, x.stream)
+                                      : launch_pdl(clear_header, dim3(1), dim3(128), 0, x.stream, static_cast<uint4*>(arena), static_cast<int>(p->header_clear_bytes / 16));
+    if (e != cudaSuccess) { p->err = "cannot clear the status word"; return E_CUDA; }
+  }
   if (!ensure_side_stream(p)) { p->err = "cannot create the second stream"; return E_CUDA; }
   const int n_groups = static_cast<int>(p->side_group.size());
   cudaStream_t side = static_cast<cudaStream_t>(p->side_stream);
