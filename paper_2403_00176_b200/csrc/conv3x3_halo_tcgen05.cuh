@@ -2,16 +2,17 @@
 //
 // The implicit-GEMM kernel (conv_tcgen05.cuh) fetches a 128-pixel tile nine times per 64 input channels, once per tap:
 // 16 KB of activations and 16 KB of weights for every 128 x 128 x 64 product, which the tensor pipe does in 290 cycles and
-// L2 -> shared memory in 420.  Here a tile's patch of TW x TH output pixels is fetched ONCE per 64 channels, with its halo:
-// one box {64 ch, TW + 2, TH + 2}, zero-filled outside the image (= the padding), whose pixels lie in shared memory as rows
-// of 128 bytes with pitch P = TW + 2.  Row m = y * P + x of the MMA is output pixel (y, x); tap (dy, dx) reads the same
-// buffer dy * P + dx rows further down, which is a shift of the operand descriptor's start address.  The two rows per patch
-// line with x >= TW are computed and dropped (P <= 31: at most an eighth of the tile at 14, 28 and 56 pixels, where patches
-// of 14 x 8, 28 x 4 and 28 x 4 pixels give as many tiles as any shape of 128 pixels does).
-// What is left to fetch per tap is the weights (one box of three dx taps per 12 MMAs) and a ninth of the patch.
-// Measured on B200: without any load but the first the main loop takes the same time, so the MMAs bound it (2470 cycles per 64
-// channels against 2304 of the pipe).  The gated network of 32 images 890 -> 833 us with the 21 layers that take this form; 512
-// channels at 14 x 14: 20 us a layer in the implicit GEMM, 15 to 17 here.
+// L2 -> shared memory in 420.  Here one box per kernel row dy and 64 channels does for the three taps of that row: the
+// TH lines of TW + 2 pixels that a patch of TW x TH output pixels needs, zero-filled outside the image (= the padding), which
+// lie in shared memory as rows of 128 bytes with pitch P = TW + 2.  Row m = y * P + x of the MMA is output pixel (y, x); tap dx
+// reads the same buffer dx rows further down, which is a shift of the operand descriptor's start address.  The two rows per
+// patch line with x >= TW are computed and dropped.  What is left to fetch per tap is the weights and a third of the patch.
+// K is summed in the order (dy, 64-channel chunk, dx, channel), as in the implicit-GEMM and row kernels: the same sums in the
+// same order, so that the three forms give the same bits.
+// Measured on B200, implicit GEMM -> here, 32 images of 56 x 56 to 128 channels: 64 channels 21.3 -> 17.0 us, 128 32.3 -> 25.6, 256
+// 58.8 -> 47.8, 512 122 -> 99 (1200 TFLOP/s); bound by the MMAs and the 85 bytes per cycle that a stage of 64 KB takes in beside them.
+// (A patch fetched once per 64 channels, K in the order (chunk, dy, dx): 24.7 us at 128 channels, 27.0 against 26.5 at 512
+// channels of 14 x 14, and other bits.)
 //
 // Warps (384 threads, persistent, 1 CTA/SM): 0 activation TMA, 1 weight TMA (constant: starts before the previous kernel has
 // ended), 3 MMA issuer, 4..11 epilogue (as in conv_tcgen05.cuh; the staging tile is packed to TW pixels per line).
@@ -25,32 +26,28 @@ namespace sod2 {
 namespace k {
 
 constexpr int HALO_BN = 128;
-constexpr int HALO_MAX_P = 31;                        // 2 * P + 130 rows of a patch buffer are read: at most 192
-constexpr int HALO_A_SLOT = 192 * 128;
-constexpr int HALO_A_STAGES = 2;
-constexpr int HALO_B_STAGE = 3 * HALO_BN * 128;       // the dx taps of one (dy, 64-channel chunk)
-constexpr int HALO_B_STAGES = 3;
-constexpr int HALO_SMEM = HALO_A_STAGES * HALO_A_SLOT + HALO_B_STAGES * HALO_B_STAGE + 2 * CONV_STAGE_OUT + 2 * HALO_BN * 4 /*bias*/ +
-                          8 * (2 * HALO_A_STAGES + 2 * HALO_B_STAGES + 6) + 16 + 1024 /*alignment*/;
+constexpr int HALO_MAX_ROWS = 128;                    // (TW + 2) * TH: the two rows read behind them end up in dropped rows only
+constexpr int HALO_A_BYTES = HALO_MAX_ROWS * 128;
+constexpr int HALO_B_BYTES = 3 * HALO_BN * 128;       // the dx taps of one (dy, 64-channel chunk)
+constexpr int HALO_STAGE = HALO_A_BYTES + HALO_B_BYTES;
+constexpr int HALO_STAGES = 3;
+constexpr int HALO_SMEM = HALO_STAGES * HALO_STAGE + 2 * CONV_STAGE_OUT + 2 * HALO_BN * 4 /*bias*/ + 8 * (2 * HALO_STAGES + 6) + 16 + 1024 /*alignment*/;
+static_assert(HALO_SMEM <= 227 * 1024, "shared memory of a CTA");
 
-// tmX: {Cin, W, H, N}, box {64, TW + 2, TH + 2, 1};  tmW: k-chunk view {64, Cout, K/64} of the weights in (dy, chunk, dx, ci)
-// order, box {64, 128, 3};  tmOut / tmRes: {Cout, W, H, N}, box {64, TW, TH, 1}.  p.TW + 2 <= HALO_MAX_P and
-// (p.TH - 1) * (p.TW + 2) + p.TW <= 128.
+// tmX: {Cin, W, H, N}, box {64, TW + 2, TH, 1};  tmW: k-chunk view {64, Cout, K/64} of the weights in (dy, chunk, dx, ci)
+// order, box {64, 128, 3};  tmOut / tmRes: {Cout, W, H, N}, box {64, TW, TH, 1}.  (p.TW + 2) * p.TH <= HALO_MAX_ROWS.
 template <int ACT, bool HASRES>
 __global__ void __launch_bounds__(CONV_THREADS, 1)
 conv3x3_halo_bf16_tcgen05(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmW,
                           const __grid_constant__ CUtensorMap tmOut, const __grid_constant__ CUtensorMap tmRes, ConvParams p) {
-  constexpr int AS = HALO_A_STAGES, BS = HALO_B_STAGES, BN = HALO_BN;
+  constexpr int ST = HALO_STAGES, BN = HALO_BN;
   extern __shared__ uint8_t smem_raw[];
-  uint8_t* patches = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  uint8_t* weights = patches + AS * HALO_A_SLOT;
-  uint8_t* out_stage = weights + BS * HALO_B_STAGE;
+  uint8_t* stages = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));   // weights, then the patch
+  uint8_t* out_stage = stages + ST * HALO_STAGE;
   float* bias_s = reinterpret_cast<float*>(out_stage + 2 * CONV_STAGE_OUT);   // [2][128]
-  uint64_t* a_full = reinterpret_cast<uint64_t*>(bias_s + 2 * BN);
-  uint64_t* a_empty = a_full + AS;
-  uint64_t* b_full = a_empty + AS;
-  uint64_t* b_empty = b_full + BS;
-  uint64_t* tmem_full = b_empty + BS;     // [2]
+  uint64_t* full = reinterpret_cast<uint64_t*>(bias_s + 2 * BN);
+  uint64_t* empty = full + ST;
+  uint64_t* tmem_full = empty + ST;       // [2]
   uint64_t* tmem_empty = tmem_full + 2;   // [2]
   uint64_t* res_full = tmem_empty + 2;    // [2]
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(res_full + 2);
@@ -58,8 +55,7 @@ conv3x3_halo_bf16_tcgen05(const __grid_constant__ CUtensorMap tmX, const __grid_
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (threadIdx.x == 0) {
-    for (int s = 0; s < AS; ++s) { ptx::mbar_init(&a_full[s], 1); ptx::mbar_init(&a_empty[s], 1); }
-    for (int s = 0; s < BS; ++s) { ptx::mbar_init(&b_full[s], 1); ptx::mbar_init(&b_empty[s], 1); }
+    for (int s = 0; s < ST; ++s) { ptx::mbar_init(&full[s], 2); ptx::mbar_init(&empty[s], 1); }
     for (int b = 0; b < 2; ++b) { ptx::mbar_init(&tmem_full[b], 1); ptx::mbar_init(&tmem_empty[b], 8); ptx::mbar_init(&res_full[b], 1); }
     *dead = 0;
     ptx::fence_barrier_init();
@@ -79,16 +75,16 @@ conv3x3_halo_bf16_tcgen05(const __grid_constant__ CUtensorMap tmX, const __grid_
   const int P = p.TW + 2;
   const int tiles_n = p.Cout / BN;
   const int cchunks = p.Cin / 64;
-  const int groups = 3 * cchunks;                    // weight stages per tile
+  const int groups = 3 * cchunks;                    // stages per tile, (dy, chunk): a multiple of three
   const int tiles_w = (p.Wo + p.TW - 1) / p.TW, tiles_h = (p.Ho + p.TH - 1) / p.TH;
-  auto weight_box = [&](ptx::Leader one, int s, int n0, int gq) {     // group gq of a tile = (chunk gq / 3, kernel row gq % 3)
-    ptx::mbar_expect_tx(one, &b_full[s], HALO_B_STAGE);
-    ptx::tma_load_3d(one, weights + s * HALO_B_STAGE, &tmW, 0, n0, ((gq % 3) * cchunks + gq / 3) * 3, &b_full[s]);
+  auto weight_box = [&](ptx::Leader one, int s, int n0, int g) {
+    ptx::mbar_expect_tx(one, &full[s], HALO_B_BYTES);
+    ptx::tma_load_3d(one, stages + s * HALO_STAGE, &tmW, 0, n0, g * 3, &full[s]);
   };
   // the first weight stages do not depend on the previous kernel
   if (warp == 1) {
     const ptx::Leader one = ptx::elect_leader();
-    for (int gq = 0; gq < BS; ++gq) weight_box(one, gq, (static_cast<int>(blockIdx.x) % tiles_n) * BN, gq);   // groups >= 3 = BS
+    for (int g = 0; g < ST; ++g) weight_box(one, g, (static_cast<int>(blockIdx.x) % tiles_n) * BN, g);   // groups >= 3 = ST
   }
   ptx::pdl_wait();
   int n_img = p.n_img;
@@ -105,66 +101,65 @@ conv3x3_halo_bf16_tcgen05(const __grid_constant__ CUtensorMap tmX, const __grid_
 
   if (warp == 0) {
     // ---- activation patches
-    const uint32_t bytes = P * (p.TH + 2) * 128;
+    const uint32_t bytes = P * p.TH * 128;
     const ptx::Leader one = ptx::elect_leader();
+    if (static_cast<int>(blockIdx.x) >= num_tiles && lane < ST) ptx::mbar_arrive(&full[lane]);   // see the weights
     int n = 0;
     for (int t = blockIdx.x; t < num_tiles; t += gridDim.x) {
       int n0, img, ho0, wo0;
       decode(t, &n0, &img, &ho0, &wo0);
       if (p.in_ids) img = p.in_ids[img];
-      for (int cc = 0; cc < cchunks; ++cc, ++n) {
-        const int s = n % AS;
-        if (n >= AS) ptx::mbar_wait_elect(&a_empty[s], ((n / AS) - 1) & 1, dead);
-        ptx::mbar_expect_tx(one, &a_full[s], bytes);
-        ptx::tma_load_4d(one, patches + s * HALO_A_SLOT, &tmX, cc * 64, wo0 - 1, ho0 - 1, img, &a_full[s]);
-      }
+      for (int dy = 0; dy < 3; ++dy)
+        for (int cc = 0; cc < cchunks; ++cc, ++n) {
+          const int s = n % ST;
+          if (n >= ST) ptx::mbar_wait_elect(&empty[s], ((n / ST) - 1) & 1, dead);
+          ptx::mbar_expect_tx(one, &full[s], bytes);
+          ptx::tma_load_4d(one, stages + s * HALO_STAGE + HALO_B_BYTES, &tmX, cc * 64, wo0 - 1, ho0 - 1 + dy, img, &full[s]);
+        }
     }
   } else if (warp == 1) {
     // ---- weights
     if (static_cast<int>(blockIdx.x) >= num_tiles) {
-      for (int s = 0; s < BS; ++s) ptx::mbar_wait_elect(&b_full[s], 0, dead);    // nothing may land after the CTA has gone
+      for (int s = 0; s < ST; ++s) ptx::mbar_wait_elect(&full[s], 0, dead);    // nothing may land after the CTA has gone
     }
     const ptx::Leader one = ptx::elect_leader();
     int n = 0;
     for (int t = blockIdx.x; t < num_tiles; t += gridDim.x) {
       const int n0 = (t % tiles_n) * BN;
-      for (int gq = 0; gq < groups; ++gq, ++n) {
-        if (n < BS) continue;
-        const int s = n % BS;
-        ptx::mbar_wait_elect(&b_empty[s], ((n / BS) - 1) & 1, dead);
-        weight_box(one, s, n0, gq);
+      for (int g = 0; g < groups; ++g, ++n) {
+        if (n < ST) continue;
+        const int s = n % ST;
+        ptx::mbar_wait_elect(&empty[s], ((n / ST) - 1) & 1, dead);
+        weight_box(one, s, n0, g);
       }
     }
   } else if (warp == 3) {
     // ---- MMA issuer: the whole warp in step, one lane issues (ptx::Leader)
     constexpr uint32_t idesc = ptx::idesc_bf16(128, BN);
     const ptx::Leader one = ptx::elect_leader();
-    // (weight stage dy holds kernel row dy of every chunk: BS == 3.  Straight-line code with the descriptors at hand: with
-    // the three rows as a loop the issuer took 82 cycles per MMA, 67 like this; the pipe takes 64)
-    static_assert(BS == 3 && AS == 2, "one weight stage per kernel row, patches in turn");
-    const uint64_t a0 = ptx::smem_desc_sw128(ptx::smem_u32(patches)), b0 = ptx::smem_desc_sw128(ptx::smem_u32(weights));
-    const uint32_t line = P * 8;             // a patch line in descriptor units of 16 bytes
-    int na = 0, j = 0;
+    // straight-line code with the descriptors at hand: a stage is twelve MMAs and nothing but a wait and a commit beside them.
+    // (Weights by single taps, or patches that stay for the three kernel rows, fetch less or finer; the arithmetic and the
+    // waits they need cost more: 32 images of 512 channels 31.8 us, 256 channels 29.3)
+    static_assert(ST == 3, "a tile is a multiple of three stages");
+    const uint64_t b0 = ptx::smem_desc_sw128(ptx::smem_u32(stages)), a0 = ptx::smem_desc_sw128(ptx::smem_u32(stages + HALO_B_BYTES));
+    uint32_t par = 0;
+    int j = 0;
     for (int t = blockIdx.x; t < num_tiles; t += gridDim.x, ++j) {
       const int acc = j & 1;
       if (j >= 2) ptx::mbar_wait_elect(&tmem_empty[acc], ((j >> 1) - 1) & 1, dead);
       const uint32_t d = tmem + acc * BN;
-      for (int cc = 0; cc < cchunks; ++cc, ++na) {
-        const int sa = na & 1;
-        const uint64_t as = a0 + sa * (HALO_A_SLOT >> 4);
-        ptx::mbar_wait_elect(&a_full[sa], (na >> 1) & 1, dead);
+      for (int r = 0; r < cchunks; ++r, par ^= 1) {
 #pragma unroll
-        for (int dy = 0; dy < 3; ++dy) {
-          ptx::mbar_wait_elect(&b_full[dy], na & 1, dead);
+        for (int s = 0; s < ST; ++s) {
+          const uint64_t ad = a0 + s * (HALO_STAGE >> 4), bd = b0 + s * (HALO_STAGE >> 4);
+          ptx::mbar_wait_elect(&full[s], par, dead);
           ptx::tc_fence_after();
-          const uint64_t ad = as + dy * line, bd = b0 + dy * (HALO_B_STAGE >> 4);
 #pragma unroll
           for (int dx = 0; dx < 3; ++dx)
 #pragma unroll
-            for (int kk = 0; kk < 4; ++kk) ptx::mma_bf16(one, d, ad + 8 * dx + 2 * kk, bd + dx * (BN * 128 / 16) + 2 * kk, idesc, (cc | dy | dx | kk) != 0);
-          ptx::mma_commit(one, &b_empty[dy]);
+            for (int kk = 0; kk < 4; ++kk) ptx::mma_bf16(one, d, ad + 8 * dx + 2 * kk, bd + dx * (BN * 128 / 16) + 2 * kk, idesc, (r | s | dx | kk) != 0);
+          ptx::mma_commit(one, &empty[s]);
         }
-        ptx::mma_commit(one, &a_empty[sa]);
       }
       ptx::mma_commit(one, &tmem_full[acc]);
     }
@@ -265,7 +260,7 @@ conv3x3_halo_bf16_tcgen05(const __grid_constant__ CUtensorMap tmX, const __grid_
           bulk_commit();
         }
         if (p.gap_sum) {
-          const uint32_t inv = 65536u / p.TW + 1;    // px / TW for px < 128 and TW <= 29: exact
+          const uint32_t inv = 65536u / p.TW + 1;    // px / TW for px < 128 and TW <= 126: exact
           gap_accumulate_tile(stage, et, p.gap_sum + static_cast<long long>(img_o) * p.Cout + np, [&](int px) {
             const int y = static_cast<int>((px * inv) >> 16);
             return y < p.TH && ho0 + y < p.Ho && wo0 + px - y * p.TW < p.Wo;

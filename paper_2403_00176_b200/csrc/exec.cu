@@ -1841,15 +1841,15 @@ struct Builder : BuildState {
       const int padded_w = ((cp.Wo + 127) / 128) * 128;
       const bool rows = ks == 3 && G.stride == 1 && G.pad == 1 && (strip ? strip_width(cp.Wo) : cp.Wo >= 96 && padded_w * 4 <= cp.Wo * 5);
       if (rows) { cp.TW = 128; cp.TH = 1; }
-      // other 3x3 / stride 1 / pad 1 layers of 128-column tiles: patches fetched once per 64 channels with their halo.  A tile
+      // other 3x3 / stride 1 / pad 1 layers of 128-column tiles: the patches of the halo kernel.  A tile
       // takes 0.62 of the implicit GEMM's time where the main loop is long, so up to 1.4 times as many of them pay
       bool halo = false;
       if (ks == 3 && G.stride == 1 && G.pad == 1 && bn == 128 && !rows) {
         const long long igemm_tiles = best / 128;
         long long fewest = -1;
         int tw_best = 0, th_best = 0;
-        for (int tw = 1; tw + 2 <= k::HALO_MAX_P && tw <= cp.Wo; ++tw) {
-          const int th = std::min((128 - tw) / (tw + 2) + 1, cp.Ho);
+        for (int tw = 1; tw + 2 <= k::HALO_MAX_ROWS && tw <= cp.Wo; ++tw) {
+          const int th = std::min(k::HALO_MAX_ROWS / (tw + 2), cp.Ho);
           const long long n = static_cast<long long>((cp.Wo + tw - 1) / tw) * ((cp.Ho + th - 1) / th);
           if (fewest < 0 || n <= fewest) { fewest = n; tw_best = tw; th_best = th; }
         }
@@ -1888,7 +1888,7 @@ struct Builder : BuildState {
         void* O = x.resolve(po);
         const void* R = hr ? x.resolve(pr) : O;
         if (cache->a != X || cache->w != Wp || cache->o != O || cache->r != R) {
-          if (!encode_bf16_nhwc(&cache->tx, X, n_in_map, H, Wd, Cin, cp.TW + (halo ? 2 : 0), cp.TH + (halo ? 2 : 0), stride) ||
+          if (!encode_bf16_nhwc(&cache->tx, X, n_in_map, H, Wd, Cin, cp.TW + (halo ? 2 : 0), cp.TH, stride) ||
               !encode_bf16_kchunks(&cache->tw, Wp, Cout, K, K, bn, halo ? 3 : kch) ||
               !encode_bf16_nhwc(&cache->to, O, n_out_map, cp.Ho, cp.Wo, Cout, cp.TW, cp.TH, 1) ||
               !encode_bf16_nhwc(&cache->tr, R, hr ? n_res_map : n_out_map, cp.Ho, cp.Wo, Cout, cp.TW, cp.TH, 1))

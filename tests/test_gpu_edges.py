@@ -6,6 +6,7 @@ import torch
 from oracle import interp as O
 from paper_2403_00176_b200 import binding as B
 from paper_2403_00176_b200 import workloads as WL
+from paper_2403_00176_b200.session import Session
 from paper_2403_00176_b200.workloads import Request, bf16_round
 from tests.gpu_harness import lockstep, run_batch
 from tests.test_gpu_parity import _check_topk_lockstep
@@ -95,6 +96,31 @@ def test_conv_halo_patches(C, shapes):
     p.run()
     for a, b in zip(outs, p.outputs()):
         assert all(np.array_equal(a[n], b[n]) for n in a)
+
+
+@pytest.mark.parametrize("cin", [64, 192, 256, 320, 512])
+def test_conv_forms_add_up_in_the_same_order(cin):
+    # kernel rows, then 64-channel chunks, then columns: halo patches (chunks resident up to 256 channels and streamed beyond), row tiles
+    # and the implicit GEMM give the same bits.  The same pixels with zeros behind them, at sizes that take different forms
+    ir = (f"sym H 1 4096\nsym W 1 4096\ninput x bf16 [1,{cin},H,W]\nconst w bf16 [128,{cin},3,3]\nconst b bf16 [128]\n"
+          "node Conv x w b -> c {kernel=3 stride=1 pad=1}\nnode Relu c -> y\noutput y\n")
+    rng = np.random.default_rng(71)
+    consts = {"w": bf16_round((rng.standard_normal((128, cin, 3, 3)) / np.sqrt(9 * cin)).astype(np.float32)), "b": bf16_round(rng.standard_normal(128).astype(np.float32))}
+    s = Session(WL.Workload("conv_forms", "bf16", ir, consts, ["H", "W"], ["y"], {}))
+    conv = [s.graph.group_info(i)["kind"] for i in range(s.graph.num_groups())].index("conv")
+    for h, w, sizes in [(37, 90, [(37, 90, "halo"), (37, 128, "rows")]), (16, 8, [(16, 8, "implicit GEMM"), (16, 30, "halo"), (16, 97, "halo")])]:
+        pixels = bf16_round(rng.standard_normal((1, cin, h, w)).astype(np.float32))
+        outs = []
+        for hh, ww, form in sizes:
+            x = np.zeros((1, cin, hh, ww), np.float32)
+            x[:, :, :h, :w] = pixels
+            p = s.prepare([Request({"H": hh, "W": ww}, {"x": x})])
+            assert p.plan.group_form(conv) == form
+            p.run()
+            p.check_device_status()
+            outs.append(p.outputs()[0]["y"][:, :, :h, :w])
+        assert all(np.array_equal(outs[0], o) for o in outs[1:])
+        assert O.rel_err(outs[0], O.run(ir, consts, {"x": pixels})["y"]) <= BF16_TOL
 
 
 @pytest.mark.parametrize("lens", [[1], [33, 64], [129, 640], list(range(1, 129, 3)) + [129, 191, 192, 193, 255, 256, 257, 300, 383, 385, 511, 512, 513, 577] + [200] * 8,
