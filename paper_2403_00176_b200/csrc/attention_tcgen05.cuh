@@ -169,7 +169,7 @@ attention_tcgen05_bf16(const __grid_constant__ CUtensorMap tmQ, const __grid_con
       const AtcReq R = reqs[it.ri];
       if (is_k) {
         const int qs = i & 1;
-        if (i >= 2) ptx::mbar_wait_elect(&q_free[qs], ((i >> 1) - 1) & 1, dead);
+        if (i >= 2) ptx::mbar_wait_warp(&q_free[qs], ((i >> 1) - 1) & 1, dead);
         ptx::mbar_expect_tx(one, &q_full[qs], ATC_Q_BYTES);
         ptx::tma_load_2d(one, sQ + qs * ATC_Q_BYTES, &tmQ, p.q_col + it.head * p.q_hs, R.q_row + it.q0, &q_full[qs]);
       }
@@ -180,7 +180,7 @@ attention_tcgen05_bf16(const __grid_constant__ CUtensorMap tmQ, const __grid_con
       const int col = is_k ? p.k_col + it.head * p.k_hs : p.v_col + it.head * p.v_hs, row = is_k ? R.k_row : R.v_row;
       for (int j = 0; j < it.nkv; ++j, ++n) {
         const int b = n % ATC_ST;
-        if (n >= ATC_ST) ptx::mbar_wait_elect(&free_[b], ((n / ATC_ST) - 1) & 1, dead);
+        if (n >= ATC_ST) ptx::mbar_wait_warp(&free_[b], ((n / ATC_ST) - 1) & 1, dead);
         ptx::mbar_expect_tx(one, &full[b], ATC_KV_BYTES);
         ptx::tma_load_2d(one, dst + b * ATC_KV_BYTES, tm, col, row + j * ATC_KB, &full[b]);
         SOD2_TRACE(0, (is_k ? 800 : 840) + n)
@@ -197,11 +197,12 @@ attention_tcgen05_bf16(const __grid_constant__ CUtensorMap tmQ, const __grid_con
       ptx::mbar_wait_warp(&q_full[i & 1], (i >> 1) & 1, dead);
       for (int j = 0; j < it.nkv; ++j, ++n) {
         const uint64_t dK = ptx::smem_desc_sw128(ptx::smem_u32(sK + (n % ATC_ST) * ATC_KV_BYTES));
-        ptx::mbar_wait_elect(&k_full[n % ATC_ST], (n / ATC_ST) & 1, dead);
-        if (n >= 2) ptx::mbar_wait_elect(&s_free[n & 1], ((n >> 1) - 1) & 1, dead);
+        ptx::mbar_wait_lanes(&k_full[n % ATC_ST], (n / ATC_ST) & 1, dead);
+        if (n >= 2) ptx::mbar_wait_lanes(&s_free[n & 1], ((n >> 1) - 1) & 1, dead);
         ptx::tc_fence_after();
 #pragma unroll
         for (int kk = 0; kk < 4; ++kk) ptx::mma_bf16(one, tmem + ATC_TMEM_S + (n & 1) * 64, dQ + 2 * kk, dK + 2 * kk, idesc_qk, kk != 0);
+        __syncwarp();
         ptx::mma_commit(one, &s_full[n & 1]);
         ptx::mma_commit(one, &k_free[n % ATC_ST]);
         if (lane == 0) { SOD2_TRACE(1, 100 + n) }
@@ -218,13 +219,14 @@ attention_tcgen05_bf16(const __grid_constant__ CUtensorMap tmQ, const __grid_con
       for (int j = 0; j < it.nkv; ++j, ++n) {
         const int steps = (it.L - j * ATC_KB + 15) >> 4;       // keys past the request are left out
         const uint32_t aV = ptx::smem_u32(sV + (n % ATC_ST) * ATC_KV_BYTES);
-        ptx::mbar_wait_elect(&v_full[n % ATC_ST], (n / ATC_ST) & 1, dead);
-        ptx::mbar_wait_elect(&p_full[n & 1], (n >> 1) & 1, dead);
+        ptx::mbar_wait_lanes(&v_full[n % ATC_ST], (n / ATC_ST) & 1, dead);
+        ptx::mbar_wait_lanes(&p_full[n & 1], (n >> 1) & 1, dead);
         ptx::tc_fence_after();
         // 16 keys per step: 8 packed columns of P in tensor memory, 16 rows (2048 B) down V
 #pragma unroll
         for (int kk = 0; kk < ATC_KB / 16; ++kk)
           if (kk < steps) ptx::mma_bf16_a_tmem(one, tmem + ATC_TMEM_O, tmem + ATC_TMEM_P + (n & 1) * 32 + kk * 8, ptx::smem_desc_sw128(aV + kk * 2048), idesc_pv, (j | kk) != 0);
+        __syncwarp();
         ptx::mma_commit(one, &o_full[n & 1]);
         ptx::mma_commit(one, &v_free[n % ATC_ST]);
         if (lane == 0) { SOD2_TRACE(1, 200 + n) }

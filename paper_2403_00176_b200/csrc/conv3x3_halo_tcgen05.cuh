@@ -112,7 +112,7 @@ conv3x3_halo_bf16_tcgen05(const __grid_constant__ CUtensorMap tmX, const __grid_
       for (int dy = 0; dy < 3; ++dy)
         for (int cc = 0; cc < cchunks; ++cc, ++n) {
           const int s = n % ST;
-          if (n >= ST) ptx::mbar_wait_elect(&empty[s], ((n / ST) - 1) & 1, dead);
+          if (n >= ST) ptx::mbar_wait_warp(&empty[s], ((n / ST) - 1) & 1, dead);
           ptx::mbar_expect_tx(one, &full[s], bytes);
           ptx::tma_load_4d(one, stages + s * HALO_STAGE + HALO_B_BYTES, &tmX, cc * 64, wo0 - 1, ho0 - 1 + dy, img, &full[s]);
         }
@@ -120,7 +120,7 @@ conv3x3_halo_bf16_tcgen05(const __grid_constant__ CUtensorMap tmX, const __grid_
   } else if (warp == 1) {
     // ---- weights
     if (static_cast<int>(blockIdx.x) >= num_tiles) {
-      for (int s = 0; s < ST; ++s) ptx::mbar_wait_elect(&full[s], 0, dead);    // nothing may land after the CTA has gone
+      for (int s = 0; s < ST; ++s) ptx::mbar_wait_warp(&full[s], 0, dead);    // nothing may land after the CTA has gone
     }
     const ptx::Leader one = ptx::elect_leader();
     int n = 0;
@@ -129,7 +129,7 @@ conv3x3_halo_bf16_tcgen05(const __grid_constant__ CUtensorMap tmX, const __grid_
       for (int g = 0; g < groups; ++g, ++n) {
         if (n < ST) continue;
         const int s = n % ST;
-        ptx::mbar_wait_elect(&empty[s], ((n / ST) - 1) & 1, dead);
+        ptx::mbar_wait_warp(&empty[s], ((n / ST) - 1) & 1, dead);
         weight_box(one, s, n0, g);
       }
     }
@@ -146,18 +146,19 @@ conv3x3_halo_bf16_tcgen05(const __grid_constant__ CUtensorMap tmX, const __grid_
     int j = 0;
     for (int t = blockIdx.x; t < num_tiles; t += gridDim.x, ++j) {
       const int acc = j & 1;
-      if (j >= 2) ptx::mbar_wait_elect(&tmem_empty[acc], ((j >> 1) - 1) & 1, dead);
+      if (j >= 2) ptx::mbar_wait_lanes(&tmem_empty[acc], ((j >> 1) - 1) & 1, dead);
       const uint32_t d = tmem + acc * BN;
       for (int r = 0; r < cchunks; ++r, par ^= 1) {
 #pragma unroll
         for (int s = 0; s < ST; ++s) {
           const uint64_t ad = a0 + s * (HALO_STAGE >> 4), bd = b0 + s * (HALO_STAGE >> 4);
-          ptx::mbar_wait_elect(&full[s], par, dead);
+          ptx::mbar_wait_lanes(&full[s], par, dead);
           ptx::tc_fence_after();
 #pragma unroll
           for (int dx = 0; dx < 3; ++dx)
 #pragma unroll
             for (int kk = 0; kk < 4; ++kk) ptx::mma_bf16(one, d, ad + 8 * dx + 2 * kk, bd + dx * (BN * 128 / 16) + 2 * kk, idesc, (r | s | dx | kk) != 0);
+          __syncwarp();
           ptx::mma_commit(one, &empty[s]);
         }
       }

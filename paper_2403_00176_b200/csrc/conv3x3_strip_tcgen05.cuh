@@ -172,7 +172,7 @@ conv3x3_strip_bf16_tcgen05(const __grid_constant__ Conv3Batch B, const __grid_co
         if (p.in_ids) img = p.in_ids[img];
         for (int i = row - 1; i <= row + len; ++i, ++n) {
           const int s = n % ST;
-          if (n >= ST) ptx::mbar_wait_elect(&empty[s], ((n / ST) - 1) & 1, dead);
+          if (n >= ST) ptx::mbar_wait_warp(&empty[s], ((n / ST) - 1) & 1, dead);
           ptx::mbar_expect_tx(one, &full[s], C3_A_BYTES);
           ptx::tma_load_4d(one, rows + s * C3_A_SLOT, &B.tx[rq], 0, w0 - 1, i, img, &full[s]);
         }
@@ -181,14 +181,15 @@ conv3x3_strip_bf16_tcgen05(const __grid_constant__ Conv3Batch B, const __grid_co
     }
   } else if (warp == 1 || warp == 3) {
     {
-      // ---- MMA issuers: rows alternate between two threads.  A row starts when the row before has completed: its issuer
+      // ---- MMA issuers: rows alternate between the leading lanes of two warps.  A row starts when the row before has completed: its issuer
       // commits to this one's `turn`, so the commit of an output row also covers what the other thread issued for it.  The
       // next row's thread has done its address arithmetic and its other waits by then.  (A thread may wait on `full` and
       // `tmem_empty` for its own rows only: its row n - 2 was issued after every earlier row had seen its barriers, so at row
-      // n each barrier is at most one phase away from the one waited for.)
+      // n each barrier is at most one phase away from the one waited for.  A warp's other lanes have left its waits before
+      // it commits, so they are no further behind.)
       // Output row o of the segment accumulates in block (j + o) % 8; input row ii (counted from the row above the segment)
       // gives to the output rows ii - 2 (dy = 2), ii - 1 and ii, as far as they belong to the segment.
-      ptx::mbar_wait_elect(w_full, 0, dead);
+      ptx::mbar_wait_lanes(w_full, 0, dead);
       const uint64_t wdesc = ptx::smem_desc_sw128(ptx::smem_u32(wres));
       const ptx::Leader one = ptx::elect_leader();
       const auto mma_commit = [&](uint64_t* bar) { ptx::mma_commit(one, bar); };
@@ -207,12 +208,12 @@ conv3x3_strip_bf16_tcgen05(const __grid_constant__ Conv3Batch B, const __grid_co
           const int c1 = min(cnt, NB - b0), c2 = cnt - c1;            // blocks before and behind the ring's end
           const uint64_t wb = wdesc + (lo - (ii - 2)) * (STRIP_TAP >> 4);
           const uint32_t d1 = tmem + b0 * 64;
-          if (fresh) ptx::mbar_wait_elect(&tmem_empty[(j + ii) % NB], ((j + ii) / NB) & 1, dead);
-          ptx::mbar_wait_elect(&full[s], (n / ST) & 1, dead);
+          if (fresh) ptx::mbar_wait_lanes(&tmem_empty[(j + ii) % NB], ((j + ii) / NB) & 1, dead);
+          ptx::mbar_wait_lanes(&full[s], (n / ST) & 1, dead);
           const uint64_t ad = ptx::smem_desc_sw128(ptx::smem_u32(rows + s * C3_A_SLOT));
           const uint32_t a_lo = static_cast<uint32_t>(ad), b_lo = static_cast<uint32_t>(wb);
           uint64_t* const done = &tmem_full[(j + ii + NB - 2) % NB];
-          if (n > 0) ptx::mbar_wait_elect(&turn[me], me ? (n >> 1) & 1 : ((n >> 1) - 1) & 1, dead);
+          if (n > 0) ptx::mbar_wait_lanes(&turn[me], me ? (n >> 1) & 1 : ((n >> 1) - 1) & 1, dead);
           ptx::tc_fence_after();
           if (c1 == 3) strip_row<3, 0>(one, d1, tmem, a_lo, b_lo);
           else
@@ -223,6 +224,7 @@ conv3x3_strip_bf16_tcgen05(const __grid_constant__ Conv3Batch B, const __grid_co
               case 5: strip_row<1, 1>(one, d1, tmem, a_lo, b_lo); break;
               case 4: strip_row<1, 0>(one, d1, tmem, a_lo, b_lo); break;
             }
+          __syncwarp();
           mma_commit(&turn[me ^ 1]);
           mma_commit(&empty[s]);
           if (ii >= 2) mma_commit(done);
@@ -270,7 +272,7 @@ conv3x3_strip_bf16_tcgen05(const __grid_constant__ Conv3Batch B, const __grid_co
       for (int u = 0; u < NSB && u < U; ++u) prepare(u);
       for (int u = 0; u < U; ++u) {
         const int bsel = u % NSB;
-        ptx::mbar_wait_elect(&stage_ready[bsel], (u / NSB) & 1, dead);
+        ptx::mbar_wait_lanes(&stage_ready[bsel], (u / NSB) & 1, dead);
         if (ptx::elect_one()) {        // (always the same lane: bulk groups belong to a thread)
           tma_store_4d(&B.to[out.rq], out_stage + bsel * CONV_STAGE_OUT, 0, out.w0, out.row, out.img);
           bulk_commit();

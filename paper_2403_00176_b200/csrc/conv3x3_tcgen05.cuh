@@ -120,7 +120,7 @@ conv3x3_rows_bf16_tcgen05(const __grid_constant__ Conv3Batch B, const __grid_con
       if (p.in_ids) img = p.in_ids[img];
       for (int ks = 0; ks < kstages; ++ks, ++n) {
         const int s = n % STAGES;
-        if (n >= STAGES) ptx::mbar_wait_elect(&empty[s], ((n / STAGES) - 1) & 1, dead);
+        if (n >= STAGES) ptx::mbar_wait_warp(&empty[s], ((n / STAGES) - 1) & 1, dead);
         const int dy = ks / cchunks, cc = ks % cchunks;
         SOD2_TRACE(0, 100 + ks)
         ptx::mbar_expect_tx(one, &full[s], C3_A_BYTES);
@@ -135,7 +135,7 @@ conv3x3_rows_bf16_tcgen05(const __grid_constant__ Conv3Batch B, const __grid_con
       const int n0 = (t / tiles_px) * BN;
       for (int ks = 0; ks < kstages; ++ks, ++n) {
         const int s = n % STAGES;
-        if (n >= STAGES) ptx::mbar_wait_elect(&empty[s], ((n / STAGES) - 1) & 1, dead);
+        if (n >= STAGES) ptx::mbar_wait_warp(&empty[s], ((n / STAGES) - 1) & 1, dead);
         ptx::mbar_expect_tx(one, &full[s], 3 * BN * 128);
         ptx::tma_load_3d(one, tiles + s * S::STAGE_BYTES + C3_A_SLOT, &tmW, 0, n0, ks * 3, &full[s]);
       }
@@ -157,14 +157,17 @@ conv3x3_rows_bf16_tcgen05(const __grid_constant__ Conv3Batch B, const __grid_con
         const int acc = j & 1;
         const bool mine = acc == me;
         if (mine) {
-          if (j >= 2) ptx::mbar_wait_elect(&tmem_empty[acc], ((j >> 1) - 1) & 1, dead);
+          if (j >= 2) ptx::mbar_wait_lanes(&tmem_empty[acc], ((j >> 1) - 1) & 1, dead);
           ptx::tc_fence_after();
         }
         const uint32_t d = tmem + acc * BN;
         for (int ks = 0; ks < kstages; ++ks, ++n) {
           const int s = n % STAGES;
-          ptx::mbar_wait_elect(&full[s], (n / STAGES) & 1, dead);
-          if (!mine) continue;
+          if (!mine) {
+            ptx::mbar_wait_warp(&full[s], (n / STAGES) & 1, dead);
+            continue;
+          }
+          ptx::mbar_wait_lanes(&full[s], (n / STAGES) & 1, dead);
           ptx::tc_fence_after();
           if (me == 0) { SOD2_TRACE(1, 200 + ks) }
           const uint32_t a = ptx::smem_u32(tiles + s * S::STAGE_BYTES);
@@ -176,6 +179,7 @@ conv3x3_rows_bf16_tcgen05(const __grid_constant__ Conv3Batch B, const __grid_con
 #pragma unroll
             for (int kk = 0; kk < 4; ++kk) ptx::mma_bf16(one, d, ad + 2 * kk, bd + 2 * kk, idesc, (ks | dx | kk) != 0);
           }
+          __syncwarp();
           ptx::mma_commit(one, &empty[s]);
           if (ks + 1 == kstages) ptx::mma_commit(one, &tmem_full[acc]);
         }
@@ -207,7 +211,7 @@ conv3x3_rows_bf16_tcgen05(const __grid_constant__ Conv3Batch B, const __grid_con
     if (ptx::elect_one()) { for (int u = 0; u < NSB && u < U; ++u) prepare(u); }
     for (int u = 0; u < U; ++u) {
       const int bsel = u % NSB;
-      ptx::mbar_wait_elect(&stage_ready[bsel], (u / NSB) & 1, dead);
+      ptx::mbar_wait_lanes(&stage_ready[bsel], (u / NSB) & 1, dead);
       const int t = blockIdx.x + (u / PASSES) * gridDim.x;
       int n0, img, h0, w0;
       const int rq = decode(t, &n0, &img, &h0, &w0);

@@ -252,14 +252,14 @@ conv_stem_bf16_tcgen05(const __grid_constant__ CUtensorMap tmW, const __grid_con
       // ---- MMA issuer
       constexpr uint32_t idesc = ptx::idesc_bf16(128, 64);
       const ptx::Leader one = ptx::elect_leader();
-      ptx::mbar_wait_elect(w_full, 0, dead);
+      ptx::mbar_wait_lanes(w_full, 0, dead);
       const uint32_t aW = ptx::smem_u32(sW);
       int it = 0;
       for (int t = blockIdx.x; t < n_tiles; t += gridDim.x, ++it) {
         const int b = it & 1;
-        ptx::mbar_wait_elect(&a_full[b], (it >> 1) & 1, dead);
+        ptx::mbar_wait_lanes(&a_full[b], (it >> 1) & 1, dead);
         SOD2_TRACE(1, 40)
-        if (it >= 2) ptx::mbar_wait_elect(&acc_free[b], ((it >> 1) - 1) & 1, dead);
+        if (it >= 2) ptx::mbar_wait_lanes(&acc_free[b], ((it >> 1) - 1) & 1, dead);
         SOD2_TRACE(1, 41)
         ptx::tc_fence_after();
         const uint32_t aA = ptx::smem_u32(sA + b * STEM_A_BYTES);
@@ -269,6 +269,7 @@ conv_stem_bf16_tcgen05(const __grid_constant__ CUtensorMap tmW, const __grid_con
 #pragma unroll
           for (int kk = 0; kk < 4; ++kk) ptx::mma_bf16(one, tmem + b * 64, ad + 2 * kk, bd + 2 * kk, idesc, (c | kk) != 0);
         }
+        __syncwarp();
         ptx::mma_commit(one, &a_free[b]);
         ptx::mma_commit(one, &acc_full[b]);
         SOD2_TRACE(1, 42)

@@ -181,7 +181,7 @@ conv_igemm_bf16_tcgen05(const __grid_constant__ CUtensorMap tmX, const __grid_co
       if (p.in_ids) img = p.in_ids[img];
       for (int ks = 0; ks < kstages; ++ks, ++n) {
         const int s = n % STAGES;
-        if (n >= STAGES) ptx::mbar_wait_elect(&empty[s], ((n / STAGES) - 1) & 1, dead);
+        if (n >= STAGES) ptx::mbar_wait_warp(&empty[s], ((n / STAGES) - 1) & 1, dead);
         int mine = 0;
         for (int c = warp; c < KCH; c += 2) ++mine;
         ptx::mbar_expect_tx(one, &full[s], mine * 128 * 128);
@@ -204,7 +204,7 @@ conv_igemm_bf16_tcgen05(const __grid_constant__ CUtensorMap tmX, const __grid_co
       const int n0 = (t / tiles_px) * BN;
       for (int ks = 0; ks < kstages; ++ks, ++n) {
         const int s = n % STAGES;
-        if (n >= STAGES) ptx::mbar_wait_elect(&empty[s], ((n / STAGES) - 1) & 1, dead);
+        if (n >= STAGES) ptx::mbar_wait_warp(&empty[s], ((n / STAGES) - 1) & 1, dead);
         ptx::mbar_expect_tx(one, &full[s], S::B_BYTES);
         ptx::tma_load_3d(one, tiles + s * S::STAGE_BYTES + S::A_BYTES, &tmW, 0, n0, ks * KCH, &full[s]);
       }
@@ -221,11 +221,11 @@ conv_igemm_bf16_tcgen05(const __grid_constant__ CUtensorMap tmX, const __grid_co
       int j = 0;
       for (int t = blockIdx.x; t < num_tiles; t += gridDim.x, ++j) {
         const int acc = j & 1;
-        if (j >= 2) ptx::mbar_wait_elect(&tmem_empty[acc], ((j >> 1) - 1) & 1, dead);
+        if (j >= 2) ptx::mbar_wait_lanes(&tmem_empty[acc], ((j >> 1) - 1) & 1, dead);
         ptx::tc_fence_after();
         const uint32_t d = tmem + acc * BN;
         for (int ks = 0; ks < kstages; ++ks) {
-          ptx::mbar_wait_elect(&full[s], par, dead);
+          ptx::mbar_wait_lanes(&full[s], par, dead);
           ptx::tc_fence_after();
           const uint64_t ad = a0 + s * (S::STAGE_BYTES >> 4), bd = b0 + s * (S::STAGE_BYTES >> 4);
 #pragma unroll
@@ -236,6 +236,7 @@ conv_igemm_bf16_tcgen05(const __grid_constant__ CUtensorMap tmX, const __grid_co
 #pragma unroll
               for (int kk = 0; kk < 4; ++kk) ptx::mma_bf16(one, d, ad + c * (128 * 8) + 2 * kk, bd + c * (BN * 8) + 2 * kk, idesc, 1);
           }
+          __syncwarp();
           ptx::mma_commit(one, &empty[s]);
           if (++s == STAGES) { s = 0; par ^= 1; }
         }

@@ -87,7 +87,7 @@ gemm_cluster_bf16_tcgen05(const __grid_constant__ CUtensorMap tmA, const __grid_
     const ptx::Leader one = ptx::elect_leader();
     for (int n = 0; n < kn; ++n) {
       const int s = n % STAGES;
-      if (n >= STAGES) ptx::mbar_wait_elect(&empty[s], ((n / STAGES) - 1) & 1, dead);
+      if (n >= STAGES) ptx::mbar_wait_warp(&empty[s], ((n / STAGES) - 1) & 1, dead);
       uint8_t* st = tiles + s * L::STAGE_BYTES;
       ptx::mbar_expect_tx(one, &full[s], warp == 0 ? L::A_BYTES : L::B_BYTES);
       if (warp == 0) ptx::tma_load_3d(one, st, &tmA, 0, m0, k0 + n, &full[s]);
@@ -101,11 +101,12 @@ gemm_cluster_bf16_tcgen05(const __grid_constant__ CUtensorMap tmA, const __grid_
     const uint64_t a0 = ptx::smem_desc_sw128(ptx::smem_u32(tiles)), b0 = ptx::smem_desc_sw128(ptx::smem_u32(tiles + L::A_BYTES));
     uint32_t s = 0, par = 0;
     for (int n = 0; n < kn; ++n) {
-      ptx::mbar_wait_elect(&full[s], par, dead);
+      ptx::mbar_wait_lanes(&full[s], par, dead);
       ptx::tc_fence_after();
       const uint64_t ad = a0 + s * (L::STAGE_BYTES >> 4), bd = b0 + s * (L::STAGE_BYTES >> 4);
 #pragma unroll
       for (int kk = 0; kk < 4; ++kk) ptx::mma_bf16(one, tmem, ad + 2 * kk, bd + 2 * kk, idesc, n != 0 || kk != 0);
+      __syncwarp();
       ptx::mma_commit(one, &empty[s]);
       if (++s == STAGES) { s = 0; par ^= 1; }
     }

@@ -209,7 +209,7 @@ gemm_pair_bf16_tcgen05(const __grid_constant__ CUtensorMap tmA, const __grid_con
       const int m0 = (wk.m * 2 + static_cast<int>(rank)) * GEMM_BM;
       for (int ks = 0; ks < kstages; ++ks, ++n) {
         const int s = n % STAGES;
-        if (n >= STAGES) ptx::mbar_wait_elect(&empty[s], ((n / STAGES) - 1) & 1, dead);
+        if (n >= STAGES) ptx::mbar_wait_warp(&empty[s], ((n / STAGES) - 1) & 1, dead);
         SOD2_PAIR_TRACE(0, n)
         if (leader) ptx::mbar_expect_tx(one, &full[s], 2 * S::A_BYTES);
         tma_load_3d_pair(one, tiles + s * S::STAGE_BYTES, &tmA, 0, m0, ks, map_to_cta(ptx::smem_u32(&full[s]), 0));
@@ -224,7 +224,7 @@ gemm_pair_bf16_tcgen05(const __grid_constant__ CUtensorMap tmA, const __grid_con
       const CUtensorMap* tmB = &maps.b[wk.w - 1];
       for (int ks = 0; ks < kstages; ++ks, ++n) {
         const int s = n % STAGES;
-        if (n >= STAGES) ptx::mbar_wait_elect(&empty[s], ((n / STAGES) - 1) & 1, dead);
+        if (n >= STAGES) ptx::mbar_wait_warp(&empty[s], ((n / STAGES) - 1) & 1, dead);
         if (leader) ptx::mbar_expect_tx(one, &full[s], 2 * wk.w * (32 * 128));
         tma_load_3d_pair(one, tiles + s * S::STAGE_BYTES + S::A_BYTES, tmB, 0, n0, ks, map_to_cta(ptx::smem_u32(&full[s]), 0));
       }
@@ -239,16 +239,17 @@ gemm_pair_bf16_tcgen05(const __grid_constant__ CUtensorMap tmA, const __grid_con
       for (PairWalk wk = share; wk.next(); ++j) {
         const int acc = j & 1;
         const uint32_t idesc = ptx::idesc_bf16(2 * GEMM_BM, 64 * wk.w);
-        if (j >= 2) ptx::mbar_wait_elect(&tmem_empty[acc], ((j >> 1) - 1) & 1, dead);
+        if (j >= 2) ptx::mbar_wait_lanes(&tmem_empty[acc], ((j >> 1) - 1) & 1, dead);
         ptx::tc_fence_after();
         const uint32_t d = tmem + acc * BN;
         for (int ks = 0; ks < kstages; ++ks) {
-          ptx::mbar_wait_elect(&full[s], par, dead);
+          ptx::mbar_wait_lanes(&full[s], par, dead);
           ptx::tc_fence_after();
           SOD2_PAIR_TRACE(1, ks)
           const uint64_t ad = a0 + s * (S::STAGE_BYTES >> 4), bd = b0 + s * (S::STAGE_BYTES >> 4);
 #pragma unroll
           for (int kk = 0; kk < 4; ++kk) mma_bf16_pair(one, d, ad + 2 * kk, bd + 2 * kk, idesc, (ks > 0) || kk != 0);
+          __syncwarp();
           mma_commit_pair(one, &empty[s]);     // frees the stage in both CTAs
           if (++s == STAGES) { s = 0; par ^= 1; }
         }
@@ -283,7 +284,7 @@ gemm_pair_bf16_tcgen05(const __grid_constant__ CUtensorMap tmA, const __grid_con
     for (int u = 0; out.live; ++u, out.step()) {
       const int bsel = u % NSB;
       const int m0 = (out.wk.m * 2 + static_cast<int>(rank)) * GEMM_BM, np = out.wk.n0 + out.ps * GEMM_PASS_COLS;
-      ptx::mbar_wait_elect(&buf_filled[bsel], (u / NSB) & 1, dead);
+      ptx::mbar_wait_lanes(&buf_filled[bsel], (u / NSB) & 1, dead);
       if (ptx::elect_one()) {        // (always the same lane: bulk groups belong to a thread)
         if (m0 < M) {
           tma_store_2d(&tmOut, out_stage + bsel * GEMM_STAGE_OUT, np, m0);

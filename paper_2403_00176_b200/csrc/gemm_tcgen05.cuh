@@ -242,7 +242,7 @@ gemm_bf16_tcgen05(const __grid_constant__ CUtensorMap tmA, const __grid_constant
       k_range(w, &ks0, &ks1);
       for (int ks = ks0; ks < ks1; ++ks, ++n) {
         const int s = n % STAGES;
-        if (n >= STAGES) ptx::mbar_wait_elect(&empty[s], ((n / STAGES) - 1) & 1, dead);
+        if (n >= STAGES) ptx::mbar_wait_warp(&empty[s], ((n / STAGES) - 1) & 1, dead);
         if (n == 0) { SOD2_TRACE(0, 2) }
         ptx::mbar_expect_tx(one, &full[s], S::A_BYTES);
         ptx::tma_load_3d(one, tiles + s * S::STAGE_BYTES, &tmA, 0, m0, ks * KCH, &full[s]);
@@ -259,7 +259,7 @@ gemm_bf16_tcgen05(const __grid_constant__ CUtensorMap tmA, const __grid_constant
       k_range(w, &ks0, &ks1);
       for (int ks = ks0; ks < ks1; ++ks, ++n) {
         const int s = n % STAGES;
-        if (n >= STAGES) ptx::mbar_wait_elect(&empty[s], ((n / STAGES) - 1) & 1, dead);
+        if (n >= STAGES) ptx::mbar_wait_warp(&empty[s], ((n / STAGES) - 1) & 1, dead);
         ptx::mbar_expect_tx(one, &full[s], S::B_BYTES);
         ptx::tma_load_3d(one, tiles + s * S::STAGE_BYTES + S::A_BYTES, &tmB, 0, n0, ks * KCH, &full[s]);
       }
@@ -277,14 +277,14 @@ gemm_bf16_tcgen05(const __grid_constant__ CUtensorMap tmA, const __grid_constant
     int j = 0;
     for (int w = blockIdx.x; w < num_tiles; w += gridDim.x, ++j) {
       const int acc = j & 1;
-      if (j >= 2) ptx::mbar_wait_elect(&tmem_empty[acc], ((j >> 1) - 1) & 1, dead);
+      if (j >= 2) ptx::mbar_wait_lanes(&tmem_empty[acc], ((j >> 1) - 1) & 1, dead);
       ptx::tc_fence_after();
       const uint32_t d = tmem + acc * BN;
       int ks0, ks1;
       k_range(w, &ks0, &ks1);
       SOD2_TRACE(1, 10 + j)
       for (int ks = ks0; ks < ks1; ++ks) {
-        ptx::mbar_wait_elect(&full[s], par, dead);
+        ptx::mbar_wait_lanes(&full[s], par, dead);
         ptx::tc_fence_after();
         const uint64_t ad = a0 + s * (S::STAGE_BYTES >> 4), bd = b0 + s * (S::STAGE_BYTES >> 4);
 #pragma unroll
@@ -295,6 +295,7 @@ gemm_bf16_tcgen05(const __grid_constant__ CUtensorMap tmA, const __grid_constant
 #pragma unroll
             for (int kk = 0; kk < 4; ++kk) ptx::mma_bf16(one, d, ad + c * (GEMM_BM * 8) + 2 * kk, bd + c * (BN * 8) + 2 * kk, idesc, 1);
         }                                 // (K ends inside the stage: KCH is 2 at most)
+        __syncwarp();                     // every lane has left the wait (mbar_wait_lanes)
         ptx::mma_commit(one, &empty[s]);  // frees the stage once these MMAs have read it
         if (++s == STAGES) { s = 0; par ^= 1; }
       }
@@ -328,7 +329,7 @@ gemm_bf16_tcgen05(const __grid_constant__ CUtensorMap tmA, const __grid_constant
     if ((SPLITK || RES) && ptx::elect_one()) { for (int u = 0; u < NSB && u < U; ++u) prepare(u); }   // else: done at barrier initialisation
     for (int u = 0; u < U; ++u) {
       const int bsel = u % NSB;
-      ptx::mbar_wait_elect(&buf_filled[bsel], (u / NSB) & 1, dead);
+      ptx::mbar_wait_lanes(&buf_filled[bsel], (u / NSB) & 1, dead);
       const int w = blockIdx.x + (u / PASSES) * gridDim.x;
       const int t = SPLITK ? w % out_tiles : w;
       const int m0 = (t % tiles_m) * GEMM_BM, np = (t / tiles_m) * BN + (u % PASSES) * PASS_COLS;

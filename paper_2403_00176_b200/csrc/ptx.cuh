@@ -96,10 +96,12 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volati
 // diverges.  Measured on B200 (ping-pong between two warps, cycles per hand-over): 125, against 231 where a role runs
 // under lane == 0 and 266 where lane 0 polls and the warp joins it; through tcgen05.commit 133 against 365 and 244.  Must
 // be called by all 32 lanes.
-// Lanes may in principle see the phase end at different tests.  `mbar_wait_elect` is for a warp whose next step is
-// elect_one(), which brings the lanes together; `mbar_wait_warp` does it itself, for what wants a warp in step at once
-// (tcgen05.ld and .st).  A __syncwarp in each wait of the producers and issuers cost a 64-token GEMM 0.2 us (of 7.5).
-__device__ __forceinline__ void mbar_wait_elect(uint64_t* bar, uint32_t parity, volatile int* dead) {
+// Lanes may see the phase end at different tests.  `mbar_wait_warp` brings them together behind the wait; `mbar_wait_lanes` leaves that
+// to its caller, who does it (__syncwarp, elect_one) before anything that lets the barrier's next phase end: the commit or
+// arrival by which a ring goes on.  A lane still in the wait would else be lost there: the parity of two phases on looks like that
+// of the phase before the awaited one.  MMA issuers have their __syncwarp between a stage's MMAs and its commit, where the
+// pipe has work: the encoder of one request 184.9 -> 185.7 us; as a vote on each test, in front of the MMAs, 187.1 -> 192.0.
+__device__ __forceinline__ void mbar_wait_lanes(uint64_t* bar, uint32_t parity, volatile int* dead) {
   if (__builtin_expect(mbar_test_wait(bar, parity), 1)) return;
   const long long give_up = clock64() + SOD2_WAIT_CYCLES;
 #pragma unroll 1
@@ -109,7 +111,7 @@ __device__ __forceinline__ void mbar_wait_elect(uint64_t* bar, uint32_t parity, 
   }
 }
 __device__ __forceinline__ void mbar_wait_warp(uint64_t* bar, uint32_t parity, volatile int* dead) {
-  mbar_wait_elect(bar, parity, dead);
+  mbar_wait_lanes(bar, parity, dead);
   __syncwarp();
 }
 // Whether the phase has ended, the same answer in every lane: what a warp may branch on around a wait, a tcgen05.ld or a
@@ -183,7 +185,8 @@ __device__ __forceinline__ bool elect_one() {
 // 190 cycles per stage beside the pipe.  Measured on B200 (cycles per MMA with a satisfied wait and a commit per stage, branch ->
 // predicate; the pipe takes 48 at N = 64, 64 at 128): N = 64 in stages of 4 / 8 / 12 MMAs 93 / 72 / 63 -> 61 / 51 / 52, N = 128
 // 97 / 82 / 75 -> 64 / 64 / 64; from N = 192 on the pipe hides either.  A warp whose lanes have seen a phase end at different
-// tests may run a stage's instructions in parts: the leader's are issued once, behind the leader's own test.
+// tests may run a stage's instructions in parts: the leader's are issued once, behind the leader's own test, and its commit
+// waits for the other lanes (mbar_wait_lanes).
 struct Leader { uint32_t on; };
 __device__ __forceinline__ Leader elect_leader() { return Leader{elect_one() ? 1u : 0u}; }
 __device__ __forceinline__ void mbar_expect_tx(Leader l, uint64_t* bar, uint32_t bytes) {

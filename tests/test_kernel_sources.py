@@ -27,3 +27,31 @@ def test_strip_convolution_orders_rows_by_completion():
     text = dict(_sources())["conv3x3_strip_tcgen05.cuh"]
     assert "mma_commit(&turn[me ^ 1])" in text and not re.search(r"mbar_arrive\w*\(&turn", text)
     assert re.search(r"tcgen05\.mma\.[^;]*%3, 1;", text) and len(re.findall(r"tcgen05\.mma\.", text)) == 1
+
+
+def test_warps_are_together_before_a_ring_goes_on():
+    # a role whose leading lane issues behind predicates has nothing but its waits to keep the other lanes from falling behind, and a
+    # lane two phases behind waits for a parity that looks like one it has seen.  Behind a wait that lanes leave one by one, the
+    # warp is brought together before the commit, arrival or load that lets the barrier's next phase end
+    sources = dict(_sources())
+    assert set(re.findall(r"\bvoid (mbar_wait\w*)\(", sources["ptx.cuh"])) == {"mbar_wait_lanes", "mbar_wait_warp"}
+    assert re.search(r"void mbar_wait_warp\([^)]*\) \{\s*mbar_wait_lanes\(bar, parity, dead\);\s*__syncwarp\(\);\s*\}", sources["ptx.cuh"])
+    events = r"\b(mbar_wait_lanes|mbar_wait_warp|__syncwarp|elect_one|elect_leader|mma_commit(?:_pair)?|mbar_arrive\w*|mbar_expect_tx|tma_load_\w+|bulk_commit|continue|void)\b[ (]"
+    users = 0
+    for name, text in sources.items():
+        if name == "ptx.cuh":
+            continue
+        apart = None
+        for m in re.finditer(events, text):
+            what, line = m.group(1), text[:m.start()].count("\n") + 1
+            if what == "mbar_wait_lanes":
+                apart, users = line, users + 1
+            elif what in ("mbar_wait_warp", "__syncwarp", "elect_one", "elect_leader", "void"):
+                apart = None
+            else:
+                assert apart is None, (name, apart, line, what)
+        assert apart is None, (name, apart)
+    assert users >= 15
+    # waits of single threads: only in kernels that have roles under one lane
+    assert {f for f, text in sources.items() if re.search(r"\bmbar_wait(_limited)?\(", text)} == {
+        "ptx.cuh", "gemm_chain_tcgen05.cuh", "conv_stem_tcgen05.cuh", "selftest_mma.cu", "noalloc.cu"}
