@@ -27,6 +27,9 @@ namespace ptx {
 // the predecessor grid has completed and its memory is visible.  Every such kernel calls pdl_wait()
 // in all threads before it touches global memory written or read by earlier kernels, so completion
 // stays transitive along the stream.  pdl_launch() lets the successor's CTAs be scheduled early.
+// Constants of the graph and packed weights may be read ahead of it: no kernel of a run writes them, and such a kernel is in a
+// run whose first launch (what clears the arena header: a memset, or a kernel that waits before it signals) lets nothing start before
+// all earlier work on the stream has ended.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 

@@ -55,3 +55,18 @@ def test_warps_are_together_before_a_ring_goes_on():
     # waits of single threads: only in kernels that have roles under one lane
     assert {f for f, text in sources.items() if re.search(r"\bmbar_wait(_limited)?\(", text)} == {
         "ptx.cuh", "gemm_chain_tcgen05.cuh", "conv_stem_tcgen05.cuh", "selftest_mma.cu", "noalloc.cu"}
+
+
+def test_a_run_starts_behind_everything_before_it():
+    # kernels read constants and packed weights ahead of their dependency wait and let their successors start early; what a caller did on
+    # the stream before the run (update a constant, prepack) is ordered by the run's first launch: nothing starts before that has waited
+    sources = dict(_sources())
+    text = sources["exec.cu"]
+    assert re.search(r"void __launch_bounds__\(128\) clear_header\([^)]*\) \{\s*ptx::pdl_wait\(\);\s*ptx::pdl_launch\(\);", text)
+    body = re.search(r"\nStatus run_plan\(.*?\n\}", text, re.S).group(0)
+    first = body.index("L->fn(xs)")
+    assert body.index("if (p->uses_header && step_lo <= 0)") < body.index("launch_pdl(clear_header") < first and body.index("cudaMemsetAsync(arena") < first
+    # kernels of plans without a header read nothing ahead: those that are programmatic dependents wait before their first load
+    for name, kernel in (("kernels_rows.cuh", "chain_elementwise"), ("kernels_compact.cuh", "nonzero_mask"), ("kernels_compact.cuh", "nonzero_write")):
+        body = re.search(r"\b%s\(.*?ptx::pdl_wait\(\);" % kernel, sources[name], re.S).group(0)
+        assert not re.search(r"->|= ?\*|reinterpret_cast", body), (kernel, body)
