@@ -397,7 +397,8 @@ def run_ours(args):
                     "gpu_launches": r["gpu_launches"], "units": r["units_batch0"], "unit": r["unit"],
                     **{k: r[k] for k in ("ms_one_request_per_inference", "ms_empty_kernel", "ratio_to_empty_kernel", "exact_edo") if k in r}}
             line["configs_note"] = ("ms / ms_graph: device time per inference (median, L2 flushed), stream-launched / replayed as one CUDA graph; "
-                                    "e2e_ms: pinned H2D + bind + plan + run + D2H; group figures: CUDA events around every launch")
+                                    "e2e_ms: pinned H2D + bind + plan + run + D2H; group figures: CUDA events around every launch; "
+                                    "sum_t_roof_over_*: null where samples skip blocks (group costs are counted at the upper bounds)")
         print(json.dumps(line))
     if world > 1:
         dist.destroy_process_group()
