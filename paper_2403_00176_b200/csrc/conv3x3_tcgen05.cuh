@@ -35,7 +35,7 @@ template <int BN, int STAGES>
 struct Conv3Smem {
   static constexpr int STAGE_BYTES = C3_A_SLOT + 3 * BN * 128;
   static constexpr int NSB = BN == 128 ? 1 : 2;   // staging buffers (what fits next to the ring)
-  static constexpr int TOTAL = STAGES * STAGE_BYTES + NSB * CONV_STAGE_OUT + 896 + 2048 + 128;
+  static constexpr int TOTAL = STAGES * STAGE_BYTES + NSB * CONV_STAGE_OUT + 2048 /*bias*/ + 8 * (2 * STAGES + 10) + 16 + 1024 /*alignment*/;
 };
 
 // B.tx: {Cin, W, H, N}, box {64, 130, 1, 1};  tmW: k-chunk view {64, Cout, K/64} of the weights in
@@ -58,7 +58,8 @@ conv3x3_rows_bf16_tcgen05(const __grid_constant__ Conv3Batch B, const __grid_con
   uint64_t* tmem_empty = tmem_full + 2;
   uint64_t* res_full = tmem_empty + 2;
   uint64_t* stage_ready = res_full + 2;
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(stage_ready + 2);
+  uint64_t* turn = stage_ready + 2;       // [2] per issuer
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(turn + 2);
   volatile int* dead = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -67,7 +68,7 @@ conv3x3_rows_bf16_tcgen05(const __grid_constant__ Conv3Batch B, const __grid_con
   if (threadIdx.x == 0) {
     for (int s = 0; s < STAGES; ++s) { ptx::mbar_init(&full[s], 2); ptx::mbar_init(&empty[s], 1); }
     for (int b = 0; b < 2; ++b) { ptx::mbar_init(&tmem_full[b], 1); ptx::mbar_init(&tmem_empty[b], 8); }
-    for (int b = 0; b < 2; ++b) { ptx::mbar_init(&res_full[b], 1); ptx::mbar_init(&stage_ready[b], 8); }
+    for (int b = 0; b < 2; ++b) { ptx::mbar_init(&res_full[b], 1); ptx::mbar_init(&stage_ready[b], 8); ptx::mbar_init(&turn[b], 1); }
     *dead = 0;
     ptx::fence_barrier_init();
     ptx::fence_proxy_async();
@@ -145,29 +146,28 @@ conv3x3_rows_bf16_tcgen05(const __grid_constant__ Conv3Batch B, const __grid_con
       // ---- two MMA issuers: warp 3 takes this CTA's even tiles (accumulator 0), warp 12 the odd ones
       // (accumulator 1).  A thread that waits on a barrier between MMAs leaves the tensor pipe idle for a
       // few hundred cycles; with two issuers one thread's wait is covered by the other's MMAs.  Both
-      // consume the same ring, stage n = j * kstages + ks of tile j, and BOTH wait on every stage in
-      // order, also on the other issuer's: a parity wait is only meaningful for a thread that has seen
-      // the barrier's previous phase, and walking all stages keeps each issuer exactly in step (the
-      // in-order producer cannot refill a slot twice while an issuer still owns an earlier stage).
+      // consume the same ring, stage n = j * kstages + ks of tile j.  A parity wait is only meaningful for a
+      // thread that knows the barrier's previous phase to have ended: the other issuer passes `turn` when it has
+      // seen its tile's last stage, and no stage of the own tile can be refilled before its own commit.
+      // (Walking the other's stages instead is no such knowledge: a warp held up there for as long as
+      // a refill takes finds the parity turned.)
       constexpr uint32_t idesc = ptx::idesc_bf16(128, BN);
       const ptx::Leader one = ptx::elect_leader();
       const int me = warp == 3 ? 0 : 1;
       int n = 0, j = 0;
       for (int t = blockIdx.x; t < num_tiles; t += gridDim.x, ++j) {
         const int acc = j & 1;
-        const bool mine = acc == me;
-        if (mine) {
-          if (j >= 2) ptx::mbar_wait_lanes(&tmem_empty[acc], ((j >> 1) - 1) & 1, dead);
-          ptx::tc_fence_after();
-        }
+        if (acc != me) { n += kstages; continue; }
+        if (j >= 1) ptx::mbar_wait_warp(&turn[me], me ? (j >> 1) & 1 : ((j >> 1) - 1) & 1, dead);
+        if (j >= 2) ptx::mbar_wait_warp(&tmem_empty[acc], ((j >> 1) - 1) & 1, dead);
         const uint32_t d = tmem + acc * BN;
         for (int ks = 0; ks < kstages; ++ks, ++n) {
           const int s = n % STAGES;
-          if (!mine) {
-            ptx::mbar_wait_warp(&full[s], (n / STAGES) & 1, dead);
-            continue;
-          }
           ptx::mbar_wait_lanes(&full[s], (n / STAGES) & 1, dead);
+          if (ks + 1 == kstages) {
+            __syncwarp();
+            if (lane == 0) ptx::mbar_arrive(&turn[me ^ 1]);
+          }
           ptx::tc_fence_after();
           if (me == 0) { SOD2_TRACE(1, 200 + ks) }
           const uint32_t a = ptx::smem_u32(tiles + s * S::STAGE_BYTES);
@@ -183,7 +183,7 @@ conv3x3_rows_bf16_tcgen05(const __grid_constant__ Conv3Batch B, const __grid_con
           ptx::mma_commit(one, &empty[s]);
           if (ks + 1 == kstages) ptx::mma_commit(one, &tmem_full[acc]);
         }
-        if (mine && me == 0) { SOD2_TRACE(1, 210) }
+        if (me == 0) { SOD2_TRACE(1, 210) }
       }
     }
   } else if (warp == 2) {

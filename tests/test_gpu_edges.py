@@ -98,6 +98,19 @@ def test_conv_halo_patches(C, shapes):
         assert all(np.array_equal(a[n], b[n]) for n in a)
 
 
+@pytest.mark.parametrize("C,H,W", [(128, 310, 110), (192, 450, 128), (128, 5, 103)])
+def test_conv_row_tiles_handed_over_between_issuers(C, H, W):
+    # row tiles of 128 and 64 channels: three and ten tiles for some CTAs (both issuers in turn, accumulators and ring reused), one for
+    # others, with a residual
+    wl = WL.cfg4(blocks=1, C=C)
+    rng = np.random.default_rng(73)
+    req = Request({"H": H, "W": W}, {"x": bf16_round(rng.uniform(-1, 1, (1, C, H, W)).astype(np.float32))})
+    s, p, outs = run_batch(wl, [req], opt_flags=B.OPT_NO_REUSE)
+    assert {p.plan.group_form(i) for i in range(s.graph.num_groups()) if s.graph.group_info(i)["kind"] == "conv"} == {"rows"}
+    errs = lockstep(wl, s, p, outs, 0, BF16_TOL)
+    assert max(errs.values()) <= BF16_TOL, errs
+
+
 @pytest.mark.parametrize("cin", [64, 192, 256, 320, 512])
 def test_conv_forms_add_up_in_the_same_order(cin):
     # kernel rows, then 64-channel chunks, then columns: halo patches (chunks resident up to 256 channels and streamed beyond), row tiles

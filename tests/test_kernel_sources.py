@@ -70,3 +70,13 @@ def test_a_run_starts_behind_everything_before_it():
     for name, kernel in (("kernels_rows.cuh", "chain_elementwise"), ("kernels_compact.cuh", "nonzero_mask"), ("kernels_compact.cuh", "nonzero_write")):
         body = re.search(r"\b%s\(.*?ptx::pdl_wait\(\);" % kernel, sources[name], re.S).group(0)
         assert not re.search(r"->|= ?\*|reinterpret_cast", body), (kernel, body)
+
+
+def test_row_convolution_hands_tiles_over_between_its_issuers():
+    # two warps issue alternate tiles out of one ring.  A warp that does not issue a tile must not wait on its stages: the other's
+    # commits let the ring go on whether or not it has looked.  It waits for its turn, which passes behind the tile's last stage
+    text = dict(_sources())["conv3x3_tcgen05.cuh"]
+    role = text[text.index("warp == 3 || warp == 12"):text.index("warp == 2", text.index("warp == 3 || warp == 12"))]
+    assert re.search(r"if \(acc != me\) \{ n \+= kstages; continue; \}\s*if \(j >= 1\) ptx::mbar_wait_warp\(&turn\[me\]", role)
+    assert re.search(r"mbar_wait_lanes\(&full\[s\][^;]*;\s*if \(ks \+ 1 == kstages\) \{\s*__syncwarp\(\);\s*if \(lane == 0\) ptx::mbar_arrive\(&turn\[me \^ 1\]\);", role)
+    assert role.count("mbar_wait_lanes(&full") == 1 and "mbar_wait_warp(&full" not in role
