@@ -1841,19 +1841,23 @@ struct Builder : BuildState {
       const int padded_w = ((cp.Wo + 127) / 128) * 128;
       const bool rows = ks == 3 && G.stride == 1 && G.pad == 1 && (strip ? strip_width(cp.Wo) : cp.Wo >= 96 && padded_w * 4 <= cp.Wo * 5);
       if (rows) { cp.TW = 128; cp.TH = 1; }
-      // other 3x3 / stride 1 / pad 1 layers of 128-column tiles: the patches of the halo kernel.  A tile
-      // takes 0.62 of the implicit GEMM's time where the main loop is long, so up to 1.4 times as many of them pay
+      // other 3x3 / stride 1 / pad 1 layers of 128-column tiles: the patches of the halo kernel, of the shape that gives the fewest,
+      // then the one that reads the fewest pixels.  A patch takes 0.80 of the implicit GEMM's tile, so they pay where their
+      // launch has up to 4/3 as many waves.  Measured, patches over implicit GEMM in time, 64 / 128 / 512 channels to 128: as many
+      // waves 0.80 to 0.92; 5 for 4 0.93 / 0.95 / 0.96; 4 for 3 0.95 / 0.97 / 1.01; 7 for 5 0.98 / 1.00 / 0.99; 3 for 2 0.98 / 1.03 / 1.07;
+      // 2 for 1 1.10 / 1.14 / 1.33.  Where the number of images is known on the device only, tiles stand for waves.
       bool halo = false;
       if (ks == 3 && G.stride == 1 && G.pad == 1 && bn == 128 && !rows) {
-        const long long igemm_tiles = best / 128;
         long long fewest = -1;
-        int tw_best = 0, th_best = 0;
+        int tw_best = 0, th_best = 0, read_best = 0;
         for (int tw = 1; tw + 2 <= k::HALO_MAX_ROWS && tw <= cp.Wo; ++tw) {
-          const int th = std::min(k::HALO_MAX_ROWS / (tw + 2), cp.Ho);
+          const int th = std::min(k::HALO_MAX_ROWS / (tw + 2), cp.Ho), read = (tw + 2) * th;
           const long long n = static_cast<long long>((cp.Wo + tw - 1) / tw) * ((cp.Ho + th - 1) / th);
-          if (fewest < 0 || n <= fewest) { fewest = n; tw_best = tw; th_best = th; }
+          if (fewest < 0 || n < fewest || (n == fewest && read < read_best)) { fewest = n; tw_best = tw; th_best = th; read_best = read; }
         }
-        halo = fewest * 5 <= igemm_tiles * 7;
+        const long long per_tile = rt ? 0 : static_cast<long long>(cp.n_img) * (Cout / bn);
+        auto waves = [&](long long tiles) { return rt ? tiles : (tiles * per_tile + p.sm_count - 1) / p.sm_count; };
+        halo = waves(fewest) * 3 <= waves(best / 128) * 4;
         if (halo) { cp.TW = tw_best; cp.TH = th_best; }
       }
       if (cp.TW * G.stride > 256 || cp.TH * G.stride > 256) return fail(E_UNSUPPORTED_OP, "convolution stride too large for the TMA box");

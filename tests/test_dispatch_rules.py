@@ -48,6 +48,19 @@ def test_gemm_forms_by_epilogue(K, N, M, tail, form):
     assert B.Graph(ir, 0).bind_dims(["M"], [[M]]).plan().group_form(0) == form
 
 
+@pytest.mark.parametrize("N,H,W,cout,form", [
+    # halo patches for up to 4/3 of the implicit GEMM's waves: as many (whatever the tiles), 5 for 4, 4 for 3; not 7 for 5, 3 for 2, 2 for 1
+    (32, 56, 56, 128, "halo"), (74, 16, 8, 128, "halo"), (20, 58, 64, 128, "halo"), (18, 64, 48, 128, "halo"), (25, 58, 64, 128, "implicit GEMM"),
+    (10, 58, 64, 128, "implicit GEMM"), (6, 64, 48, 128, "implicit GEMM"), (4, 64, 48, 128, "halo"), (4, 64, 48, 256, "halo"), (5, 64, 48, 256, "implicit GEMM"),
+    # row tiles from four fifths of 128 pixels on; tiles of 64 columns stay
+    (1, 20, 102, 128, "halo"), (1, 20, 103, 128, "rows"), (1, 20, 102, 192, "implicit GEMM")])
+def test_convolution_forms(N, H, W, cout, form):
+    ir = f"input x bf16 [{N},128,{H},{W}]\nconst w bf16 [{cout},128,3,3]\nnode Conv x w -> y {{kernel=3 stride=1 pad=1}}\noutput y\n"
+    g = B.Graph(ir, 0)
+    conv = [g.group_info(i)["kind"] for i in range(g.num_groups())].index("conv")
+    assert g.bind_dims([], [[]]).plan().group_form(conv) == form
+
+
 def test_projection_blocks_copy_no_samples():
     # the executed and the skipped branch of a projection block are convolutions: both read the Switch input and write the Combine
     # output through the id lists, so the groups around them launch nothing; with copies asked for, they do
