@@ -231,7 +231,9 @@ sod2_status sod2_plan_io_counts(const sod2_plan_t* p, int* inputs, int* outputs)
  * reads), else 0. */
 sod2_status sod2_plan_group_on_side_stream(const sod2_plan_t* p, int group, int* on_side);
 /* Which form of its kernel a group takes for the bound shapes: GEMM "tile 64", "tile 128", "tile 256", "pair", "cluster 2",
- * "cluster 4" or "cluster 8"; attention "tcgen05" or "mma.sync"; "mixed" where launches of one group differ, empty otherwise. */
+ * "cluster 4" or "cluster 8"; attention "tcgen05" or "mma.sync"; convolution "strip", "rows", "halo" or "implicit GEMM";
+ * LayerNorm "in the selection" where the token selection before it writes its rows; "mixed" where launches of one group
+ * differ, empty otherwise. */
 sod2_status sod2_plan_group_form(const sod2_plan_t* p, int group, char* buf, size_t len);
 /* True shape of an output after a run (execution-determined extents are read back from the device;
  * synchronises cuda_stream). */

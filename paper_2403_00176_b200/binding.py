@@ -394,7 +394,7 @@ class Plan(_Handle):
         return bool(v.value)
 
     def group_form(self, group: int) -> str:
-        """Form of its kernel that a GEMM, attention or convolution group takes for the bound shapes."""
+        """Form of its kernel that a group takes for the bound shapes, as listed at sod2_plan_group_form."""
         t = C.create_string_buffer(32)
         _check(lib.sod2_plan_group_form(self.h, group, t, 32), self.h)
         return t.value.decode()

@@ -323,7 +323,7 @@ struct Plan {
   bool sm_count_known = false;
   bool uses_header = true;                // false: no kernel of the plan writes the status word, a ticket or a count: nothing to clear or read
   std::vector<double> group_flops, group_bytes;   // algorithmic cost per group for the bound shapes
-  std::vector<const char*> group_form;            // kernel form a GEMM, attention or convolution group's launches take ("mixed": several), or null
+  std::vector<const char*> group_form;            // kernel form a group's launches take (sod2_plan_group_form) ("mixed": several), or null
   // Runs of consecutive GEMM groups that execute as one persistent kernel (gemm_chain_tcgen05.cuh): decided after
   // view resolution and before liveness, because the members run concurrently: everything a member reads stays
   // live, and everything a member writes is live, over the whole run.

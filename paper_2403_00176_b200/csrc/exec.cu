@@ -1426,7 +1426,10 @@ struct Builder : BuildState {
         }
         return cudaGetLastError();
       });
-      if (L) p.launches.back()->share = {{gi, 0.8}, {gi + 1, 0.2}};     // about the bytes of the two
+      if (L) {
+        p.launches.back()->share = {{gi, 0.8}, {gi + 1, 0.2}};     // about the bytes of the two
+        form(gi + 1, "in the selection");
+      }
     }
     return OK;
   }

@@ -168,7 +168,13 @@ def test_topk_keep_with_the_layernorm_behind_it(D, H):
     rng = np.random.default_rng(67)
     name, sym = wl.ir.split("input ")[1].split()[0], wl.sym_names[0]
     reqs = [Request({sym: n}, {name: bf16_round((rng.standard_normal((1, n, D)) * rng.uniform(0.5, 2.0, (1, n, 1)) + rng.standard_normal((1, n, 1))).astype(np.float32))}) for n in lens]
-    _check_topk_lockstep(wl, reqs, 2)
+    s, p, outs = _check_topk_lockstep(wl, reqs, 2)
+    kinds = [s.graph.group_info(i)["kind"] for i in range(s.graph.num_groups())]
+    assert p.plan.group_form(kinds.index("topk_keep") + 1) == ("in the selection" if D <= 512 else "")
+    # with the arena's space reused, which the launch's reads and writes must allow
+    _, _, reused = run_batch(wl, reqs)
+    for a, b in zip(outs, reused):
+        assert all(np.array_equal(a[n], b[n]) for n in a)
 
 
 @pytest.mark.parametrize("K,N,M,act,residual", [(768, 768, 7169, None, True), (768, 2312, 4224, "Gelu", False), (3072, 768, 4100, "Relu", True), (3072, 776, 11009, None, False), (768, 392, 12700, None, True)])

@@ -2,6 +2,7 @@
 the exhaustive optimum on small random graphs (the paper reports 1.05x of optimal for its plan)."""
 import itertools
 import random
+import re
 
 import numpy as np
 import pytest
@@ -55,6 +56,24 @@ def test_arena_invariants(mk):
     p2 = g2.bind_dims(wl.sym_names, [[r.syms[s] for s in wl.sym_names] for r in wl.batch(0)]).plan()
     _, mem2 = _check_invariants(p2, wl.ir)
     assert mem2["arena_bytes"] >= mem2["sum_bytes"]
+
+
+@pytest.mark.parametrize("D,together", [(64, True), (512, True), (576, False)])
+def test_a_selection_and_the_layernorm_in_its_launch_live_together(D, together):
+    # one launch selects the kept rows and writes them normalised (up to 512 columns): what it reads stays until the LayerNorm's
+    # step, and the normalised rows are there from the selection's step on; wider rows are normalised by a launch of their own
+    wl = WL.cfg3(layers=3, D=D, H=D // 64, F=2 * D)
+    g = B.Graph(wl.ir)
+    p = g.bind_dims(wl.sym_names, [[40], [7], [300]]).plan()
+    kinds = [g.group_info(i)["kind"] for i in range(g.num_groups())]
+    steps = [i for i, k in enumerate(kinds) if k == "topk_keep"][:-1]        # the last one's rows leave as they are
+    assert len(steps) == 2 and all(kinds[i + 1] == "layernorm" for i in steps)
+    slots, _ = _check_invariants(p, wl.ir)
+    for l, i in enumerate(steps):
+        assert p.group_form(i + 1) == ("in the selection" if together else "")
+        normed = re.search(rf"node LayerNormalization keep{l} \S+ \S+ -> (\S+)", wl.ir).group(1)
+        assert slots[f"y{l}"]["last_use_step"] == (i + 1 if together else i)
+        assert slots[normed]["def_step"] == (i if together else i + 1)
 
 
 def _random_chain_graph(rnd, n_ops):
