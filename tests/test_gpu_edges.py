@@ -80,16 +80,22 @@ def test_conv_strips_segments_and_ring(shapes):
         assert all(np.array_equal(a[n], b[n]) for n in a)
 
 
-@pytest.mark.parametrize("C,shapes", [(128, [(14, 14), (28, 28), (56, 56), (5, 29), (31, 30), (1, 1)]), (256, [(7, 7), (17, 43), (33, 64)]), (384, [(2, 15)])])
+@pytest.mark.parametrize("C,shapes", [(128, [(14, 14), (28, 28), (56, 56), (5, 29), (31, 30), (1, 1)]), (256, [(7, 7), (17, 43), (33, 64)]), (384, [(2, 15)]),
+                                      (384, [(130, 98)]), (128, [(2400, 14)])])
 def test_conv_halo_patches(C, shapes):
-    # patches that fill their 128 rows and that do not, lines of the widest pitch (29 pixels), images smaller than a patch and a
-    # pixel larger, two and three channel tiles, tiles in a CTA's second round
+    # patches that fill their 128 rows and that do not, images smaller than a patch and a pixel larger, lines of a whole tile, two and
+    # three channel tiles; and launches in which CTAs take three tiles (accumulators, bias and residual buffers, and the ring from
+    # tile to tile)
     wl = WL.cfg4(blocks=2, C=C)
     rng = np.random.default_rng(61)
     reqs = [Request({"H": h, "W": w}, {"x": bf16_round(rng.uniform(-1, 1, (1, C, h, w)).astype(np.float32))}) for h, w in shapes]
     s, p, outs = run_batch(wl, reqs, opt_flags=B.OPT_NO_REUSE)
     forms = {p.plan.group_form(i) for i in range(s.graph.num_groups()) if s.graph.group_info(i)["kind"] == "conv"}
     assert forms == {"halo"}, forms
+    if shapes[0][0] > 100:
+        (h, w), = shapes
+        patches = min(-(-w // tw) * -(-h // min(128 // (tw + 2), h)) for tw in range(1, min(w, 126) + 1))
+        assert patches * (C // 128) > 2 * torch.cuda.get_device_properties(0).multi_processor_count
     for r, req in enumerate(reqs):
         errs = lockstep(wl, s, p, outs, r, BF16_TOL)
         assert max(errs.values()) <= BF16_TOL, (req.syms, errs)
