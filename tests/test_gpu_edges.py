@@ -143,6 +143,64 @@ def test_conv_forms_add_up_in_the_same_order(cin):
             assert O.rel_err(outs[0], O.run(ir, consts, {"x": pixels})["y"]) <= BF16_TOL
 
 
+@pytest.mark.parametrize("cin,cout,side,kernel,form", [(64, 64, (20, 70), 3, "strip"), (64, 128, (14, 14), 3, "halo"), (128, 128, (20, 110), 3, "rows"),
+                                                       (64, 192, (9, 11), 3, "implicit GEMM"), (128, 128, (9, 11), 1, "implicit GEMM")])
+def test_skipped_samples_through_a_convolution(cin, cout, side, kernel, form):
+    # a block whose skipped samples go through a convolution with a ReLU, in every form that reads and writes through the skipped ids, and an
+    # identity block behind it: against the oracle, against whole-sample copies, without reuse, and with the counts read back
+    n, (h, w) = 7, side
+    lines, consts, rng = [f"input x bf16 [{n},64,{h},{w}]", "fconst zero f32 [] = 0.0"], {}, np.random.default_rng(79)
+
+    def const(name, shape, scale, at=0.0):
+        lines.append(f"const {name} bf16 [{','.join(map(str, shape))}]")
+        consts[name] = bf16_round((rng.standard_normal(shape) * scale + at).astype(np.float32))
+
+    const("w", (cin, 64, 1, 1), 1 / 8)
+    lines += ["node Conv x w -> stem {kernel=1 stride=1 pad=0}"]
+    src, c = "stem", cin
+    for b in range(2):
+        const(f"gw{b}", (c, 1), 1.0)
+        const(f"gb{b}", (1,), 0.0)
+        const(f"w{b}", (cout, c, 3, 3), (2 / (9 * c)) ** 0.5)
+        const(f"v{b}", (cout, cout, 3, 3), (2 / (9 * cout)) ** 0.5)
+        lines += [f"iconst s{b} i64 [2] = {n} {c}", f"node GlobalAveragePool {src} -> p{b}", f"node Reshape p{b} s{b} -> r{b}", f"node MatMul r{b} gw{b} -> m{b}",
+                  f"node Add m{b} gb{b} -> z{b}", f"node Greater z{b} zero -> gate{b}", f"node Switch {src} gate{b} -> e{b} k{b}",
+                  f"node Conv e{b} w{b} -> c{b} {{kernel=3 stride=1 pad=1}}", f"node Relu c{b} -> d{b}", f"node Conv d{b} v{b} -> f{b} {{kernel=3 stride=1 pad=1}}",
+                  f"node Relu f{b} -> y{b}"]
+        skipped = f"k{b}"
+        if b == 0:
+            const("u", (cout, c, kernel, kernel), (2 / (kernel * kernel * c)) ** 0.5)
+            const("ub", (cout,), 0.1)
+            lines += [f"node Conv k0 u ub -> q {{kernel={kernel} stride=1 pad={kernel // 2}}}", "node Relu q -> t"]
+            skipped = "t"
+        lines.append(f"node Combine y{b} {skipped} gate{b} -> blk{b}")
+        src, c = f"blk{b}", cout
+    ir = "\n".join(lines + [f"node GlobalAveragePool {src} -> gap", "output gap", "output gate0", "output gate1"]) + "\n"
+    ir = "\n".join(sorted(ir.splitlines(), key=lambda l: {"node": 1, "output": 2}.get(l.split()[0], 0))) + "\n"
+    x = rng.standard_normal((n, 64, h, w)) + rng.standard_normal((n, 64, 1, 1))
+    wl = WL.Workload("skipped_convolution", "bf16", ir, consts, [], ["gap", "gate0", "gate1"], {})
+    # the gates of both blocks near the middle of their samples' logits, by the oracle
+    req = Request({}, {"x": bf16_round(x.astype(np.float32))})
+    for b in range(2):
+        z = np.sort(O.run(ir, consts, req.inputs)[f"z{b}"].reshape(-1))
+        consts[f"gb{b}"] = bf16_round(np.array([-(z[3] + z[4]) / 2], np.float32))
+    runs = {}
+    for flags in (B.OPT_NO_REUSE, 0, B.OPT_COPY_REGROUP):
+        s, p, outs = run_batch(wl, [req], opt_flags=flags)
+        runs[flags] = outs[0]
+        if flags == B.OPT_NO_REUSE:
+            errs = lockstep(wl, s, p, outs, 0, BF16_TOL)
+            assert {"blk0", "blk1"} <= set(errs) and max(v for v in errs.values()) <= BF16_TOL, errs
+        if not flags & B.OPT_COPY_REGROUP:
+            forms = {p.plan.group_form(i) for i in range(s.graph.num_groups()) if s.graph.group_info(i)["kind"] == "conv"}
+            assert forms - {"implicit GEMM"} == ({form} if kernel == 3 else {"halo"}) - {"implicit GEMM"}     # (the first is 1x1)
+            p.run_exact()
+            assert all(np.array_equal(a, runs[flags][name]) for name, a in p.outputs()[0].items())
+    assert all(0 < runs[0][f"gate{b}"].sum() < n for b in range(2))
+    for flags in (0, B.OPT_COPY_REGROUP):
+        assert all(np.array_equal(runs[flags][name], runs[B.OPT_NO_REUSE][name]) for name in runs[0]), flags
+
+
 @pytest.mark.parametrize("lens", [[1], [33, 64], [129, 640], list(range(1, 129, 3)) + [129, 191, 192, 193, 255, 256, 257, 300, 383, 385, 511, 512, 513, 577] + [200] * 8,
                                   list(range(2, 130, 3)) + [128, 129, 191, 192, 193, 255, 256, 257, 300, 383, 385, 511, 512, 513, 577] + [200] * 7])
 def test_attention_blocks_items_and_tables(lens):
