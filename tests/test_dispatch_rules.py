@@ -39,7 +39,8 @@ def test_attention_forms():
     (768, 3072, 1000, "gelu", "tile 128"), (768, 3072, 1806, "gelu", "tile 128"), (768, 3072, 2900, "gelu", "tile 256"), (768, 3072, 12700, "gelu", "pair"),
     (384, 1536, 3600, "gelu", "tile 128"), (384, 1536, 6000, "gelu", "tile 256"),
     # a residual and fewer than 24 chunks; 24 and more by the main loop
-    (768, 768, 3600, "residual", "tile 128"), (1472, 768, 2400, "residual", "tile 128"), (1536, 768, 2400, "residual", "tile 128"), (768, 768, 7169, "residual", "pair"),
+    (768, 768, 3600, "residual", "tile 128"), (1472, 768, 2400, "residual", "tile 128"), (1536, 768, 2400, "residual", "tile 128"), (1472, 1920, 3650, "residual", "tile 128"), (1536, 1920, 3650, "residual", "tile 256"),
+    (768, 768, 7169, "residual", "pair"),
     # up to 8 chunks whatever the tail
     (512, 1152, 4500, "", "tile 128"), (576, 1152, 4500, "", "tile 256")])
 def test_gemm_forms_by_epilogue(K, N, M, tail, form):
