@@ -281,7 +281,9 @@ sod2_status sod2_selftest_bounded_wait(void* dev_status_word, void* cuda_stream)
  * per CTA (pair = 0: tcgen05.mma.cta_group::1, 128 x n_cols x 16, both CTAs of every cluster at once) or one per CTA
  * pair (pair = 1: cta_group::2, 256 x n_cols x 16) issues `iters` bf16 MMAs on fixed shared-memory operands, in
  * stages of `per_stage` instructions.  handshake: 0 = MMAs only, 1 = a tcgen05.commit after every stage, 2 = the
- * full / empty barrier handshake of the GEMM main loops after every stage (all waits satisfied at once).
+ * full / empty barrier handshake of the GEMM main loops after every stage (all waits satisfied at once), 3 = what an
+ * issuer of the kernels does for a stage: a satisfied wait of a whole warp, whose leading lane issues and commits behind
+ * predicates (per_stage 4, 8 or 12).
  * *cycles_per_mma (host) = SM cycles of the first issuing thread / iters.  n_cols in {64, 128, 256}; per_stage in
  * 1..64 and dividing iters; iters <= 65536.  Allocates and frees one small device buffer; synchronises cuda_stream.
  * Every wait in the kernel is bounded.  Errors: SOD2_E_INVALID_ARG, SOD2_E_CUDA, SOD2_E_TIMEOUT (a wait ran out);

@@ -141,7 +141,8 @@ def sod2_selftest_bounded_wait(dev_status_word: int, stream: int) -> None:
 
 def sod2_selftest_mma_rate(pair: bool, n_cols: int, per_stage: int, handshake: int, stream: int, iters: int = 4096, clusters: int = 74) -> float:
     """SM cycles per tcgen05.mma (128 x n_cols x 16 on one CTA, 256 x n_cols x 16 on a CTA pair) issued in stages of
-    `per_stage`; handshake 0 = MMAs only, 1 = commit per stage, 2 = full / empty barrier handshake per stage."""
+    `per_stage`; handshake 0 = MMAs only, 1 = commit per stage, 2 = full / empty barrier handshake per stage,
+    3 = a satisfied wait of a whole warp and a commit per stage, its leading lane issuing behind predicates."""
     out = C.c_double()
     _check(lib.sod2_selftest_mma_rate(int(bool(pair)), n_cols, per_stage, handshake, iters, clusters, C.c_void_p(stream), C.byref(out)))
     return out.value

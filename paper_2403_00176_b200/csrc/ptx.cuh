@@ -186,10 +186,10 @@ __device__ __forceinline__ bool elect_one() {
 // The lane that issues for its warp, elected once per role.  What it issues (MMAs, commits, TMA loads) is predicated and not
 // branched on: a branch on elect_one() around a stage's instructions, and the __syncwarp behind it, cost the issuing warp 130 to
 // 190 cycles per stage beside the pipe.  Measured on B200 (cycles per MMA with a satisfied wait and a commit per stage, branch ->
-// predicate; the pipe takes 48 at N = 64, 64 at 128): N = 64 in stages of 4 / 8 / 12 MMAs 93 / 72 / 63 -> 61 / 51 / 52, N = 128
-// 97 / 82 / 75 -> 64 / 64 / 64; from N = 192 on the pipe hides either.  A warp whose lanes have seen a phase end at different
-// tests may run a stage's instructions in parts: the leader's are issued once, behind the leader's own test, and its commit
-// waits for the other lanes (mbar_wait_lanes).
+// predicate with the __syncwarp before the commit; the pipe takes 48 at N = 64, 64 at 128): N = 64 in stages of 4 / 8 / 12 MMAs 93 / 72 /
+// 63 -> 69 / 59 / 55, N = 128 97 / 82 / 75 -> 67 / 66 / 65; from N = 192 on the pipe hides either (sod2_selftest_mma_rate, handshake 3).
+// A warp whose lanes have seen a phase end at different tests may run a stage's instructions in parts: the leader's are
+// issued once, behind the leader's own test, and its commit waits for the other lanes (mbar_wait_lanes).
 struct Leader { uint32_t on; };
 __device__ __forceinline__ Leader elect_leader() { return Leader{elect_one() ? 1u : 0u}; }
 __device__ __forceinline__ void mbar_expect_tx(Leader l, uint64_t* bar, uint32_t bytes) {

@@ -1,11 +1,12 @@
 // Self-test / measurement entry point: the issue rate of tcgen05.mma, for one CTA and for a CTA pair.
 // One thread per CTA (or per pair) issues `iters` bf16 MMAs of shape 128 x N x 16 (256 x N x 16 for a pair) on
-// operands that sit in shared memory for the whole run; nothing is loaded, the data is irrelevant.  Three issue
+// operands that sit in shared memory for the whole run; nothing is loaded, the data is irrelevant.  Issue
 // patterns: MMAs only; a tcgen05.commit after every stage of `per_stage` instructions; the full / empty barrier
 // handshake of the GEMM main loops (the issuing thread waits for `full`, commits to `empty`, a second thread waits
 // for `empty` and arrives on `full`), whose waits are always satisfied at once.  The result says how much of the
 // issuing thread's own work the tensor pipe overlaps: none of it (a stage costs its MMA cycles plus the wait, the
-// fence and the commit), identically for both forms.  The paper has no counterpart of this call: it documents the
+// fence and the commit), identically for both forms.  A fourth pattern is what an issuer of the kernels does: a whole
+// warp waits (for a phase that has ended), its leading lane issues a stage behind predicates (ptx::Leader) and commits it.  The paper has no counterpart of this call: it documents the
 // machine facts the kernels were shaped by, and lets a test pin them.
 // Every wait is bounded; a wait that runs out makes the call return SOD2_E_TIMEOUT.
 #include <cuda_runtime.h>
@@ -23,7 +24,8 @@ constexpr int MR_SLOTS = 4;
 constexpr int MR_SLOT_BYTES = 49152;       // A: 128 rows x 128 B, B: up to 256 rows x 128 B
 constexpr int MR_SMEM = MR_SLOTS * MR_SLOT_BYTES + 1024 + 256;
 
-template <int PAIR, int N, int HS>
+// WS: instructions per stage where a whole warp issues (HS == 3), straight-line as in the kernels.
+template <int PAIR, int N, int HS, int WS>
 __global__ void __launch_bounds__(128, 1) mma_rate_kernel(long long* out, int iters, int per_stage) {
   extern __shared__ uint8_t raw[];
   uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(raw) + 1023) & ~uintptr_t(1023));
@@ -47,8 +49,30 @@ __global__ void __launch_bounds__(128, 1) mma_rate_kernel(long long* out, int it
   k::cluster_sync_all();
   ptx::tc_fence_after();
   const uint32_t tmem = *slot;
-  const bool issuer = threadIdx.x == 0 && (!PAIR || rank == 0);
-  if (issuer) {
+  const bool issuer = threadIdx.x < (HS == 3 ? 32 : 1) && (!PAIR || rank == 0);
+  if (HS == 3 && issuer) {
+    constexpr uint32_t idesc = ptx::idesc_bf16(PAIR ? 256 : 128, N);
+    const ptx::Leader one = ptx::elect_leader();
+    const uint64_t ad0 = ptx::smem_desc_sw128(ptx::smem_u32(base)), bd0 = ptx::smem_desc_sw128(ptx::smem_u32(base + 16384));
+    uint32_t sl = 0;
+    const auto mma = [&](uint64_t ad, uint64_t bd) {
+      if (PAIR) k::mma_bf16_pair(one, tmem, ad, bd, idesc, 1); else ptx::mma_bf16(one, tmem, ad, bd, idesc, 1);
+    };
+    const long long t0 = clock64();
+    for (int it = 0; it < iters; it += WS) {
+      ptx::mbar_wait_lanes(bar + 2 + sl, 1, dead);       // nobody arrives here: the phase before the first has ended
+      ptx::tc_fence_after();
+      const uint64_t ad = ad0 + sl * (MR_SLOT_BYTES >> 4), bd = bd0 + sl * (MR_SLOT_BYTES >> 4);
+#pragma unroll
+      for (int g = 0; g < WS; ++g) mma(ad + 2 * (g & 3), bd + 2 * (g & 3));
+      __syncwarp();
+      if (PAIR) k::mma_commit_pair(one, bar + 6 + sl); else ptx::mma_commit(one, bar + 6 + sl);
+      if (++sl == MR_SLOTS) sl = 0;
+    }
+    if (PAIR) k::mma_commit_pair(one, bar); else ptx::mma_commit(one, bar);
+    ptx::mbar_wait_warp(bar, 0, dead);
+    if (threadIdx.x == 0) out[blockIdx.x * 2] = clock64() - t0;
+  } else if (issuer) {
     constexpr uint32_t idesc = ptx::idesc_bf16(PAIR ? 256 : 128, N);
     const uint64_t ad0 = ptx::smem_desc_sw128(ptx::smem_u32(base)), bd0 = ptx::smem_desc_sw128(ptx::smem_u32(base + 16384));
     int sl = 0;
@@ -93,9 +117,9 @@ __global__ void __launch_bounds__(128, 1) mma_rate_kernel(long long* out, int it
   if (threadIdx.x < 32) { if (PAIR) k::tmem_dealloc_pair(tmem, 512); else ptx::tmem_dealloc(tmem, 512); }
 }
 
-template <int PAIR, int N, int HS>
+template <int PAIR, int N, int HS, int WS = 4>
 cudaError_t launch_rate(long long* out, int iters, int per_stage, int clusters, cudaStream_t st) {
-  auto kern = mma_rate_kernel<PAIR, N, HS>;
+  auto kern = mma_rate_kernel<PAIR, N, HS, WS>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, MR_SMEM);
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
@@ -116,7 +140,11 @@ cudaError_t launch_rate_hs(int hs, long long* out, int iters, int per_stage, int
   switch (hs) {
     case 0: return launch_rate<PAIR, N, 0>(out, iters, per_stage, clusters, st);
     case 1: return launch_rate<PAIR, N, 1>(out, iters, per_stage, clusters, st);
-    default: return launch_rate<PAIR, N, 2>(out, iters, per_stage, clusters, st);
+    case 2: return launch_rate<PAIR, N, 2>(out, iters, per_stage, clusters, st);
+    default:
+      if (per_stage == 4) return launch_rate<PAIR, N, 3, 4>(out, iters, per_stage, clusters, st);
+      if (per_stage == 8) return launch_rate<PAIR, N, 3, 8>(out, iters, per_stage, clusters, st);
+      return launch_rate<PAIR, N, 3, 12>(out, iters, per_stage, clusters, st);
   }
 }
 
@@ -129,9 +157,9 @@ extern "C" sod2_status sod2_selftest_mma_rate(int pair, int n_cols, int per_stag
   auto fail = [&](sod2_status s, const std::string& m) { set_thread_error(m); return s; };
   if (!cycles_per_mma) return fail(SOD2_E_INVALID_ARG, "sod2_selftest_mma_rate: null result pointer");
   if (n_cols != 64 && n_cols != 128 && n_cols != 256) return fail(SOD2_E_INVALID_ARG, "sod2_selftest_mma_rate: n_cols must be 64, 128 or 256");
-  if (per_stage < 1 || per_stage > 64 || iters < per_stage || iters > (1 << 16) || iters % per_stage || handshake < 0 || handshake > 2 ||
-      clusters < 1 || clusters > 74)
-    return fail(SOD2_E_INVALID_ARG, "sod2_selftest_mma_rate: per_stage in 1..64 dividing iters <= 65536, handshake in 0..2, clusters in 1..74");
+  if (per_stage < 1 || per_stage > 64 || iters < per_stage || iters > (1 << 16) || iters % per_stage || handshake < 0 || handshake > 3 ||
+      clusters < 1 || clusters > 74 || (handshake == 3 && per_stage != 4 && per_stage != 8 && per_stage != 12))
+    return fail(SOD2_E_INVALID_ARG, "sod2_selftest_mma_rate: per_stage in 1..64 (4, 8 or 12 with handshake 3) dividing iters <= 65536, handshake in 0..3, clusters in 1..74");
   cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
   long long* out = nullptr;
   const size_t bytes = static_cast<size_t>(2 * clusters) * 2 * sizeof(long long);

@@ -222,6 +222,18 @@ def test_attention_blocks_items_and_tables(lens):
         assert np.array_equal(a["y"], b["y"])
 
 
+def test_issue_behind_predicates_keeps_up_with_the_pipe():
+    # cycles per MMA where a warp waits, its leading lane issues a stage behind predicates and commits it, in stages of 4, 8 and 12: the
+    # tensor pipe's 64 at 128 columns and 128 at 256 within a tenth; at 64 columns 43 to 69, where the pipe's 48 do not hide all of the
+    # issuer's work.  One thread's handshake takes 95 to 162.  Printed with -s
+    st = torch.cuda.current_stream().cuda_stream
+    rate = {(pair, n, k): [B.sod2_selftest_mma_rate(pair, n, k, hs, st, iters=4032 if k == 12 else 4096) for hs in (2, 3)]
+            for pair in (False, True) for n in (64, 128, 256) for k in (4, 8, 12)}
+    print({key: [round(v, 1) for v in r] for key, r in rate.items()})
+    for (pair, n, k), (thread, warp) in rate.items():
+        assert warp <= {64: 74.0, 128: 72.0, 256: 133.0}[n] and warp < thread + 1.0
+
+
 @pytest.mark.parametrize("D,H", [(64, 1), (256, 4), (320, 5), (512, 8), (576, 9)])
 def test_topk_keep_with_the_layernorm_behind_it(D, H):
     # the kept rows of the first layer leave normalised for the second, in the launch that selects them: rows of one and two
