@@ -321,6 +321,9 @@ struct Plan {
   int gpu_launches = 0;
   int sm_count = 148;                     // persistent kernels launch one CTA per SM
   bool sm_count_known = false;
+  // whether the header is cleared by a kernel, which counts as a launch, or by a memset (a first kernel that is a plain launch,
+  // as the layout changes are, waits longer for a kernel's end: 110.1 against 109.2 us for one image)
+  bool clear_by_kernel = false;
   bool uses_header = true;                // false: no kernel of the plan writes the status word, a ticket or a count: nothing to clear or read
   std::vector<double> group_flops, group_bytes;   // algorithmic cost per group for the bound shapes
   std::vector<const char*> group_form;            // kernel form a group's launches take (sod2_plan_group_form) ("mixed": several), or null

@@ -2058,9 +2058,9 @@ struct Builder : BuildState {
           }
         }
         // accumulating in the convolution's epilogue costs about as much per byte as the pooling pass it
-        // replaces; what it saves is the pass's two launches, which only outweighs it on the smaller tensors.  The strip
-        // kernel's epilogue has the time (it waits 1500 cycles a row for the main loop): any size (32 x 64 x 112 x 112: 785 -> 757 us
-        // for the gated network)
+        // replaces; what it saves is the pass's two launches, which only outweighs it on the smaller tensors.  In the strip
+        // kernel, which has 64 columns to add up beside a main loop of 1360 cycles a row, it costs less than the pass (9 us a layer
+        // of 51 MB against a pass of 51 MB and two launches): any size (32 x 64 x 112 x 112: 785 -> 757 us for the gated network)
         if (writer >= 0) {
           const Group& Wg = c.groups[writer];
           const auto& wd = g.tensors[Wg.w].S.dims;
@@ -2405,6 +2405,8 @@ struct Builder : BuildState {
       if (!p.stage_of) cost(G);
     }
     if (p.build_state) *p.build_state = *this;
+    p.clear_by_kernel = p.launches.empty() || p.launches[0]->group < 0 || c.groups[p.launches[0]->group].kind != GKind::LAYOUT;
+    p.gpu_launches += p.uses_header && p.clear_by_kernel;
     if (p.front_reserve) {
       // staged plan: scratch and index lists at the fixed places behind the header that the first stage chose
       const size_t sc = (scratch_need + 255) & ~size_t(255), ax = (aux_need + 255) & ~size_t(255);
@@ -2773,17 +2775,15 @@ Status run_plan(Plan* p, const void* const* inputs, void* const* outputs, void* 
   }
   RunCtx x{inputs, outputs, static_cast<char*>(arena), static_cast<char*>(p->c->packed_ws), static_cast<cudaStream_t>(stream), p};
   if (p->uses_header && step_lo <= 0) {
-    // (layout changes are plain launches, which wait for a kernel's end longer than for a memset: 109.2 against 110.1 us)
-    const bool plain_first = !p->launches.empty() && p->launches[0]->group >= 0 && p->c->groups[p->launches[0]->group].kind == GKind::LAYOUT;
-    const cudaError_t e = plain_first ? cudaMemsetAsync(arena, 0, p->header_clear_bytes, x.stream)
-                                      : launch_pdl(clear_header, dim3(1), dim3(128), 0, x.stream, static_cast<uint4*>(arena), static_cast<int>(p->header_clear_bytes / 16));
+    const cudaError_t e = p->clear_by_kernel ? launch_pdl(clear_header, dim3(1), dim3(128), 0, x.stream, static_cast<uint4*>(arena), static_cast<int>(p->header_clear_bytes / 16))
+                                             : cudaMemsetAsync(arena, 0, p->header_clear_bytes, x.stream);
     if (e != cudaSuccess) { p->err = "cannot clear the status word"; return E_CUDA; }
   }
   if (!ensure_side_stream(p)) { p->err = "cannot create the second stream"; return E_CUDA; }
   const int n_groups = static_cast<int>(p->side_group.size());
   cudaStream_t side = static_cast<cudaStream_t>(p->side_stream);
   bool open_fork = false;
-  int64_t enqueued = 0;
+  int64_t enqueued = p->uses_header && p->clear_by_kernel && step_lo <= 0;
   for (size_t i = 0; i < p->launches.size(); ++i) {
     auto& L = p->launches[i];
     const int g = L->group;
