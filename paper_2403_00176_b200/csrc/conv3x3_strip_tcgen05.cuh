@@ -1,7 +1,7 @@
 // 3x3 / stride 1 / pad 1 convolution, 64 -> 64 channels (channels-last, bf16, tcgen05), in vertical strips.
 //
-// An MMA of N = 64 columns occupies the tensor pipe for about 72 cycles, one of N = 192 for 96: with one tap per
-// instruction a 64-channel layer cannot pass half of the pipe's rate.  Here an instruction carries the three dy taps of
+// An MMA of N = 64 columns occupies the tensor pipe for 48 cycles, one of N = 192 for 96: with one tap per
+// instruction a 64-channel layer cannot pass two thirds of the pipe's rate.  Here an instruction carries the three dy taps of
 // one dx: the operand B is [dy = 2 | dy = 1 | dy = 0] x 64 output channels, and the result is what input row i gives to
 // the output rows i - 1, i and i + 1, whose accumulators lie side by side in tensor memory (a ring of eight 64-column
 // blocks; where the three blocks wrap around its end the instruction is cut in two).  Tensor-core instructions are only
@@ -81,8 +81,10 @@ __device__ __forceinline__ void strip_hand_over(uint32_t tmem, int blk, int q, i
 
 // B.tx: {64, W, H, N}, box {64, 130, 1, 1};  tmW: k-chunk view {64, 64, 9} of the weights in (dy, dx, ci) order, box
 // {64, 64, 1};  B.to / B.tr: {64, W, H, N}, box {64, 128, 1, 1}.  B.tile_start as for the row-halo kernel.
-// GAP: p.gap_sum receives the channel sums (the code for it costs the kernel registers: one image of 227 x 341 111.2 -> 113.0 us with
-// it everywhere).  The additions fit under the main loop: the gated network of 32 images pools three tensors of 51 MB less, 785 -> 757 us.
+// GAP: p.gap_sum receives the channel sums.  The conversions to fp64 then bound the epilogue (a layer of 32 gated images of 112 x 112
+// takes 27 us with them and 18 without), but the pooling passes over three tensors of 51 MB that they replace take longer: the
+// gated network of 32 images 785 -> 757 us.  A template parameter because the code for them costs registers: one image of 227 x
+// 341 111.2 -> 113.0 us with it everywhere.
 template <int ACT, bool HASRES, bool GAP>
 __global__ void __launch_bounds__(STRIP_THREADS, 1)
 conv3x3_strip_bf16_tcgen05(const __grid_constant__ Conv3Batch B, const __grid_constant__ CUtensorMap tmW, ConvParams p) {
