@@ -217,33 +217,7 @@ conv3x3_halo_bf16_tcgen05(const __grid_constant__ CUtensorMap tmX, const __grid_
         float v[32];
         bias_act32<ACT>(v, r, bias_t + ps * 64 + half * 32);
         if constexpr (HASRES) ptx::mbar_wait_warp(&res_full[u & 1], (u >> 1) & 1, dead);
-        if (live) {
-          uint4 pk[4];
-          if constexpr (HASRES) {
-            uint4 rv[4];
-#pragma unroll
-            for (int g = 0; g < 4; ++g) rv[g] = *reinterpret_cast<const uint4*>(obase + (((half * 4 + g) ^ (row & 7)) << 4));
-#pragma unroll
-            for (int g = 0; g < 4; ++g) {
-              const __nv_bfloat162* h = reinterpret_cast<const __nv_bfloat162*>(&rv[g]);
-              __nv_bfloat162* oh = reinterpret_cast<__nv_bfloat162*>(&pk[g]);
-#pragma unroll
-              for (int i = 0; i < 4; ++i) {
-                const float2 f = __bfloat1622float2(h[i]);
-                oh[i] = __floats2bfloat162_rn(fmaxf(v[g * 8 + 2 * i] + f.x, relu2_floor), fmaxf(v[g * 8 + 2 * i + 1] + f.y, relu2_floor));
-              }
-            }
-          } else {
-#pragma unroll
-            for (int g = 0; g < 4; ++g) {
-              __nv_bfloat162* oh = reinterpret_cast<__nv_bfloat162*>(&pk[g]);
-#pragma unroll
-              for (int i = 0; i < 4; ++i) oh[i] = __floats2bfloat162_rn(v[g * 8 + 2 * i], v[g * 8 + 2 * i + 1]);
-            }
-          }
-#pragma unroll
-          for (int g = 0; g < 4; ++g) *reinterpret_cast<uint4*>(obase + (((half * 4 + g) ^ (row & 7)) << 4)) = pk[g];
-        }
+        if (live) conv_pixel_to_staging<HASRES>(v, obase, row, half, relu2_floor);
         ptx::fence_proxy_async();
         if (et == 0) bulk_wait_read0();              // the pass before has left its buffer
         conv_epi_bar();

@@ -309,32 +309,8 @@ conv3x3_strip_bf16_tcgen05(const __grid_constant__ Conv3Batch B, const __grid_co
       float v[32];
       bias_act32<ACT>(v, r, bias_s + half * 32);
       uint8_t* obase = out_stage + bsel * CONV_STAGE_OUT + row * 128;
-      uint4 rv[4];        // residual loads together, then the arithmetic, then the stores (never reordered by the compiler)
       ptx::mbar_wait_warp(&res_full[bsel], (j / NSB) & 1, dead);
-      uint4 pk[4];
-      if constexpr (HASRES) {
-#pragma unroll
-        for (int u = 0; u < 4; ++u) rv[u] = *reinterpret_cast<const uint4*>(obase + (((half * 4 + u) ^ (row & 7)) << 4));
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          const __nv_bfloat162* h = reinterpret_cast<const __nv_bfloat162*>(&rv[u]);
-          __nv_bfloat162* oh = reinterpret_cast<__nv_bfloat162*>(&pk[u]);
-#pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            const float2 f = __bfloat1622float2(h[i]);
-            oh[i] = __floats2bfloat162_rn(fmaxf(v[u * 8 + 2 * i] + f.x, relu2_floor), fmaxf(v[u * 8 + 2 * i + 1] + f.y, relu2_floor));
-          }
-        }
-      } else {
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          __nv_bfloat162* oh = reinterpret_cast<__nv_bfloat162*>(&pk[u]);
-#pragma unroll
-          for (int i = 0; i < 4; ++i) oh[i] = __floats2bfloat162_rn(v[u * 8 + 2 * i], v[u * 8 + 2 * i + 1]);
-        }
-      }
-#pragma unroll
-      for (int u = 0; u < 4; ++u) *reinterpret_cast<uint4*>(obase + (((half * 4 + u) ^ (row & 7)) << 4)) = pk[u];
+      conv_pixel_to_staging<HASRES>(v, obase, row, half, relu2_floor);
       if constexpr (GAP) {
         group_bar();                               // every row of the tile is in the staging buffer
         int img, trow, w0;

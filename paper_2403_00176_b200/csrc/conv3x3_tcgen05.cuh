@@ -279,33 +279,7 @@ conv3x3_rows_bf16_tcgen05(const __grid_constant__ Conv3Batch B, const __grid_con
         }
         ptx::mbar_wait_warp(&res_full[bsel], (u / NSB) & 1, dead);
         if (et == 0) { SOD2_TRACE(3, 410) }
-        if (live) {
-          uint4 pk[4];
-          if constexpr (HASRES) {
-            uint4 rv[4];
-#pragma unroll
-            for (int g = 0; g < 4; ++g) rv[g] = *reinterpret_cast<const uint4*>(obase + (((half * 4 + g) ^ (row & 7)) << 4));
-#pragma unroll
-            for (int g = 0; g < 4; ++g) {
-              const __nv_bfloat162* h = reinterpret_cast<const __nv_bfloat162*>(&rv[g]);
-              __nv_bfloat162* oh = reinterpret_cast<__nv_bfloat162*>(&pk[g]);
-#pragma unroll
-              for (int i = 0; i < 4; ++i) {
-                const float2 f = __bfloat1622float2(h[i]);
-                oh[i] = __floats2bfloat162_rn(fmaxf(v[g * 8 + 2 * i] + f.x, relu2_floor), fmaxf(v[g * 8 + 2 * i + 1] + f.y, relu2_floor));
-              }
-            }
-          } else {
-#pragma unroll
-            for (int g = 0; g < 4; ++g) {
-              __nv_bfloat162* oh = reinterpret_cast<__nv_bfloat162*>(&pk[g]);
-#pragma unroll
-              for (int i = 0; i < 4; ++i) oh[i] = __floats2bfloat162_rn(v[g * 8 + 2 * i], v[g * 8 + 2 * i + 1]);
-            }
-          }
-#pragma unroll
-          for (int g = 0; g < 4; ++g) *reinterpret_cast<uint4*>(obase + (((half * 4 + g) ^ (row & 7)) << 4)) = pk[g];
-        }
+        if (live) conv_pixel_to_staging<HASRES>(v, obase, row, half, relu2_floor);
         if (p.gap_sum) {
           conv_epi_bar();                               // every row of the tile is in the staging buffer
           if (live) {

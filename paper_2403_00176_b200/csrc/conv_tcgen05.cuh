@@ -67,6 +67,38 @@ __device__ __forceinline__ void tma_store_4d(const void* tmap, const void* src, 
 }
 __device__ __forceinline__ void conv_epi_bar() { asm volatile("bar.sync 1, 256;" ::: "memory"); }
 
+// 32 channels of a pixel (half 0 or 1 of a 64-channel pass) as bf16 into its row of a staging buffer, added to the residual that lies
+// there (then max with relu2_floor) where HASRES.  16-byte granules are XOR-ed with the row (128-byte swizzle).  The residual's loads
+// together, then the arithmetic, then the stores: the compiler never reorders them.
+template <bool HASRES>
+__device__ __forceinline__ void conv_pixel_to_staging(const float* v, uint8_t* obase, int row, int half, float relu2_floor) {
+  uint4 pk[4];
+  if constexpr (HASRES) {
+    uint4 rv[4];
+#pragma unroll
+    for (int g = 0; g < 4; ++g) rv[g] = *reinterpret_cast<const uint4*>(obase + (((half * 4 + g) ^ (row & 7)) << 4));
+#pragma unroll
+    for (int g = 0; g < 4; ++g) {
+      const __nv_bfloat162* h = reinterpret_cast<const __nv_bfloat162*>(&rv[g]);
+      __nv_bfloat162* oh = reinterpret_cast<__nv_bfloat162*>(&pk[g]);
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const float2 f = __bfloat1622float2(h[i]);
+        oh[i] = __floats2bfloat162_rn(fmaxf(v[g * 8 + 2 * i] + f.x, relu2_floor), fmaxf(v[g * 8 + 2 * i + 1] + f.y, relu2_floor));
+      }
+    }
+  } else {
+#pragma unroll
+    for (int g = 0; g < 4; ++g) {
+      __nv_bfloat162* oh = reinterpret_cast<__nv_bfloat162*>(&pk[g]);
+#pragma unroll
+      for (int i = 0; i < 4; ++i) oh[i] = __floats2bfloat162_rn(v[g * 8 + 2 * i], v[g * 8 + 2 * i + 1]);
+    }
+  }
+#pragma unroll
+  for (int g = 0; g < 4; ++g) *reinterpret_cast<uint4*>(obase + (((half * 4 + g) ^ (row & 7)) << 4)) = pk[g];
+}
+
 // Sum over the valid pixels of one staged [128 pixels x 64 channels] bf16 tile (128-byte rows, 16-byte
 // granules XOR-ed with the row), by the 256 epilogue threads, in fp64 (a bf16 value is exact in fp64; masked
 // pixels add +0.0).  valid(px) tells whether tile pixel px lies in the image.
@@ -297,32 +329,8 @@ conv_igemm_bf16_tcgen05(const __grid_constant__ CUtensorMap tmX, const __grid_co
         }
         float v[32];
         bias_act32<ACT>(v, r, bias_t + ps * 64 + half * 32);
-        uint4 pk[4];
-        if constexpr (HASRES) {
-          ptx::mbar_wait_warp(&res_full[u & 1], (u >> 1) & 1, dead);
-          uint4 rv[4];
-#pragma unroll
-          for (int g = 0; g < 4; ++g) rv[g] = *reinterpret_cast<const uint4*>(obase + (((half * 4 + g) ^ (row & 7)) << 4));
-#pragma unroll
-          for (int g = 0; g < 4; ++g) {
-            const __nv_bfloat162* h = reinterpret_cast<const __nv_bfloat162*>(&rv[g]);
-            __nv_bfloat162* oh = reinterpret_cast<__nv_bfloat162*>(&pk[g]);
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-              const float2 f = __bfloat1622float2(h[i]);
-              oh[i] = __floats2bfloat162_rn(fmaxf(v[g * 8 + 2 * i] + f.x, relu2_floor), fmaxf(v[g * 8 + 2 * i + 1] + f.y, relu2_floor));
-            }
-          }
-        } else {
-#pragma unroll
-          for (int g = 0; g < 4; ++g) {
-            __nv_bfloat162* oh = reinterpret_cast<__nv_bfloat162*>(&pk[g]);
-#pragma unroll
-            for (int i = 0; i < 4; ++i) oh[i] = __floats2bfloat162_rn(v[g * 8 + 2 * i], v[g * 8 + 2 * i + 1]);
-          }
-        }
-#pragma unroll
-        for (int g = 0; g < 4; ++g) *reinterpret_cast<uint4*>(obase + (((half * 4 + g) ^ (row & 7)) << 4)) = pk[g];
+        if constexpr (HASRES) ptx::mbar_wait_warp(&res_full[u & 1], (u >> 1) & 1, dead);
+        conv_pixel_to_staging<HASRES>(v, obase, row, half, relu2_floor);
         ptx::fence_proxy_async();
         if (et == 0) bulk_wait_read0();              // the pass before has left its buffer
         conv_epi_bar();
